@@ -18,6 +18,7 @@
 #include <cstddef>
 #include <cuda_runtime.h>
 
+#include "copy_rows.cuh"
 #include "dvm_generic.h"
 #include "f32_state.cuh"
 #include "pclb_internal.h"
@@ -173,25 +174,6 @@ __global__ void __launch_bounds__(kGenThreads)
   if (u_r) u_r[n] = (T)(m.ux * c + m.uy * s);
   if (u_t) u_t[n] = (T)(m.uy * c - m.ux * s);
   if (temp) temp[n] = (T)m.E;
-}
-
-template <class T>
-__global__ void __launch_bounds__(kGenThreads)
-    gen_pack_kernel(const T* __restrict__ f, T* __restrict__ out, const __grid_constant__ StepParams p) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  const int t = blockIdx.y, q = blockIdx.z;
-  if (r >= p.n_r) return;
-  out[((size_t)q * p.n_theta + t) * p.n_r + r] = f[(size_t)q * p.rows * p.pitch + (size_t)(t + kGhostRows) * p.pitch + r];
-}
-
-template <class T>
-__global__ void __launch_bounds__(kGenThreads)
-    gen_unpack_kernel(const T* __restrict__ in, T* __restrict__ f, const __grid_constant__ StepParams p,
-                      const __grid_constant__ DvmG d) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  const int t = blockIdx.y, q = blockIdx.z;
-  if (r >= p.n_r) return;
-  gen_store<T>(f, p, d, q, t, r, in[((size_t)q * p.n_theta + t) * p.n_r + r]);
 }
 
 // Radial ghost layers of wall `side` at row t: layer l sits at r = -1 - l
@@ -394,15 +376,12 @@ cudaError_t gen_launch_moments(const T* f, T* rho, T* ur, T* ut, T* temp, const 
 
 template <class T>
 cudaError_t gen_launch_pack(const T* f, T* out, const StepParams& p, const DvmG& d, cudaStream_t s) {
-  gen_pack_kernel<T><<<dim3((p.n_r + kGenThreads - 1) / kGenThreads, p.n_theta, d.q), kGenThreads, 0, s>>>(f, out, p);
-  return cudaGetLastError();
+  return launch_copy_rows<T, false>(f, out, d.q, p, RecvLabels{}, s);
 }
 
 template <class T>
 cudaError_t gen_launch_unpack(const T* in, T* f, const StepParams& p, const DvmG& d, cudaStream_t s) {
-  gen_unpack_kernel<T><<<dim3((p.n_r + kGenThreads - 1) / kGenThreads, p.n_theta, d.q), kGenThreads, 0, s>>>(
-      in, f, p, d);
-  return cudaGetLastError();
+  return launch_copy_rows<T, true>(in, f, d.q, p, recv_labels(d, d.q), s);
 }
 
 cudaError_t gen_launch_step_f64(const double* f, double* f_out, double* ghost, const StepParams& p, const DvmG& d,

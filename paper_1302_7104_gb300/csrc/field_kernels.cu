@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <float.h>
 
+#include "copy_rows.cuh"
 #include "device_common.cuh"
 #include "f32_eq2.cuh"
 #include "f32_state.cuh"
@@ -144,24 +145,6 @@ __global__ void moments_kernel(const T* __restrict__ f, T* rho, T* u_r, T* u_t, 
   if (temp) temp[n] = m.E;
 }
 
-template <class T>
-__global__ void pack_kernel(const T* __restrict__ f, T* __restrict__ out, const __grid_constant__ StepParams p) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  const int t = blockIdx.y, q = blockIdx.z;
-  if (r >= p.n_r) return;
-  out[((size_t)q * p.n_theta + t) * p.n_r + r] =
-      f[(size_t)q * p.rows * p.pitch + (size_t)(t + kGhostRows) * p.pitch + r];
-}
-
-template <class T>
-__global__ void unpack_kernel(const T* __restrict__ in, T* __restrict__ f, const __grid_constant__ StepParams p,
-                              const __grid_constant__ DvmConst<T> d) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  const int t = blockIdx.y, q = blockIdx.z;
-  if (r >= p.n_r) return;
-  store_with_ghosts<T>(f, p, d, q, t, r, in[((size_t)q * p.n_theta + t) * p.n_r + r]);
-}
-
 // Global integrals with weight r dr dtheta, in double.  Each block reduces a
 // fixed grid-stride subset in a fixed order, so results are reproducible.
 template <class T>
@@ -254,16 +237,12 @@ cudaError_t launch_moments(const T* f, T* rho, T* ur, T* ut, T* temp, const Step
 
 template <class T>
 cudaError_t launch_pack(const T* f, T* out, const StepParams& p, cudaStream_t s) {
-  dim3 grid((p.n_r + kRowThreads - 1) / kRowThreads, p.n_theta, kQ);
-  pack_kernel<T><<<grid, kRowThreads, 0, s>>>(f, out, p);
-  return cudaGetLastError();
+  return launch_copy_rows<T, false>(f, out, kQ, p, RecvLabels{}, s);
 }
 
 template <class T>
 cudaError_t launch_unpack(const T* in, T* f, const StepParams& p, const DvmConst<T>& d, cudaStream_t s) {
-  dim3 grid((p.n_r + kRowThreads - 1) / kRowThreads, p.n_theta, kQ);
-  unpack_kernel<T><<<grid, kRowThreads, 0, s>>>(in, f, p, d);
-  return cudaGetLastError();
+  return launch_copy_rows<T, true>(in, f, kQ, p, recv_labels(d, kQ), s);
 }
 
 template <class T>
