@@ -180,17 +180,29 @@ __device__ __forceinline__ NodeState<float> node_moments(const float* f, Stride 
   return st;
 }
 
+// FP64 sums over the pairs of opposite directions of each shell: with the
+// octagon's unit vectors (1,0), (s,s), (0,1), (-s,s) a shell takes 22 FP64
+// operations instead of 32 (four per label), and FP64 issue is what bounds
+// every caller (a quarter SM starts one warp-wide FP64 operation per 76 cycles).
 template <class Stride>
 __device__ __forceinline__ NodeState<double> node_moments(const double* f, Stride stride,
                                                           const DvmConst<double>& d) {
-  double s0 = 0.0, sx = 0.0, sy = 0.0, se = 0.0;
+  double s0 = f[0], sx = 0.0, sy = 0.0, se = 0.0;
+  const double c = d.cx[2];   // 1 / sqrt 2
 #pragma unroll
-  for (int q = 0; q < kQ; ++q) {
-    const double v = f[q * stride];
-    s0 += v;
-    sx = fma(d.vx[q], v, sx);
-    sy = fma(d.vy[q], v, sy);
-    se = fma(d.half_v2[d.shell[q]], v, se);
+  for (int k = 1; k <= 4; ++k) {
+    double S = 0.0, D[kNDirs / 2];
+#pragma unroll
+    for (int i = 0; i < kNDirs / 2; ++i) {
+      const int q = 1 + (k - 1) * kNDirs + i;
+      const double a = f[q * stride], b = f[(q + kNDirs / 2) * stride];
+      S += a + b;
+      D[i] = a - b;
+    }
+    s0 += S;
+    sx = fma(d.speed[k], fma(c, D[1] - D[3], D[0]), sx);
+    sy = fma(d.speed[k], fma(c, D[1] + D[3], D[2]), sy);
+    se = fma(d.half_v2[k], S, se);
   }
   const double inv = 1.0 / s0;
   const double ux = sx * inv, uy = sy * inv;
@@ -328,6 +340,33 @@ __device__ __forceinline__ T feq_q(const EqParams<T>& p, T vx, T vy, int k) {
   const T x = vx * p.uxE + vy * p.uyE;
   const T poly = p.a0 + x * (p.a1 + x * (p.a1h + x * (T(1.0 / 6.0) + x * T(1.0 / 24.0))));
   return p.w[k] * poly;
+}
+
+// The equilibrium folded per shell for the pairs of opposite velocities, FP64:
+// with y = c_i.u/E for the first direction of a pair, f^eq(+-v_k c_i) = ev +- od,
+// ev = A + y^2 (B + y^2 C), od = y (O1 + y^2 O3).
+struct EqShells64 {
+  double A[4], B[4], C[4], O1[4], O3[4];   // shells k = 1..4
+  double y[kNDirs / 2];
+};
+
+__device__ __forceinline__ EqShells64 eq_shells(const EqParams<double>& e, const DvmConst<double>& d) {
+  EqShells64 g;
+#pragma unroll
+  for (int k = 1; k <= 4; ++k) {
+    const double v = d.speed[k], hv = d.half_v2[k], wv = e.w[k] * v, wh = e.w[k] * hv;
+    g.A[k - 1] = e.w[k] * e.a0;
+    g.B[k - 1] = wh * e.a1;                        // w v^2 a1 / 2
+    g.C[k - 1] = wh * (hv * (1.0 / 6.0));          // w v^4 / 24
+    g.O1[k - 1] = wv * e.a1;
+    g.O3[k - 1] = wv * (hv * (1.0 / 3.0));         // w v^3 / 6
+  }
+  const double c = d.cx[2];   // 1 / sqrt 2; directions (1,0), (s,s), (0,1), (-s,s)
+  g.y[0] = e.uxE;
+  g.y[1] = c * (e.uyE + e.uxE);
+  g.y[2] = e.uyE;
+  g.y[3] = c * (e.uyE - e.uxE);
+  return g;
 }
 
 // ---------------------------------------------------------------------------

@@ -335,17 +335,6 @@ __global__ void __launch_bounds__(kGenThreads)
     }
 }
 
-__global__ void gen_diag_final_kernel(const double* partials, int n_blocks, double* out, double n_nodes) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double s[6] = {0, 0, 0, 0, DBL_MAX, DBL_MAX};
-  for (int b = 0; b < n_blocks; ++b)
-    for (int i = 0; i < 6; ++i)
-      s[i] = i < 4 ? s[i] + partials[(size_t)b * 8 + i] : fmin(s[i], partials[(size_t)b * 8 + i]);
-  for (int i = 0; i < 6; ++i) out[i] = s[i];
-  out[6] = n_nodes;
-  out[7] = 0.0;
-}
-
 template <int SCH>
 cudaError_t gen_step_scheme(const double* f, double* f_out, double* ghost, const StepParams& p, const DvmG& d,
                             cudaStream_t s) {
@@ -434,8 +423,8 @@ template <class T>
 cudaError_t gen_launch_diagnostics(const T* f, double* partials, double* out, const StepParams& p, const DvmG& d,
                                    double dr, double dth, double r_in, cudaStream_t s) {
   gen_diag_partial_kernel<T><<<kDiagBlocks, kGenThreads, 0, s>>>(f, partials, p, d, dr, dth, r_in);
-  gen_diag_final_kernel<<<1, 32, 0, s>>>(partials, kDiagBlocks, out, (double)p.n_r * p.n_theta);
-  return cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
+  return e != cudaSuccess ? e : launch_diag_final(partials, kDiagBlocks, out, (double)p.n_r * p.n_theta, s);
 }
 
 #define PCLB_GEN_INSTANTIATE(T)                                                                               \

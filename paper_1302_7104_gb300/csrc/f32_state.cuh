@@ -53,8 +53,9 @@ __device__ __forceinline__ void shell_sums(const float* f, Stride stride, const 
   }
 }
 
+// raw (if given): the moments rho, j_x, j_y and e = rho (E + u^2/2) themselves.
 template <class Stride>
-__device__ __forceinline__ State32 state32(const float* f, Stride stride, const DvmConst<float>& d) {
+__device__ __forceinline__ State32 state32(const float* f, Stride stride, const DvmConst<float>& d, ff* raw = nullptr) {
   ff rho = ff_of(f[0]), jx = ff_of(0.f), jy = ff_of(0.f), e = ff_of(0.f);
   // (shell, shell added to it, speed, v^2/2): 1; 2+3 with v_2; 3 with v_3 - v_2; 4
 #pragma unroll
@@ -76,6 +77,7 @@ __device__ __forceinline__ State32 state32(const float* f, Stride stride, const 
     jy = ff_add(jy, ff_mul(sp, ff{Y, Yl}));
     e = ff_add(e, ff_mul(hv, ff_of(S)));
   }
+  if (raw) { raw[0] = rho; raw[1] = jx; raw[2] = jy; raw[3] = e; }
   State32 s;
   const ff inv = ff_recip(rho);
   s.rho = rho;

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <float.h>
 
+#include <algorithm>
+
 #include "copy_rows.cuh"
 #include "device_common.cuh"
 #include "f32_eq2.cuh"
@@ -12,6 +14,8 @@
 #include "pclb_internal.h"
 
 namespace pclb {
+
+constexpr int kDiagThreads32 = 512;   // two blocks per SM, 32 warps
 
 // Write value v of label q at interior row t, column r of the stored layout,
 // together with its copies in the azimuthal ghost rows (Eq. 40).
@@ -25,26 +29,34 @@ __device__ __forceinline__ void store_with_ghosts(T* f, const StepParams& p, con
   if (t < 2) f[(size_t)d.recv_hi[q] * plane + (size_t)(p.n_theta + kGhostRows + t) * p.pitch + r] = v;
 }
 
-template <class T>
-__global__ void set_state_kernel(T* __restrict__ f, const T* __restrict__ rho, const T* __restrict__ u_r,
-                                 const T* __restrict__ u_t, const T* __restrict__ temp,
-                                 const __grid_constant__ StepParams p, const __grid_constant__ DvmConst<T> d,
+// FP64 path.  Bound: FP64 issue (see node_moments).  Per shell the polynomial
+// of Eq. (10) in x = v_k y_i, y_i = c_i.u/E, is folded into w ev = A + y^2 (B +
+// y^2 C) and w od = y (O1 + y^2 O3): six operations per pair of opposite
+// velocities, where Horner's rule in x takes seven per label.
+__global__ void set_state_kernel(double* __restrict__ f, const double* __restrict__ rho, const double* __restrict__ u_r,
+                                 const double* __restrict__ u_t, const double* __restrict__ temp,
+                                 const __grid_constant__ StepParams p, const __grid_constant__ DvmConst<double> d,
                                  int t_begin) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   const int t = blockIdx.y + t_begin;
   if (r >= p.n_r || t >= p.n_theta) return;
   const size_t n = (size_t)t * p.n_r + r;
-  const T c = (T)p.cos_t[t], s = (T)p.sin_t[t];
-  const T R = rho[n], ur = u_r[n], ut = u_t[n], E = temp[n];  // E = T for gamma = 2
-  if (!(R > T(0) && E > T(0))) atomicOr(p.status, PCLB_FLAG_NONPHYS);
-  const T ux = ur * c - ut * s, uy = ur * s + ut * c;
-  const EqParams<T> e = eq_params<T>((double)R, ux, uy, (double)E, d);
+  const double c = p.cos_t[t], s = p.sin_t[t];
+  const double R = rho[n], ur = u_r[n], ut = u_t[n], E = temp[n];  // E = T for gamma = 2
+  if (!(R > 0.0 && E > 0.0)) atomicOr(p.status, PCLB_FLAG_NONPHYS);
+  const EqParams<double> e = eq_params<double>(R, ur * c - ut * s, ur * s + ut * c, E, d);
+  const EqShells64 g = eq_shells(e, d);
+  store_with_ghosts<double>(f, p, d, 0, t, r, e.w[0] * e.a0);
 #pragma unroll
-  for (int k = 0; k < 5; ++k) {
-    const int q_begin = k == 0 ? 0 : 1 + (k - 1) * kNDirs;
-    const int q_end = k == 0 ? 1 : q_begin + kNDirs;
-    for (int q = q_begin; q < q_end; ++q)
-      store_with_ghosts<T>(f, p, d, q, t, r, feq_q<T>(e, d.vx[q], d.vy[q], k));
+  for (int i = 0; i < kNDirs / 2; ++i) {
+    const double y = g.y[i], y2 = y * y;
+#pragma unroll
+    for (int k = 1; k <= 4; ++k) {
+      const int q = 1 + (k - 1) * kNDirs + i;
+      const double ev = fma(y2, fma(y2, g.C[k - 1], g.B[k - 1]), g.A[k - 1]), z = fma(y2, g.O3[k - 1], g.O1[k - 1]);
+      store_with_ghosts<double>(f, p, d, q, t, r, fma(y, z, ev));
+      store_with_ghosts<double>(f, p, d, q + kNDirs / 2, t, r, fma(-y, z, ev));
+    }
   }
 }
 
@@ -145,28 +157,9 @@ __global__ void moments_kernel(const T* __restrict__ f, T* rho, T* u_r, T* u_t, 
   if (temp) temp[n] = m.E;
 }
 
-// Global integrals with weight r dr dtheta, in double.  Each block reduces a
-// fixed grid-stride subset in a fixed order, so results are reproducible.
-template <class T>
-__global__ void diag_partial_kernel(const T* __restrict__ f, double* partials, const __grid_constant__ StepParams p,
-                                    const __grid_constant__ DvmConst<T> d, double dr, double dth, double r_in) {
-  const size_t plane = (size_t)p.rows * p.pitch;
-  const size_t n_nodes = (size_t)p.n_r * p.n_theta;
-  double acc[4] = {0, 0, 0, 0};
-  double mn[2] = {DBL_MAX, DBL_MAX};
-  for (size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x; n < n_nodes;
-       n += (size_t)gridDim.x * blockDim.x) {
-    const int t = (int)(n / p.n_r), r = (int)(n % p.n_r);
-    double rho, ux, uy, E;
-    node_state_double(f + (size_t)(t + kGhostRows) * p.pitch + r, plane, d, rho, ux, uy, E);
-    const double w = (r_in + r * dr) * dr * dth;
-    acc[0] += w * rho;
-    acc[1] += w * rho * ux;
-    acc[2] += w * rho * uy;
-    acc[3] += w * rho * (E + 0.5 * (ux * ux + uy * uy));
-    mn[0] = fmin(mn[0], rho);
-    mn[1] = fmin(mn[1], E);
-  }
+// Block reduction of the six integrals of a block (four sums, two minima) in a
+// fixed order, written to the block's partial slot.
+__device__ __forceinline__ void diag_block_reduce(const double (&acc)[4], const double (&mn)[2], double* partials) {
   __shared__ double red[6][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double v[6] = {acc[0], acc[1], acc[2], acc[3], mn[0], mn[1]};
@@ -179,25 +172,103 @@ __global__ void diag_partial_kernel(const T* __restrict__ f, double* partials, c
     if (lane == 0) red[i][warp] = v[i];
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    const int nw = blockDim.x / 32;
-    for (int i = 0; i < 6; ++i) {
-      double s = red[i][0];
-      for (int w = 1; w < nw; ++w) s = i < 4 ? s + red[i][w] : fmin(s, red[i][w]);
-      partials[(size_t)blockIdx.x * 8 + i] = s;
-    }
+  if (threadIdx.x < 6) {
+    const int nw = blockDim.x / 32, i = threadIdx.x;
+    double s = red[i][0];
+    for (int w = 1; w < nw; ++w) s = i < 4 ? s + red[i][w] : fmin(s, red[i][w]);
+    partials[(size_t)blockIdx.x * 8 + i] = s;
   }
 }
 
-__global__ void diag_final_kernel(const double* partials, int n_blocks, double* out, double n_nodes) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double s[6] = {0, 0, 0, 0, DBL_MAX, DBL_MAX};
-  for (int b = 0; b < n_blocks; ++b)
-    for (int i = 0; i < 6; ++i)
-      s[i] = i < 4 ? s[i] + partials[(size_t)b * 8 + i] : fmin(s[i], partials[(size_t)b * 8 + i]);
-  for (int i = 0; i < 6; ++i) out[i] = s[i];
-  out[6] = n_nodes;
-  out[7] = 0.0;
+// Global integrals with weight r dr dtheta, in double.  Each block reduces a
+// fixed grid-stride subset in a fixed order, so results are reproducible.
+__global__ void diag_partial_kernel(const double* __restrict__ f, double* partials, const __grid_constant__ StepParams p,
+                                    const __grid_constant__ DvmConst<double> d, double dr, double dth, double r_in) {
+  const size_t plane = (size_t)p.rows * p.pitch;
+  const size_t n_nodes = (size_t)p.n_r * p.n_theta;
+  double acc[4] = {0, 0, 0, 0};
+  double mn[2] = {DBL_MAX, DBL_MAX};
+  for (size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x; n < n_nodes;
+       n += (size_t)gridDim.x * blockDim.x) {
+    const int t = (int)(n / p.n_r), r = (int)(n % p.n_r);
+    const NodeState<double> m = node_moments(f + (size_t)(t + kGhostRows) * p.pitch + r, plane, d);
+    const double w = (r_in + r * dr) * dr * dth;
+    acc[0] += w * m.rho;
+    acc[1] += w * m.rho * m.ux;
+    acc[2] += w * m.rho * m.uy;
+    acc[3] += w * m.rho * (m.E + 0.5 * (m.ux * m.ux + m.uy * m.uy));
+    mn[0] = fmin(mn[0], m.rho);
+    mn[1] = fmin(mn[1], m.E);
+  }
+  diag_block_reduce(acc, mn, partials);
+}
+
+// FP32: the same integrals from the raw float-float moments (rho, j, e =
+// rho (E + u^2/2)), without FP64 work per node: a thread adds up to `rows`
+// nodes of one column in float-float and enters the double sums once, weighted
+// by the column's r dr dtheta.  The form above spent ~30 FP64 operations per
+// node (conversions, weights and sums; 121 us on 1024 x 2048, FP64-bound),
+// this one is bound by the read of f.
+__global__ void __launch_bounds__(kDiagThreads32, 2)
+    diag_partial_f32_kernel(const float* __restrict__ f, double* partials, const __grid_constant__ StepParams p,
+                            const __grid_constant__ DvmConst<float> d, double dr, double dth, double r_in, int rows) {
+  const size_t plane = (size_t)p.rows * p.pitch;
+  const size_t items = (size_t)((p.n_theta + rows - 1) / rows) * p.n_r;
+  double acc[4] = {0, 0, 0, 0};
+  float mh[2] = {FLT_MAX, FLT_MAX}, ml[2] = {0.f, 0.f};   // least rho and E so far, float-float
+  bool any = false;
+  for (size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x; n < items; n += (size_t)gridDim.x * blockDim.x) {
+    const int r = (int)(n % p.n_r), t0 = (int)(n / p.n_r) * rows, t1 = min(t0 + rows, p.n_theta);
+    ff s[4] = {ff_of(0.f), ff_of(0.f), ff_of(0.f), ff_of(0.f)};
+#pragma unroll 1
+    for (int t = t0; t < t1; ++t) {
+      ff m[4];
+      const State32 st = state32(f + (size_t)(t + kGhostRows) * p.pitch + r, plane, d, m);
+      // a node whose velocity or temperature is not finite makes its sums NaN
+      m[1].hi += st.ux.hi - st.ux.hi;
+      m[2].hi += st.uy.hi - st.uy.hi;
+      m[3].hi += st.E.hi - st.E.hi;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) s[i] = ff_add(s[i], m[i]);
+      auto least = [&](int i, ff x) {
+        if (x.hi < mh[i] || (x.hi == mh[i] && x.lo < ml[i])) { mh[i] = x.hi; ml[i] = x.lo; }
+      };
+      least(0, st.rho);
+      least(1, st.E);
+    }
+    any = true;
+    const double w = (r_in + r * dr) * dr * dth;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i] += w * ((double)s[i].hi + s[i].lo);
+  }
+  const double mn[2] = {any && mh[0] < FLT_MAX ? (double)mh[0] + ml[0] : DBL_MAX,
+                        any && mh[1] < FLT_MAX ? (double)mh[1] + ml[1] : DBL_MAX};
+  diag_block_reduce(acc, mn, partials);
+}
+
+// The blocks' partials to the result: warp i adds (or takes the least of) the
+// i-th integral, lanes over blocks (one thread over all of them took 112 us).
+__global__ void __launch_bounds__(192) diag_final_kernel(const double* partials, int n_blocks, double* out, double n_nodes) {
+  const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double s = i < 4 ? 0.0 : DBL_MAX;
+  for (int b = lane; b < n_blocks; b += 32) {
+    const double v = partials[(size_t)b * 8 + i];
+    s = i < 4 ? s + v : fmin(s, v);
+  }
+  for (int off = 16; off > 0; off >>= 1) {
+    const double o = __shfl_down_sync(0xffffffffu, s, off);
+    s = i < 4 ? s + o : fmin(s, o);
+  }
+  if (lane == 0) out[i] = s;
+  if (threadIdx.x == 0) {
+    out[6] = n_nodes;
+    out[7] = 0.0;
+  }
+}
+
+cudaError_t launch_diag_final(const double* partials, int n_blocks, double* out, double n_nodes, cudaStream_t s) {
+  diag_final_kernel<<<1, 192, 0, s>>>(partials, n_blocks, out, n_nodes);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -217,7 +288,7 @@ cudaError_t launch_set_state(T* f, const T* rho, const T* ur, const T* ut, const
     set_state_f32_kernel<<<grid, kSetThreads32, 0, s>>>(f, rho, ur, ut, temp, p, d, t_begin);
   } else {
     const dim3 grid((p.n_r + kRowThreads - 1) / kRowThreads, t_end - t_begin);
-    set_state_kernel<T><<<grid, kRowThreads, 0, s>>>(f, rho, ur, ut, temp, p, d, t_begin);
+    set_state_kernel<<<grid, kRowThreads, 0, s>>>(f, rho, ur, ut, temp, p, d, t_begin);
   }
   return cudaGetLastError();
 }
@@ -249,11 +320,16 @@ template <class T>
 cudaError_t launch_diagnostics(const T* f, double* partials, double* out, const StepParams& p,
                                const DvmConst<T>& d, double dr, double dth, double r_in,
                                cudaStream_t s) {
-  diag_partial_kernel<T><<<kDiagBlocks, 256, 0, s>>>(f, partials, p, d, dr, dth, r_in);
+  if constexpr (sizeof(T) == 4) {
+    // rows per thread: as many as keep every thread of the grid at work, at most 8
+    const size_t per = (size_t)p.n_r * p.n_theta / ((size_t)kDiagBlocks * kDiagThreads32);
+    diag_partial_f32_kernel<<<kDiagBlocks, kDiagThreads32, 0, s>>>(f, partials, p, d, dr, dth, r_in,
+                                                                   (int)std::min<size_t>(8, std::max<size_t>(1, per)));
+  } else {
+    diag_partial_kernel<<<kDiagBlocks, 256, 0, s>>>(f, partials, p, d, dr, dth, r_in);
+  }
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  diag_final_kernel<<<1, 32, 0, s>>>(partials, kDiagBlocks, out, (double)p.n_r * p.n_theta);
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : launch_diag_final(partials, kDiagBlocks, out, (double)p.n_r * p.n_theta, s);
 }
 
 #define PCLB_INSTANTIATE(T)                                                                         \

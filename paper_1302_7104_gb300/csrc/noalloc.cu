@@ -73,18 +73,6 @@ __global__ void diag_rows_kernel(const T* __restrict__ f, double* __restrict__ p
   }
 }
 
-__global__ void diag_rows_final(const double* __restrict__ partials, int n_rows, double* out,
-                                double n_nodes) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double s[6] = {0, 0, 0, 0, DBL_MAX, DBL_MAX};
-  for (int b = 0; b < n_rows; ++b)
-    for (int i = 0; i < 6; ++i)
-      s[i] = i < 4 ? s[i] + partials[(size_t)b * 8 + i] : fmin(s[i], partials[(size_t)b * 8 + i]);
-  for (int i = 0; i < 6; ++i) out[i] = s[i];
-  out[6] = n_nodes;
-  out[7] = 0.0;
-}
-
 // Device address of the scratch array, looked up once per device with that
 // device current (a host-side reference to the array is not a device address).
 std::mutex g_setup_mutex;
@@ -155,9 +143,7 @@ cudaError_t launch_rows(const void* f, double* scratch, const pclb_grid& g, cons
                                                             g.n_theta, d, dr, dth, g.r_in);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  diag_rows_final<<<1, 32, 0, s>>>(scratch, g.n_theta, scratch + (size_t)kNoAllocMaxRows * 8,
-                                   (double)g.n_r * g.n_theta);
-  return cudaGetLastError();
+  return launch_diag_final(scratch, g.n_theta, scratch + (size_t)kNoAllocMaxRows * 8, (double)g.n_r * g.n_theta, s);
 }
 
 }  // namespace

@@ -147,6 +147,9 @@ AdjScratch adjoint_scratch(unsigned char* base, int n_theta, int elem);
 
 constexpr int kDiagBlocks = 304;    // 2 x 152 SMs
 
+// Adds up the blocks' partials of the global integrals (field_kernels.cu).
+cudaError_t launch_diag_final(const double* partials, int n_blocks, double* out, double n_nodes, cudaStream_t s);
+
 // Host helpers shared by the C-ABI translation units (defined in pclb_abi.cu).
 pclb_status validate_problem(const pclb_grid* g, const pclb_dvm* d, pclb_precision prec);
 template <class T>
