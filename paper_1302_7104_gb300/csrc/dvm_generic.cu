@@ -21,6 +21,7 @@
 #include "copy_rows.cuh"
 #include "dvm_generic.h"
 #include "f32_state.cuh"
+#include "gen_state.cuh"
 #include "pclb_internal.h"
 
 namespace pclb {
@@ -51,16 +52,24 @@ __device__ __forceinline__ GenState gen_state_of(double s0, double sx, double sy
   return m;
 }
 
-// Moments (Eqs. 3-5): rho = sum f, rho u = sum f v, rho (E + u^2/2) = sum f v^2/2.
-template <class T>
-__device__ GenState gen_moments_node(const T* f, size_t plane, const DvmG& d) {
-  double s0 = 0.0, sx = 0.0, sy = 0.0, se = 0.0;
-  for (int q = 0; q < d.q; ++q) {
-    const double v = (double)f[(size_t)q * plane];
-    s0 += v;
-    sx = fma(d.vx[q], v, sx);
-    sy = fma(d.vy[q], v, sy);
-    se = fma(d.half_v2[d.shell[q]], v, se);
+// Moments (Eqs. 3-5): rho = sum f, rho u = sum f v, rho (E + u^2/2) = sum f
+// v^2/2, over the pairs of opposite velocities (2.5 FP64 operations per label
+// instead of 4; FP64 issue bounds every caller).
+__device__ GenState gen_moments_node(const double* f, size_t plane, const DvmG& d) {
+  const int half = d.n_dirs / 2;
+  double s0 = f[0], sx = 0.0, sy = 0.0, se = 0.0;
+  for (int k = 1; k <= 4; ++k) {
+    double S = 0.0;
+#pragma unroll 4
+    for (int i = 0; i < half; ++i) {
+      const int q = 1 + (k - 1) * d.n_dirs + i;
+      const double a = f[(size_t)q * plane], b = f[(size_t)(q + half) * plane];
+      S += a + b;
+      sx = fma(d.vx[q], a - b, sx);
+      sy = fma(d.vy[q], a - b, sy);
+    }
+    s0 += S;
+    se = fma(d.half_v2[k], S, se);
   }
   return gen_state_of(s0, sx, sy, se);
 }
@@ -143,26 +152,33 @@ __device__ __forceinline__ void gen_store(T* f, const StepParams& p, const DvmG&
 }
 
 // ---------------------------------------------------------------------------
-template <class T>
 __global__ void __launch_bounds__(kGenThreads)
-    gen_set_state_kernel(T* __restrict__ f, const T* __restrict__ rho, const T* __restrict__ u_r,
-                         const T* __restrict__ u_t, const T* __restrict__ temp, const __grid_constant__ StepParams p,
-                         const __grid_constant__ DvmG d) {
+    gen_set_state_kernel(double* __restrict__ f, const double* __restrict__ rho, const double* __restrict__ u_r,
+                         const double* __restrict__ u_t, const double* __restrict__ temp,
+                         const __grid_constant__ StepParams p, const __grid_constant__ DvmG d) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   const int t = blockIdx.y;
   if (r >= p.n_r) return;
   const size_t n = (size_t)t * p.n_r + r;
   const double c = p.cos_t[t], s = p.sin_t[t];
-  const double R = (double)rho[n], ur = (double)u_r[n], ut = (double)u_t[n], E = (double)temp[n];  // E = T
+  const double R = rho[n], ur = u_r[n], ut = u_t[n], E = temp[n];  // E = T
   if (!(R > 0.0 && E > 0.0)) atomicOr(p.status, PCLB_FLAG_NONPHYS);
-  const GenEq e = gen_eq(R, ur * c - ut * s, ur * s + ut * c, E, d);
-  for (int q = 0; q < d.q; ++q) gen_store<T>(f, p, d, q, t, r, (T)gen_feq(e, d, q));
+  const GenEqC<double> e = gen_eq_c<double>(gen_eq(R, ur * c - ut * s, ur * s + ut * c, E, d));
+  gen_store<double>(f, p, d, 0, t, r, e.w[0] * e.a0);
+  const int half = d.n_dirs / 2;
+  for (int k = 1; k <= 4; ++k)
+    for (int i = 0; i < half; ++i) {
+      const int q = 1 + (k - 1) * d.n_dirs + i;
+      double fp, fm;
+      gen_feq_pair<double>(e, d.vx[q], d.vy[q], k, fp, fm);
+      gen_store<double>(f, p, d, q, t, r, fp);
+      gen_store<double>(f, p, d, q + half, t, r, fm);
+    }
 }
 
-template <class T>
 __global__ void __launch_bounds__(kGenThreads)
-    gen_moments_kernel(const T* __restrict__ f, T* rho, T* u_r, T* u_t, T* temp, const __grid_constant__ StepParams p,
-                       const __grid_constant__ DvmG d) {
+    gen_moments_kernel(const double* __restrict__ f, double* rho, double* u_r, double* u_t, double* temp,
+                       const __grid_constant__ StepParams p, const __grid_constant__ DvmG d) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   const int t = blockIdx.y;
   if (r >= p.n_r) return;
@@ -170,26 +186,109 @@ __global__ void __launch_bounds__(kGenThreads)
   const GenState m = gen_moments_node(f + (size_t)(t + kGhostRows) * p.pitch + r, plane, d);
   const size_t n = (size_t)t * p.n_r + r;
   const double c = p.cos_t[t], s = p.sin_t[t];
-  if (rho) rho[n] = (T)m.rho;
-  if (u_r) u_r[n] = (T)(m.ux * c + m.uy * s);
-  if (u_t) u_t[n] = (T)(m.uy * c - m.ux * s);
-  if (temp) temp[n] = (T)m.E;
+  if (rho) rho[n] = m.rho;
+  if (u_r) u_r[n] = m.ux * c + m.uy * s;
+  if (u_t) u_t[n] = m.uy * c - m.ux * s;
+  if (temp) temp[n] = m.E;
+}
+
+// FP32 storage: f = f^eq of the fields, evaluated in float-float and rounded
+// once per label.  Per node and shell the polynomial of Eq. (10) in x = v_k
+// y_i, y_i = c_i.u/E, is folded into w ev = A + y^2 (B + y^2 C) and w od = y
+// (O1 + y^2 O3), so that a pair of opposite velocities takes three multiply-adds,
+// a product and two rounded sums.
+template <int ND>
+__global__ void __launch_bounds__(kGenThreads)
+    gen_set_state_f32_kernel(float* __restrict__ f, const float* __restrict__ rho, const float* __restrict__ u_r,
+                             const float* __restrict__ u_t, const float* __restrict__ temp,
+                             const __grid_constant__ StepParams p, const __grid_constant__ DvmG d,
+                             const __grid_constant__ DvmG32 c) {
+  constexpr int H = ND / 2;
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  const int t = blockIdx.y;
+  if (r >= p.n_r) return;
+  const size_t n = (size_t)t * p.n_r + r;
+  const ff R = ff_of(rho[n]), E = ff_of(temp[n]), ur = ff_of(u_r[n]), ut = ff_of(u_t[n]);   // E = T
+  if (!(R.hi > 0.f && E.hi > 0.f)) atomicOr(p.status, PCLB_FLAG_NONPHYS);
+  const float4 cs = p.cs_ff[t];
+  const ff co{cs.x, cs.y}, si{cs.z, cs.w};
+  const ff ux = ff_add(ff_mul(ur, co), ff_neg(ff_mul(ut, si))), uy = ff_add(ff_mul(ur, si), ff_mul(ut, co));
+  const ff invE = ff_recip(E);
+  const ff uxE = ff_mul(ux, invE), uyE = ff_mul(uy, invE);
+  const ff u2E = ff_add(ff_mul(ux, uxE), ff_mul(uy, uyE));   // u^2 / E
+  const ff a1 = ff_add(ff_of(1.f), ff_scale(u2E, -0.5f));
+  const ff a0 = ff_add(a1, ff_scale(ff_mul(u2E, u2E), 0.125f));
+  ff sum = ff_of(0.f);
+  ff A[4], B[4], C[4], O1[4], O3[4];
+  const ff sixth{1.0f / 6.0f, (float)(1.0 / 6.0 - (double)(1.0f / 6.0f))};
+#pragma unroll
+  for (int k = 1; k <= 4; ++k) {
+    ff F{c.Fch[k][3], c.Fcl[k][3]};
+#pragma unroll
+    for (int j = 2; j >= 0; --j) F = ff_mul_add(F, E, ff{c.Fch[k][j], c.Fcl[k][j]});
+    F = ff_mul(F, E);
+    sum = ff_add(sum, F);
+    const ff w = ff_mul(R, F), v{c.sph[k], c.spl[k]}, wv = ff_mul(w, v), hv{c.hvh[k], c.hvl[k]};   // hv = v^2/2
+    A[k - 1] = ff_mul(w, a0);
+    B[k - 1] = ff_mul(ff_mul(w, hv), a1);
+    O1[k - 1] = ff_mul(wv, a1);
+    O3[k - 1] = ff_scale(ff_mul(ff_mul(wv, hv), sixth), 2.f);            // w v^3 / 6
+    C[k - 1] = ff_mul(ff_mul(ff_mul(w, hv), hv), sixth);                  // w v^4 / 24
+  }
+  const ff w0 = ff_mul(R, ff_add(ff_of(1.f), ff_mul(ff{-c.B0h, -c.B0l}, sum)));
+  const ff f0 = ff_mul(w0, a0);
+  gen_store<float>(f, p, d, 0, t, r, f0.hi + f0.lo);
+#pragma unroll 1
+  for (int i = 0; i < H; ++i) {
+    const ff y = ff_add(ff_mul(ff{c.cxh[i], c.cxl[i]}, uxE), ff_mul(ff{c.cyh[i], c.cyl[i]}, uyE));
+    const ff y2 = ff_mul(y, y);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const ff ev = ff_mul_add(y2, ff_mul_add(y2, C[k], B[k]), A[k]);
+      const ff od = ff_mul(y, ff_mul_add(y2, O3[k], O1[k]));
+      float h, e;
+      two_sum(ev.hi, od.hi, h, e);
+      gen_store<float>(f, p, d, 1 + k * ND + i, t, r, h + (e + (ev.lo + od.lo)));
+      two_sum(ev.hi, -od.hi, h, e);
+      gen_store<float>(f, p, d, 1 + k * ND + i + H, t, r, h + (e + (ev.lo - od.lo)));
+    }
+  }
+}
+
+template <int ND>
+__global__ void __launch_bounds__(kGenThreads)
+    gen_moments_f32_kernel(const float* __restrict__ f, float* rho, float* u_r, float* u_t, float* temp,
+                           const __grid_constant__ StepParams p, const __grid_constant__ DvmG32 c) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  const int t = blockIdx.y;
+  if (r >= p.n_r) return;
+  const size_t plane = (size_t)p.rows * p.pitch;
+  const State32 m = gen_state32<ND>(f + (size_t)(t + kGhostRows) * p.pitch + r, plane, c);
+  const size_t n = (size_t)t * p.n_r + r;
+  const float4 cs = p.cs_ff[t];
+  const ff co{cs.x, cs.y}, si{cs.z, cs.w};
+  auto put = [&](float* o, ff x) {
+    if (o) o[n] = x.hi + x.lo;
+  };
+  put(rho, m.rho);
+  put(u_r, ff_add(ff_mul(m.ux, co), ff_mul(m.uy, si)));
+  put(u_t, ff_add(ff_mul(m.uy, co), ff_neg(ff_mul(m.ux, si))));
+  put(temp, m.E);
 }
 
 // Radial ghost layers of wall `side` at row t: layer l sits at r = -1 - l
 // (inner) or n_r + l (outer).  Eq. (39) applied twice to the wall node a and
 // the next node b: g0 = 2a - b, g1 = 2 g0 - a, for the components the
 // boundary kind extrapolates; the others prescribed.
-template <class T>
 __global__ void __launch_bounds__(kGenThreads)
-    gen_ghost_kernel(const T* __restrict__ f, T* __restrict__ ghost, const __grid_constant__ StepParams p,
+    gen_ghost_kernel(const double* __restrict__ f, double* __restrict__ ghost, const __grid_constant__ StepParams p,
                      const __grid_constant__ DvmG d) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int side = blockIdx.y;
   if (t >= p.n_theta) return;
   const size_t plane = (size_t)p.rows * p.pitch;
   const int ra = side == 0 ? 0 : p.n_r - 1, step = side == 0 ? 1 : -1;
-  const T* fa = f + (size_t)(t + kGhostRows) * p.pitch + ra;
+  const double* fa = f + (size_t)(t + kGhostRows) * p.pitch + ra;
   const GenState a = gen_moments_node(fa, plane, d);
   const GenState b = gen_moments_node(fa + step, plane, d);
   double g[2][4];
@@ -217,11 +316,11 @@ __global__ void __launch_bounds__(kGenThreads)
   for (int l = 0; l < 2; ++l) {
     ok = ok && g[l][0] > 0.0 && g[l][3] > 0.0;
     const GenEq e = gen_eq(g[l][0], g[l][1], g[l][2], g[l][3], d);
-    T* out = ghost + ((size_t)(side * 2 + l) * p.n_theta + t) * d.q;
+    double* out = ghost + ((size_t)(side * 2 + l) * p.n_theta + t) * d.q;
     for (int q = 0; q < d.q; ++q) {
       double v = gen_feq(e, d, q);
-      if (neq) v += (double)fa[(size_t)q * plane] - gen_feq(ea, d, q);
-      out[q] = (T)v;
+      if (neq) v += fa[(size_t)q * plane] - gen_feq(ea, d, q);
+      out[q] = v;
     }
   }
   if (!ok) atomicOr(p.status, PCLB_FLAG_NONPHYS);
@@ -299,16 +398,30 @@ __global__ void __launch_bounds__(kGenThreads)
 
 // Global integrals with weight r dr dtheta (as pclb_diagnostics): per block a
 // fixed grid-stride subset in a fixed order, then one thread sums the blocks.
-template <class T>
+// The node state in double: FP64 storage by double sums, FP32 by the
+// float-float sums of gen_state32.
+template <int ND>
+__device__ __forceinline__ GenState gen_diag_state(const double* f, size_t plane, const DvmG& d, const DvmG32&) {
+  return gen_moments_node(f, plane, d);
+}
+template <int ND>
+__device__ __forceinline__ GenState gen_diag_state(const float* f, size_t plane, const DvmG&, const DvmG32& c) {
+  const State32 s = gen_state32<ND>(f, plane, c);
+  return GenState{(double)s.rho.hi + s.rho.lo, (double)s.ux.hi + s.ux.lo, (double)s.uy.hi + s.uy.lo,
+                  (double)s.E.hi + s.E.lo, s.ok};
+}
+
+template <class T, int ND>
 __global__ void __launch_bounds__(kGenThreads)
     gen_diag_partial_kernel(const T* __restrict__ f, double* partials, const __grid_constant__ StepParams p,
-                            const __grid_constant__ DvmG d, double dr, double dth, double r_in) {
+                            const __grid_constant__ DvmG d, const __grid_constant__ DvmG32 c, double dr, double dth,
+                            double r_in) {
   const size_t plane = (size_t)p.rows * p.pitch;
   const size_t n_nodes = (size_t)p.n_r * p.n_theta;
   double v[6] = {0, 0, 0, 0, DBL_MAX, DBL_MAX};
   for (size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x; n < n_nodes; n += (size_t)gridDim.x * blockDim.x) {
     const int t = (int)(n / p.n_r), r = (int)(n % p.n_r);
-    const GenState m = gen_moments_node(f + (size_t)(t + kGhostRows) * p.pitch + r, plane, d);
+    const GenState m = gen_diag_state<ND>(f + (size_t)(t + kGhostRows) * p.pitch + r, plane, d, c);
     const double w = (r_in + r * dr) * dr * dth;
     v[0] += w * m.rho;
     v[1] += w * m.rho * m.ux;
@@ -339,7 +452,7 @@ template <int SCH>
 cudaError_t gen_step_scheme(const double* f, double* f_out, double* ghost, const StepParams& p, const DvmG& d,
                             cudaStream_t s) {
   // one thread per wall row, in warps, so that the rows spread over the SMs
-  gen_ghost_kernel<double><<<dim3((p.n_theta + 31) / 32, 2), 32, 0, s>>>(f, ghost, p, d);
+  gen_ghost_kernel<<<dim3((p.n_theta + 31) / 32, 2), 32, 0, s>>>(f, ghost, p, d);
   gen_step_kernel<SCH><<<dim3((p.n_r + kGenThreads - 1) / kGenThreads, p.n_theta), kGenThreads, 0, s>>>(
       f, f_out, ghost, p, d);
   return cudaGetLastError();
@@ -349,17 +462,27 @@ cudaError_t gen_step_scheme(const double* f, double* f_out, double* ghost, const
 
 template <class T>
 cudaError_t gen_launch_set_state(T* f, const T* rho, const T* ur, const T* ut, const T* temp, const StepParams& p,
-                                 const DvmG& d, cudaStream_t s) {
-  gen_set_state_kernel<T><<<dim3((p.n_r + kGenThreads - 1) / kGenThreads, p.n_theta), kGenThreads, 0, s>>>(
-      f, rho, ur, ut, temp, p, d);
+                                 const DvmG& d, const DvmG32& c, cudaStream_t s) {
+  const dim3 grid((p.n_r + kGenThreads - 1) / kGenThreads, p.n_theta);
+  if constexpr (sizeof(T) == 8)
+    gen_set_state_kernel<<<grid, kGenThreads, 0, s>>>(f, rho, ur, ut, temp, p, d);
+  else if (d.n_dirs == 16)
+    gen_set_state_f32_kernel<16><<<grid, kGenThreads, 0, s>>>(f, rho, ur, ut, temp, p, d, c);
+  else
+    gen_set_state_f32_kernel<24><<<grid, kGenThreads, 0, s>>>(f, rho, ur, ut, temp, p, d, c);
   return cudaGetLastError();
 }
 
 template <class T>
 cudaError_t gen_launch_moments(const T* f, T* rho, T* ur, T* ut, T* temp, const StepParams& p, const DvmG& d,
-                               cudaStream_t s) {
-  gen_moments_kernel<T><<<dim3((p.n_r + kGenThreads - 1) / kGenThreads, p.n_theta), kGenThreads, 0, s>>>(
-      f, rho, ur, ut, temp, p, d);
+                               const DvmG32& c, cudaStream_t s) {
+  const dim3 grid((p.n_r + kGenThreads - 1) / kGenThreads, p.n_theta);
+  if constexpr (sizeof(T) == 8)
+    gen_moments_kernel<<<grid, kGenThreads, 0, s>>>(f, rho, ur, ut, temp, p, d);
+  else if (d.n_dirs == 16)
+    gen_moments_f32_kernel<16><<<grid, kGenThreads, 0, s>>>(f, rho, ur, ut, temp, p, c);
+  else
+    gen_moments_f32_kernel<24><<<grid, kGenThreads, 0, s>>>(f, rho, ur, ut, temp, p, c);
   return cudaGetLastError();
 }
 
@@ -421,21 +544,24 @@ void fill_dvm_generic32(DvmG32& c, const pclb_dvm& d, const DvmG& g) {
 
 template <class T>
 cudaError_t gen_launch_diagnostics(const T* f, double* partials, double* out, const StepParams& p, const DvmG& d,
-                                   double dr, double dth, double r_in, cudaStream_t s) {
-  gen_diag_partial_kernel<T><<<kDiagBlocks, kGenThreads, 0, s>>>(f, partials, p, d, dr, dth, r_in);
+                                   const DvmG32& c, double dr, double dth, double r_in, cudaStream_t s) {
+  if (d.n_dirs == 16)
+    gen_diag_partial_kernel<T, 16><<<kDiagBlocks, kGenThreads, 0, s>>>(f, partials, p, d, c, dr, dth, r_in);
+  else
+    gen_diag_partial_kernel<T, 24><<<kDiagBlocks, kGenThreads, 0, s>>>(f, partials, p, d, c, dr, dth, r_in);
   const cudaError_t e = cudaGetLastError();
   return e != cudaSuccess ? e : launch_diag_final(partials, kDiagBlocks, out, (double)p.n_r * p.n_theta, s);
 }
 
 #define PCLB_GEN_INSTANTIATE(T)                                                                               \
   template cudaError_t gen_launch_set_state<T>(T*, const T*, const T*, const T*, const T*, const StepParams&, \
-                                               const DvmG&, cudaStream_t);                                    \
+                                               const DvmG&, const DvmG32&, cudaStream_t);                     \
   template cudaError_t gen_launch_moments<T>(const T*, T*, T*, T*, T*, const StepParams&, const DvmG&,        \
-                                             cudaStream_t);                                                   \
+                                             const DvmG32&, cudaStream_t);                                    \
   template cudaError_t gen_launch_pack<T>(const T*, T*, const StepParams&, const DvmG&, cudaStream_t);        \
   template cudaError_t gen_launch_unpack<T>(const T*, T*, const StepParams&, const DvmG&, cudaStream_t);      \
   template cudaError_t gen_launch_diagnostics<T>(const T*, double*, double*, const StepParams&, const DvmG&,  \
-                                                 double, double, double, cudaStream_t);
+                                                 const DvmG32&, double, double, double, cudaStream_t);
 PCLB_GEN_INSTANTIATE(float)
 PCLB_GEN_INSTANTIATE(double)
 

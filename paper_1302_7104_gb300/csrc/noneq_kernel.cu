@@ -29,6 +29,7 @@
 #include "device_common.cuh"
 #include "dvm_generic.h"
 #include "f32_state.cuh"
+#include "gen_state.cuh"
 #include "pclb_internal.h"
 
 namespace pclb {
@@ -160,9 +161,10 @@ __global__ void __launch_bounds__(kNeqThreads)
 
 // The same for the N_i = 16 and 24 sets of Table I (Q = 65, 97, built to
 // reproduce the same equilibrium moments, Eqs. 6-9): the node's moments in
-// double (one pass over its Q values), the central moments in the storage
-// type with the velocities of the set (float tables for FP32).
-template <class T>
+// double, or in float-float for FP32 storage (one pass over its Q values), the
+// central moments in the storage type with the velocities of the set (float
+// tables for FP32).
+template <class T, int ND>
 __global__ void __launch_bounds__(kNeqThreads)
     noneq_gen_kernel(const T* __restrict__ f, T* __restrict__ out, int groups, const __grid_constant__ StepParams p,
                      const __grid_constant__ DvmG d, const __grid_constant__ DvmG32 c) {
@@ -172,16 +174,27 @@ __global__ void __launch_bounds__(kNeqThreads)
   const size_t plane = (size_t)p.rows * p.pitch;
   const T* fn = f + (size_t)(t + kGhostRows) * p.pitch + r;
   // rho, rho u, rho (E + u^2/2) (Eqs. 3-5), then u and E
-  double s0 = 0.0, sx = 0.0, sy = 0.0, se = 0.0;
-  for (int q = 0; q < d.q; ++q) {
-    const double v = (double)fn[(size_t)q * plane];
-    s0 += v;
-    sx = fma(d.vx[q], v, sx);
-    sy = fma(d.vy[q], v, sy);
-    se = fma(d.half_v2[d.shell[q]], v, se);
+  double s0, uxd, uyd, E;
+  if constexpr (sizeof(T) == 4) {
+    const State32 m = gen_state32<ND>(fn, plane, c);
+    s0 = (double)m.rho.hi + m.rho.lo;
+    uxd = (double)m.ux.hi + m.ux.lo;
+    uyd = (double)m.uy.hi + m.uy.lo;
+    E = (double)m.E.hi + m.E.lo;
+  } else {
+    double sx = 0.0, sy = 0.0, se = 0.0;
+    s0 = 0.0;
+    for (int q = 0; q < d.q; ++q) {
+      const double v = fn[(size_t)q * plane];
+      s0 += v;
+      sx = fma(d.vx[q], v, sx);
+      sy = fma(d.vy[q], v, sy);
+      se = fma(d.half_v2[d.shell[q]], v, se);
+    }
+    uxd = sx / s0;
+    uyd = sy / s0;
+    E = (se - 0.5 * (sx * uxd + sy * uyd)) / s0;
   }
-  const double uxd = sx / s0, uyd = sy / s0;
-  const double E = (se - 0.5 * (sx * uxd + sy * uyd)) / s0;
   if (!(s0 > 0.0 && E > 0.0 && isfinite(E) && isfinite(uxd) && isfinite(uyd))) atomicOr(p.status, PCLB_FLAG_NONPHYS);
   const double rE = s0 * E, rE2 = 2.0 * s0 * E * E;
   const T rho = (T)s0, ux = (T)uxd, uy = (T)uyd;
@@ -250,7 +263,10 @@ template <class T>
 cudaError_t launch_noneq_gen(const T* f, T* out, int groups, const StepParams& p, const DvmG& d, const DvmG32& c,
                              cudaStream_t s) {
   dim3 grid((p.n_r + kNeqThreads - 1) / kNeqThreads, p.n_theta);
-  noneq_gen_kernel<T><<<grid, kNeqThreads, 0, s>>>(f, out, groups, p, d, c);
+  if (d.n_dirs == 16)
+    noneq_gen_kernel<T, 16><<<grid, kNeqThreads, 0, s>>>(f, out, groups, p, d, c);
+  else
+    noneq_gen_kernel<T, 24><<<grid, kNeqThreads, 0, s>>>(f, out, groups, p, d, c);
   return cudaGetLastError();
 }
 

@@ -51,16 +51,17 @@ cudaError_t launch_adjoint(const CUtensorMap*, const CUtensorMap*, const CUtenso
                            cudaEvent_t);
 template <class T>
 cudaError_t gen_launch_set_state(T*, const T*, const T*, const T*, const T*, const StepParams&, const DvmG&,
-                                 cudaStream_t);
+                                 const DvmG32&, cudaStream_t);
 template <class T>
-cudaError_t gen_launch_moments(const T*, T*, T*, T*, T*, const StepParams&, const DvmG&, cudaStream_t);
+cudaError_t gen_launch_moments(const T*, T*, T*, T*, T*, const StepParams&, const DvmG&, const DvmG32&,
+                               cudaStream_t);
 template <class T>
 cudaError_t gen_launch_pack(const T*, T*, const StepParams&, const DvmG&, cudaStream_t);
 template <class T>
 cudaError_t gen_launch_unpack(const T*, T*, const StepParams&, const DvmG&, cudaStream_t);
 template <class T>
-cudaError_t gen_launch_diagnostics(const T*, double*, double*, const StepParams&, const DvmG&, double, double,
-                                   double, cudaStream_t);
+cudaError_t gen_launch_diagnostics(const T*, double*, double*, const StepParams&, const DvmG&, const DvmG32&, double,
+                                   double, double, cudaStream_t);
 template <class T>
 cudaError_t launch_moments_vjp(const T*, const T*, const T*, const T*, const T*, T*, const StepParams&,
                                const DvmConst<T>&, cudaStream_t);
@@ -876,10 +877,10 @@ pclb_status pclb_set_state(pclb_ctx* ctx, const void* rho, const void* u_r, cons
   cudaError_t e;
   if (generic(ctx) && ctx->prec == PCLB_FP32)
     e = gen_launch_set_state<float>(fbuf<float>(ctx, ctx->cur), (const float*)rho, (const float*)u_r,
-                                    (const float*)u_theta, (const float*)T, ctx->sp, ctx->dvmg, ctx->stream);
+                                    (const float*)u_theta, (const float*)T, ctx->sp, ctx->dvmg, dvmg32(ctx), ctx->stream);
   else if (generic(ctx))
     e = gen_launch_set_state<double>(fbuf<double>(ctx, ctx->cur), (const double*)rho, (const double*)u_r,
-                                     (const double*)u_theta, (const double*)T, ctx->sp, ctx->dvmg, ctx->stream);
+                                     (const double*)u_theta, (const double*)T, ctx->sp, ctx->dvmg, dvmg32(ctx), ctx->stream);
   else if (ctx->prec == PCLB_FP32)
     e = launch_set_state<float>(fbuf<float>(ctx, ctx->cur), (const float*)rho, (const float*)u_r,
                                 (const float*)u_theta, (const float*)T, ctx->sp, ctx->dvm32, ctx->stream);
@@ -1014,10 +1015,10 @@ pclb_status pclb_moments(pclb_ctx* ctx, void* rho, void* u_r, void* u_theta, voi
   cudaError_t e;
   if (generic(ctx) && ctx->prec == PCLB_FP32)
     e = gen_launch_moments<float>(fbuf<float>(ctx, ctx->cur), (float*)rho, (float*)u_r, (float*)u_theta,
-                                  (float*)T, ctx->sp, ctx->dvmg, ctx->stream);
+                                  (float*)T, ctx->sp, ctx->dvmg, dvmg32(ctx), ctx->stream);
   else if (generic(ctx))
     e = gen_launch_moments<double>(fbuf<double>(ctx, ctx->cur), (double*)rho, (double*)u_r, (double*)u_theta,
-                                   (double*)T, ctx->sp, ctx->dvmg, ctx->stream);
+                                   (double*)T, ctx->sp, ctx->dvmg, dvmg32(ctx), ctx->stream);
   else if (ctx->prec == PCLB_FP32)
     e = launch_moments<float>(fbuf<float>(ctx, ctx->cur), (float*)rho, (float*)u_r, (float*)u_theta,
                               (float*)T, ctx->sp, ctx->dvm32, ctx->stream);
@@ -1059,9 +1060,9 @@ pclb_status pclb_diagnostics(pclb_ctx* ctx, double* out) {
   cudaError_t e;
   if (generic(ctx))
     e = ctx->prec == PCLB_FP32 ? gen_launch_diagnostics<float>(fbuf<float>(ctx, ctx->cur), partials, dout, ctx->sp,
-                                                               ctx->dvmg, dr, dth, ctx->grid.r_in, ctx->stream)
+                                                               ctx->dvmg, dvmg32(ctx), dr, dth, ctx->grid.r_in, ctx->stream)
                                : gen_launch_diagnostics<double>(fbuf<double>(ctx, ctx->cur), partials, dout,
-                                                                ctx->sp, ctx->dvmg, dr, dth, ctx->grid.r_in,
+                                                                ctx->sp, ctx->dvmg, dvmg32(ctx), dr, dth, ctx->grid.r_in,
                                                                 ctx->stream);
   else
     e = ctx->prec == PCLB_FP32 ? launch_diagnostics<float>(fbuf<float>(ctx, ctx->cur), partials, dout, ctx->sp,
