@@ -37,7 +37,6 @@
 
 #include "device_common.cuh"
 #include "adjoint_common.cuh"
-#include "ghost_cols.cuh"
 #include "f32_state.cuh"
 #include "pclb_internal.h"
 

@@ -129,6 +129,11 @@ __device__ __forceinline__ double recip_newton1(double n) {
   return fma(r, fma(-n, r, 1.0), r);
 }
 
+// 1/x of a node's density or temperature: FP64 by two Newton steps (4 FP64
+// operations; the division takes about 10 and a branch).
+__device__ __forceinline__ float recip_state(float x) { return 1.0f / x; }
+__device__ __forceinline__ double recip_state(double x) { return recip_newton(x); }
+
 __device__ __forceinline__ double recip_refined(double x) {
   // Newton-Raphson step y1 = y0 (2 - x y0) on a single-precision seed.
   double y0 = (double)__frcp_rn((float)x);
@@ -180,6 +185,18 @@ __device__ __forceinline__ NodeState<float> node_moments(const float* f, Stride 
   return st;
 }
 
+// Velocity and temperature from the sums rho, rho u, rho (E + u^2/2).
+__device__ __forceinline__ NodeState<double> node_state64(double s0, double sx, double sy, double se) {
+  const double inv = recip_newton(s0);
+  const double ux = sx * inv, uy = sy * inv;
+  const double E = (se - 0.5 * (sx * ux + sy * uy)) * inv;
+  NodeState<double> st;
+  st.rho = s0; st.ux = ux; st.uy = uy; st.E = E;
+  st.rho_d = s0; st.E_d = E;
+  st.ok = (s0 > 0.0) && (E > 0.0) && isfinite(se) && isfinite(sx) && isfinite(sy);
+  return st;
+}
+
 // FP64 sums over the pairs of opposite directions of each shell: with the
 // octagon's unit vectors (1,0), (s,s), (0,1), (-s,s) a shell takes 22 FP64
 // operations instead of 32 (four per label), and FP64 issue is what bounds
@@ -204,14 +221,7 @@ __device__ __forceinline__ NodeState<double> node_moments(const double* f, Strid
     sy = fma(d.speed[k], fma(c, D[1] + D[3], D[2]), sy);
     se = fma(d.half_v2[k], S, se);
   }
-  const double inv = 1.0 / s0;
-  const double ux = sx * inv, uy = sy * inv;
-  const double E = (se - 0.5 * (sx * ux + sy * uy)) * inv;
-  NodeState<double> st;
-  st.rho = s0; st.ux = ux; st.uy = uy; st.E = E;
-  st.rho_d = s0; st.E_d = E;
-  st.ok = (s0 > 0.0) && (E > 0.0) && isfinite(se) && isfinite(sx) && isfinite(sy);
-  return st;
+  return node_state64(s0, sx, sy, se);
 }
 
 // ---------------------------------------------------------------------------
@@ -325,7 +335,7 @@ __device__ __forceinline__ EqParams<T> eq_params(double rho, T ux, T uy, double 
   EqParams<T> p;
   shell_weights(rho, E, d, p.w);
   const T Ef = (T)E;
-  const T invE = T(1) / Ef;
+  const T invE = recip_state(Ef);
   const T u2E = (ux * ux + uy * uy) * invE;   // u^2 / E
   p.a1 = T(1) - T(0.5) * u2E;
   p.a0 = p.a1 + T(0.125) * u2E * u2E;

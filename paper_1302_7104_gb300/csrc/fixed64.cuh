@@ -1,0 +1,119 @@
+// FP64 values as 64-bit fixed-point numbers, for the FP64 step's sums,
+// differences and convection increments.
+//
+// GB300 starts one warp-wide FP64 operation per quarter SM every 64-76
+// cycles (measured), while 64-bit integer sums take 4, 32 x 32 -> 64-bit
+// products 5 and float operations about 1.  A distribution value f is held as
+// x = f 2^(1081 - ek), |x| < 2^59, with ek the largest biased exponent of its
+// shell in the tile's window: one unit is at most 2^-58 of the largest value,
+// finer than the double's own spacing for every value within 2^-5 of it, where
+// the conversion is exact.  Sums and differences of these numbers are exact;
+// products drop less than two units.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace pclb {
+
+// Exponents for which fx_to_double stays inside the normal range; NaN and
+// infinity (0x7ff) are outside.
+constexpr int kFxMinExp = 128, kFxMaxExp = 1900;
+
+// f as fixed point; its biased exponent must not exceed ek.
+__device__ __forceinline__ int64_t fx_from_double(double f, int ek) {
+  const int hi = __double2hiint(f);
+  const uint32_t mh = ((uint32_t)hi & 0xfffffu) | 0x100000u;
+  uint64_t m = ((uint64_t)mh << 32 | (uint32_t)__double2loint(f)) << 6;
+  m >>= min(ek - ((hi >> 20) & 0x7ff), 63);
+  const int64_t s = hi >> 31;
+  return (int64_t)(m ^ s) - s;
+}
+
+// The double nearest x 2^(ek - 1081) (|x| < 2^63).
+__device__ __forceinline__ double fx_to_double(int64_t x, int ek) {
+  const int64_t s = x >> 63;
+  uint64_t u = (uint64_t)((x ^ s) - s);
+  const int lz = __clzll((long long)u);
+  u <<= lz & 63;                                        // leading bit at 63
+  const uint64_t r = (u >> 11) + ((u >> 10) & 1);       // 53 bits, the carry runs into the exponent
+  const uint32_t hi = (uint32_t)(r >> 32) + ((uint32_t)(ek + 4 - lz) << 20) + ((uint32_t)s & 0x80000000u);
+  return u == 0 ? 0.0 : __hiloint2double((int)hi, (int)(uint32_t)r);
+}
+
+// c in [0, 1] as a fraction in units of 2^-63 (c < 2^-960 counts as 0).
+__device__ __forceinline__ uint64_t fx_fraction(double c) {
+  const int hi = __double2hiint(c);
+  const uint32_t mh = ((uint32_t)hi & 0xfffffu) | 0x100000u;
+  const uint64_t m = ((uint64_t)mh << 32 | (uint32_t)__double2loint(c)) << 11;   // 2^63 <= m < 2^64
+  const int sh = 1023 - (hi >> 20);                     // c = m 2^-63 2^-sh
+  const uint64_t one = 1ull << 63, x = sh > 63 ? 0 : m >> sh;
+  return x < one ? x : one;
+}
+
+// a c 2^-63 for a < 2^61, c <= 2^63 (below the exact product by less than 2).
+__device__ __forceinline__ uint64_t fx_mul(uint64_t a, uint64_t c) {
+  const uint32_t al = (uint32_t)a, ah = (uint32_t)(a >> 32), cl = (uint32_t)c, ch = (uint32_t)(c >> 32);
+  const uint64_t mid = (uint64_t)al * ch + (uint64_t)ah * cl;
+  return (uint64_t)(2u * ah) * ch + (mid >> 31);
+}
+
+// a c 2^-63 for fractions a, c <= 2^63.
+__device__ __forceinline__ uint64_t fx_mul_frac(uint64_t a, uint64_t c) {
+  const uint32_t al = (uint32_t)a, ah = (uint32_t)(a >> 32), cl = (uint32_t)c, ch = (uint32_t)(c >> 32);
+  const uint64_t mid = (uint64_t)al * ch + (uint64_t)ah * cl;   // < 2^64: the low words are below 2^32
+  return 2 * ((uint64_t)ah * ch) + (mid >> 31);
+}
+
+__device__ __forceinline__ uint64_t fx_abs(int64_t x) {
+  const int64_t s = x >> 63;
+  return (uint64_t)((x ^ s) - s);
+}
+__device__ __forceinline__ int64_t fx_signed(uint64_t a, int64_t s) { return ((int64_t)a ^ s) - s; }   // s: 0 or -1
+
+__device__ __forceinline__ float fx_float(uint64_t u) {
+  return fmaf(__uint2float_rn((uint32_t)(u >> 32)), 4294967296.0f, __uint2float_rn((uint32_t)u));
+}
+__device__ __forceinline__ float fx_float(int64_t x) {
+  return fmaf(__int2float_rn((int32_t)(x >> 32)), 4294967296.0f, __uint2float_rn((uint32_t)x));
+}
+
+// Courant data of one direction, alpha = |C|: M(D, Dp) = D (alpha^2 + 2 K v)
+// with K = alpha (1 - alpha) and v = |D| / (|D| + |Dp|) where D and Dp have one
+// sign, v = 1 where they have not (Eq. 28: a D + K |D| (D - Dp)/(|D| + |Dp|)).
+struct FxCourant {
+  uint64_t a2;    // alpha^2, units 2^-63
+  uint64_t k40;   // 2 K rounded down to units of 2^-40
+  float k2, klo;  // 2 K 2^29, and what k40 leaves off, times 2^52
+};
+
+__device__ __forceinline__ FxCourant fx_courant(uint64_t alpha) {
+  FxCourant c;
+  c.a2 = fx_mul_frac(alpha, alpha);
+  const uint64_t k = 2 * (alpha - c.a2);
+  c.k40 = k >> 23;
+  c.k2 = __uint2float_rn((uint32_t)(k >> 32)) * 0.25f;
+  c.klo = __uint2float_rn((uint32_t)k & 0x7fffffu) * 0.00048828125f;
+  return c;
+}
+
+// M of Eq. (28) in upwind form, |D|, |Dp| < 2^60.  v is formed to ~2^-46: a
+// float quotient rounded to i0 2^-23, its exact integer remainder, and the
+// remainder's float quotient.  Where D = 0 the quotients may be anything (0 / 0):
+// the result is c |D| = 0 in integers.
+__device__ __forceinline__ int64_t fx_mwb(int64_t D, int64_t Dp, const FxCourant& c) {
+  const int64_t s = D >> 63;
+  const uint64_t a = (uint64_t)((D ^ s) - s), n = a + fx_abs(Dp);
+  const uint64_t num = (int32_t)((uint32_t)(D >> 32) ^ (uint32_t)(Dp >> 32)) < 0 ? n : a;
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fx_float(n)));
+  const float v0 = fx_float(num) * r;
+  const uint32_t i0 = __float_as_uint(__fadd_rn(v0, 1.0f)) - 0x3f800000u;   // v0 in units of 2^-23, rounded
+  const int64_t rem = (int64_t)((num << 23) - n * (uint64_t)i0);            // |rem| <= 4 n < 2^63
+  const float q = fx_float(rem) * r;                                        // the rest of v, units of 2^-23
+  const int32_t i1 = __float2int_rn(fmaf(c.k2, q, c.klo * v0));             // units of 2^-52
+  const uint64_t coef = c.a2 + c.k40 * (uint64_t)i0 + (uint64_t)((int64_t)i1 * 2048);
+  return fx_signed(fx_mul(a, coef), s);
+}
+
+}  // namespace pclb

@@ -318,9 +318,27 @@ pclb_status encode_node_map(pclb_ctx* ctx, const void* base, CUtensorMap* out) {
   return encode_map(ctx, base, kAdjRows32, out, kTileR);
 }
 
-pclb_status make_tmap(pclb_ctx* ctx, int which) {
-  return encode_map(ctx, ctx->ws + ctx->lay.f[which], ctx->prec == PCLB_FP32 ? kTileT32 + 4 : kWinT,
-                    &ctx->tmap[which]);
+// Tile rows of the FP64 MWB step: small tiles while the chip could not be
+// filled with large ones (152 SMs, one CTA each).
+int step_tile_rows(const pclb_grid* g, pclb_precision prec) {
+  const long long tiles = (long long)((g->n_r + kTileR - 1) / kTileR) * ((g->n_theta + kTileT - 1) / kTileT);
+  return prec == PCLB_FP64 && tiles <= kSmallGridTiles64 ? kTileTSmall : kTileT;
+}
+
+// Window rows of the step's TMA boxes: the small tiles are the FP64 MWB
+// step's only (the other schemes run 16-row tiles).
+int step_box_rows(const pclb_ctx* ctx) {
+  if (ctx->prec == PCLB_FP32) return kTileT32 + 4;
+  return (ctx->scheme == PCLB_SCHEME_MWB ? ctx->sp.tile_rows : kTileT) + 4;
+}
+
+// Both f buffers' descriptors for the current scheme.
+pclb_status make_tmaps(pclb_ctx* ctx) {
+  for (int w = 0; w < 2; ++w) {
+    const pclb_status st = encode_map(ctx, ctx->ws + ctx->lay.f[w], step_box_rows(ctx), &ctx->tmap[w]);
+    if (st != PCLB_OK) return st;
+  }
+  return PCLB_OK;
 }
 
 pclb_status bounded_sync(pclb_ctx* ctx, int timeout_ms) {
@@ -792,6 +810,7 @@ pclb_status pclb_create(const pclb_grid* grid, const pclb_dvm* dvm, double tau, 
   sp.dt_dth = dt / dth;
   sp.decay = std::exp(-dt / tau);
   sp.scheme = PCLB_SCHEME_MWB;
+  sp.tile_rows = step_tile_rows(grid, prec);
   sp.wait_ns = kDefaultWaitNs;
   sp.bc_kind[0] = bc->kind[0];
   sp.bc_kind[1] = bc->kind[1];
@@ -835,10 +854,10 @@ pclb_status pclb_create(const pclb_grid* grid, const pclb_dvm* dvm, double tau, 
   ctx->cur_lam = 0;
   ctx->has_lam = false;
   const size_t adj_bufs[5] = {lay.f[0], lay.f[1], lay.adj_f, lay.lam[0], lay.lam[1]};
-  for (int w = 0; w < 7; ++w) {
-    pclb_status s2 = w < 2 ? make_tmap(ctx, w)
-                           : encode_map(ctx, ctx->ws + adj_bufs[w - 2], adj_box_rows(ctx), &ctx->tmap_adj[w - 2]);
-    if (s2 == PCLB_OK && w >= 2) s2 = encode_node_map(ctx, ctx->ws + adj_bufs[w - 2], &ctx->tmap_node[w - 2]);
+  for (int w = 0; w < 6; ++w) {
+    pclb_status s2 = w == 0 ? make_tmaps(ctx)
+                            : encode_map(ctx, ctx->ws + adj_bufs[w - 1], adj_box_rows(ctx), &ctx->tmap_adj[w - 1]);
+    if (s2 == PCLB_OK && w >= 1) s2 = encode_node_map(ctx, ctx->ws + adj_bufs[w - 1], &ctx->tmap_node[w - 1]);
     if (s2 != PCLB_OK) {
       std::snprintf(g_err, sizeof(g_err), "%s", ctx->err);
       delete ctx;
@@ -954,7 +973,7 @@ pclb_status pclb_step_states(pclb_ctx* ctx, const void* f_from, void* f_to) {
                             ctx->stream);
   } else {
     CUtensorMap map;
-    pclb_status st = encode_map(ctx, f_from, ctx->prec == PCLB_FP32 ? kTileT32 + 4 : kWinT, &map);
+    pclb_status st = encode_map(ctx, f_from, step_box_rows(ctx), &map);
     if (st != PCLB_OK) return st;
     e = ctx->prec == PCLB_FP32 ? launch_step_f32(&map, (float*)f_to, ctx->sp, ctx->dvm32, ctx->stream)
                                : launch_step<double>(&map, (double*)f_to, ctx->sp, ctx->dvm64, ctx->stream);
@@ -1222,7 +1241,7 @@ pclb_status pclb_set_scheme(pclb_ctx* ctx, int32_t scheme, int32_t relaxation) {
   ctx->relaxation = relaxation;
   ctx->sp.scheme = scheme;
   ctx->sp.decay = relaxation == PCLB_RELAX_EULER ? 1.0 - ctx->dt / ctx->tau : std::exp(-ctx->dt / ctx->tau);
-  return PCLB_OK;
+  return make_tmaps(ctx);   // the FP64 schemes differ in their tiles
 }
 
 pclb_status pclb_set_wait_limit(pclb_ctx* ctx, uint64_t limit_ns) {

@@ -1,5 +1,6 @@
-// Fused time step of the polar-coordinate FDLB model: one launch advances
-// every node by the combined scheme of Eq. (38).
+// Fused FP64 time step of the polar-coordinate FDLB model with the compared
+// convection schemes (Sec. II B 3): one launch advances every node by the
+// combined scheme of Eq. (38).  The MWB step is step_kernel_f64.cu.
 //
 // Tile work (one CTA = kTileR x kTileT interior nodes):
 //   1. one thread issues 33 TMA box copies (one per velocity plane) of the
@@ -8,13 +9,11 @@
 //   2. every thread computes the moments (Eqs. 3-5) of its node(s) and
 //      factors their equilibrium (Eqs. 10-11);
 //   3. CTAs whose window covers a wall compute the radial ghost columns in
-//      shared memory: moments of the two wall nodes, Eq. (39) extrapolation
-//      (or prescribed values), f = f^eq (Sec. II C 1) -- ghosts never touch
-//      global memory;
+//      shared memory (ghost_cols.cuh) -- ghosts never touch global memory;
 //   4. for every pair of opposite velocities (sharing their Courant entry,
 //      staged per tile row in shared memory, and the even and odd parts of
 //      the equilibrium polynomial): relaxation (Eq. 19) minus the convection
-//      increments (Eq. 28 or the compared schemes) in r and theta read from
+//      increments (the compared schemes) in r and theta read from
 //      the window, stored straight to the output; rows next to the azimuthal
 //      seam are also written into the output's ghost rows (Eq. 40, label
 //      rotated by N_f) so the next step's window is one contiguous box.
@@ -40,26 +39,15 @@ static_assert((kPlane * 4) % 128 == 0, "TMA destinations must stay 128-byte alig
 
 template <class T>
 constexpr int step_smem_bytes() {
-  // planes, Courant table [pair][row] of 4 values, barrier slot
-  return kQ * kPlane * (int)sizeof(T) + kPairs64 * kTileT * 4 * (int)sizeof(T) + 128;
+  // planes, Courant table [pair][row] of 4 values, ghost columns' scratch, barrier slot
+  return (kQ * kPlane + kPairs64 * kTileT * 4 + kGhostScratch64<kTileT>) * (int)sizeof(T) + 128;
 }
 
 // Convection increment (upwind form, see device_common.cuh) from
 // a = |C| and K = a (1 - a) given by the Courant table.
-// Limiter part of the MWB increment, h = |D| (D - Dp) / (|D| + |Dp|), 0 when
-// D = Dp = 0.  One Newton step on the reciprocal: h then carries a relative
-// error <= 1e-12, i.e. K h <= 2.5e-13 |D| (K <= 1/4) in the update.
-__device__ __forceinline__ double mwb_h(double D, double Dp) {
-  const double den = fabs(D) + fabs(Dp);
-  // den >= 2^-1022 (the smallest normal number), tested on the high word of
-  // the non-negative den with an integer compare (keeps the FP64 pipe free)
-  return __double2hiint(den) >= 0x00100000 ? fabs(D) * (D - Dp) * recip_newton1(den) : 0.0;
-}
-
 template <int SCH>
 __device__ __forceinline__ double convect_aK(double a, double K, double f0, double u1, double u2, double d1) {
   const double D = f0 - u1, Dp = u1 - u2;
-  if (SCH == PCLB_SCHEME_MWB) return a * D + K * mwb_h(D, Dp);
   if (SCH == PCLB_SCHEME_WB) return a * D + 0.5 * K * (D - Dp);
   if (SCH == PCLB_SCHEME_UPWIND2) return a * D + 0.5 * a * (D - Dp);
   return a * D + 0.5 * K * ((d1 - f0) - D);
@@ -72,7 +60,8 @@ __global__ void __launch_bounds__(kThreads64, 1)
   extern __shared__ __align__(128) unsigned char smem_raw[];
   T* sm = reinterpret_cast<T*>(smem_raw);
   T* tab = sm + kQ * kPlane;                           // [pair][row][a_r, k_r, a_w, flags]
-  uint64_t* bar = reinterpret_cast<uint64_t*>(tab + kPairs64 * kTileT * 4);
+  T* scratch = tab + kPairs64 * kTileT * 4;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(scratch + kGhostScratch64<kTileT>);
 
   const int r0 = blockIdx.x * kTileR;
   const int t0 = (blockIdx.y + ty0) * kTileT;   // ty0: first tile row of the launch
@@ -135,20 +124,14 @@ __global__ void __launch_bounds__(kThreads64, 1)
   if (!ok) atomicOr(p.status, PCLB_FLAG_NONPHYS);
 
   // ---- 3. radial ghost columns (inside the window only) -------------------
-  if (r0 == 0 && warp == 0 && lane < kTileT) {
-    const int tt = t0 + lane;
-    if (tt < p.n_theta) fill_ghost_columns<T, kPlane>(sm, 2 + lane, 0, kLeft, tt, p, d);
-  }
-  const int cw_out = p.n_r - 1 - r0 + kLeft;   // window column of the outer wall node
-  if (cw_out + 1 <= kLeft + kTileR + 1 && warp == 1 && lane < kTileT) {
-    const int tt = t0 + lane;
-    if (tt < p.n_theta) fill_ghost_columns<T, kPlane>(sm, 2 + lane, 1, cw_out, tt, p, d);
-  }
-  __syncthreads();
+  if (r0 == 0 || p.n_r - 1 - r0 <= kTileR)
+    ghost_columns_f64<kTileT, kPlane>(sm, scratch, r0, t0, p, d);
+  else
+    __syncthreads();
 
   // ---- 4. relaxation minus MWB increments, per pair of opposite velocities --
   const T inv_r = (r < p.n_r) ? (T)p.inv_r[r] : T(1);
-  const T decay = (T)p.decay, omd = T(1) - decay;
+  const T decay = (T)p.decay;
   const size_t plane_out = (size_t)p.rows * p.pitch;
   auto store = [&](int q, int c, T out) {
     T* dst = f_out + (size_t)q * plane_out + r;
@@ -187,37 +170,17 @@ __global__ void __launch_bounds__(kThreads64, 1)
         const T x = vx * eq[c].uxE + vy * eq[c].uyE, x2 = x * x;
         const T ev = eq[c].a0 + x2 * (eq[c].a1h + x2 * T(1.0 / 24.0));
         const T od = x * (eq[c].a1 + x2 * T(1.0 / 6.0));
-        const T fe1 = SCH == PCLB_SCHEME_MWB ? T(0) : eq[c].w[k] * (ev + od);
-        const T fe2 = SCH == PCLB_SCHEME_MWB ? T(0) : eq[c].w[k] * (ev - od);
+        const T fe1 = eq[c].w[k] * (ev + od), fe2 = eq[c].w[k] * (ev - od);
         const T* fp1 = sm + q1 * kPlane + row[c] * kWinR + col;
         const T* fp2 = sm + q2 * kPlane + row[c] * kWinR + col;
         const bool lw = SCH == PCLB_SCHEME_LW;
         const T a = fp1[0], b = fp2[0];
-        T o1, o2;
-        if constexpr (SCH == PCLB_SCHEME_MWB) {
-          // relaxation minus a D + K h in r and theta, as one chain of fused
-          // multiply-adds
-          // (1 - d) f^eq + d f0 = (1 - d) rho F_k P + d f0
-          const T wd = omd * eq[c].w[k];
-          auto mwb = [&](T f0, T P, const T* fp, int s_r, int s_t) {
-            const T u1 = fp[s_r], v1 = fp[s_t];
-            const T Dr = f0 - u1, Dt = f0 - v1;
-            T o = fma(wd, P, decay * f0);
-            o = fma(-ar, Dr, o);
-            o = fma(-kr, mwb_h(Dr, u1 - fp[2 * s_r]), o);
-            o = fma(-at, Dt, o);
-            return fma(-kt, mwb_h(Dt, v1 - fp[2 * s_t]), o);
-          };
-          o1 = mwb(a, ev + od, fp1, sr, st);
-          o2 = mwb(b, ev - od, fp2, -sr, -st);
-        } else {
-          o1 = fe1 + (a - fe1) * decay -
-               convect_aK<SCH>(ar, kr, a, fp1[sr], fp1[2 * sr], lw ? fp1[-sr] : T(0)) -
-               convect_aK<SCH>(at, kt, a, fp1[st], fp1[2 * st], lw ? fp1[-st] : T(0));
-          o2 = fe2 + (b - fe2) * decay -
-               convect_aK<SCH>(ar, kr, b, fp2[-sr], fp2[-2 * sr], lw ? fp2[sr] : T(0)) -
-               convect_aK<SCH>(at, kt, b, fp2[-st], fp2[-2 * st], lw ? fp2[st] : T(0));
-        }
+        const T o1 = fe1 + (a - fe1) * decay -
+                     convect_aK<SCH>(ar, kr, a, fp1[sr], fp1[2 * sr], lw ? fp1[-sr] : T(0)) -
+                     convect_aK<SCH>(at, kt, a, fp1[st], fp1[2 * st], lw ? fp1[-st] : T(0));
+        const T o2 = fe2 + (b - fe2) * decay -
+                     convect_aK<SCH>(ar, kr, b, fp2[-sr], fp2[-2 * sr], lw ? fp2[sr] : T(0)) -
+                     convect_aK<SCH>(at, kt, b, fp2[-st], fp2[-2 * st], lw ? fp2[st] : T(0));
         store(q1, c, o1);
         store(q2, c, o2);
       }
@@ -239,8 +202,12 @@ static cudaError_t launch_scheme(const CUtensorMap* tmap_in, T* f_out, const Ste
   return cudaGetLastError();
 }
 
-// Tile rows [ty_begin, ty_end) of the grid (ty_end < 0: to the last tile row);
-// an empty range launches nothing.
+cudaError_t launch_step_f64_mwb(const CUtensorMap*, double*, const StepParams&, const DvmConst<double>&, cudaStream_t,
+                                int, int);
+
+// Tile rows [ty_begin, ty_end) of the grid, kTileT nodes each (ty_end < 0: to
+// the last tile row); an empty range launches nothing.  tmap_in: boxes of
+// step_box_rows(p, scheme) window rows.
 template <class T>
 cudaError_t launch_step(const CUtensorMap* tmap_in, T* f_out, const StepParams& p,
                         const DvmConst<T>& d, cudaStream_t stream, int ty_begin, int ty_end) {
@@ -251,7 +218,7 @@ cudaError_t launch_step(const CUtensorMap* tmap_in, T* f_out, const StepParams& 
     case PCLB_SCHEME_LW: return launch_scheme<T, PCLB_SCHEME_LW>(tmap_in, f_out, p, d, stream, ty_begin, ty_end);
     case PCLB_SCHEME_UPWIND2:
       return launch_scheme<T, PCLB_SCHEME_UPWIND2>(tmap_in, f_out, p, d, stream, ty_begin, ty_end);
-    default: return launch_scheme<T, PCLB_SCHEME_MWB>(tmap_in, f_out, p, d, stream, ty_begin, ty_end);
+    default: return launch_step_f64_mwb(tmap_in, f_out, p, d, stream, ty_begin, ty_end);
   }
 }
 

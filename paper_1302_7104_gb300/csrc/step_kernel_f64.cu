@@ -1,0 +1,361 @@
+// Fused FP64 time step (Eq. 38 with the MWB increments of Eq. 28): one launch
+// advances every node.  The other convection schemes run step_kernel.cu.
+//
+// What bounds it: FP64 issue.  A quarter SM starts one warp-wide FP64
+// operation per 64-76 cycles (measured), so the ~34 FP64 operations per update
+// of a plain evaluation took 34 ms on 4096 x 4096, where HBM needs 1.3 ms.
+// Everything that is a sum, a difference or a convection increment is
+// therefore done in 64-bit fixed point (fixed64.cuh) on the integer and float
+// pipes; FP64 keeps the node state, the equilibrium factors and the final
+// sums (~7 operations per update), so results keep double precision.
+//
+// Tile work (one CTA, 512 threads; kTileR x TT nodes, 16 / TT warps per row):
+//   1. one thread issues 33 TMA box copies (one per velocity plane) of the
+//      window [r0-4, r0+36) x [t0-2, t0+TT+2) into shared memory;
+//   2. tiles at a wall form the radial ghost columns in the window, in FP64
+//      (ghost_cols.cuh);
+//   3. the block finds the largest exponent of each shell's planes and
+//      converts the window in place to fixed point;
+//   4. the sums of Eqs. 3-5 per shell as integers, then the node state and the
+//      equilibrium factors in FP64;
+//   5. per pair of opposite velocities: d f - M_r - M_theta in fixed point,
+//      turned to double once, plus (1 - d) f^eq in FP64; rows next to the
+//      azimuthal seam also store the output's ghost rows (Eq. 40).
+// A tile whose window holds NaN or infinity, exponents near the ends of the
+// range, a node that is not physical, or densities more than 2^8 below the
+// largest value (the fixed-point unit would be coarse for them) is loaded
+// again and evaluated in FP64 throughout.
+//
+// TT = 16: one thread per node, for grids that fill the chip with such tiles.
+// TT = 4: the four shells of a row on four warps, for small grids, where the
+// time of one tile is the time of the step.
+#include <cuda.h>
+#include <cuda_runtime.h>
+
+#include "device_common.cuh"
+#include "fixed64.cuh"
+#include "ghost_cols.cuh"
+#include "pclb_internal.h"
+
+namespace pclb {
+
+namespace {
+
+constexpr int kThreadsFx = 512;
+constexpr int kPairsFx = 4 * kNDirs / 2;   // pairs of opposite velocities
+constexpr int kHalfDirs = kNDirs / 2;
+constexpr int kGroupsFx = 5;               // exponent groups: the rest plane and the four shells
+
+struct FxTab {
+  FxCourant r;      // radial
+  uint64_t at;      // |C_theta| at the tile's first column, units 2^-63
+  int fl, pad;      // bit 0: v_r < 0, bit 1: v_theta < 0 for the first label of the pair
+};
+
+template <int TT>
+struct FxSize {
+  static constexpr int split = 16 / TT;                       // warps per row
+  static constexpr int plane = kWinR * (TT + 4);
+  static constexpr int planes_bytes = kQ * plane * 8;
+  static constexpr int tab_bytes = kPairsFx * TT * (int)sizeof(FxTab);
+  static constexpr int ghost_bytes = kGhostScratch64<TT> * 8;
+  // split > 1: per node the shells' sums (S, X, Y), then w_1..4, w_0, a0, a1, u/E, rho
+  static constexpr int node_bytes = split > 1 ? 32 * TT * 12 * 8 : 0;
+  static constexpr int scratch = ghost_bytes > node_bytes ? ghost_bytes : node_bytes;
+  static constexpr int smem = planes_bytes + tab_bytes + scratch + 128;
+  static_assert((plane * 8) % 128 == 0, "TMA destinations must stay 128-byte aligned");
+  static_assert(smem <= 232448, "shared memory of one CTA");
+};
+
+// The pairs of one node in FP64 throughout, for the tiles described above: w
+// the node in the window (doubles), planes PLANE apart.
+template <int PLANE, class Store>
+__device__ __noinline__ void general_node(const double* w, const EqParams<double>& eq, const double* courant, double inv_r,
+                                          double decay, const DvmConst<double>& d, Store store) {
+  const double omd = 1.0 - decay;
+#pragma unroll 1
+  for (int pair = 0; pair < kPairsFx; ++pair) {
+    const int k = 1 + pair / kHalfDirs, q1 = 1 + (k - 1) * kNDirs + pair % kHalfDirs, q2 = q1 + kHalfDirs;
+    const double* e = courant + pair * 4;
+    const double ar = e[0], kr = e[1], at = e[2] * inv_r, kt = at - at * at;
+    const int fl = (int)e[3], sr = (fl & 1) ? 1 : -1, st = (fl & 2) ? kWinR : -kWinR;
+    const double x = d.vx[q1] * eq.uxE + d.vy[q1] * eq.uyE, x2 = x * x;
+    const double ev = eq.a0 + x2 * (eq.a1h + x2 * (1.0 / 24.0)), od = x * (eq.a1 + x2 * (1.0 / 6.0));
+    const double wd = omd * eq.w[k];
+    auto mwb = [&](const double* fp, double P, int s_r, int s_t) {
+      // |D| (D - Dp) / (|D| + |Dp|), small differences scaled up by a power of two
+      auto h = [](double D, double Dp) {
+        const bool small = fmax(fabs(D), fabs(Dp)) < 0x1p-500;
+        if (small) { D *= 0x1p+500; Dp *= 0x1p+500; }
+        const double den = fabs(D) + fabs(Dp);
+        const double v = den >= 0x1p-1000 ? fabs(D) * recip_newton1(den) * (D - Dp) : 0.0;
+        return small ? v * 0x1p-500 : v;
+      };
+      const double f0 = fp[0], u1 = fp[s_r], v1 = fp[s_t], Dr = f0 - u1, Dt = f0 - v1;
+      double o = fma(wd, P, decay * f0);
+      o = fma(-ar, Dr, o);
+      o = fma(-kr, h(Dr, u1 - fp[2 * s_r]), o);
+      o = fma(-at, Dt, o);
+      return fma(-kt, h(Dt, v1 - fp[2 * s_t]), o);
+    };
+    store(q1, mwb(w + (size_t)q1 * PLANE, ev + od, sr, st));
+    store(q2, mwb(w + (size_t)q2 * PLANE, ev - od, -sr, -st));
+  }
+}
+
+}  // namespace
+
+template <int TT>
+__global__ void __launch_bounds__(kThreadsFx, 1)
+    step_kernel_f64(const __grid_constant__ CUtensorMap tmap_in, double* __restrict__ f_out,
+                    const __grid_constant__ StepParams p, const __grid_constant__ DvmConst<double> d, int ty0) {
+  using SZ = FxSize<TT>;
+  constexpr int PLANE = SZ::plane, SPLIT = SZ::split;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  double* sm = reinterpret_cast<double*>(smem_raw);
+  int64_t* fx = reinterpret_cast<int64_t*>(smem_raw);
+  FxTab* tab = reinterpret_cast<FxTab*>(smem_raw + SZ::planes_bytes);                      // [pair][row]
+  double* scratch = reinterpret_cast<double*>(smem_raw + SZ::planes_bytes + SZ::tab_bytes);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + SZ::planes_bytes + SZ::tab_bytes + SZ::scratch);
+  int* top = reinterpret_cast<int*>(bar + 2);   // [kGroupsFx] largest high words
+
+  const int r0 = blockIdx.x * kTileR;
+  const int t0 = (blockIdx.y + ty0) * TT;   // ty0: first tile row of the launch
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+
+  auto load = [&](uint64_t* b) {   // thread 0: window rows [t0-2, t0+TT+2) are stored rows [t0, t0+TT+4)
+    mbar_arrive_expect_tx(b, (uint32_t)(kQ * PLANE * 8));
+#pragma unroll 1
+    for (int q = 0; q < kQ; ++q) tma_load_3d(sm + q * PLANE, &tmap_in, r0 - kLeft, t0, q, b);
+  };
+  if (tid == 0) {
+    tma_prefetch_desc(&tmap_in);
+    mbar_init(&bar[0], 1);
+    mbar_init(&bar[1], 1);
+    mbar_fence_init();
+    load(&bar[0]);
+  }
+  const double inv_r0 = p.inv_r[r0];
+  if (tid < kPairsFx * TT) {   // Courant entries of the tile rows
+    const int pair = tid / TT, rl = tid % TT;
+    const double* e = p.courant64 + ((size_t)(min(t0 + rl, p.n_theta - 1) + kGhostRows) * kPairsFx + pair) * 4;
+    FxTab t;
+    t.r = fx_courant(fx_fraction(e[0]));
+    t.at = fx_fraction(e[2] * inv_r0);
+    t.fl = (int)e[3];
+    t.pad = 0;
+    tab[pair * TT + rl] = t;
+  }
+  if (tid < kGroupsFx) top[tid] = 0;
+  // The whole block gives the tile up if any thread's wait ran out (block
+  // barriers follow, so the decision must be uniform); thread 0 then gives
+  // the copies one more bounded chance to land before the block exits.
+  __syncthreads();
+  auto wait = [&](uint64_t* b) {
+    if (__syncthreads_or(p.wait_ns == 0 || !mbar_wait_bounded(b, 0, p.wait_ns))) {   // 0: give up at once
+      if (tid == 0) {
+        atomicOr(p.status, PCLB_FLAG_TIMEOUT);
+        mbar_wait_bounded(b, 0, kDefaultWaitNs);
+      }
+      return false;
+    }
+    return true;
+  };
+  if (!wait(&bar[0])) return;
+
+  const bool wall_tile = r0 == 0 || p.n_r - 1 - r0 <= kTileR;
+  if (wall_tile) ghost_columns_f64<TT, PLANE>(sm, scratch, r0, t0, p, d);
+
+  // ---- largest exponent of each shell, then the window in fixed point --------
+  {
+    const int* hi = reinterpret_cast<const int*>(sm) + 1;
+#pragma unroll
+    for (int g = 0; g < kGroupsFx; ++g) {
+      const int first = g == 0 ? 0 : (1 + (g - 1) * kNDirs) * PLANE, n = g == 0 ? PLANE : kNDirs * PLANE;
+      int m = 0;
+      for (int i = tid; i < n; i += kThreadsFx) m = max(m, hi[2 * (first + i)] & 0x7fffffff);
+      m = __reduce_max_sync(0xffffffffu, (unsigned)m);
+      if (lane == 0) atomicMax(&top[g], m);
+    }
+  }
+  __syncthreads();
+  int ek[kGroupsFx];
+  bool general = false;
+  double most = 0.0;   // bound of the values in the window
+#pragma unroll
+  for (int g = 0; g < kGroupsFx; ++g) {
+    ek[g] = top[g] >> 20;
+    general = general || ek[g] < kFxMinExp || ek[g] > kFxMaxExp;
+    most = fmax(most, __hiloint2double(top[g] & 0x7ff00000, 0));
+  }
+  if (!general) {
+#pragma unroll
+    for (int g = 0; g < kGroupsFx; ++g) {
+      const int first = g == 0 ? 0 : (1 + (g - 1) * kNDirs) * PLANE, n = g == 0 ? PLANE : kNDirs * PLANE;
+      for (int i = tid; i < n; i += kThreadsFx) fx[first + i] = fx_from_double(sm[first + i], ek[g]);
+    }
+  }
+  __syncthreads();
+
+  // ---- the node state and the equilibrium factors ------------------------------
+  const int rl = warp % TT, split = warp / TT;   // tile row; the shells of this warp
+  const int r = r0 + lane, t = t0 + rl;
+  const int node = (rl + 2) * kWinR + kLeft + lane;
+  const bool valid = r < p.n_r && t < p.n_theta;
+  const double decay = p.decay;
+  EqParams<double> eq;
+  double f0 = 0.0;
+  // the sums S, X = sum c_x f, Y of shell k
+  auto shell_sums = [&](int k, double o[3]) {
+    const int64_t* f = fx + (1 + (k - 1) * kNDirs) * PLANE + node;
+    int64_t S = 0, D[kHalfDirs];
+#pragma unroll
+    for (int i = 0; i < kHalfDirs; ++i) {
+      const int64_t a = f[i * PLANE], b = f[(i + kHalfDirs) * PLANE];
+      S += a + b;
+      D[i] = a - b;
+    }
+    const int e = k == 1 ? ek[1] : (k == 2 ? ek[2] : (k == 3 ? ek[3] : ek[4]));
+    const double c = d.cx[2];
+    o[0] = fx_to_double(S, e);
+    o[1] = fma(c, fx_to_double(D[1] - D[3], e), fx_to_double(D[0], e));
+    o[2] = fma(c, fx_to_double(D[1] + D[3], e), fx_to_double(D[2], e));
+  };
+  auto factors = [&](const NodeState<double>& m) {
+    eq = valid ? eq_params<double>(m.rho, m.ux, m.uy, m.E, d) : eq_params<double>(1.0, 0.0, 0.0, 1.0, d);
+    // not physical, or more than 2^8 below the window's largest value: too coarse a unit
+    if (valid && !(m.ok && m.rho >= most * 0.00390625)) general = true;
+  };
+  if constexpr (SPLIT == 1) {
+    if (!general) {
+      f0 = fx_to_double(fx[node], ek[0]);
+      double s0 = f0, sx = 0.0, sy = 0.0, se = 0.0;
+#pragma unroll 1
+      for (int k = 1; k <= 4; ++k) {
+        double s[3];
+        shell_sums(k, s);
+        s0 += s[0];
+        sx = fma(d.speed[k], s[1], sx);
+        sy = fma(d.speed[k], s[2], sy);
+        se = fma(d.half_v2[k], s[0], se);
+      }
+      factors(node_state64(s0, sx, sy, se));
+    }
+  } else {
+    // shell split + 1 by this warp, the state by the row's first warp
+    double* part = scratch + (rl * 32 + lane) * 12;
+    if (!general) shell_sums(split + 1, part + 3 * split);
+    __syncthreads();
+    if (!general && split == 0) {
+      f0 = fx_to_double(fx[node], ek[0]);
+      double s0 = f0, sx = 0.0, sy = 0.0, se = 0.0;
+#pragma unroll
+      for (int k = 1; k <= 4; ++k) {
+        s0 += part[3 * (k - 1)];
+        sx = fma(d.speed[k], part[3 * (k - 1) + 1], sx);
+        sy = fma(d.speed[k], part[3 * (k - 1) + 2], sy);
+        se = fma(d.half_v2[k], part[3 * (k - 1)], se);
+      }
+      factors(node_state64(s0, sx, sy, se));
+#pragma unroll
+      for (int k = 1; k <= 4; ++k) part[k - 1] = eq.w[k];
+      part[4] = eq.a0; part[5] = eq.a1; part[6] = eq.uxE; part[7] = eq.uyE;
+    }
+    __syncthreads();
+    if (!general && split > 0) {
+#pragma unroll
+      for (int k = 1; k <= 4; ++k) eq.w[k] = part[k - 1];
+      eq.a0 = part[4]; eq.a1 = part[5]; eq.uxE = part[6]; eq.uyE = part[7];
+    }
+  }
+  general = __syncthreads_or(general);
+
+  // ---- output ------------------------------------------------------------------
+  const size_t plane_out = (size_t)p.rows * p.pitch;
+  double* out = f_out + (size_t)(t + kGhostRows) * p.pitch + r;
+  auto store = [&](int q, double v) {
+    out[(size_t)q * plane_out] = v;
+    if (t >= p.n_theta - 2)   // also the low ghost rows (theta <= 0) of the receiving label
+      f_out[(size_t)d.recv_lo[q] * plane_out + (size_t)(t - (p.n_theta - 2)) * p.pitch + r] = v;
+    if (t < 2)                // and the high ghost rows (theta > 2 pi n_f / n_dirs)
+      f_out[(size_t)d.recv_hi[q] * plane_out + (size_t)(p.n_theta + kGhostRows + t) * p.pitch + r] = v;
+  };
+  if (general) {   // the window again, as doubles
+    if (tid == 0) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      load(&bar[1]);
+    }
+    if (!wait(&bar[1])) return;
+    if (wall_tile) ghost_columns_f64<TT, PLANE>(sm, scratch, r0, t0, p, d);
+    if (split != 0 || !valid) return;
+    const NodeState<double> m = node_moments(sm + node, PLANE, d);
+    if (!m.ok) atomicOr(p.status, PCLB_FLAG_NONPHYS);
+    eq = eq_params<double>(m.rho, m.ux, m.uy, m.E, d);
+    const double fe = eq.w[0] * eq.a0;
+    store(0, fe + (sm[node] - fe) * decay);
+    general_node<PLANE>(sm + node, eq, p.courant64 + (size_t)(t + kGhostRows) * kPairsFx * 4, p.inv_r[r], decay, d, store);
+    return;
+  }
+  if (!valid) return;
+  const double omd = 1.0 - decay;
+  if (split == 0) {   // rest velocity: no convection
+    const double fe = eq.w[0] * eq.a0;
+    store(0, fe + (f0 - fe) * decay);
+  }
+  const uint64_t dfx = fx_fraction(fabs(decay));
+  const int64_t dsign = decay < 0.0 ? -1 : 0;
+  const uint64_t ratio = fx_fraction(p.inv_r[r] * recip_newton(inv_r0));   // 1/r relative to the tile's first column
+  const double c45 = d.cx[2];
+  const double y1 = c45 * (eq.uyE + eq.uxE), y3 = c45 * (eq.uyE - eq.uxE);
+#pragma unroll 1
+  for (int k = SPLIT == 1 ? 1 : split + 1; k <= (SPLIT == 1 ? 4 : split + 1); ++k) {
+    const int e = k == 1 ? ek[1] : (k == 2 ? ek[2] : (k == 3 ? ek[3] : ek[4]));
+    // (1 - d) f^eq of the shell's pairs: ev +- od, ev = A + y^2 (B + y^2 C), od = y (O1 + y^2 O3)
+    const double w = omd * (k == 1 ? eq.w[1] : (k == 2 ? eq.w[2] : (k == 3 ? eq.w[3] : eq.w[4])));
+    const double hv = d.half_v2[k], wv = w * d.speed[k], wh = w * hv;
+    const double A = w * eq.a0, B = wh * eq.a1, C = wh * (hv * (1.0 / 6.0)), O1 = wv * eq.a1, O3 = wv * (hv * (1.0 / 3.0));
+#pragma unroll 1
+    for (int i = 0; i < kHalfDirs; ++i) {
+      const int q1 = 1 + (k - 1) * kNDirs + i, q2 = q1 + kHalfDirs;
+      const FxTab& te = tab[((k - 1) * kHalfDirs + i) * TT + rl];
+      const FxCourant cr = te.r, ct = fx_courant(fx_mul_frac(te.at, ratio));
+      const int fl = te.fl;
+      const int sr = (fl & 1) ? 1 : -1;               // v_r < 0 for q1: upwind at larger r
+      const int st = (fl & 2) ? kWinR : -kWinR;       // v_theta < 0 for q1: upwind at larger theta
+      // d f - M_r - M_theta of a label whose upwind neighbours sit at s_r and s_t
+      auto carried = [&](const int64_t* x, int s_r, int s_t) {
+        const int64_t x0 = x[0], u1 = x[s_r], u2 = x[2 * s_r], v1 = x[s_t], v2 = x[2 * s_t];
+        const int64_t keep = fx_signed(fx_mul(fx_abs(x0), dfx), (x0 >> 63) ^ dsign);
+        return fx_to_double(keep - fx_mwb(x0 - u1, u1 - u2, cr) - fx_mwb(x0 - v1, v1 - v2, ct), e);
+      };
+      const double g1 = carried(fx + q1 * PLANE + node, sr, st), g2 = carried(fx + q2 * PLANE + node, -sr, -st);
+      const double y = i == 0 ? eq.uxE : (i == 1 ? y1 : (i == 2 ? eq.uyE : y3)), y2 = y * y;
+      const double ev = fma(y2, fma(y2, C, B), A), z = fma(y2, O3, O1);
+      store(q1, fma(y, z, ev + g1));
+      store(q2, fma(-y, z, ev + g2));
+    }
+  }
+}
+
+template <int TT>
+static cudaError_t launch_tile_rows(const CUtensorMap* tmap_in, double* f_out, const StepParams& p,
+                                    const DvmConst<double>& d, cudaStream_t stream, int ty_begin, int ty_end) {
+  static std::atomic<unsigned long long> configured{0};   // per instantiation and device
+  const cudaError_t e = set_smem_once(step_kernel_f64<TT>, FxSize<TT>::smem, configured);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((p.n_r + kTileR - 1) / kTileR, ty_end - ty_begin);
+  step_kernel_f64<TT><<<grid, kThreadsFx, FxSize<TT>::smem, stream>>>(*tmap_in, f_out, p, d, ty_begin);
+  return cudaGetLastError();
+}
+
+// Tile rows [ty_begin, ty_end) of kTileT nodes each.
+cudaError_t launch_step_f64_mwb(const CUtensorMap* tmap_in, double* f_out, const StepParams& p,
+                                const DvmConst<double>& d, cudaStream_t stream, int ty_begin, int ty_end) {
+  if (p.tile_rows == kTileT) return launch_tile_rows<kTileT>(tmap_in, f_out, p, d, stream, ty_begin, ty_end);
+  constexpr int per = kTileT / kTileTSmall;
+  const int last = (p.n_theta + kTileTSmall - 1) / kTileTSmall;
+  return launch_tile_rows<kTileTSmall>(tmap_in, f_out, p, d, stream, ty_begin * per,
+                                       ty_end * per < last ? ty_end * per : last);
+}
+
+}  // namespace pclb

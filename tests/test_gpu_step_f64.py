@@ -1,0 +1,96 @@
+"""The FP64 step in fixed point (step_kernel_f64.cu): its tiles of 4 and 16
+rows, the edges of its grid rule, and the states that leave fixed point
+(thin gas beside dense gas in one tile, magnitudes near the ends of the double
+range, NaN), against the oracle.
+
+Tolerance: 1e-12 of max|f| per step, as the other FP64 parity tests; a state
+scaled by a power of two scales the result exactly in the oracle, so scaled
+cases use the same relative tolerance.
+"""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_1302_7104_gb300 import inputs as I
+from paper_1302_7104_gb300 import pclb as P
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def _noisy(w, seed=3, noise=0.01):
+    f = O.set_state(w)
+    return np.ascontiguousarray(f * (1.0 + noise * np.random.default_rng(seed).normal(size=f.shape)))
+
+
+def _step(w, f, n=1):
+    with P.PCLB(w, precision="fp64") as g:
+        got = g.set_f(torch.as_tensor(f, device="cuda")).step(n).get_f().cpu().numpy()
+        return got, g.status_flags()
+
+
+# 32 x 16-node tiles: up to 76 of them take tiles of 4 rows
+@pytest.mark.parametrize("n_r,n_t", [(3, 2), (33, 4), (32, 5), (35, 17), (64, 608), (64, 609), (2432, 16), (2433, 17),
+                                     (31, 1217)])
+@pytest.mark.parametrize("bc", [(I.BC_EXTRAP, I.BC_EXTRAP), (I.BC_WALL | I.BC_NEQ, I.BC_DIRICHLET | I.BC_NEQ)])
+def test_step_matches_oracle_at_the_edges_of_the_tile_rule(n_r, n_t, bc):
+    w = I.random_smooth(n_r, n_t, seed=n_r + n_t, bc_kind=bc, amp=0.02 if n_r < 8 else 0.2)
+    f = _noisy(w)
+    got, _ = _step(w, f, 2)
+    want = O.run(w, f, 2)
+    assert np.max(np.abs(got - want)) <= 2e-12 * np.max(np.abs(want))
+
+
+def _contrast(w, ratio):
+    """Density falling by `ratio` across the middle of a 32-node tile."""
+    w.rho = np.where(np.arange(w.n_r) < 16, 1.0, 1.0 / ratio) * np.ones_like(w.rho)
+    return w
+
+
+@pytest.mark.parametrize("n_t", [40, 1300])            # tiles of 4 and of 16 rows
+@pytest.mark.parametrize("ratio", [200.0, 300.0, 1e6, 1e12])
+def test_thin_gas_beside_dense_gas_keeps_its_own_precision(n_t, ratio):
+    """Every node to 1e-12 of its own row's scale: the thin side (radial nodes
+    20..31, four nodes off the jump) against the largest value there."""
+    w = _contrast(I.random_smooth(64, n_t, seed=5), ratio)
+    f = _noisy(w)
+    got, _ = _step(w, f)
+    want = O.run(w, f, 1)
+    assert np.max(np.abs(got - want)) <= 1e-12 * np.max(np.abs(want))
+    thin = np.s_[:, :, 20:32]
+    assert np.max(np.abs(got[thin] - want[thin])) <= 1e-12 * np.max(np.abs(want[thin]))
+
+
+@pytest.mark.parametrize("n_t", [24, 1300])
+@pytest.mark.parametrize("scale", [2.0 ** -1000, 2.0 ** -880, 2.0 ** -300, 2.0 ** 300, 2.0 ** 860, 2.0 ** 1000])
+def test_states_of_any_magnitude(n_t, scale):
+    w = I.random_smooth(40, n_t, seed=6)
+    f = _noisy(w)
+    got, flags = _step(w, f * scale)
+    want = O.run(w, f, 1)
+    assert flags == 0
+    assert np.max(np.abs(got / scale - want)) <= 1e-12 * np.max(np.abs(want))
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+def test_non_finite_values_stay_local_and_are_flagged(bad):
+    w = I.random_smooth(100, 40, seed=7)
+    f = _noisy(w)
+    f[5, 20, 50] = bad
+    got, flags = _step(w, f)
+    assert flags & P.FLAG_NONPHYS
+    want = O.run(w, np.where(np.isfinite(f), f, 0.1), 1)
+    far = np.ones(f.shape, dtype=bool)
+    far[:, 18:23, 48:53] = False
+    assert not np.isfinite(got[5, 20, 50])
+    assert np.max(np.abs(got[far] - want[far])) <= 1e-12 * np.max(np.abs(want))
+
+
+def test_zero_planes_and_equal_neighbours():
+    """A shell that is exactly zero, and a uniform state (every difference 0)."""
+    w = I.uniform(70, 24)
+    f = O.set_state(w)
+    f[9:17] = 0.0
+    got, _ = _step(w, f)
+    want = O.run(w, f, 1)
+    assert np.max(np.abs(got - want)) <= 1e-12 * np.max(np.abs(want))
