@@ -185,6 +185,13 @@ __device__ __forceinline__ NodeState<float> node_moments(const float* f, Stride 
   return st;
 }
 
+// x > 0 and isfinite(x) on the bit patterns (an FP64 compare costs an FP64 issue slot).
+__device__ __forceinline__ bool positive64(double x) {
+  const long long b = __double_as_longlong(x);
+  return b > 0 && b <= 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool finite64(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+
 // Velocity and temperature from the sums rho, rho u, rho (E + u^2/2).
 __device__ __forceinline__ NodeState<double> node_state64(double s0, double sx, double sy, double se) {
   const double inv = recip_newton(s0);
@@ -193,7 +200,7 @@ __device__ __forceinline__ NodeState<double> node_state64(double s0, double sx, 
   NodeState<double> st;
   st.rho = s0; st.ux = ux; st.uy = uy; st.E = E;
   st.rho_d = s0; st.E_d = E;
-  st.ok = (s0 > 0.0) && (E > 0.0) && isfinite(se) && isfinite(sx) && isfinite(sy);
+  st.ok = positive64(s0) && positive64(E) && finite64(se) && finite64(sx) && finite64(sy);
   return st;
 }
 
@@ -364,12 +371,12 @@ __device__ __forceinline__ EqShells64 eq_shells(const EqParams<double>& e, const
   EqShells64 g;
 #pragma unroll
   for (int k = 1; k <= 4; ++k) {
-    const double v = d.speed[k], hv = d.half_v2[k], wv = e.w[k] * v, wh = e.w[k] * hv;
+    const double wa = e.w[k] * e.a1;
     g.A[k - 1] = e.w[k] * e.a0;
-    g.B[k - 1] = wh * e.a1;                        // w v^2 a1 / 2
-    g.C[k - 1] = wh * (hv * (1.0 / 6.0));          // w v^4 / 24
-    g.O1[k - 1] = wv * e.a1;
-    g.O3[k - 1] = wv * (hv * (1.0 / 3.0));         // w v^3 / 6
+    g.B[k - 1] = wa * d.half_v2[k];
+    g.C[k - 1] = e.w[k] * d.v4_24[k];
+    g.O1[k - 1] = wa * d.speed[k];
+    g.O3[k - 1] = e.w[k] * d.v3_6[k];
   }
   const double c = d.cx[2];   // 1 / sqrt 2; directions (1,0), (s,s), (0,1), (-s,s)
   g.y[0] = e.uxE;

@@ -184,6 +184,8 @@ void fill_dvm(DvmConst<T>& c, const pclb_dvm& d, const pclb_grid& g) {
     c.speed_lo[k] = (T)(d.speeds[k] - (double)c.speed[k]);
     c.half_v2[k] = (T)hv2;
     c.half_v2_lo[k] = (T)(hv2 - (double)c.half_v2[k]);
+    c.v3_6[k] = (T)(d.speeds[k] * hv2 / 3.0);
+    c.v4_24[k] = (T)(hv2 * hv2 / 6.0);
   }
   c.B0 = (T)d.B[0];
   {

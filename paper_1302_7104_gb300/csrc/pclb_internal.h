@@ -55,6 +55,7 @@ struct DvmConst {
   T cx[kQ], cy[kQ];           // unit direction (cos phi_i, sin phi_i); 0 for q = 0
   T speed[5];                 // v_k
   T half_v2[5];               // v_k^2 / 2
+  T v3_6[5], v4_24[5];        // v_k^3 / 6, v_k^4 / 24
   T Fc[5][4];                 // F_k(E) = sum_{n=1..4} Fc[k][n-1] E^n, k = 1..4 (Eq. 11a)
   T Fc_lo[5][4];              // Fc - (double)Fc rounded to T: the low part of a float-float pair
   // Low parts (value - (double)hi, rounded to T) of the velocity constants, so

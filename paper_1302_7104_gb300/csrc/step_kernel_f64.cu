@@ -181,12 +181,12 @@ __global__ void __launch_bounds__(kThreadsFx, 1)
   __syncthreads();
   int ek[kGroupsFx];
   bool general = false;
-  double most = 0.0;   // bound of the values in the window
+  int most = 0;   // high word of the largest value in the window
 #pragma unroll
   for (int g = 0; g < kGroupsFx; ++g) {
     ek[g] = top[g] >> 20;
     general = general || ek[g] < kFxMinExp || ek[g] > kFxMaxExp;
-    most = fmax(most, __hiloint2double(top[g] & 0x7ff00000, 0));
+    most = max(most, top[g]);
   }
   if (!general) {
 #pragma unroll
@@ -202,10 +202,10 @@ __global__ void __launch_bounds__(kThreadsFx, 1)
   const int r = r0 + lane, t = t0 + rl;
   const int node = (rl + 2) * kWinR + kLeft + lane;
   const bool valid = r < p.n_r && t < p.n_theta;
-  const double decay = p.decay;
+  const double decay = p.decay, omd = 1.0 - decay;
   EqParams<double> eq;
   double f0 = 0.0;
-  // the sums S, X = sum c_x f, Y of shell k
+  // the sums S, X = sum c_x f, Y of shell k (1 / sqrt 2 as a fraction of 2^63)
   auto shell_sums = [&](int k, double o[3]) {
     const int64_t* f = fx + (1 + (k - 1) * kNDirs) * PLANE + node;
     int64_t S = 0, D[kHalfDirs];
@@ -216,15 +216,16 @@ __global__ void __launch_bounds__(kThreadsFx, 1)
       D[i] = a - b;
     }
     const int e = k == 1 ? ek[1] : (k == 2 ? ek[2] : (k == 3 ? ek[3] : ek[4]));
-    const double c = d.cx[2];
+    auto diagonal = [](int64_t x) { return fx_signed(fx_mul(fx_abs(x), 0x5a827999fcef3242ull), x >> 63); };
     o[0] = fx_to_double(S, e);
-    o[1] = fma(c, fx_to_double(D[1] - D[3], e), fx_to_double(D[0], e));
-    o[2] = fma(c, fx_to_double(D[1] + D[3], e), fx_to_double(D[2], e));
+    o[1] = fx_to_double(D[0] + diagonal(D[1] - D[3]), e);
+    o[2] = fx_to_double(D[2] + diagonal(D[1] + D[3]), e);
   };
+  // factors of (1 - d) f^eq: w_k = (1 - d) rho F_k
   auto factors = [&](const NodeState<double>& m) {
-    eq = valid ? eq_params<double>(m.rho, m.ux, m.uy, m.E, d) : eq_params<double>(1.0, 0.0, 0.0, 1.0, d);
+    eq = valid ? eq_params<double>(omd * m.rho, m.ux, m.uy, m.E, d) : eq_params<double>(1.0, 0.0, 0.0, 1.0, d);
     // not physical, or more than 2^8 below the window's largest value: too coarse a unit
-    if (valid && !(m.ok && m.rho >= most * 0.00390625)) general = true;
+    if (valid && !(m.ok && __double2hiint(m.rho) >= most - (8 << 20))) general = true;
   };
   if constexpr (SPLIT == 1) {
     if (!general) {
@@ -297,26 +298,27 @@ __global__ void __launch_bounds__(kThreadsFx, 1)
     return;
   }
   if (!valid) return;
-  const double omd = 1.0 - decay;
-  if (split == 0) {   // rest velocity: no convection
-    const double fe = eq.w[0] * eq.a0;
-    store(0, fe + (f0 - fe) * decay);
-  }
+  if (split == 0) store(0, fma(decay, f0, eq.w[0] * eq.a0));   // rest velocity: no convection
   const uint64_t dfx = fx_fraction(fabs(decay));
   const int64_t dsign = decay < 0.0 ? -1 : 0;
   const uint64_t ratio = fx_fraction(p.inv_r[r] * recip_newton(inv_r0));   // 1/r relative to the tile's first column
   const double c45 = d.cx[2];
   const double y1 = c45 * (eq.uyE + eq.uxE), y3 = c45 * (eq.uyE - eq.uxE);
+  // A pair's results are stored one pair later, so that the FP64 pipe works
+  // on them beside the next pair's integer part.
+  int q_last = 0;
+  double o1, o2;
 #pragma unroll 1
   for (int k = SPLIT == 1 ? 1 : split + 1; k <= (SPLIT == 1 ? 4 : split + 1); ++k) {
     const int e = k == 1 ? ek[1] : (k == 2 ? ek[2] : (k == 3 ? ek[3] : ek[4]));
     // (1 - d) f^eq of the shell's pairs: ev +- od, ev = A + y^2 (B + y^2 C), od = y (O1 + y^2 O3)
-    const double w = omd * (k == 1 ? eq.w[1] : (k == 2 ? eq.w[2] : (k == 3 ? eq.w[3] : eq.w[4])));
-    const double hv = d.half_v2[k], wv = w * d.speed[k], wh = w * hv;
-    const double A = w * eq.a0, B = wh * eq.a1, C = wh * (hv * (1.0 / 6.0)), O1 = wv * eq.a1, O3 = wv * (hv * (1.0 / 3.0));
+    const double w = k == 1 ? eq.w[1] : (k == 2 ? eq.w[2] : (k == 3 ? eq.w[3] : eq.w[4])), wa = w * eq.a1;
+    const double A = w * eq.a0, B = wa * d.half_v2[k], C = w * d.v4_24[k], O1 = wa * d.speed[k], O3 = w * d.v3_6[k];
 #pragma unroll 1
     for (int i = 0; i < kHalfDirs; ++i) {
       const int q1 = 1 + (k - 1) * kNDirs + i, q2 = q1 + kHalfDirs;
+      const double y = i == 0 ? eq.uxE : (i == 1 ? y1 : (i == 2 ? eq.uyE : y3)), y2 = y * y;
+      const double ev = fma(y2, fma(y2, C, B), A), z = fma(y2, O3, O1);
       const FxTab& te = tab[((k - 1) * kHalfDirs + i) * TT + rl];
       const FxCourant cr = te.r, ct = fx_courant(fx_mul_frac(te.at, ratio));
       const int fl = te.fl;
@@ -329,12 +331,17 @@ __global__ void __launch_bounds__(kThreadsFx, 1)
         return fx_to_double(keep - fx_mwb(x0 - u1, u1 - u2, cr) - fx_mwb(x0 - v1, v1 - v2, ct), e);
       };
       const double g1 = carried(fx + q1 * PLANE + node, sr, st), g2 = carried(fx + q2 * PLANE + node, -sr, -st);
-      const double y = i == 0 ? eq.uxE : (i == 1 ? y1 : (i == 2 ? eq.uyE : y3)), y2 = y * y;
-      const double ev = fma(y2, fma(y2, C, B), A), z = fma(y2, O3, O1);
-      store(q1, fma(y, z, ev + g1));
-      store(q2, fma(-y, z, ev + g2));
+      if (q_last) {
+        store(q_last, o1);
+        store(q_last + kHalfDirs, o2);
+      }
+      o1 = fma(y, z, ev + g1);
+      o2 = fma(-y, z, ev + g2);
+      q_last = q1;
     }
   }
+  store(q_last, o1);
+  store(q_last + kHalfDirs, o2);
 }
 
 template <int TT>
