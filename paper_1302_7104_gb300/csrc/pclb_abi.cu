@@ -320,18 +320,18 @@ pclb_status encode_node_map(pclb_ctx* ctx, const void* base, CUtensorMap* out) {
   return encode_map(ctx, base, kAdjRows32, out, kTileR);
 }
 
-// Tile rows of the FP64 MWB step: small tiles while the chip could not be
-// filled with large ones (152 SMs, one CTA each).
-int step_tile_rows(const pclb_grid* g, pclb_precision prec) {
+// Tile rows of the octagon's step: small tiles while the chip (152 SMs) could
+// not be filled with large ones.
+int step_tile_rows(const pclb_grid* g, const pclb_dvm* d, pclb_precision prec) {
   const long long tiles = (long long)((g->n_r + kTileR - 1) / kTileR) * ((g->n_theta + kTileT - 1) / kTileT);
-  return prec == PCLB_FP64 && tiles <= kSmallGridTiles64 ? kTileTSmall : kTileT;
+  return d->n_dirs == kNDirs && tiles <= (prec == PCLB_FP64 ? kSmallGridTiles64 : kSmallGridTiles32) ? kTileTSmall
+                                                                                                     : kTileT;
 }
 
-// Window rows of the step's TMA boxes: the small tiles are the FP64 MWB
-// step's only (the other schemes run 16-row tiles).
+// Window rows of the step's TMA boxes (in FP64 the small tiles are the MWB
+// step's only, the other schemes run 16-row tiles).
 int step_box_rows(const pclb_ctx* ctx) {
-  if (ctx->prec == PCLB_FP32) return kTileT32 + 4;
-  return (ctx->scheme == PCLB_SCHEME_MWB ? ctx->sp.tile_rows : kTileT) + 4;
+  return (ctx->prec == PCLB_FP32 || ctx->scheme == PCLB_SCHEME_MWB ? ctx->sp.tile_rows : kTileT) + 4;
 }
 
 // Both f buffers' descriptors for the current scheme.
@@ -812,7 +812,7 @@ pclb_status pclb_create(const pclb_grid* grid, const pclb_dvm* dvm, double tau, 
   sp.dt_dth = dt / dth;
   sp.decay = std::exp(-dt / tau);
   sp.scheme = PCLB_SCHEME_MWB;
-  sp.tile_rows = step_tile_rows(grid, prec);
+  sp.tile_rows = step_tile_rows(grid, dvm, prec);
   sp.wait_ns = kDefaultWaitNs;
   sp.bc_kind[0] = bc->kind[0];
   sp.bc_kind[1] = bc->kind[1];

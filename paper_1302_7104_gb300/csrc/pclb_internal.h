@@ -28,8 +28,9 @@ constexpr int kTileT = 16;
 constexpr int kTileT32 = 16;
 constexpr int kStepThreads32 = 16 * kTileT32;
 constexpr int kCtasPerSm32 = 2;
-constexpr int kTileTSmall = 4;      // FP64 step on small grids (step_kernel_f64.cu)
-constexpr int kSmallGridTiles64 = 76;   // at most this many 32 x 16 tiles: small tiles
+constexpr int kTileTSmall = 4;      // the steps of the octagon on small grids
+// at most this many 32 x 16 tiles: small tiles
+constexpr int kSmallGridTiles64 = 76, kSmallGridTiles32 = 76;
 constexpr int kWinR = kTileR + 8;   // 40 columns
 constexpr int kWinT = kTileT + 4;   // 20 rows
 constexpr int kLeft = 4;            // column of interior r0 inside the window
@@ -105,7 +106,7 @@ struct StepParams {
   const double* courant64;    // the same table in double: [n_theta + 4][pairs][4] (flags as value)
   const float* inv_r_f;       // [n_r] 1 / r_i in float
   const float4* cs_ff;        // [n_theta] cos theta_i, sin theta_i as float-float pairs (hi, lo, hi, lo)
-  int tile_rows;              // tile rows of the FP64 step, kTileT or kTileTSmall
+  int tile_rows;              // tile rows of the step, kTileT or kTileTSmall
   uint32_t* status;           // device status word (PCLB_FLAG_*)
   uint64_t wait_ns;           // a step's wait for its own window copies before it gives the tile up
 };
@@ -144,6 +145,25 @@ inline cudaError_t set_smem_once(F* fn, int bytes, std::atomic<unsigned long lon
   e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess && bit) done.fetch_or(bit, std::memory_order_release);
   return e;
+}
+
+// Launches fn so that its start overlaps the end of the kernel before it on
+// the stream (programmatic dependent launch): fn calls pdl_wait() before it
+// touches anything that kernel reads or writes.
+template <class... P, class... A>
+inline cudaError_t launch_overlapped(void (*fn)(P...), dim3 grid, int threads, int smem, cudaStream_t stream,
+                                     const A&... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, fn, args...);
 }
 
 size_t adjoint_scratch_bytes(int n_theta, int elem);

@@ -1,9 +1,9 @@
 // Fused FP32 time step of the polar-coordinate FDLB model (Eq. 38), the hot
 // kernel of the library.
 //
-// Work per CTA: a tile of 32 (r) x 16 (theta) nodes, 256 threads.  One thread
+// Work per CTA: a tile of 32 (r) x TT (theta) nodes, 256 threads.  One thread
 // issues 33 TMA box copies (one per velocity plane) of the window
-// [r0-4, r0+36) x [t0-2, t0+18) into shared memory, in four groups with a
+// [r0-4, r0+36) x [t0-2, t0+TT+2) into shared memory, in four groups with a
 // barrier each (rest + shell 1, shells 2, 3, 4), while the others copy the
 // tile's rows of the host-computed Courant table.  Each thread then owns two
 // radially adjacent nodes of one row and processes them together with packed
@@ -12,7 +12,7 @@
 //     (Eqs. 11a-b) in float-float arithmetic, so that the rounded equilibrium
 //     keeps the collision invariants of the exact one;
 //   * radial ghost columns for tiles at a wall (Eq. 39, f = f^eq), computed in
-//     shared memory;
+//     shared memory by one warp per wall;
 //   * for every pair (q, q') of opposite velocities of a shell: v_q.u/E from
 //     float-float constants, the even and odd parts of the equilibrium
 //     polynomial (Eq. 10) shared by q and q'; then per velocity the relaxation
@@ -22,6 +22,14 @@
 //     and added once to the relaxed value, so that they cost one rounding at
 //     the magnitude of f instead of four (this halves the FP32 path's drift
 //     from the FP64 one over long runs).
+// TT = 16: one thread per node pair, for grids that fill the chip with such
+// tiles.  TT = 4: four threads per node pair, a shell each (the node state
+// formed by all four), and two warps of their own for the ghost columns; for
+// small grids, where the latency of one tile is the time of the step.  The results
+// do not depend on TT.
+// Consecutive steps overlap their starts: a step's launch, barrier set-up and
+// table rows run while the step before it drains (programmatic dependent
+// launch); its window copies wait for that step.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -36,13 +44,18 @@ namespace pclb {
 namespace {
 
 constexpr int kPairs = 4 * kHalf;                    // 16
-constexpr int kPlaneF = kWinR * (kTileT32 + 4);      // floats per plane window
-constexpr int kPlanesBytes = kQ * kPlaneF * 4;       // 105600
-constexpr int kTabBytes = kPairs * kTileT32 * 16;    // one float4 per (pair, row)
-constexpr int kSmemF32 = kPlanesBytes + kTabBytes + 128;
-// every plane window is a TMA destination: 128-byte aligned (a tile height
-// whose window breaks this faults with a misaligned address)
-static_assert((kPlaneF * 4) % 128 == 0 && kPlanesBytes % 16 == 0, "TMA destinations must stay 128-byte aligned");
+template <int TT>
+struct F32Size {
+  static constexpr int split = 16 / TT;                          // threads per node pair
+  static constexpr int plane = kWinR * (TT + 4);                 // floats per plane window
+  static constexpr int planes_bytes = kQ * plane * 4;            // 105600 for TT = 16
+  static constexpr int tab_bytes = kPairs * TT * 16;             // one float4 per (pair, row)
+  static constexpr int smem = planes_bytes + tab_bytes + 128;
+  static constexpr int threads = kStepThreads32 + (split > 1 ? 64 : 0);   // two warps for the ghost columns
+  // every plane window is a TMA destination: 128-byte aligned (a tile height
+  // whose window breaks this faults with a misaligned address)
+  static_assert((plane * 4) % 128 == 0 && planes_bytes % 16 == 0, "TMA destinations must stay 128-byte aligned");
+};
 constexpr int kGroups = 4;
 __device__ __forceinline__ int group_first(int g) { return g == 0 ? 0 : 1 + g * kNDirs; }
 __device__ __forceinline__ int group_planes(int g) { return g == 0 ? 1 + kNDirs : kNDirs; }
@@ -52,17 +65,17 @@ __device__ __forceinline__ f2 ld2(const float* p) { return *reinterpret_cast<con
 // Sums over one shell (plus, optionally, a second shell added direction by
 // direction) of f, c_x f and c_y f for both nodes, with the octagon's exact
 // unit vectors as float-float constants.
-template <int K, int KADD>
+template <int K, int KADD, int PL>
 __device__ __forceinline__ void shell_sums2(const float* f, f2& S, f2& X, f2& Xl, f2& Y, f2& Yl) {
   S = bc2(0.f); X = bc2(0.f); Xl = bc2(0.f); Y = bc2(0.f); Yl = bc2(0.f);
 #pragma unroll
   for (int i = 0; i < kHalf; ++i) {
     const int q = 1 + (K - 1) * kNDirs + i;
-    f2 fa = ld2(f + q * kPlaneF), fb = ld2(f + (q + kHalf) * kPlaneF);
+    f2 fa = ld2(f + q * PL), fb = ld2(f + (q + kHalf) * PL);
     if (KADD > 0) {
       const int qa = 1 + (KADD - 1) * kNDirs + i;
-      fa = add2(fa, ld2(f + qa * kPlaneF));
-      fb = add2(fb, ld2(f + (qa + kHalf) * kPlaneF));
+      fa = add2(fa, ld2(f + qa * PL));
+      fb = add2(fb, ld2(f + (qa + kHalf) * PL));
     }
     S = add2(S, add2(fa, fb));
     const f2 dd = sub2(fa, fb);
@@ -83,13 +96,13 @@ __device__ __forceinline__ void shell_sums2(const float* f, f2& S, f2& X, f2& Xl
 // Moments (Eqs. 3-5) and temperature recovery of the two nodes.  ready(g)
 // is called before plane group g (the rest plane and shell 1, then shells 2,
 // 3, 4) is first read, so the sums start while later groups still land.
-template <class Ready>
+template <int PL, class Ready>
 __device__ __forceinline__ State2 state2(const float* f, const DvmConst<float>& d, Ready ready) {
   ready(0);
   ff2 rho = ff2_of(ld2(f)), jx = ff2_of(bc2(0.f)), jy = jx, e = jx;
   f2 S, X, Xl, Y, Yl;
   // shell 1
-  shell_sums2<1, 0>(f, S, X, Xl, Y, Yl);
+  shell_sums2<1, 0, PL>(f, S, X, Xl, Y, Yl);
   rho = ff2_add(rho, ff2_of(S));
   jx = ff2_add(jx, ff2_mul(ffc(d.speed[1], d.speed_lo[1]), ff2{X, Xl}));
   jy = ff2_add(jy, ff2_mul(ffc(d.speed[1], d.speed_lo[1]), ff2{Y, Yl}));
@@ -97,19 +110,19 @@ __device__ __forceinline__ State2 state2(const float* f, const DvmConst<float>& 
   // shells 2 + 3 direction by direction, with the speed and v^2/2 of shell 2
   ready(1);
   ready(2);
-  shell_sums2<2, 3>(f, S, X, Xl, Y, Yl);
+  shell_sums2<2, 3, PL>(f, S, X, Xl, Y, Yl);
   rho = ff2_add(rho, ff2_of(S));
   jx = ff2_add(jx, ff2_mul(ffc(d.speed[2], d.speed_lo[2]), ff2{X, Xl}));
   jy = ff2_add(jy, ff2_mul(ffc(d.speed[2], d.speed_lo[2]), ff2{Y, Yl}));
   e = ff2_add(e, ff2_mul(ffc(d.half_v2[2], d.half_v2_lo[2]), ff2_of(S)));
   // shell 3 again with the differences v_3 - v_2, (v_3^2 - v_2^2)/2
-  shell_sums2<3, 0>(f, S, X, Xl, Y, Yl);
+  shell_sums2<3, 0, PL>(f, S, X, Xl, Y, Yl);
   jx = ff2_add(jx, ff2_mul(ffc(d.dv23, d.dv23_lo), ff2{X, Xl}));
   jy = ff2_add(jy, ff2_mul(ffc(d.dv23, d.dv23_lo), ff2{Y, Yl}));
   e = ff2_add(e, ff2_mul(ffc(d.dh23, d.dh23_lo), ff2_of(S)));
   // shell 4
   ready(3);
-  shell_sums2<4, 0>(f, S, X, Xl, Y, Yl);
+  shell_sums2<4, 0, PL>(f, S, X, Xl, Y, Yl);
   rho = ff2_add(rho, ff2_of(S));
   jx = ff2_add(jx, ff2_mul(ffc(d.speed[4], d.speed_lo[4]), ff2{X, Xl}));
   jy = ff2_add(jy, ff2_mul(ffc(d.speed[4], d.speed_lo[4]), ff2{Y, Yl}));
@@ -125,64 +138,72 @@ __device__ __forceinline__ State2 state2(const float* f, const DvmConst<float>& 
   return s;
 }
 
-// Ghost columns of one wall for tile row `row` (window row index), Sec. II C 1.
-__device__ __noinline__ void ghost_columns_f32(float* sm, int row, int side, int cw, int t,
-                                               const StepParams& p, const DvmConst<float>& d) {
+// Ghost columns of one wall (wall node at window column cw) for the tile's TT
+// rows, by one warp, Sec. II C 1: lane (row, node) forms the state of the wall
+// node a or of the next node b, then lane (row, layer) the layer's state and
+// its equilibrium; with TT = 4 the four groups of lanes hold the same states and
+// store a shell each.  (One lane per row forming both states and both layers
+// took about 8 of the 19 us of a small step.)
+template <int TT>
+__device__ __noinline__ void ghost_columns_f32(float* sm, int lane, int side, int cw, int t0, const StepParams& p,
+                                               const DvmConst<float>& d) {
+  constexpr int PL = F32Size<TT>::plane;
   const int step = side == 0 ? 1 : -1;
-  const State32 a = state32(sm + row * kWinR + cw, kPlaneF, d);
-  const State32 b = state32(sm + row * kWinR + cw + step, kPlaneF, d);
-  State32 g[2];
+  const int row = 2 + lane % TT, layer = (lane / TT) & 1, group = lane / (2 * TT);
+  const int t = min(t0 + lane % TT, p.n_theta - 1);
+  const State32 m = state32(sm + row * kWinR + cw + (layer == 0 ? 0 : step), PL, d);
+  // the other node's state (lane a holds a, lane b holds b)
+  auto other = [&](ff x) { return ff{__shfl_xor_sync(0xffffffffu, x.hi, TT), __shfl_xor_sync(0xffffffffu, x.lo, TT)}; };
+  const State32 o{other(m.rho), other(m.ux), other(m.uy), other(m.E),
+                  __shfl_xor_sync(0xffffffffu, (int)m.ok, TT) != 0};
+  const State32 a = layer == 0 ? m : o, b = layer == 0 ? o : m;
   // Eq. (39), applied twice: g0 = 2a - b, g1 = 2 g0 - a = 3a - 2b.
-  g[0].rho = ff_add(ff_scale(a.rho, 2.f), ff_neg(b.rho));
-  g[0].E = ff_add(ff_scale(a.E, 2.f), ff_neg(b.E));
-  g[0].ux = ff_add(ff_scale(a.ux, 2.f), ff_neg(b.ux));
-  g[0].uy = ff_add(ff_scale(a.uy, 2.f), ff_neg(b.uy));
-  g[1].rho = ff_add(ff_scale(g[0].rho, 2.f), ff_neg(a.rho));
-  g[1].E = ff_add(ff_scale(g[0].E, 2.f), ff_neg(a.E));
-  g[1].ux = ff_add(ff_scale(g[0].ux, 2.f), ff_neg(a.ux));
-  g[1].uy = ff_add(ff_scale(g[0].uy, 2.f), ff_neg(a.uy));
+  auto extrapolated = [&](ff xa, ff xb) {
+    const ff g0 = ff_add(ff_scale(xa, 2.f), ff_neg(xb));
+    return layer == 0 ? g0 : ff_add(ff_scale(g0, 2.f), ff_neg(xa));
+  };
+  State32 g;
+  g.rho = extrapolated(a.rho, b.rho);
+  g.E = extrapolated(a.E, b.E);
+  g.ux = extrapolated(a.ux, b.ux);
+  g.uy = extrapolated(a.uy, b.uy);
   const int kind = p.bc_kind[side] & ~PCLB_BC_NEQ;
   const bool neq = (p.bc_kind[side] & PCLB_BC_NEQ) != 0;
   if (kind != PCLB_BC_EXTRAP) {
     const double c = p.cos_t[t], s = p.sin_t[t];
-    for (int layer = 0; layer < 2; ++layer) {
-      const double* v = p.bc_vals + (size_t)((side * 2 + layer) * 4) * p.n_theta + t;
-      const double ur = v[1 * p.n_theta], ut = v[2 * p.n_theta];
-      g[layer].ux = ff_from(ur * c - ut * s);
-      g[layer].uy = ff_from(ur * s + ut * c);
-      if (kind == PCLB_BC_DIRICHLET) {
-        g[layer].rho = ff_from(v[0]);
-        g[layer].E = ff_from(v[3 * p.n_theta]);
-      }
+    const double* v = p.bc_vals + (size_t)((side * 2 + layer) * 4) * p.n_theta + t;
+    const double ur = v[1 * p.n_theta], ut = v[2 * p.n_theta];
+    g.ux = ff_from(ur * c - ut * s);
+    g.uy = ff_from(ur * s + ut * c);
+    if (kind == PCLB_BC_DIRICHLET) {
+      g.rho = ff_from(v[0]);
+      g.E = ff_from(v[3 * p.n_theta]);
     }
   }
-  bool ok = a.ok && b.ok;
+  const int col = cw - step * (1 + layer);
+  if (t0 + lane % TT >= p.n_theta) return;
+  if (!(a.ok && b.ok && g.rho.hi > 0.f && g.E.hi > 0.f)) atomicOr(p.status, PCLB_FLAG_NONPHYS);
+  if (col < 0 || col >= kWinR) return;
   // equilibrium of the wall node, for the departure it hands to its ghosts
   Eq32 ea{};
   if (neq) ea = eq32(a, d);
   const float* fa = sm + row * kWinR + cw;
-  for (int layer = 0; layer < 2; ++layer) {
-    ok = ok && g[layer].rho.hi > 0.f && g[layer].E.hi > 0.f;
-    const int col = cw - step * (1 + layer);
-    if (col < 0 || col >= kWinR) continue;
-    const Eq32 e = eq32(g[layer], d);
-    float* gp = sm + row * kWinR + col;
-    gp[0] = feq32(e, d, 0, 0, 1.f) + (neq ? fa[0] - feq32(ea, d, 0, 0, 1.f) : 0.f);
+  const Eq32 e = eq32(g, d);
+  float* gp = sm + row * kWinR + col;
+  if (group == 0) gp[0] = feq32(e, d, 0, 0, 1.f) + (neq ? fa[0] - feq32(ea, d, 0, 0, 1.f) : 0.f);
 #pragma unroll 1
-    for (int k = 1; k <= 4; ++k)
+  for (int k = TT == 16 ? 1 : group + 1; k <= (TT == 16 ? 4 : group + 1); ++k)
 #pragma unroll
-      for (int i = 0; i < kHalf; ++i) {
-        const int q = 1 + (k - 1) * kNDirs + i;
-        float v1 = feq32(e, d, k, i, 1.f), v2 = feq32(e, d, k, i, -1.f);
-        if (neq) {
-          v1 += fa[q * kPlaneF] - feq32(ea, d, k, i, 1.f);
-          v2 += fa[(q + kHalf) * kPlaneF] - feq32(ea, d, k, i, -1.f);
-        }
-        gp[q * kPlaneF] = v1;
-        gp[(q + kHalf) * kPlaneF] = v2;
+    for (int i = 0; i < kHalf; ++i) {
+      const int q = 1 + (k - 1) * kNDirs + i;
+      float v1 = feq32(e, d, k, i, 1.f), v2 = feq32(e, d, k, i, -1.f);
+      if (neq) {
+        v1 += fa[q * PL] - feq32(ea, d, k, i, 1.f);
+        v2 += fa[(q + kHalf) * PL] - feq32(ea, d, k, i, -1.f);
       }
-  }
-  if (!ok) atomicOr(p.status, PCLB_FLAG_NONPHYS);
+      gp[q * PL] = v1;
+      gp[(q + kHalf) * PL] = v2;
+    }
 }
 
 __device__ __forceinline__ float rcp_approx(float x) {
@@ -202,17 +223,19 @@ __device__ __forceinline__ f2 limiter2(f2 D, f2 Dp) {
 
 }  // namespace
 
-template <int SCH>
-__global__ void __launch_bounds__(kStepThreads32, kCtasPerSm32)
+template <int SCH, int TT>
+__global__ void __launch_bounds__(F32Size<TT>::threads, kCtasPerSm32)
     step_kernel_f32(const __grid_constant__ CUtensorMap tmap_in, float* __restrict__ f_out,
                     const __grid_constant__ StepParams p, const __grid_constant__ DvmConst<float> d, int ty0) {
+  using SZ = F32Size<TT>;
+  constexpr int PL = SZ::plane, SPLIT = SZ::split;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float* sm = reinterpret_cast<float*>(smem_raw);
-  float4* tab = reinterpret_cast<float4*>(smem_raw + kPlanesBytes);
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + kPlanesBytes + kTabBytes);
+  float4* tab = reinterpret_cast<float4*>(smem_raw + SZ::planes_bytes);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + SZ::planes_bytes + SZ::tab_bytes);
 
   const int r0 = blockIdx.x * kTileR;
-  const int t0 = (blockIdx.y + ty0) * kTileT32;   // ty0: first tile row of the launch
+  const int t0 = (blockIdx.y + ty0) * TT;   // ty0: first tile row of the launch
   const int tid = threadIdx.x;
 
   // Thread 0 initialises the barriers and issues the copies at once; the
@@ -222,25 +245,31 @@ __global__ void __launch_bounds__(kStepThreads32, kCtasPerSm32)
     tma_prefetch_desc(&tmap_in);
     for (int g = 0; g < kGroups; ++g) mbar_init(&bar[g], 1);
     mbar_fence_init();
+  }
+  // Courant entries of the tile rows: table layout [pair][row] (read before
+  // the wait: no step writes them)
+  const int te_pair = tid / TT, te_row = tid % TT;
+  float4 te;
+  if (tid < kPairs * TT) te = p.courant[(size_t)(min(t0 + te_row, p.n_theta - 1) + kGhostRows) * kPairs + te_pair];
+  pdl_wait();      // the step before this one has written f and read f_out
+  pdl_launch();    // the next one may start its set-up
+  if (tid == 0) {
 #pragma unroll 1
     for (int g = 0; g < kGroups; ++g) {
       const int q0 = group_first(g), n = group_planes(g);
-      mbar_arrive_expect_tx(&bar[g], (uint32_t)(n * kPlaneF * 4));
+      mbar_arrive_expect_tx(&bar[g], (uint32_t)(n * PL * 4));
 #pragma unroll 1
-      for (int q = q0; q < q0 + n; ++q) tma_load_3d(sm + q * kPlaneF, &tmap_in, r0 - kLeft, t0, q, &bar[g]);
+      for (int q = q0; q < q0 + n; ++q) tma_load_3d(sm + q * PL, &tmap_in, r0 - kLeft, t0, q, &bar[g]);
     }
   }
-  {  // Courant entries of the tile rows: table layout [pair][row]
-    const int pair = tid / kTileT32, rl = tid % kTileT32;
-    const int t = min(t0 + rl, p.n_theta - 1);
-    tab[pair * kTileT32 + rl] = p.courant[(size_t)(t + kGhostRows) * kPairs + pair];
-  }
+  if (tid < kPairs * TT) tab[te_pair * TT + te_row] = te;
   __syncthreads();   // table visible (while the copies are still landing)
   bool ok = true;
 
   // ---- per-thread nodes: row rl, radial cells j2 and j2 + 1 -----------------
   const int warp = tid >> 5, lane = tid & 31;
-  const int rl = 2 * warp + (lane >> 4);          // tile row 0..15
+  const int rl = (2 * warp + (lane >> 4)) % TT;    // tile row
+  const int split = SPLIT == 1 ? 0 : warp / (TT / 2);   // SPLIT > 1: shell split + 1; the two warps after those: ghost columns
   const int j2 = 2 * (lane & 15);                  // even radial offset 0..30
   const int row = rl + 2;                          // window row
   const int col = kLeft + j2;                      // window column of the first node
@@ -250,12 +279,25 @@ __global__ void __launch_bounds__(kStepThreads32, kCtasPerSm32)
   const bool v0 = row_ok && r < p.n_r, v1 = row_ok && r + 1 < p.n_r;
   const float* win = sm + row * kWinR + col;
 
+  const int cw_out = p.n_r - 1 - r0 + kLeft;
+  const bool inner = r0 == 0, outer = cw_out <= kLeft + kTileR;   // tiles at a wall
+  auto ready = [&](int g) {
+    if (ok) ok = p.wait_ns != 0 && mbar_wait_bounded(&bar[g], 0, p.wait_ns);   // 0: give up at once
+  };
+  if constexpr (SPLIT > 1) {
+    if (warp >= kStepThreads32 / 32) {   // the ghost columns' warps: one per wall
+      const int side = warp - kStepThreads32 / 32;
+      if (!inner && !outer) return;
+      for (int g = 0; g < kGroups; ++g) ready(g);
+      if (ok && (side == 0 ? inner : outer)) ghost_columns_f32<TT>(sm, lane, side, side == 0 ? kLeft : cw_out, t0, p, d);
+      __syncthreads_or(!ok);
+      return;
+    }
+  }
+
   Eq2 eq;
   {
-    auto ready = [&](int g) {
-      if (ok) ok = p.wait_ns != 0 && mbar_wait_bounded(&bar[g], 0, p.wait_ns);   // 0: give up at once
-    };
-    State2 s = state2(win, d, ready);
+    State2 s = state2<PL>(win, d, ready);
     const bool ok0 = s.rho.hi.x > 0.f && s.E.hi.x > 0.f && isfinite(s.E.hi.x) && isfinite(s.ux.hi.x) &&
                      isfinite(s.uy.hi.x);
     const bool ok1 = s.rho.hi.y > 0.f && s.E.hi.y > 0.f && isfinite(s.E.hi.y) && isfinite(s.ux.hi.y) &&
@@ -270,12 +312,11 @@ __global__ void __launch_bounds__(kStepThreads32, kCtasPerSm32)
   }
 
   // ---- radial ghost columns (tiles at a wall only) ----------------------------
-  const int cw_out = p.n_r - 1 - r0 + kLeft;
-  if (r0 == 0 || cw_out <= kLeft + kTileR) {
-    if (ok && r0 == 0 && warp == 0 && lane < kTileT32 && t0 + lane < p.n_theta)
-      ghost_columns_f32(sm, 2 + lane, 0, kLeft, t0 + lane, p, d);
-    if (ok && cw_out <= kLeft + kTileR && warp == 1 && lane < kTileT32 && t0 + lane < p.n_theta)
-      ghost_columns_f32(sm, 2 + lane, 1, cw_out, t0 + lane, p, d);
+  if (inner || outer) {
+    if constexpr (SPLIT == 1) {
+      if (ok && inner && warp == 0) ghost_columns_f32<TT>(sm, lane, 0, kLeft, t0, p, d);
+      if (ok && outer && warp == 1) ghost_columns_f32<TT>(sm, lane, 1, cw_out, t0, p, d);
+    }
     if (__syncthreads_or(!ok)) {   // ghost columns visible; a copy that timed out stops the tile
       if (tid == 0) {
         atomicOr(p.status, PCLB_FLAG_TIMEOUT);
@@ -297,7 +338,7 @@ __global__ void __launch_bounds__(kStepThreads32, kCtasPerSm32)
   const size_t plane_out = (size_t)p.rows * p.pitch;
   float* out_row = f_out + (size_t)(t + kGhostRows) * p.pitch + r;
   // tiles away from the radial walls and the seam take the plain store
-  const bool plain_tile = r0 + kTileR <= p.n_r && t0 >= 2 && t0 + kTileT32 <= p.n_theta - 2;
+  const bool plain_tile = r0 + kTileR <= p.n_r && t0 >= 2 && t0 + TT <= p.n_theta - 2;
   auto store = [&](int q, f2 o) {
     if (plain_tile) {
       __stcs(reinterpret_cast<float2*>(out_row + (size_t)q * plane_out), o);   // not read again before the next step
@@ -320,7 +361,7 @@ __global__ void __launch_bounds__(kStepThreads32, kCtasPerSm32)
     }
   };
 
-  {  // rest velocity: no convection
+  if (split == 0) {  // rest velocity: no convection
     const f2 f0 = ld2(win);
     const f2 e0 = mul2(eq.w[0], eq.a0);
     store(0, fma2(sub2(f0, e0), decay, e0));
@@ -333,7 +374,7 @@ __global__ void __launch_bounds__(kStepThreads32, kCtasPerSm32)
   // MWB a D + K h(D, Dp); WB a D + K (D - Dp)/2; LW a D + K (Dd - D)/2 with
   // Dd the downwind difference; second-order upwind a D + a (D - Dp)/2.
   auto update = [&](int q, int sr, int st, f2 nar, f2 nkr, f2 nat, f2 nkt, f2 fe) {
-    const float* w = win + q * kPlaneF;
+    const float* w = win + q * PL;
     const f2 C = ld2(w);
     const f2 S = ld2(w + 2 * sr);                 // (j-2, j-1) or (j+2, j+3)
     const f2 T1 = ld2(w + st * kWinR);
@@ -366,14 +407,14 @@ __global__ void __launch_bounds__(kStepThreads32, kCtasPerSm32)
   // Shells run as a loop (keeps the hot body small for the instruction
   // cache); the four direction pairs of a shell are unrolled.
 #pragma unroll 1
-  for (int k = 1; k <= 4; ++k) {
+  for (int k = SPLIT == 1 ? 1 : split + 1; k <= (SPLIT == 1 ? 4 : split + 1); ++k) {
     const f2 sh = bc2(d.speed[k]), sl = bc2(d.speed_lo[k]);
     const f2 wk = k == 1 ? eq.w[1] : (k == 2 ? eq.w[2] : (k == 3 ? eq.w[3] : eq.w[4]));
     const int qb = 1 + (k - 1) * kNDirs;
 #pragma unroll
     for (int i = 0; i < kHalf; ++i) {
       const int q = qb + i;
-      const float4 tb = tab[((k - 1) * kHalf + i) * kTileT32 + rl];
+      const float4 tb = tab[((k - 1) * kHalf + i) * TT + rl];
       const int fl = __float_as_int(tb.w);
       const int sr = (fl & 1) ? 1 : -1;            // v_r < 0: upwind at larger r
       const int st = (fl & 2) ? 1 : -1;            // v_theta < 0: upwind at larger theta
@@ -388,21 +429,33 @@ __global__ void __launch_bounds__(kStepThreads32, kCtasPerSm32)
   }
 }
 
+template <int SCH, int TT>
+static cudaError_t launch_tile_rows_f32(const CUtensorMap* tmap_in, float* f_out, const StepParams& p,
+                                        const DvmConst<float>& d, cudaStream_t stream, int ty_begin, int ty_end) {
+  static std::atomic<unsigned long long> configured{0};   // per instantiation and device
+  {
+    const cudaError_t e = set_smem_once(step_kernel_f32<SCH, TT>, F32Size<TT>::smem, configured);
+    if (e != cudaSuccess) return e;
+  }
+  const dim3 grid((p.n_r + kTileR - 1) / kTileR, ty_end - ty_begin);
+  return launch_overlapped(step_kernel_f32<SCH, TT>, grid, F32Size<TT>::threads, F32Size<TT>::smem, stream, *tmap_in,
+                           f_out, p, d, ty_begin);
+}
+
 template <int SCH>
 static cudaError_t launch_scheme_f32(const CUtensorMap* tmap_in, float* f_out, const StepParams& p,
                                      const DvmConst<float>& d, cudaStream_t stream, int ty_begin, int ty_end) {
-  static std::atomic<unsigned long long> configured{0};   // per instantiation and device
-  {
-    const cudaError_t e = set_smem_once(step_kernel_f32<SCH>, kSmemF32, configured);
-    if (e != cudaSuccess) return e;
-  }
-  dim3 grid((p.n_r + kTileR - 1) / kTileR, ty_end - ty_begin);
-  step_kernel_f32<SCH><<<grid, kStepThreads32, kSmemF32, stream>>>(*tmap_in, f_out, p, d, ty_begin);
-  return cudaGetLastError();
+  if (p.tile_rows == kTileT32)
+    return launch_tile_rows_f32<SCH, kTileT32>(tmap_in, f_out, p, d, stream, ty_begin, ty_end);
+  constexpr int per = kTileT32 / kTileTSmall;
+  const int last = (p.n_theta + kTileTSmall - 1) / kTileTSmall;
+  return launch_tile_rows_f32<SCH, kTileTSmall>(tmap_in, f_out, p, d, stream, ty_begin * per,
+                                                ty_end * per < last ? ty_end * per : last);
 }
 
-// Tile rows [ty_begin, ty_end) of the grid (ty_end < 0: to the last tile row);
-// an empty range launches nothing.
+// Tile rows [ty_begin, ty_end) of the grid, kTileT32 nodes each (ty_end < 0:
+// to the last tile row); an empty range launches nothing.  tmap_in: boxes of
+// p.tile_rows + 4 window rows.
 cudaError_t launch_step_f32(const CUtensorMap* tmap_in, float* f_out, const StepParams& p,
                             const DvmConst<float>& d, cudaStream_t stream, int ty_begin, int ty_end) {
   if (ty_end < 0) ty_end = (p.n_theta + kTileT32 - 1) / kTileT32;
