@@ -76,6 +76,7 @@ namespace {
 
 thread_local char g_err[512] = "";
 constexpr int kDefaultTimeoutMs = 120000;
+constexpr int kSpinUs = 2000;   // bounded_sync polls without pause this long
 
 struct HostCtx : pclb_ctx {
   std::vector<double> cos_t, sin_t, inv_r, bc_vals;
@@ -362,11 +363,14 @@ pclb_status bounded_sync(pclb_ctx* ctx, int timeout_ms) {
       st = cuda_fail(ctx, e, "stream work failed");
       break;
     }
-    const auto ms = std::chrono::duration_cast<std::chrono::milliseconds>(std::chrono::steady_clock::now() - t0).count();
-    if (ms > timeout_ms) {
+    const auto waited = std::chrono::steady_clock::now() - t0;
+    if (waited > std::chrono::milliseconds(timeout_ms)) {
       st = fail(ctx, PCLB_ETIMEOUT, "stream did not finish within %d ms", timeout_ms);
       break;
     }
+    // Short waits poll without a pause: the shortest sleep costs the host
+    // ~55 us, as long as a whole kernel here.
+    if (waited < std::chrono::microseconds(kSpinUs)) continue;
     std::this_thread::sleep_for(std::chrono::microseconds(sleep_us));
     if (sleep_us < 20) sleep_us *= 2;
   }
