@@ -312,7 +312,7 @@ pclb_status pclb_load_state(pclb_ctx* ctx, const void* state);
  * 16-byte aligned, distinct); the context's own state is left alone.  Lets a
  * backward pass recompute a segment's states straight into the buffers the
  * adjoint steps read.  Asynchronous, one kernel launch (two for n_dirs 16,
- * 24). */
+ * 24 in FP64). */
 pclb_status pclb_step_states(pclb_ctx* ctx, const void* f_from, void* f_to);
 
 /* Set / read the adjoint variable: device, [Q][n_theta][n_r], context

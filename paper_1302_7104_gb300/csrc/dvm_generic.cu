@@ -237,7 +237,14 @@ __global__ void __launch_bounds__(kGenThreads)
   }
   const ff w0 = ff_mul(R, ff_add(ff_of(1.f), ff_mul(ff{-c.B0h, -c.B0l}, sum)));
   const ff f0 = ff_mul(w0, a0);
-  gen_store<float>(f, p, d, 0, t, r, f0.hi + f0.lo);
+  const size_t plane = (size_t)p.rows * p.pitch;
+  float* row = f + (size_t)(t + kGhostRows) * p.pitch + r;
+  const bool seam = t < 2 || t >= p.n_theta - 2;   // the row also feeds azimuthal ghost rows
+  auto put = [&](int q, float v) {
+    if (seam) gen_store<float>(f, p, d, q, t, r, v);
+    else row[(size_t)q * plane] = v;
+  };
+  put(0, f0.hi + f0.lo);
 #pragma unroll 1
   for (int i = 0; i < H; ++i) {
     const ff y = ff_add(ff_mul(ff{c.cxh[i], c.cxl[i]}, uxE), ff_mul(ff{c.cyh[i], c.cyl[i]}, uyE));
@@ -248,9 +255,9 @@ __global__ void __launch_bounds__(kGenThreads)
       const ff od = ff_mul(y, ff_mul_add(y2, O3[k], O1[k]));
       float h, e;
       two_sum(ev.hi, od.hi, h, e);
-      gen_store<float>(f, p, d, 1 + k * ND + i, t, r, h + (e + (ev.lo + od.lo)));
+      put(1 + k * ND + i, h + (e + (ev.lo + od.lo)));
       two_sum(ev.hi, -od.hi, h, e);
-      gen_store<float>(f, p, d, 1 + k * ND + i + H, t, r, h + (e + (ev.lo - od.lo)));
+      put(1 + k * ND + i + H, h + (e + (ev.lo - od.lo)));
     }
   }
 }

@@ -28,10 +28,9 @@ void fill_dvm_generic32(DvmG32& c, const pclb_dvm& d, const DvmG& g);
 cudaError_t gen_launch_step_f64(const double* f, double* f_out, double* ghost, const StepParams& p, const DvmG& d,
                                 cudaStream_t s);
 
-// One FP32 step of the N_i = 16 or 24 set: its radial ghost layers into
-// ghost [side][layer][n_theta][Q], then the tiled kernel; tmap describes f
+// One FP32 step of the N_i = 16 or 24 set (the tiled kernel); tmap describes f
 // (box kWinR x (kTileT32 + 4) x 1 over Q planes).
-cudaError_t gen_tiled_step_f32(const CUtensorMap* tmap, const float* f, float* f_out, float* ghost,
-                               const StepParams& p, const DvmG& d, const DvmG32& c, cudaStream_t s);
+cudaError_t gen_tiled_step_f32(const CUtensorMap* tmap, const float* f, float* f_out, const StepParams& p,
+                               const DvmG& d, const DvmG32& c, cudaStream_t s);
 
 }  // namespace pclb

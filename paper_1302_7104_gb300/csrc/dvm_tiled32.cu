@@ -20,10 +20,12 @@
 //     in r and theta, summed first and added once, with the float Courant
 //     table of the pair; streaming stores, plus the azimuthal ghost rows of
 //     the seam (Eq. 40).
-// The radial ghost nodes (Sec. II C 1) come from a small per-wall buffer that
-// a ghost kernel (one thread per wall row, float-float as the node state)
-// writes before the step; tiles at a wall copy them into the window's ghost
-// columns once each pair's planes have landed.
+// Tiles at a wall form the states of the radial ghost layers (Sec. II C 1)
+// themselves, one thread per wall row in float-float, into shared memory, and
+// write the layers' equilibrium into the window's ghost columns once each
+// pair's planes have landed.  (A separate ghost kernel before the step took
+// 15 us of it on 1024 x 1024, with the chip idle.)
+// Consecutive steps overlap their set-up (programmatic dependent launch).
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -42,7 +44,7 @@ constexpr int kTThreads = 16 * kTileT32;            // 256: two nodes each
 constexpr int kTPlane = kWinR * (kTileT32 + 4);     // floats per plane window (800)
 constexpr int kTStages = 4;                         // ring depth (stages in flight)
 constexpr int kTPPS = 2;                            // pairs per stage: one wait and one barrier per two pairs
-constexpr int kGhostThreads = 32;                   // ghost kernel: one thread per wall row
+constexpr int kGhostF = 36;                         // floats of one wall row's ghost factors
 static_assert((kTPlane * 4) % 128 == 0, "TMA destinations must stay 128-byte aligned");
 
 template <int ND>
@@ -50,7 +52,8 @@ struct TiledSize {
   static constexpr int Q = 1 + 4 * ND, H = ND / 2, NP = 4 * H;   // labels, pairs per shell, pairs
   static constexpr int ring_bytes = kTStages * kTPPS * 2 * kTPlane * 4;
   static constexpr int tab_bytes = NP * kTileT32 * 16;           // one float4 per (pair, row)
-  static constexpr int smem = ring_bytes + tab_bytes + 8 * kTStages + 64;
+  static constexpr int ghost_bytes = 2 * kTileT32 * kGhostF * 4;   // both walls' rows
+  static constexpr int smem = ring_bytes + tab_bytes + ghost_bytes + 8 * kTStages + 64;
 };
 
 __device__ __forceinline__ f2 ldg2(const float* p) { return __ldg(reinterpret_cast<const float2*>(p)); }
@@ -181,21 +184,17 @@ __device__ __forceinline__ ff2 ff2_from_double(double v) {
   return ff2{bc2(h), bc2((float)(v - (double)h))};
 }
 
-// Radial ghost layers of wall `side` at row t into ghost [side][layer][n_theta][Q]
-// (Sec. II C 1): Eq. (39) applied twice to the wall node a and the next node
-// b, g0 = 2a - b and g1 = 2 g0 - a = 3a - 2b, for the components the boundary
-// kind extrapolates, the others prescribed; the ghost distribution is the
-// equilibrium of that state, plus the wall node's departure from equilibrium
-// for non-equilibrium ghosts.  All in float-float and float, as the step's
-// node state: the two layers are the two halves of the packed arithmetic.
+// The radial ghost layers of wall `side` at row t (Sec. II C 1): Eq. (39) applied
+// twice to the wall node a and the next node b, g0 = 2a - b and g1 = 2 g0 - a =
+// 3a - 2b, for the components the boundary kind extrapolates, the others
+// prescribed; the ghost distribution is the equilibrium of that state, plus
+// the wall node's departure from equilibrium for non-equilibrium ghosts.  All
+// in float-float and float, as the step's node state: the two layers are the
+// two halves of the packed arithmetic.  Writes their equilibrium factors (11
+// pairs) and those of the wall node (11) to out.
 template <int ND>
-__global__ void __launch_bounds__(kGhostThreads)
-    tiled_ghost_f32(const float* __restrict__ f, float* __restrict__ ghost, const __grid_constant__ StepParams p,
-                    const __grid_constant__ DvmG d, const __grid_constant__ DvmG32 c) {
-  constexpr int Q = 1 + 4 * ND, H = ND / 2;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  const int side = blockIdx.y;
-  if (t >= p.n_theta) return;
+__device__ __noinline__ void tiled_ghost_state(const float* __restrict__ f, float* out, int side, int t,
+                                               const StepParams& p, const DvmG32& c) {
   const size_t plane = (size_t)p.rows * p.pitch;
   const int ra = side == 0 ? 0 : p.n_r - 1, rb = side == 0 ? 1 : p.n_r - 2;
   const float* fa = f + (size_t)(t + kGhostRows) * p.pitch + ra;
@@ -213,7 +212,6 @@ __global__ void __launch_bounds__(kGhostThreads)
     g[i] = ff2_add(ff2_mul(A, ff2{mk2(2.f, 3.f), bc2(0.f)}), ff2_mul(B, ff2{mk2(-1.f, -2.f), bc2(0.f)}));
   }
   const int kind = p.bc_kind[side] & ~PCLB_BC_NEQ;
-  const bool neq = (p.bc_kind[side] & PCLB_BC_NEQ) != 0;
   if (kind != PCLB_BC_EXTRAP) {
     const double cs = p.cos_t[t], sn = p.sin_t[t];
     ff2 v[4];
@@ -236,31 +234,31 @@ __global__ void __launch_bounds__(kGhostThreads)
   ok = ok && g[0].hi.x > 0.f && g[3].hi.x > 0.f && g[0].hi.y > 0.f && g[3].hi.y > 0.f;
   if (!ok) atomicOr(p.status, PCLB_FLAG_NONPHYS);
   const TEq eg = tiled_factors(g[0], g[1], g[2], g[3], c);
-  float* out0 = ghost + ((size_t)(side * 2 + 0) * p.n_theta + t) * Q;
-  float* out1 = ghost + ((size_t)(side * 2 + 1) * p.n_theta + t) * Q;
-  {
-    f2 v = mul2(eg.w[0], eg.a0);
-    if (neq) v = add2(v, bc2(fa[0] - ea.w[0].x * ea.a0.x));
-    out0[0] = v.x;
-    out1[0] = v.y;
+  f2* o = reinterpret_cast<f2*>(out);
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    o[k] = eg.w[k];
+    out[22 + k] = ea.w[k].x;
   }
-#pragma unroll 1
-  for (int pr = 0; pr < 4 * H; ++pr) {
-    const int k = 1 + pr / H, q1 = 1 + (k - 1) * ND + pr % H, q2 = q1 + H;
-    const f2 wg = k == 1 ? eg.w[1] : (k == 2 ? eg.w[2] : (k == 3 ? eg.w[3] : eg.w[4]));
-    f2 gp, gm;
-    tiled_feq_pair(eg, wg, c.vx[q1], c.vy[q1], gp, gm);
-    if (neq) {
-      const f2 wa = k == 1 ? ea.w[1] : (k == 2 ? ea.w[2] : (k == 3 ? ea.w[3] : ea.w[4]));
-      f2 ap, am;
-      tiled_feq_pair(ea, wa, c.vx[q1], c.vy[q1], ap, am);
-      gp = add2(gp, bc2(fa[(size_t)q1 * plane] - ap.x));
-      gm = add2(gm, bc2(fa[(size_t)q2 * plane] - am.x));
-    }
-    out0[q1] = gp.x;
-    out1[q1] = gp.y;
-    out0[q2] = gm.x;
-    out1[q2] = gm.y;
+  o[5] = eg.a0; o[6] = eg.a1; o[7] = eg.a1h; o[8] = eg.uxE; o[9] = eg.uyE;
+  out[27] = ea.a0.x; out[28] = ea.a1.x; out[29] = ea.a1h.x; out[30] = ea.uxE.x; out[31] = ea.uyE.x;
+}
+
+// Ghost values of labels q1 and its opposite at one wall row: both layers (the
+// halves of gp, gm), the departure of the wall node (values a1, a2) added for
+// non-equilibrium ghosts.
+__device__ __forceinline__ void tiled_ghost_pair(const float* s, int k, float vx, float vy, bool neq, float a1, float a2,
+                                                 f2& gp, f2& gm) {
+  const f2* o = reinterpret_cast<const f2*>(s);
+  TEq e;
+  e.a0 = o[5]; e.a1 = o[6]; e.a1h = o[7]; e.uxE = o[8]; e.uyE = o[9];
+  tiled_feq_pair(e, o[k], vx, vy, gp, gm);
+  if (neq) {
+    e.a0 = bc2(s[27]); e.a1 = bc2(s[28]); e.a1h = bc2(s[29]); e.uxE = bc2(s[30]); e.uyE = bc2(s[31]);
+    f2 ap, am;
+    tiled_feq_pair(e, bc2(s[22 + k]), vx, vy, ap, am);
+    gp = add2(gp, bc2(a1 - ap.x));
+    gm = add2(gm, bc2(a2 - am.x));
   }
 }
 
@@ -303,14 +301,15 @@ __device__ __forceinline__ void tupd(const float* w, f2 nar, f2 nkr, f2 nat, f2 
 template <int ND, int SCH>
 __global__ void __launch_bounds__(kTThreads, 3)
     tiled_step_f32(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ f, float* __restrict__ f_out,
-                   const float* __restrict__ ghost, const __grid_constant__ StepParams p,
-                   const __grid_constant__ DvmG d, const __grid_constant__ DvmG32 c) {
+                   const __grid_constant__ StepParams p, const __grid_constant__ DvmG d,
+                   const __grid_constant__ DvmG32 c) {
   using TS = TiledSize<ND>;
-  constexpr int H = TS::H, NP = TS::NP, Q = TS::Q;
+  constexpr int H = TS::H, NP = TS::NP;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float* ring = reinterpret_cast<float*>(smem_raw);
   float4* tab = reinterpret_cast<float4*>(smem_raw + TS::ring_bytes);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + TS::ring_bytes + TS::tab_bytes);
+  float* gfac = reinterpret_cast<float*>(smem_raw + TS::ring_bytes + TS::tab_bytes);   // [side][row][kGhostF]
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + TS::ring_bytes + TS::tab_bytes + TS::ghost_bytes);
 
   const int r0 = blockIdx.x * kTileR;
   const int t0 = blockIdx.y * kTileT32;
@@ -333,14 +332,25 @@ __global__ void __launch_bounds__(kTThreads, 3)
     tma_prefetch_desc(&tmap);
     for (int s = 0; s < kTStages; ++s) mbar_init(&full[s], 1);
     mbar_fence_init();
-    for (int s = 0; s < kTStages && s < NS; ++s) issue(s, s);
   }
+  pdl_wait();      // the step before this one has written f and read f_out
+  pdl_launch();    // the next one may start its set-up
+  if (tid == 0)
+    for (int s = 0; s < kTStages && s < NS; ++s) issue(s, s);
   for (int i = tid; i < NP * kTileT32; i += kTThreads) {   // Courant entries: [pair][row]
     const int pr = i / kTileT32, rl = i % kTileT32;
     const int t = min(t0 + rl, p.n_theta - 1);
     tab[i] = p.courant[(size_t)(t + kGhostRows) * NP + pr];
   }
-  __syncthreads();   // barriers initialised, table visible
+  // wall tiles: the ghost layers' states, a warp per wall
+  const int cw_out = p.n_r - 1 - r0 + kLeft;
+  const bool inner = r0 == 0, outer = cw_out <= kLeft + kTileR;
+  if (inner || outer) {
+    const int side = tid >> 5, rr = tid & 31;
+    if (side < 2 && rr < kTileT32 && t0 + rr < p.n_theta && (side == 0 ? inner : outer))
+      tiled_ghost_state<ND>(f, gfac + (side * kTileT32 + rr) * kGhostF, side, t0 + rr, p, c);
+  }
+  __syncthreads();   // barriers initialised, table and ghost states visible
 
   const int warp = tid >> 5, lane = tid & 31;
   const int rl = 2 * warp + (lane >> 4);       // tile row 0..15
@@ -394,8 +404,6 @@ __global__ void __launch_bounds__(kTThreads, 3)
 
   // wall tiles: ghost columns of both walls (inner: window columns kLeft - 1,
   // kLeft - 2; outer: cw_out + 1, cw_out + 2) for the tile rows
-  const int cw_out = p.n_r - 1 - r0 + kLeft;
-  const bool inner = r0 == 0, outer = cw_out <= kLeft + kTileR;
   const int row = rl + 2, col = kLeft + j2;
   bool ok = true;
 #pragma unroll 1
@@ -404,17 +412,19 @@ __global__ void __launch_bounds__(kTThreads, 3)
     if (ok) ok = p.wait_ns != 0 && mbar_wait_bounded(&full[s], (uint32_t)((sg / kTStages) & 1), p.wait_ns);
     float* stg = ring + s * kTPPS * 2 * kTPlane;
     if (inner || outer) {
-      // per pair: 2 walls x 2 labels x 2 layers x 16 rows
-      for (int it = tid; it < kTPPS * 128 && ok; it += kTThreads) {
-        const int P = it >> 7, side = (it >> 6) & 1, L = (it >> 5) & 1, layer = (it >> 4) & 1, rr = it & 15;
-        const int pr = sg * kTPPS + P;
-        const int q1 = 1 + (pr / H) * ND + pr % H, q2 = q1 + H;
-        const int tt = t0 + rr;
-        if ((side == 0 ? inner : outer) && tt < p.n_theta) {
-          const int cg = side == 0 ? kLeft - 1 - layer : cw_out + 1 + layer;
-          if (cg >= 0 && cg < kWinR)
-            stg[P * 2 * kTPlane + L * kTPlane + (rr + 2) * kWinR + cg] =
-                ghost[((size_t)(side * 2 + layer) * p.n_theta + tt) * Q + (L ? q2 : q1)];
+      // per pair: 2 walls x 16 rows, both labels and layers
+      if (tid < kTPPS * 32 && ok) {
+        const int P = tid >> 5, side = (tid >> 4) & 1, rr = tid & 15;
+        const int pr = sg * kTPPS + P, k = 1 + pr / H, q1 = 1 + (k - 1) * ND + pr % H;
+        if ((side == 0 ? inner : outer) && t0 + rr < p.n_theta) {
+          float* w = stg + P * 2 * kTPlane + (rr + 2) * kWinR;
+          const int ca = side == 0 ? kLeft : cw_out, step = side == 0 ? -1 : 1;
+          f2 gp, gm;
+          tiled_ghost_pair(gfac + (side * kTileT32 + rr) * kGhostF, k, c.vx[q1], c.vy[q1],
+                           (p.bc_kind[side] & PCLB_BC_NEQ) != 0, w[ca], w[kTPlane + ca], gp, gm);
+          const int c0 = ca + step, c1 = ca + 2 * step;
+          if (c0 >= 0 && c0 < kWinR) { w[c0] = gp.x; w[kTPlane + c0] = gm.x; }
+          if (c1 >= 0 && c1 < kWinR) { w[c1] = gp.y; w[kTPlane + c1] = gm.y; }
         }
       }
       __syncthreads();
@@ -475,8 +485,8 @@ __global__ void __launch_bounds__(kTThreads, 3)
 }
 
 template <int ND, int SCH>
-cudaError_t launch_tiled(const CUtensorMap* tmap, const float* f, float* f_out, const float* ghost, const StepParams& p,
-                         const DvmG& d, const DvmG32& c, cudaStream_t s) {
+cudaError_t launch_tiled(const CUtensorMap* tmap, const float* f, float* f_out, const StepParams& p, const DvmG& d,
+                         const DvmG32& c, cudaStream_t s) {
   static std::atomic<unsigned long long> configured{0};
   constexpr int smem = TiledSize<ND>::smem;
   {
@@ -484,37 +494,27 @@ cudaError_t launch_tiled(const CUtensorMap* tmap, const float* f, float* f_out, 
     if (e != cudaSuccess) return e;
   }
   const dim3 grid((p.n_r + kTileR - 1) / kTileR, (p.n_theta + kTileT32 - 1) / kTileT32);
-  tiled_step_f32<ND, SCH><<<grid, kTThreads, smem, s>>>(*tmap, f, f_out, ghost, p, d, c);
-  return cudaGetLastError();
+  return launch_overlapped(tiled_step_f32<ND, SCH>, grid, kTThreads, smem, s, *tmap, f, f_out, p, d, c);
 }
 
 template <int ND>
-cudaError_t launch_tiled_nd(const CUtensorMap* tmap, const float* f, float* f_out, const float* ghost,
-                            const StepParams& p, const DvmG& d, const DvmG32& c, cudaStream_t s) {
+cudaError_t launch_tiled_nd(const CUtensorMap* tmap, const float* f, float* f_out, const StepParams& p, const DvmG& d,
+                            const DvmG32& c, cudaStream_t s) {
   switch (p.scheme) {
-    case PCLB_SCHEME_WB: return launch_tiled<ND, PCLB_SCHEME_WB>(tmap, f, f_out, ghost, p, d, c, s);
-    case PCLB_SCHEME_LW: return launch_tiled<ND, PCLB_SCHEME_LW>(tmap, f, f_out, ghost, p, d, c, s);
-    case PCLB_SCHEME_UPWIND2: return launch_tiled<ND, PCLB_SCHEME_UPWIND2>(tmap, f, f_out, ghost, p, d, c, s);
-    default: return launch_tiled<ND, PCLB_SCHEME_MWB>(tmap, f, f_out, ghost, p, d, c, s);
+    case PCLB_SCHEME_WB: return launch_tiled<ND, PCLB_SCHEME_WB>(tmap, f, f_out, p, d, c, s);
+    case PCLB_SCHEME_LW: return launch_tiled<ND, PCLB_SCHEME_LW>(tmap, f, f_out, p, d, c, s);
+    case PCLB_SCHEME_UPWIND2: return launch_tiled<ND, PCLB_SCHEME_UPWIND2>(tmap, f, f_out, p, d, c, s);
+    default: return launch_tiled<ND, PCLB_SCHEME_MWB>(tmap, f, f_out, p, d, c, s);
   }
 }
 
 }  // namespace
 
-// One FP32 step of the N_i = 16 or 24 set: the radial ghost layers, then the
-// tiled kernel over the whole grid (the same stream orders them).  tmap describes f (box kWinR x
+// One FP32 step of the N_i = 16 or 24 set.  tmap describes f (box kWinR x
 // (kTileT32 + 4) x 1, Q planes).
-cudaError_t gen_tiled_step_f32(const CUtensorMap* tmap, const float* f, float* f_out, float* ghost,
-                               const StepParams& p, const DvmG& d, const DvmG32& c, cudaStream_t s) {
-  const dim3 ggrid((p.n_theta + kGhostThreads - 1) / kGhostThreads, 2);
-  if (d.n_dirs == 16) {
-    tiled_ghost_f32<16><<<ggrid, kGhostThreads, 0, s>>>(f, ghost, p, d, c);
-    const cudaError_t e = cudaGetLastError();
-    return e != cudaSuccess ? e : launch_tiled_nd<16>(tmap, f, f_out, ghost, p, d, c, s);
-  }
-  tiled_ghost_f32<24><<<ggrid, kGhostThreads, 0, s>>>(f, ghost, p, d, c);
-  const cudaError_t e = cudaGetLastError();
-  return e != cudaSuccess ? e : launch_tiled_nd<24>(tmap, f, f_out, ghost, p, d, c, s);
+cudaError_t gen_tiled_step_f32(const CUtensorMap* tmap, const float* f, float* f_out, const StepParams& p,
+                               const DvmG& d, const DvmG32& c, cudaStream_t s) {
+  return d.n_dirs == 16 ? launch_tiled_nd<16>(tmap, f, f_out, p, d, c, s) : launch_tiled_nd<24>(tmap, f, f_out, p, d, c, s);
 }
 
 }  // namespace pclb

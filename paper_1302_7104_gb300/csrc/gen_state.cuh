@@ -35,13 +35,22 @@ __device__ __forceinline__ void gen_raw_moments(const float* f, size_t plane, co
   constexpr int H = ND / 2;
   m[0] = ff_of(f[0]);
   m[1] = m[2] = m[3] = ff_of(0.f);
+  // a shell's values are loaded while the shell before it is summed
+  float v[ND], next[ND];
+  auto load = [&](int k, float* o) {
+#pragma unroll
+    for (int i = 0; i < ND; ++i) o[i] = __ldg(f + (size_t)(1 + (k - 1) * ND + i) * plane);
+  };
+  load(1, next);
 #pragma unroll 1
   for (int k = 1; k <= 4; ++k) {
-    const float* fk = f + (size_t)(1 + (k - 1) * ND) * plane;
+#pragma unroll
+    for (int i = 0; i < ND; ++i) v[i] = next[i];
+    if (k < 4) load(k + 1, next);
     ff S = ff_of(0.f), X = S, Y = S;
 #pragma unroll
     for (int i = 0; i < H; ++i) {
-      const float a = fk[(size_t)i * plane], b = fk[(size_t)(i + H) * plane];
+      const float a = v[i], b = v[i + H];
       float sh, sl, dh, dl;
       two_sum(a, b, sh, sl);
       two_sum(a, -b, dh, dl);   // opposite unit vectors

@@ -422,8 +422,7 @@ pclb_status do_step(pclb_ctx* ctx, int n) {
     cudaError_t e;
     if (generic(ctx)) {
       if constexpr (sizeof(T) == 4)
-        e = gen_tiled_step_f32(&ctx->tmap[src], fbuf<float>(ctx, src), fbuf<float>(ctx, dst),
-                               reinterpret_cast<float*>(ctx->ws + ctx->lay.gen_ghost), ctx->sp, ctx->dvmg,
+        e = gen_tiled_step_f32(&ctx->tmap[src], fbuf<float>(ctx, src), fbuf<float>(ctx, dst), ctx->sp, ctx->dvmg,
                                dvmg32(ctx), ctx->stream);
       else
         e = gen_launch_step_f64(fbuf<double>(ctx, src), fbuf<double>(ctx, dst),
@@ -970,9 +969,7 @@ pclb_status pclb_step_states(pclb_ctx* ctx, const void* f_from, void* f_to) {
     CUtensorMap map;
     pclb_status st = encode_map(ctx, f_from, kTileT32 + 4, &map);
     if (st != PCLB_OK) return st;
-    e = gen_tiled_step_f32(&map, (const float*)f_from, (float*)f_to,
-                           reinterpret_cast<float*>(ctx->ws + ctx->lay.gen_ghost), ctx->sp, ctx->dvmg, dvmg32(ctx),
-                           ctx->stream);
+    e = gen_tiled_step_f32(&map, (const float*)f_from, (float*)f_to, ctx->sp, ctx->dvmg, dvmg32(ctx), ctx->stream);
   } else if (generic(ctx)) {
     e = gen_launch_step_f64((const double*)f_from, (double*)f_to,
                             reinterpret_cast<double*>(ctx->ws + ctx->lay.gen_ghost), ctx->sp, ctx->dvmg,
