@@ -155,15 +155,35 @@ __device__ __forceinline__ void to_moment_cotangent(T rho, T ux, T uy, T E, cons
   g[3] = G[3] * inv;
 }
 
-// The FP32 pair kernel over tiles a0 .. a0 + na - 1 and b0 .. (nx blocks in
-// r), all theta tiles (adjoint_f32x2.cu); tmap_fn, tmap_ln: descriptors of f
-// and lam with one tile per box, for its node phase.  walls: the tiles may
-// include wall tiles (radial tile 0 or r0 >= n_r - 33); false only for a
-// launch of interior tiles, which then runs the instance without wall code.
+// Order of the tiles in an adjoint launch: the tiles at a wall (radial tile 0
+// and those from first_outer on) first, as they take longest, then the rest
+// with the radial index running fastest.
+struct AdjOrder {
+  int nt, ny;        // radial and azimuthal tiles
+  int first_outer;   // >= 1
+  int blocks() const { return nt * ny; }
+  __device__ __forceinline__ bool wall(int b) const { return b < (1 + nt - first_outer) * ny; }
+  __device__ __forceinline__ void tile(int b, int& tx, int& ty) const {
+    const int nw = 1 + nt - first_outer, walls = nw * ny;
+    if (b < walls) {
+      tx = b % nw == 0 ? 0 : first_outer + b % nw - 1;
+      ty = b / nw;
+    } else {
+      const int ni = nt - nw;
+      tx = 1 + (b - walls) % ni;
+      ty = (b - walls) / ni;
+    }
+  }
+};
+
+template <class T>
+struct WallScratch;
+
+// The FP32 adjoint step (adjoint_f32x2.cu); tmap_fn, tmap_ln: descriptors of f
+// and lam with one tile per box, for its node phase.
 cudaError_t launch_adjoint_pairs_f32(const CUtensorMap* tmap_f, const CUtensorMap* tmap_l, const CUtensorMap* tmap_fn,
-                                     const CUtensorMap* tmap_ln, const float* f,
-                                     const float* lam_in, float* lam_out, const EqParams<float>* ghost,
-                                     const float* gwall, const float* gdir, int a0, int na, int b0, int nx,
-                                     bool walls, const StepParams& p, const DvmConst<float>& d, cudaStream_t s);
+                                     const CUtensorMap* tmap_ln, const float* f, const float* lam_in, float* lam_out,
+                                     const WallScratch<float>& ws, const AdjOrder& order, const StepParams& p,
+                                     const DvmConst<float>& d, cudaStream_t s);
 
 }  // namespace pclb

@@ -24,6 +24,7 @@
 #include <atomic>
 
 #include "adjoint_common.cuh"
+#include "adjoint_walls.cuh"
 #include "device_common.cuh"
 #include "f32_state.cuh"
 #include "f32x2.cuh"
@@ -386,17 +387,14 @@ __device__ __forceinline__ f2 gather_az2(const float* P) {
   return sub2(sub2(add2(lds2(P), lds2(P + DB + W)), lds2(P + W)), lds2(P + DB + 2 * W));
 }
 
-// WALLS: the launch may contain wall tiles (the tiles of radial index 0 and
-// those within 33 columns of n_r); the interior launch is the instance
-// without any wall code.
+// One tile.  WALLS: a tile at a wall (radial tile 0 or r0 >= n_r - 33), else
+// the instance without any wall code.
 template <bool WALLS>
-__global__ void __launch_bounds__(kAThr, 3)
-    adjoint_pair_f32x2(const __grid_constant__ CUtensorMap tmap_f, const __grid_constant__ CUtensorMap tmap_l,
-                       const __grid_constant__ CUtensorMap tmap_fn, const __grid_constant__ CUtensorMap tmap_ln,
-                       const float* __restrict__ f, const float* __restrict__ lam_in, float* __restrict__ lam_out,
-                       const EqParams<float>* __restrict__ ghost, const float* __restrict__ gwall,
-                       const float* __restrict__ gdir, int a0, int na,
-                       int b0, const __grid_constant__ StepParams p, const __grid_constant__ DvmConst<float> d) {
+__device__ __forceinline__ void adjoint_tile(const CUtensorMap& tmap_f, const CUtensorMap& tmap_l,
+                                             const CUtensorMap& tmap_fn, const CUtensorMap& tmap_ln,
+                                             const float* __restrict__ f, const float* __restrict__ lam_in,
+                                             float* __restrict__ lam_out, const WallScratch<float>& ws, int tx, int ty,
+                                             bool last_tile, const StepParams& p, const DvmConst<float>& d) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float* ring = reinterpret_cast<float*>(smem_raw);
   float* prod = reinterpret_cast<float*>(smem_raw + kRingBytes);
@@ -405,10 +403,8 @@ __global__ void __launch_bounds__(kAThr, 3)
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + kRingBytes + kProdBytes + kInvrBytes + kTabBytes);
   uint64_t* pbar = bar + kAS;                   // the node phase's two halves
 
-  // radial tile: blocks 0 .. na - 1 take tiles a0 .., the rest tiles b0 ..
-  const int tx = (int)blockIdx.x < na ? a0 + (int)blockIdx.x : b0 + (int)blockIdx.x - na;
   const int r0 = tx * kTileR;
-  const int t0 = blockIdx.y * kTT;
+  const int t0 = ty * kTT;
   const int tid = threadIdx.x;
 
   auto issue_pair = [&](int pr, int s) {
@@ -441,8 +437,24 @@ __global__ void __launch_bounds__(kAThr, 3)
     tma_prefetch_desc(&tmap_ln);
     for (int s = 0; s < kAS + 2; ++s) mbar_init(&bar[s], 1);
     mbar_fence_init();
+  }
+  pdl_wait();      // the step before this one has written lam and read lam_out
+  pdl_launch();    // the next one may start its set-up
+  if (tid == 0) {
     issue_group(0);
     issue_group(1);
+  }
+  // wall tiles: the ghost states of this tile's rows and their cotangent
+  const int cw_out = p.n_r - 1 - r0 + kLeft;
+  const bool inner = r0 == 0, outer = cw_out <= kLeft + kTileR;
+  const int slots[2] = {0, WallScratch<float>::slot(1, last_tile)};
+  static_assert(sizeof(WallShared<float, kTT>) <= kTabBytes, "wall scratch inside the Courant table");
+  if constexpr (WALLS) {
+    __syncthreads();
+    for (int side = 0; side < 2; ++side)
+      if (side == 0 ? inner : outer)
+        adjoint_walls<float, kTT>(f, lam_in, side, slots[side], t0, ws, *reinterpret_cast<WallShared<float, kTT>*>(ctab),
+                                  p, d);
   }
   auto prime_pairs = [&]() {
     for (int s = 0; s < kAS && s < kANP; ++s) issue_pair(s, s);
@@ -514,7 +526,8 @@ __global__ void __launch_bounds__(kAThr, 3)
       auto wall = [&](int rr) {
         float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
         auto add = [&](int side, int node) {
-          const float4 x = *reinterpret_cast<const float4*>(gwall + ((size_t)(side * 2 + node) * p.n_theta + t) * 4);
+          const float4 x =
+              *reinterpret_cast<const float4*>(ws.gwall + ((size_t)(slots[side] * 2 + node) * p.n_theta + t) * 4);
           w.x += x.x; w.y += x.y; w.z += x.z; w.w += x.w;
         };
         if (rr == 0) add(0, 0);
@@ -561,12 +574,10 @@ __global__ void __launch_bounds__(kAThr, 3)
 
   // wall tiles: the ghost states of the rows this thread fills (threads 0..15
   // the inner wall, 32..47 the outer wall, one tile row each)
-  const int cw_out = p.n_r - 1 - r0 + kLeft;
-  const bool inner = r0 == 0, outer = cw_out <= kLeft + kTileR;
   const bool wall_tile = WALLS && (inner || outer);
   const int gside = tid >> 5, grow = tid & 31;
   const bool fills = wall_tile && tid < 64 && grow < kTT && t0 + grow < p.n_theta && (gside == 0 ? inner : outer);
-  const EqParams<float>* eg = ghost + (size_t)(gside * 3) * p.n_theta + t0 + grow;   // layer l at + l n_theta
+  const EqParams<float>* eg = ws.ghost + (size_t)(slots[gside & 1] * 3) * p.n_theta + t0 + grow;   // layer l at + l n_theta
   const bool gneq = (p.bc_kind[gside & 1] & PCLB_BC_NEQ) != 0;   // its ghosts carry the wall node's departure
 
   bool ok = true;
@@ -700,7 +711,7 @@ __global__ void __launch_bounds__(kAThr, 3)
         for (int sd = 0; sd < 2; ++sd) {
           if (!(p.bc_kind[sd] & PCLB_BC_NEQ)) continue;
           const int rw = sd == 0 ? 0 : p.n_r - 1;
-          const float* gd = gdir + ((size_t)sd * p.n_theta + t) * kQ;
+          const float* gd = ws.gdir + ((size_t)slots[sd] * p.n_theta + t) * kQ;
           if (r == rw) { o1.x += gd[q1]; o2.x += gd[q2]; }
           if (r + 1 == rw) { o1.y += gd[q1]; o2.y += gd[q2]; }
         }
@@ -721,33 +732,31 @@ __global__ void __launch_bounds__(kAThr, 3)
   }
 }
 
-template <bool WALLS>
-cudaError_t launch_pairs(const CUtensorMap* tmap_f, const CUtensorMap* tmap_l, const CUtensorMap* tmap_fn,
-                                const CUtensorMap* tmap_ln, const float* f, const float* lam_in, float* lam_out,
-                                const EqParams<float>* ghost, const float* gwall, const float* gdir, int a0, int na,
-                                int b0, int nx, const StepParams& p, const DvmConst<float>& d, cudaStream_t s) {
-  static std::atomic<unsigned long long> configured{0};   // per instance and device
-  {
-    const cudaError_t e = set_smem_once(adjoint_pair_f32x2<WALLS>, kASmem, configured);
-    if (e != cudaSuccess) return e;
-  }
-  const dim3 grid((unsigned)nx, (unsigned)((p.n_theta + kTT - 1) / kTT));
-  adjoint_pair_f32x2<WALLS><<<grid, kAThr, kASmem, s>>>(*tmap_f, *tmap_l, *tmap_fn, *tmap_ln, f, lam_in, lam_out,
-                                                        ghost, gwall, gdir, a0, na, b0, p, d);
-  return cudaGetLastError();
+__global__ void __launch_bounds__(kAThr, 3)
+    adjoint_pair_f32x2(const __grid_constant__ CUtensorMap tmap_f, const __grid_constant__ CUtensorMap tmap_l,
+                       const __grid_constant__ CUtensorMap tmap_fn, const __grid_constant__ CUtensorMap tmap_ln,
+                       const float* __restrict__ f, const float* __restrict__ lam_in, float* __restrict__ lam_out,
+                       const __grid_constant__ WallScratch<float> ws, const __grid_constant__ AdjOrder order,
+                       const __grid_constant__ StepParams p, const __grid_constant__ DvmConst<float> d) {
+  int tx, ty;
+  order.tile(blockIdx.x, tx, ty);
+  if (order.wall(blockIdx.x))
+    adjoint_tile<true>(tmap_f, tmap_l, tmap_fn, tmap_ln, f, lam_in, lam_out, ws, tx, ty, tx == order.nt - 1, p, d);
+  else
+    adjoint_tile<false>(tmap_f, tmap_l, tmap_fn, tmap_ln, f, lam_in, lam_out, ws, tx, ty, false, p, d);
 }
 
 }  // namespace
 
 cudaError_t launch_adjoint_pairs_f32(const CUtensorMap* tmap_f, const CUtensorMap* tmap_l, const CUtensorMap* tmap_fn,
-                                     const CUtensorMap* tmap_ln, const float* f,
-                                     const float* lam_in, float* lam_out, const EqParams<float>* ghost,
-                                     const float* gwall, const float* gdir, int a0, int na, int b0, int nx,
-                                     bool walls, const StepParams& p, const DvmConst<float>& d, cudaStream_t s) {
-  return walls ? launch_pairs<true>(tmap_f, tmap_l, tmap_fn, tmap_ln, f, lam_in, lam_out, ghost, gwall, gdir, a0, na,
-                                    b0, nx, p, d, s)
-               : launch_pairs<false>(tmap_f, tmap_l, tmap_fn, tmap_ln, f, lam_in, lam_out, ghost, gwall, gdir, a0,
-                                     na, b0, nx, p, d, s);
+                                     const CUtensorMap* tmap_ln, const float* f, const float* lam_in, float* lam_out,
+                                     const WallScratch<float>& ws, const AdjOrder& order, const StepParams& p,
+                                     const DvmConst<float>& d, cudaStream_t s) {
+  static std::atomic<unsigned long long> configured{0};
+  const cudaError_t e = set_smem_once(adjoint_pair_f32x2, kASmem, configured);
+  if (e != cudaSuccess) return e;
+  return launch_overlapped(adjoint_pair_f32x2, dim3((unsigned)order.blocks()), kAThr, kASmem, s, *tmap_f, *tmap_l,
+                           *tmap_fn, *tmap_ln, f, lam_in, lam_out, ws, order, p, d);
 }
 
 }  // namespace pclb

@@ -17,26 +17,30 @@
 // sign(x) with sign(0) = 0 (the switch function on its active branch); at
 // D = Dp = 0 the derivative of h is 0.
 //
-// Two kernels:
-//   * adjoint_wall_kernel, one warp per wall and row: the ghost states
-//     (Eq. 39 or prescribed) and the cotangent g_wall they return, written to
-//     small global buffers;
-//   * adjoint_pair_kernel, tiles of 32 (r) x TT (theta) nodes, one node per
-//     thread.  Each thread first forms g of its node from f^n and lam^{n+1}
-//     read from global memory (a reduction over the 33 labels).  Then the
-//     velocities, in pairs of opposite labels, stream their f and lam windows
-//     over [r0-4, r0+36) x [t0-2, t0+TT+2) through a ring of shared-memory
-//     stages filled by TMA while earlier pairs compute.  Each pair runs in two
-//     phases: (A) every node whose upwind stencil can reach the tile forms
-//     lam(n) dM(n)/dD and lam(n) dM(n)/dDp once, in r and in theta; (B) every
-//     tile node gathers the products of the nodes that read it and adds
-//     d lam + psi . ((1-d) g + g_wall).  One barrier per pair separates the
-//     phases; a stage is refilled as soon as its pair's phase (A) is done.
+// One launch per step, tiles of 32 (r) x TT (theta) nodes: the FP32 kernel is
+// adjoint_f32x2.cu (two nodes per thread), the FP64 kernel adjoint_pair_kernel
+// below (one node per thread).
+//   * Tiles at a wall first form their rows' ghost states (Eq. 39 or
+//     prescribed) and the cotangent g_wall they return (adjoint_walls.cuh).
+//     They come first in the launch.  (As a kernel of its own on a side
+//     stream, with the wall tiles after it, this took 19 us (FP32) and 31 us
+//     (FP64) of each step with most of the chip idle, and four event calls.)
+//   * Each thread forms g of its node from f^n and lam^{n+1} read from global
+//     memory (a reduction over the 33 labels).  Then the velocities, in pairs
+//     of opposite labels, stream their f and lam windows over [r0-4, r0+36) x
+//     [t0-2, t0+TT+2) through a ring of shared-memory stages filled by TMA
+//     while earlier pairs compute.  Each pair runs in two phases: (A) every
+//     node whose upwind stencil can reach the tile forms lam(n) dM(n)/dD and
+//     lam(n) dM(n)/dDp once, in r and in theta; (B) every tile node gathers
+//     the products of the nodes that read it and adds d lam + psi . ((1-d) g +
+//     g_wall).  One barrier per pair separates the phases; a stage is refilled
+//     as soon as its pair's phase (A) is done.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
 #include "device_common.cuh"
 #include "adjoint_common.cuh"
+#include "adjoint_walls.cuh"
 #include "f32_state.cuh"
 #include "pclb_internal.h"
 
@@ -58,6 +62,9 @@ struct alignas(4 * sizeof(T)) CourEntry {
   T a_r, k_r, a_w;
   int fl;
 };
+
+// bytes of one part of the wall scratch, aligned for the next
+static size_t scratch_part(size_t bytes) { return (bytes + 255) & ~(size_t)255; }
 
 constexpr int kAdjStages = 2;   // ring depth of the pair-streaming kernel (2 measured best of 1..4)
 static_assert(sizeof(EqParams<float>) == 10 * sizeof(float) && sizeof(EqParams<double>) == 10 * sizeof(double),
@@ -84,45 +91,6 @@ struct AdjSize {
 
 namespace {
 
-
-template <class T>
-struct Cour {
-  T a_r, k_r, a_w;
-  int up_r, up_t;   // upwind offsets in r (columns) and theta (rows): -1 or +1
-};
-
-__device__ __forceinline__ void courant_entry(const StepParams& p, int row, int pair, float& ar, float& kr,
-                                              float& aw, int& fl) {
-  const float4 e = p.courant[(size_t)row * (4 * kNDirs / 2) + pair];
-  ar = e.x; kr = e.y; aw = e.z; fl = __float_as_int(e.w);
-}
-__device__ __forceinline__ void courant_entry(const StepParams& p, int row, int pair, double& ar, double& kr,
-                                              double& aw, int& fl) {
-  const double* e = p.courant64 + ((size_t)row * (4 * kNDirs / 2) + pair) * 4;
-  ar = e[0]; kr = e[1]; aw = e[2]; fl = (int)e[3];
-}
-
-// Courant data of label q at stored row `row` (ghost rows included), from
-// the table of opposite-velocity pairs.
-template <class T>
-__device__ __forceinline__ Cour<T> courant(const StepParams& p, const DvmConst<T>& d, int q, int row) {
-  Cour<T> c;
-  if (q == 0) {
-    c.a_r = T(0); c.k_r = T(0); c.a_w = T(0); c.up_r = -1; c.up_t = -1;
-    return c;
-  }
-  const int k = d.shell[q];
-  const int i = (q - 1) % kNDirs;
-  const bool second = i >= kNDirs / 2;
-  const int pair = (k - 1) * (kNDirs / 2) + (second ? i - kNDirs / 2 : i);
-  int fl;
-  courant_entry(p, row, pair, c.a_r, c.k_r, c.a_w, fl);
-  const bool vr_neg = ((fl & 1) != 0) != second;   // the partner has the opposite velocity
-  const bool vt_neg = ((fl & 2) != 0) != second;
-  c.up_r = vr_neg ? 1 : -1;
-  c.up_t = vt_neg ? 1 : -1;
-  return c;
-}
 
 // (rho, u_x, u_y, E) of one node for the cotangent of the equilibrium (FP64;
 // the FP32 pair kernel forms the state of its two nodes in float-float).
@@ -214,177 +182,7 @@ __device__ __forceinline__ void gather_azimuthal_mixed(const T* pb, int pa, int 
   }
 }
 
-// f^eq_q of a node state (rho and E in double as the step evaluates them).
-template <class T>
-__device__ __forceinline__ T adj_feq(const EqParams<T>& e, const DvmConst<T>& d, int q) {
-  return feq_q<T>(e, d.vx[q], d.vy[q], d.shell[q]);
-}
-
 }  // namespace
-
-// ---------------------------------------------------------------------------
-// Walls: one warp per side s (0 inner, 1 outer) and row t.  It forms the
-// equilibrium parameters of the two ghost layers (Eq. 39, or the prescribed
-// states) and the cotangent g_wall that the ghosts return to the wall node
-// (node 0) and the next node inward (node 1); lanes 0..15 take one pair of
-// opposite velocities each, a warp reduction sums them.
-// ghost [side][layer][n_theta] EqParams; gwall [side][node][n_theta][4].
-// ---------------------------------------------------------------------------
-template <class T>
-__global__ void __launch_bounds__(128)
-    adjoint_wall_kernel(const T* __restrict__ f, const T* __restrict__ lam, EqParams<T>* __restrict__ ghost,
-                        T* __restrict__ gwall, T* __restrict__ gdir, const __grid_constant__ StepParams p,
-                        const __grid_constant__ DvmConst<T> d) {
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  const int side = warp & 1, t = warp >> 1;
-  if (t >= p.n_theta) return;                          // uniform across the warp
-  const int plane = p.rows * p.pitch;
-  const int srow = t + kGhostRows;
-  const int step = side == 0 ? 1 : -1;                // towards the interior
-  const int out = -step;                              // the upwind offset that reads the ghosts
-  const int ra = side == 0 ? 0 : p.n_r - 1;
-  const T* fa = f + (size_t)srow * p.pitch + ra;
-  const T* fb = fa + step;
-  const T* la = lam + (size_t)srow * p.pitch + ra;
-  const T* lb = la + step;
-  const NodeState<T> a = node_moments(fa, plane, d);
-  const NodeState<T> b = node_moments(fb, plane, d);
-  const int kind = p.bc_kind[side] & ~PCLB_BC_NEQ;
-  double grho[2], gE[2];
-  T gux[2], guy[2];
-  grho[0] = 2.0 * a.rho_d - b.rho_d;  grho[1] = 2.0 * grho[0] - a.rho_d;   // Eq. (39), applied twice
-  gE[0] = 2.0 * a.E_d - b.E_d;        gE[1] = 2.0 * gE[0] - a.E_d;
-  gux[0] = T(2) * a.ux - b.ux;        gux[1] = T(2) * gux[0] - a.ux;
-  guy[0] = T(2) * a.uy - b.uy;        guy[1] = T(2) * guy[0] - a.uy;
-  if (kind != PCLB_BC_EXTRAP) {
-    const double c = p.cos_t[t], s = p.sin_t[t];
-    for (int l = 0; l < 2; ++l) {
-      const double* v = p.bc_vals + (size_t)((side * 2 + l) * 4) * p.n_theta + t;
-      gux[l] = (T)(v[1 * p.n_theta] * c - v[2 * p.n_theta] * s);
-      guy[l] = (T)(v[1 * p.n_theta] * s + v[2 * p.n_theta] * c);
-      if (kind == PCLB_BC_DIRICHLET) {
-        grho[l] = v[0];
-        gE[l] = v[3 * p.n_theta];
-      }
-    }
-  }
-  const EqParams<T> e0 = eq_params<T>(grho[0], gux[0], guy[0], gE[0], d);
-  const EqParams<T> e1 = eq_params<T>(grho[1], gux[1], guy[1], gE[1], d);
-  const bool neq = (p.bc_kind[side] & PCLB_BC_NEQ) != 0;
-  // non-equilibrium ghosts also carry the wall node's departure f_q(a) -
-  // f^eq_q(a): its equilibrium parameters go to the third slot (zero for
-  // other walls, whose pair kernels do not read it; neq is uniform across
-  // the warp, which serves one side)
-  EqParams<T> ea{};
-  if (neq) ea = eq_params<T>(a.rho_d, a.ux, a.uy, a.E_d, d);
-  if (lane == 0) {
-    if (!(grho[0] > 0.0 && grho[1] > 0.0 && gE[0] > 0.0 && gE[1] > 0.0)) atomicOr(p.status, PCLB_FLAG_NONPHYS);
-    ghost[(size_t)(side * 3 + 0) * p.n_theta + t] = e0;
-    ghost[(size_t)(side * 3 + 1) * p.n_theta + t] = e1;
-    ghost[(size_t)(side * 3 + 2) * p.n_theta + t] = ea;
-    gdir[((size_t)side * p.n_theta + t) * kQ] = T(0);   // the rest velocity reads no ghost
-  }
-  // per layer: the sums A, Bx, By, Cs, Dx, Fq of eq_cotangent over this
-  // lane's pair; layer 2: those at the wall node's own state for the
-  // departure of non-equilibrium ghosts
-  T c[3][6];
-#pragma unroll
-  for (int l = 0; l < 3; ++l)
-#pragma unroll
-    for (int j = 0; j < 6; ++j) c[l][j] = T(0);
-  constexpr int half = kNDirs / 2;
-  if (lane < 4 * half) {
-    const int k = 1 + lane / half;
-    const int q1 = 1 + (k - 1) * kNDirs + lane % half;
-    // cotangent of the ghost values f_q(layer l) = -sum_n lam_q(n) dM_q(n)/df_q(ghost l):
-    // the wall node a reads (a, g0, g1), the next node b reads (b, a, g0)
-    T lg[2][2];                                        // [label][layer]
-#pragma unroll
-    for (int L = 0; L < 2; ++L) {
-      const int q = q1 + L * half;
-      const Cour<T> cr = courant<T>(p, d, q, srow);
-      lg[L][0] = lg[L][1] = T(0);
-      if (cr.up_r == out) {
-        const T f_a = fa[(size_t)q * plane], f_b = fb[(size_t)q * plane];
-        // the ghost values as the step forms them (plus the departure f_q(a)
-        // - f^eq_q(a) for non-equilibrium ghosts)
-        const T dep = neq ? f_a - adj_feq<T>(ea, d, q) : T(0);
-        const T g0 = adj_feq<T>(e0, d, q) + dep, g1 = adj_feq<T>(e1, d, q) + dep;
-        T MDa, MPa, MDb, MPb;
-        mwb_partials<T>(cr.a_r, cr.k_r, f_a - g0, g0 - g1, MDa, MPa);
-        mwb_partials<T>(cr.a_r, cr.k_r, f_b - f_a, f_a - g0, MDb, MPb);
-        const T lam_a = la[(size_t)q * plane], lam_b = lb[(size_t)q * plane];
-        lg[L][0] = lam_a * (MDa - MPa) + lam_b * MPb;
-        lg[L][1] = lam_a * MPa;
-      }
-    }
-    // the ghost values' cotangents flow, for non-equilibrium ghosts, straight
-    // to f_q(a) (coefficient 1) and, with the opposite sign, through f^eq_q(a)
-    gdir[((size_t)side * p.n_theta + t) * kQ + q1] = lg[0][0] + lg[0][1];
-    gdir[((size_t)side * p.n_theta + t) * kQ + q1 + half] = lg[1][0] + lg[1][1];
-    const T lneq[2] = {neq ? -(lg[0][0] + lg[0][1]) : T(0), neq ? -(lg[1][0] + lg[1][1]) : T(0)};
-#pragma unroll
-    for (int l = 0; l < 3; ++l) {
-      if (l == 2 && !neq) break;                      // the departure's terms: non-equilibrium ghosts only
-      const T E = l < 2 ? (T)gE[l] : a.E, ux = l < 2 ? gux[l] : a.ux, uy = l < 2 ? guy[l] : a.uy;
-      const T lp = l < 2 ? lg[0][l] : lneq[0], lm = l < 2 ? lg[1][l] : lneq[1];
-      const T* cf = d.Fc[k];
-      const T F = E * (cf[0] + E * (cf[1] + E * (cf[2] + E * cf[3])));
-      const T Fd = cf[0] + E * (T(2) * cf[1] + E * (T(3) * cf[2] + E * T(4) * cf[3]));
-      const T invE = recip1(E);
-      const T s = (ux * ux + uy * uy) * invE;
-      const T a1 = T(1) - T(0.5) * s;
-      const T a0 = a1 + T(0.125) * s * s;
-      T Ak = 0, Bxk = 0, Byk = 0, Ck = 0, Dk = 0;
-      pair_terms<T>(d.vx[q1], d.vy[q1], ux * invE, uy * invE, s, a0, a1, lp, lm, Ak, Bxk, Byk, Ck, Dk);
-      c[l][0] = F * Ak; c[l][1] = F * Bxk; c[l][2] = F * Byk; c[l][3] = F * Ck; c[l][4] = F * Dk; c[l][5] = Fd * Ak;
-    }
-  }
-#pragma unroll
-  for (int l = 0; l < 3; ++l) {
-    if (l == 2 && !neq) break;
-#pragma unroll
-    for (int j = 0; j < 6; ++j)
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) c[l][j] += __shfl_xor_sync(0xffffffffu, c[l][j], o);
-  }
-  if (lane != 0) return;
-  T Gl[3][4];
-#pragma unroll
-  for (int l = 0; l < 3; ++l) {
-    // G of eq_cotangent at the ghost state, and at the wall node's state for
-    // the departure (the rest velocity returns nothing)
-    if (l == 2 && !neq) {
-      Gl[2][0] = Gl[2][1] = Gl[2][2] = Gl[2][3] = T(0);
-      break;
-    }
-    const T rho = l < 2 ? (T)grho[l] : a.rho, E = l < 2 ? (T)gE[l] : a.E;
-    const T ux = l < 2 ? gux[l] : a.ux, uy = l < 2 ? guy[l] : a.uy;
-    const T invE = recip1(E);
-    const T s = (ux * ux + uy * uy) * invE;
-    Gl[l][0] = c[l][0];
-    Gl[l][1] = rho * (c[l][1] + T(2) * ux * c[l][3]) * invE;
-    Gl[l][2] = rho * (c[l][2] + T(2) * uy * c[l][3]) * invE;
-    Gl[l][3] = rho * (c[l][5] - (c[l][4] + s * c[l][3]) * invE);
-  }
-  // back through the extrapolation g0 = 2a - b, g1 = 3a - 2b (extrapolated components only)
-  const bool ext_rho_E = kind != PCLB_BC_DIRICHLET;
-  const bool ext_u = kind == PCLB_BC_EXTRAP;
-  T Ga[4], Gb[4];
-  for (int j = 0; j < 4; ++j) {
-    const bool ext = (j == 0 || j == 3) ? ext_rho_E : ext_u;
-    Ga[j] = (ext ? T(2) * Gl[0][j] + T(3) * Gl[1][j] : T(0)) + (neq ? Gl[2][j] : T(0));
-    Gb[j] = ext ? -Gl[0][j] - T(2) * Gl[1][j] : T(0);
-  }
-  T ga[4], gb[4];
-  to_moment_cotangent<T>(a.rho, a.ux, a.uy, a.E, Ga, ga);
-  to_moment_cotangent<T>(b.rho, b.ux, b.uy, b.E, Gb, gb);
-  for (int j = 0; j < 4; ++j) {
-    gwall[((size_t)(side * 2 + 0) * p.n_theta + t) * 4 + j] = ga[j];
-    gwall[((size_t)(side * 2 + 1) * p.n_theta + t) * 4 + j] = gb[j];
-  }
-}
 
 // ---------------------------------------------------------------------------
 // Pair-streaming part.
@@ -393,9 +191,8 @@ template <class T>
 __global__ void __launch_bounds__(AdjSize<T>::threads, AdjTile<T>::min_blocks)
     adjoint_pair_kernel(const __grid_constant__ CUtensorMap tmap_f, const __grid_constant__ CUtensorMap tmap_l,
                         const T* __restrict__ f, const T* __restrict__ lam_in, T* __restrict__ lam_out,
-                        const EqParams<T>* __restrict__ ghost, const T* __restrict__ gwall,
-                        const T* __restrict__ gdir, int a0, int na, int b0, const __grid_constant__ StepParams p,
-                        const __grid_constant__ DvmConst<T> d) {
+                        const __grid_constant__ WallScratch<T> ws, const __grid_constant__ AdjOrder order,
+                        const __grid_constant__ StepParams p, const __grid_constant__ DvmConst<T> d) {
   constexpr int TT = AdjTile<T>::TT;
   constexpr int PLANE = AdjSize<T>::plane;
   constexpr int NP = AdjSize<T>::npairs, RC = AdjSize<T>::rcols, PROD = AdjSize<T>::prod;
@@ -410,10 +207,10 @@ __global__ void __launch_bounds__(AdjSize<T>::threads, AdjTile<T>::min_blocks)
   CourEntry<T>* ctab = reinterpret_cast<CourEntry<T>*>(invr + kTileR);   // [TT + 4][NP]
   uint64_t* bar = reinterpret_cast<uint64_t*>(ctab + (TT + 4) * NP);     // [S]
 
-  // radial tile: blocks 0 .. na - 1 take tiles a0 .., the rest tiles b0 ..
-  const int tx = (int)blockIdx.x < na ? a0 + (int)blockIdx.x : b0 + (int)blockIdx.x - na;
+  int tx, ty;
+  order.tile(blockIdx.x, tx, ty);
   const int r0 = tx * kTileR;
-  const int t0 = blockIdx.y * TT;
+  const int t0 = ty * TT;
   const int tid = threadIdx.x;
   const int lane = tid & 31, rowl = tid >> 5;
 
@@ -434,6 +231,16 @@ __global__ void __launch_bounds__(AdjSize<T>::threads, AdjTile<T>::min_blocks)
     for (int s = 0; s < S; ++s) mbar_init(&bar[s], 1);
     mbar_fence_init();
   }
+  pdl_wait();      // the step before this one has written lam and read lam_out
+  pdl_launch();    // the next one may start its set-up
+  // wall tiles: the ghost states of this tile's rows and their cotangent
+  const int cw_out = p.n_r - 1 - r0 + kLeft;
+  const bool inner = r0 == 0, outer = cw_out <= kLeft + kTileR;
+  const int slots[2] = {0, WallScratch<T>::slot(1, tx == order.nt - 1)};
+  static_assert(sizeof(WallShared<T, TT>) <= (TT + 4) * NP * sizeof(CourEntry<T>), "wall scratch inside the Courant table");
+  for (int side = 0; side < 2; ++side)
+    if (side == 0 ? inner : outer)
+      adjoint_walls<T, TT>(f, lam_in, side, slots[side], t0, ws, *reinterpret_cast<WallShared<T, TT>*>(ctab), p, d);
   if (tid < kTileR) invr[tid] = r0 + tid < p.n_r ? (T)p.inv_r[r0 + tid] : T(1);
   // Courant entries of the stored rows t0 .. t0 + TT + 3 (theta rows t0 - 2 .. t0 + TT + 1)
   for (int i = tid; i < (TT + 4) * NP; i += blockDim.x) {
@@ -484,7 +291,7 @@ __global__ void __launch_bounds__(AdjSize<T>::threads, AdjTile<T>::min_blocks)
     // the cotangent the ghost nodes return to the two nodes next to each wall
     auto add_wall = [&](int side, int node) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) gs[j] += gwall[((size_t)(side * 2 + node) * p.n_theta + t) * 4 + j];
+      for (int j = 0; j < 4; ++j) gs[j] += ws.gwall[((size_t)(slots[side] * 2 + node) * p.n_theta + t) * 4 + j];
     };
     if (r == 0) add_wall(0, 0);
     if (r == 1) add_wall(0, 1);
@@ -505,12 +312,10 @@ __global__ void __launch_bounds__(AdjSize<T>::threads, AdjTile<T>::min_blocks)
   if (valid) store(0, decay * lam_in[(size_t)srow * p.pitch + r] + gs[0] + gs[3] * d.half_v2[0]);
 
   // wall tiles: the ghost states of the rows this thread fills (warp 0: inner, warp 1: outer)
-  const int cw_out = p.n_r - 1 - r0 + kLeft;
-  const bool inner = r0 == 0, outer = cw_out <= kLeft + kTileR;
   const bool wall_tile = inner || outer;
   const int gside = rowl == 0 ? 0 : 1;
   const bool fills = wall_tile && rowl < 2 && lane < TT && t0 + lane < p.n_theta && (gside == 0 ? inner : outer);
-  const EqParams<T>* eg = ghost + (size_t)(gside * 3) * p.n_theta + t0 + lane;   // layer l at + l n_theta
+  const EqParams<T>* eg = ws.ghost + (size_t)(slots[gside] * 3) * p.n_theta + t0 + lane;   // layer l at + l n_theta
   const bool gneq = (p.bc_kind[gside] & PCLB_BC_NEQ) != 0;   // its ghosts carry the wall node's departure
 
   bool ok = true;
@@ -641,8 +446,8 @@ __global__ void __launch_bounds__(AdjSize<T>::threads, AdjTile<T>::min_blocks)
         // non-equilibrium ghosts hand their cotangent straight to f_q of the wall node
         for (int sd = 0; sd < 2; ++sd)
           if ((p.bc_kind[sd] & PCLB_BC_NEQ) && r == (sd == 0 ? 0 : p.n_r - 1)) {
-            o1 += gdir[((size_t)sd * p.n_theta + t) * kQ + q1];
-            o2 += gdir[((size_t)sd * p.n_theta + t) * kQ + q2];
+            o1 += ws.gdir[((size_t)slots[sd] * p.n_theta + t) * kQ + q1];
+            o2 += ws.gdir[((size_t)slots[sd] * p.n_theta + t) * kQ + q2];
           }
       }
       store(q1, o1);
@@ -661,80 +466,47 @@ __global__ void __launch_bounds__(AdjSize<T>::threads, AdjTile<T>::min_blocks)
   }
 }
 
-// The tiles that read the wall kernel's output (ghost columns, g_wall) are
-// tile 0 and the tiles with r0 >= n_r - 33; they run on the side stream after
-// the wall kernel while the interior tiles run on the main stream.
 template <class T>
 cudaError_t launch_adjoint(const CUtensorMap* tmap_f, const CUtensorMap* tmap_l, const CUtensorMap* tmap_fn,
-                           const CUtensorMap* tmap_ln, const T* f, const T* lam_in,
-                           T* lam_out, const AdjScratch& ws, const StepParams& p, const DvmConst<T>& d,
-                           cudaStream_t stream, cudaStream_t side, cudaEvent_t ev_fork, cudaEvent_t ev_join) {
-  EqParams<T>* ghost = reinterpret_cast<EqParams<T>*>(ws.ghost);
-  T* gwall = reinterpret_cast<T*>(ws.gwall);
-  const int nt = (p.n_r + kTileR - 1) / kTileR;
-  const int t_hi = p.n_r - 33 > 0 ? (p.n_r - 33 + kTileR - 1) / kTileR : 0;   // first tile with r0 >= n_r - 33
-  const int b0 = t_hi > 1 ? t_hi : 1;
-  const int n_interior = t_hi > 1 ? t_hi - 1 : 0;                              // tiles 1 .. t_hi - 1
-  cudaError_t e = cudaEventRecord(ev_fork, stream);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(side, ev_fork, 0);
-  if (e != cudaSuccess) return e;
-  // per-label cotangents of non-equilibrium ghosts: [side][n_theta][Q] after gwall
-  T* gdir = reinterpret_cast<T*>(ws.gwall + (((size_t)16 * p.n_theta * sizeof(T) + 255) & ~(size_t)255));
-  adjoint_wall_kernel<T><<<(2 * p.n_theta + 3) / 4, 128, 0, side>>>(f, lam_in, ghost, gwall, gdir, p, d);
+                           const CUtensorMap* tmap_ln, const T* f, const T* lam_in, T* lam_out, unsigned char* scratch,
+                           const StepParams& p, const DvmConst<T>& d, cudaStream_t stream) {
+  WallScratch<T> ws;
+  ws.ghost = reinterpret_cast<EqParams<T>*>(scratch);
+  ws.gwall = reinterpret_cast<T*>(scratch + scratch_part((size_t)9 * p.n_theta * 10 * sizeof(T)));
+  ws.gdir = reinterpret_cast<T*>(reinterpret_cast<unsigned char*>(ws.gwall) +
+                                 scratch_part((size_t)24 * p.n_theta * sizeof(T)));
+  constexpr int rows = sizeof(T) == 4 ? kAdjRows32 : kAdjRows64;
+  AdjOrder order;
+  order.nt = (p.n_r + kTileR - 1) / kTileR;
+  order.ny = (p.n_theta + rows - 1) / rows;
+  // tile 0 and the tiles with r0 >= n_r - 33 are wall tiles
+  order.first_outer = p.n_r - 33 > 0 ? (p.n_r - 33 + kTileR - 1) / kTileR : 0;
+  if (order.first_outer < 1) order.first_outer = 1;
   if constexpr (sizeof(T) == 4) {
     // FP32: the packed two-nodes-per-thread pair kernel (adjoint_f32x2.cu)
-    e = cudaGetLastError();
-    if (e == cudaSuccess)
-      e = launch_adjoint_pairs_f32(tmap_f, tmap_l, tmap_fn, tmap_ln, f, lam_in, lam_out, ghost, gwall, gdir, 0, 1, b0,
-                                   1 + (nt - b0), true, p, d, side);
-    // tiles 1 .. t_hi - 1 have r0 > 0 and r0 < n_r - 33: no wall tile among them
-    if (e == cudaSuccess && n_interior > 0)
-      e = launch_adjoint_pairs_f32(tmap_f, tmap_l, tmap_fn, tmap_ln, f, lam_in, lam_out, ghost, gwall, gdir, 1, n_interior,
-                                   0, n_interior, false, p, d, stream);
+    return launch_adjoint_pairs_f32(tmap_f, tmap_l, tmap_fn, tmap_ln, f, lam_in, lam_out, ws, order, p, d, stream);
   } else {
     static std::atomic<unsigned long long> configured{0};
     constexpr int smem = AdjSize<T>::smem;
-    e = set_smem_once(adjoint_pair_kernel<T>, smem, configured);
+    const cudaError_t e = set_smem_once(adjoint_pair_kernel<T>, smem, configured);
     if (e != cudaSuccess) return e;
-    constexpr int TT = AdjTile<T>::TT;
-    const unsigned gy = (unsigned)((p.n_theta + TT - 1) / TT);
-    adjoint_pair_kernel<T><<<dim3(1 + (nt - b0), gy), AdjSize<T>::threads, smem, side>>>(
-        *tmap_f, *tmap_l, f, lam_in, lam_out, ghost, gwall, gdir, 0, 1, b0, p, d);
-    if (n_interior > 0)
-      adjoint_pair_kernel<T><<<dim3(n_interior, gy), AdjSize<T>::threads, smem, stream>>>(
-          *tmap_f, *tmap_l, f, lam_in, lam_out, ghost, gwall, gdir, 1, n_interior, 0, p, d);
-    e = cudaGetLastError();
+    return launch_overlapped(adjoint_pair_kernel<T>, dim3((unsigned)order.blocks()), AdjSize<T>::threads, smem, stream,
+                             *tmap_f, *tmap_l, f, lam_in, lam_out, ws, order, p, d);
   }
-  if (e != cudaSuccess) return e;
-  e = cudaEventRecord(ev_join, side);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, ev_join, 0);
-  return e;
 }
 
 size_t adjoint_scratch_bytes(int n_theta, int elem) {
-  // ghost: 2 x 3 EqParams (10 values) per row (two ghost layers and the wall
-  // node); gwall: 2 x 2 x 4 per row; the non-equilibrium ghosts' per-label
-  // cotangents: 2 x Q per row
-  const size_t b = (size_t)6 * n_theta * 10 * elem, c = (size_t)16 * n_theta * elem;
-  const size_t g = (size_t)2 * n_theta * kQ * elem;
-  auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-  return up(b) + up(c) + up(g);
-}
-
-AdjScratch adjoint_scratch(unsigned char* base, int n_theta, int elem) {
-  AdjScratch s;
-  s.ghost = base;
-  s.gwall = base + (((size_t)6 * n_theta * 10 * elem + 255) & ~(size_t)255);
-  return s;
+  // the parts of WallScratch: three slots of 3 EqParams (10 values), of 2 x 4
+  // values and of Q values per row
+  return scratch_part((size_t)9 * n_theta * 10 * elem) + scratch_part((size_t)24 * n_theta * elem) +
+         scratch_part((size_t)3 * n_theta * kQ * elem);
 }
 
 template cudaError_t launch_adjoint<float>(const CUtensorMap*, const CUtensorMap*, const CUtensorMap*,
-                                           const CUtensorMap*, const float*, const float*, float*,
-                                           const AdjScratch&, const StepParams&, const DvmConst<float>&, cudaStream_t,
-                                           cudaStream_t, cudaEvent_t, cudaEvent_t);
+                                           const CUtensorMap*, const float*, const float*, float*, unsigned char*,
+                                           const StepParams&, const DvmConst<float>&, cudaStream_t);
 template cudaError_t launch_adjoint<double>(const CUtensorMap*, const CUtensorMap*, const CUtensorMap*,
-                                            const CUtensorMap*, const double*, const double*,
-                                            double*, const AdjScratch&, const StepParams&, const DvmConst<double>&,
-                                            cudaStream_t, cudaStream_t, cudaEvent_t, cudaEvent_t);
+                                            const CUtensorMap*, const double*, const double*, double*, unsigned char*,
+                                            const StepParams&, const DvmConst<double>&, cudaStream_t);
 
 }  // namespace pclb

@@ -46,9 +46,7 @@ template <class T>
 cudaError_t launch_noneq_gen(const T*, T*, int, const StepParams&, const DvmG&, const DvmG32&, cudaStream_t);
 template <class T>
 cudaError_t launch_adjoint(const CUtensorMap*, const CUtensorMap*, const CUtensorMap*, const CUtensorMap*, const T*,
-                           const T*, T*, const AdjScratch&,
-                           const StepParams&, const DvmConst<T>&, cudaStream_t, cudaStream_t, cudaEvent_t,
-                           cudaEvent_t);
+                           const T*, T*, unsigned char*, const StepParams&, const DvmConst<T>&, cudaStream_t);
 template <class T>
 cudaError_t gen_launch_set_state(T*, const T*, const T*, const T*, const T*, const StepParams&, const DvmG&,
                                  const DvmG32&, cudaStream_t);
@@ -440,24 +438,12 @@ pclb_status do_step(pclb_ctx* ctx, int n) {
 
 template <class T>
 pclb_status do_adjoint(pclb_ctx* ctx, const CUtensorMap* tmap_f, const CUtensorMap* tmap_fn, const void* f) {
-  if (!ctx->side) {
-    // created on first use: the side stream (highest priority, so that the
-    // wall tiles are scheduled as soon as their inputs are ready) and the
-    // fork / join events
-    int lo = 0, hi = 0;
-    cudaError_t e = cudaDeviceGetStreamPriorityRange(&lo, &hi);
-    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&ctx->side, cudaStreamNonBlocking, hi);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "adjoint side stream");
-  }
   const int src = ctx->cur_lam, dst = 1 - ctx->cur_lam;
-  const AdjScratch ws = adjoint_scratch(ctx->ws + ctx->lay.adj_scratch, ctx->grid.n_theta, (int)sizeof(T));
   cudaError_t e = launch_adjoint<T>(tmap_f, &ctx->tmap_adj[3 + src], tmap_fn, &ctx->tmap_node[3 + src],
                                     reinterpret_cast<const T*>(f),
                                     reinterpret_cast<const T*>(ctx->ws + ctx->lay.lam[src]),
-                                    reinterpret_cast<T*>(ctx->ws + ctx->lay.lam[dst]), ws, ctx->sp, dvm_of<T>(ctx),
-                                    ctx->stream, ctx->side, ctx->ev_fork, ctx->ev_join);
+                                    reinterpret_cast<T*>(ctx->ws + ctx->lay.lam[dst]),
+                                    ctx->ws + ctx->lay.adj_scratch, ctx->sp, dvm_of<T>(ctx), ctx->stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "adjoint kernel launch");
   ctx->cur_lam = dst;
   return PCLB_OK;
@@ -879,9 +865,6 @@ pclb_status pclb_destroy(pclb_ctx* ctx) {
   if (st != PCLB_OK) std::snprintf(g_err, sizeof(g_err), "%s", ctx->err);
   drop_graphs(ctx);
   if (ctx->capture) cudaStreamDestroy(ctx->capture);
-  if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
-  if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
-  if (ctx->side) cudaStreamDestroy(ctx->side);
   destroy_io(ctx);
   delete static_cast<HostCtx*>(ctx);
   return st;

@@ -122,16 +122,11 @@ struct Layout {
   size_t partials;            // double [kDiagBlocks][8] reduction partials
   size_t diag_out;            // double [8]
   size_t stage;               // host-I/O staging: 8 fields [n_theta][n_r]
-  size_t adj_scratch;         // adjoint ghost states and wall cotangents
+  size_t adj_scratch;         // the adjoint's wall scratch (adjoint_walls.cuh)
   size_t gen_ghost;           // N_i = 16, 24: radial ghost values [side][layer][n_theta][Q]
   size_t total;
 };
 
-// Scratch of one adjoint step (device pointers inside the workspace).
-struct AdjScratch {
-  unsigned char* ghost;       // [side][layer][n_theta] EqParams of the radial ghost layers
-  unsigned char* gwall;       // [side][node][n_theta][4] cotangent the ghosts return
-};
 // Raises kernel fn's dynamic shared-memory limit to `bytes` once per device
 // (the attribute belongs to each device's context); `done` holds one bit per
 // device ordinal.
@@ -167,7 +162,6 @@ inline cudaError_t launch_overlapped(void (*fn)(P...), dim3 grid, int threads, i
 }
 
 size_t adjoint_scratch_bytes(int n_theta, int elem);
-AdjScratch adjoint_scratch(unsigned char* base, int n_theta, int elem);
 
 constexpr int kDiagBlocks = 304;    // 2 x 152 SMs
 
@@ -195,14 +189,12 @@ struct pclb_ctx {
   int32_t scheme = 0;       // pclb_scheme
   int32_t relaxation = 0;   // pclb_relaxation
   cudaStream_t stream;
-  cudaStream_t side = nullptr;        // high-priority stream for the adjoint's wall work
   cudaStream_t capture = nullptr;     // private stream for capturing step graphs
   struct StepGraph {
     int32_t n, cur;                   // steps and starting buffer of the captured sequence
     cudaGraphExec_t exec;
   } graphs[4] = {};
   int32_t n_graphs = 0;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   // pclb_run_host with page-locked buffers: the host transfers of each
   // azimuthal slab run on two copy streams and its set-state kernel on a
   // third stream while the steps of other slabs run on `stream` and io_alt
