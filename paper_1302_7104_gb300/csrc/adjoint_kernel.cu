@@ -35,31 +35,30 @@
 //     the products of the nodes that read it and adds d lam + psi . ((1-d) g +
 //     g_wall).  One barrier per pair separates the phases; a stage is refilled
 //     as soon as its pair's phase (A) is done.
+// The FP64 kernel is bound by FP64 issue (a warp-wide operation per ~76 cycles
+// and quarter SM); the partials are therefore formed in integers
+// (fx_mwb_partials, 10 of 14 FP64 operations less per label and direction).
+// TT = 8 rows; 4 on grids whose tiles would leave SMs idle.
 #include <cuda.h>
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "device_common.cuh"
 #include "adjoint_common.cuh"
 #include "adjoint_walls.cuh"
+#include "fixed64.cuh"
 #include "f32_state.cuh"
 #include "pclb_internal.h"
 
 namespace pclb {
 
-template <class T>
-struct AdjTile;
-template <>
-struct AdjTile<double> {
-  static constexpr int TT = kAdjRows64;
-  static constexpr int min_blocks = 3;   // at most 85 registers
-};
-
-// Courant entry of one pair of opposite velocities at one theta row:
-// (|C_r|, |C_r|(1 - |C_r|), |v_theta| dt / dtheta, flags) with flag bit 0 set
-// when v_r < 0 and bit 1 when v_theta < 0 for the first label of the pair.
-template <class T>
-struct alignas(4 * sizeof(T)) CourEntry {
-  T a_r, k_r, a_w;
+// Courant entry of one pair of opposite velocities at one theta row, in units
+// of 2^-63: alpha^2 and 2 alpha (1 - alpha) of alpha = |C_r|, and |C_theta| at
+// the tile's first column; flag bit 0 set when v_r < 0 and bit 1 when v_theta
+// < 0 for the first label of the pair.
+struct alignas(32) CourEntry {
+  uint64_t a2, k2, at;
   int fl;
 };
 
@@ -70,23 +69,23 @@ constexpr int kAdjStages = 2;   // ring depth of the pair-streaming kernel (2 me
 static_assert(sizeof(EqParams<float>) == 10 * sizeof(float) && sizeof(EqParams<double>) == 10 * sizeof(double),
               "ghost-state scratch holds 10 values per EqParams");
 
-template <class T>
+template <int TT>
 struct AdjSize {
-  static constexpr int TT = AdjTile<T>::TT;
   static constexpr int threads = 32 * TT;
+  static constexpr int min_blocks = 24 / TT;   // at most 85 registers
   static constexpr int plane = kWinR * (TT + 4);
   static constexpr int npairs = 4 * kNDirs / 2;
   // products of one label: radial A, B over TT rows x 36 columns (tile
   // columns -2 .. 33), azimuthal A, B over TT + 4 rows (-2 .. TT + 1) x 32
   static constexpr int rcols = kTileR + 4;
   static constexpr int prod = 2 * TT * rcols + 2 * (TT + 4) * kTileR;
-  static constexpr int ring_bytes = kAdjStages * 4 * plane * (int)sizeof(T);   // f, f', lam, lam' per stage
-  static constexpr int prod_bytes = 2 * 2 * prod * (int)sizeof(T);             // 2 buffers x 2 labels
-  static constexpr int invr_bytes = kTileR * (int)sizeof(T);
-  static constexpr int tab_bytes = (TT + 4) * npairs * (int)sizeof(CourEntry<T>);
-  static constexpr int smem = ring_bytes + prod_bytes + invr_bytes + tab_bytes + 128;
+  static constexpr int ring_bytes = kAdjStages * 4 * plane * 8;   // f, f', lam, lam' per stage
+  static constexpr int prod_bytes = 2 * 2 * prod * 8;             // 2 buffers x 2 labels
+  static constexpr int ratio_bytes = kTileR * 8;
+  static constexpr int tab_bytes = (TT + 4) * npairs * (int)sizeof(CourEntry);
+  static constexpr int smem = ring_bytes + prod_bytes + ratio_bytes + tab_bytes + 128;
   // the ring's planes are TMA destinations: 128-byte aligned
-  static_assert((plane * (int)sizeof(T)) % 128 == 0, "TMA destinations must stay 128-byte aligned");
+  static_assert((plane * 8) % 128 == 0, "TMA destinations must stay 128-byte aligned");
 };
 
 namespace {
@@ -106,40 +105,42 @@ __device__ __forceinline__ void adj_node_state(const double* f, int plane, const
 // upwind side at offset U, q2 (the opposite velocity) at -U.  sf, sl: the
 // pair's f and lam planes (q2 at +PLANE); o: the node in a plane; pr: its
 // product slot (M_D products; the M_Dp ones at +DB, q2's at +PROD).
-template <class T, int U, int PLANE, int PROD, int DB>
-__device__ __forceinline__ void radial_pair(const T* sf, const T* sl, T* pb, int o, int pr, T a, T K, T lam[2]) {
-  T MD, MP;
-  const T* f1 = sf + o;
-  mwb_partials<T>(a, K, f1[0] - f1[U], f1[U] - f1[2 * U], MD, MP);
-  lam[0] = sl[o];
-  pb[pr] = lam[0] * MD;
-  pb[pr + DB] = lam[0] * MP;
-  const T* f2 = sf + PLANE + o;
-  mwb_partials<T>(a, K, f2[0] - f2[-U], f2[-U] - f2[-2 * U], MD, MP);
-  lam[1] = sl[PLANE + o];
-  pb[PROD + pr] = lam[1] * MD;
-  pb[PROD + pr + DB] = lam[1] * MP;
+template <int U, int PLANE, int PROD, int DB>
+__device__ __forceinline__ void radial_pair(const double* sf, const double* sl, double* pb, int o, int pr, uint64_t a2,
+                                            uint64_t k2, double lam[2]) {
+#pragma unroll
+  for (int L = 0; L < 2; ++L) {
+    constexpr int kU[2] = {U, -U};
+    const double* f = sf + L * PLANE + o;
+    double MD, MP;
+    fx_mwb_partials(f[0] - f[kU[L]], f[kU[L]] - f[2 * kU[L]], a2, k2, MD, MP);
+    lam[L] = sl[L * PLANE + o];
+    pb[L * PROD + pr] = lam[L] * MD;
+    pb[L * PROD + pr + DB] = lam[L] * MP;
+  }
 }
 
-template <class T, int U, int PLANE, int PROD, int DB>
-__device__ __forceinline__ void azimuthal_pair(const T* sf, const T lam[2], T* pb, int o, int pa, T a, T K) {
-  T MD, MP;
-  const T* f1 = sf + o;
-  mwb_partials<T>(a, K, f1[0] - f1[U], f1[U] - f1[2 * U], MD, MP);
-  pb[pa] = lam[0] * MD;
-  pb[pa + DB] = lam[0] * MP;
-  const T* f2 = sf + PLANE + o;
-  mwb_partials<T>(a, K, f2[0] - f2[-U], f2[-U] - f2[-2 * U], MD, MP);
-  pb[PROD + pa] = lam[1] * MD;
-  pb[PROD + pa + DB] = lam[1] * MP;
+template <int U, int PLANE, int PROD, int DB>
+__device__ __forceinline__ void azimuthal_pair(const double* sf, const double lam[2], double* pb, int o, int pa,
+                                               uint64_t a2, uint64_t k2) {
+#pragma unroll
+  for (int L = 0; L < 2; ++L) {
+    constexpr int kU[2] = {U, -U};
+    const double* f = sf + L * PLANE + o;
+    double MD, MP;
+    fx_mwb_partials(f[0] - f[kU[L]], f[kU[L]] - f[2 * kU[L]], a2, k2, MD, MP);
+    pb[L * PROD + pa] = lam[L] * MD;
+    pb[L * PROD + pa + DB] = lam[L] * MP;
+  }
 }
 
 // One label at one halo node, upwind side at offset U.
-template <class T, int U>
-__device__ __forceinline__ void azimuthal_one(const T* fw, const T* lw, T* pa, int DB, T a, T K) {
-  T MD, MP;
-  mwb_partials<T>(a, K, fw[0] - fw[U], fw[U] - fw[2 * U], MD, MP);
-  const T lam = lw[0];
+template <int U>
+__device__ __forceinline__ void azimuthal_one(const double* fw, const double* lw, double* pa, int DB, uint64_t a2,
+                                              uint64_t k2) {
+  double MD, MP;
+  fx_mwb_partials(fw[0] - fw[U], fw[U] - fw[2 * U], a2, k2, MD, MP);
+  const double lam = lw[0];
   pa[0] = lam * MD;
   pa[DB] = lam * MP;
 }
@@ -187,15 +188,16 @@ __device__ __forceinline__ void gather_azimuthal_mixed(const T* pb, int pa, int 
 // ---------------------------------------------------------------------------
 // Pair-streaming part.
 // ---------------------------------------------------------------------------
-template <class T>
-__global__ void __launch_bounds__(AdjSize<T>::threads, AdjTile<T>::min_blocks)
+template <int TT>
+__global__ void __launch_bounds__(AdjSize<TT>::threads, AdjSize<TT>::min_blocks)
     adjoint_pair_kernel(const __grid_constant__ CUtensorMap tmap_f, const __grid_constant__ CUtensorMap tmap_l,
-                        const T* __restrict__ f, const T* __restrict__ lam_in, T* __restrict__ lam_out,
-                        const __grid_constant__ WallScratch<T> ws, const __grid_constant__ AdjOrder order,
-                        const __grid_constant__ StepParams p, const __grid_constant__ DvmConst<T> d) {
-  constexpr int TT = AdjTile<T>::TT;
-  constexpr int PLANE = AdjSize<T>::plane;
-  constexpr int NP = AdjSize<T>::npairs, RC = AdjSize<T>::rcols, PROD = AdjSize<T>::prod;
+                        const double* __restrict__ f, const double* __restrict__ lam_in, double* __restrict__ lam_out,
+                        const __grid_constant__ WallScratch<double> ws, const __grid_constant__ AdjOrder order,
+                        const __grid_constant__ StepParams p, const __grid_constant__ DvmConst<double> d) {
+  using T = double;
+  using SZ = AdjSize<TT>;
+  constexpr int PLANE = SZ::plane;
+  constexpr int NP = SZ::npairs, RC = SZ::rcols, PROD = SZ::prod;
   constexpr int S = kAdjStages;
   // offsets inside one label's products
   constexpr int AR = 0, BR = TT * RC, AT = 2 * TT * RC, BT = 2 * TT * RC + (TT + 4) * kTileR;
@@ -203,8 +205,8 @@ __global__ void __launch_bounds__(AdjSize<T>::threads, AdjTile<T>::min_blocks)
   extern __shared__ __align__(128) unsigned char smem_raw[];
   T* ring = reinterpret_cast<T*>(smem_raw);                 // [stage][f q1, f q2, lam q1, lam q2][PLANE]
   T* prod = ring + S * 4 * PLANE;                             // [buffer][label][products]
-  T* invr = prod + 2 * 2 * PROD;                              // 1/r of the tile columns
-  CourEntry<T>* ctab = reinterpret_cast<CourEntry<T>*>(invr + kTileR);   // [TT + 4][NP]
+  uint64_t* ratio = reinterpret_cast<uint64_t*>(prod + 2 * 2 * PROD);   // 1/r of the tile columns relative to the first
+  CourEntry* ctab = reinterpret_cast<CourEntry*>(ratio + kTileR);        // [TT + 4][NP]
   uint64_t* bar = reinterpret_cast<uint64_t*>(ctab + (TT + 4) * NP);     // [S]
 
   int tx, ty;
@@ -237,16 +239,24 @@ __global__ void __launch_bounds__(AdjSize<T>::threads, AdjTile<T>::min_blocks)
   const int cw_out = p.n_r - 1 - r0 + kLeft;
   const bool inner = r0 == 0, outer = cw_out <= kLeft + kTileR;
   const int slots[2] = {0, WallScratch<T>::slot(1, tx == order.nt - 1)};
-  static_assert(sizeof(WallShared<T, TT>) <= (TT + 4) * NP * sizeof(CourEntry<T>), "wall scratch inside the Courant table");
+  static_assert(sizeof(WallShared<T, TT>) <= (TT + 4) * NP * sizeof(CourEntry), "wall scratch inside the Courant table");
   for (int side = 0; side < 2; ++side)
     if (side == 0 ? inner : outer)
       adjoint_walls<T, TT>(f, lam_in, side, slots[side], t0, ws, *reinterpret_cast<WallShared<T, TT>*>(ctab), p, d);
-  if (tid < kTileR) invr[tid] = r0 + tid < p.n_r ? (T)p.inv_r[r0 + tid] : T(1);
+  const double inv_r0 = p.inv_r[r0];
+  if (tid < kTileR) ratio[tid] = r0 + tid < p.n_r ? fx_fraction(p.inv_r[r0 + tid] * recip_newton(inv_r0)) : 0;
   // Courant entries of the stored rows t0 .. t0 + TT + 3 (theta rows t0 - 2 .. t0 + TT + 1)
   for (int i = tid; i < (TT + 4) * NP; i += blockDim.x) {
     const int srow = t0 + i / NP, pr = i % NP;
-    CourEntry<T> e{T(0), T(0), T(0), 0};
-    if (srow < p.rows) courant_entry(p, srow, pr, e.a_r, e.k_r, e.a_w, e.fl);
+    CourEntry e{0, 0, 0, 0};
+    if (srow < p.rows) {
+      const double* c = p.courant64 + ((size_t)srow * NP + pr) * 4;
+      const uint64_t alpha = fx_fraction(c[0]);
+      e.a2 = fx_mul_frac(alpha, alpha);
+      e.k2 = 2 * (alpha - e.a2);
+      e.at = fx_fraction(c[2] * inv_r0);
+      e.fl = (int)c[3];
+    }
     ctab[i] = e;
   }
   __syncthreads();
@@ -301,7 +311,7 @@ __global__ void __launch_bounds__(AdjSize<T>::threads, AdjTile<T>::min_blocks)
   const int o_node = row * kWinR + col;                 // this node in a window plane
   const int p_rad = AR + rowl * RC + lane + 2;          // its radial product slot
   const int p_az = AT + row * kTileR + lane;            // its azimuthal product slot
-  const T my_invr = invr[lane];
+  const uint64_t my_ratio = ratio[lane];
   auto store = [&](int q, T v) {
     lam_out[(size_t)q * plane_out + (size_t)srow * p.pitch + r] = v;
     if (t >= p.n_theta - 2)
@@ -360,33 +370,41 @@ __global__ void __launch_bounds__(AdjSize<T>::threads, AdjTile<T>::min_blocks)
     // branch in which the stencil offsets are constants.
     const T* sfp = st;                                    // f q1, f q2 at +PLANE
     const T* slp = st + 2 * PLANE;                        // lam q1, lam q2 at +PLANE
-    const CourEntry<T> e = ctab[row * NP + pair];
+    const CourEntry e = ctab[row * NP + pair];
     const int fl_c = e.fl;                                // flags of this node's row
     T lam_c[2];                                           // lam^{n+1} of both labels at this node
     if (fl_c & 1)
-      radial_pair<T, 1, PLANE, PROD, BR - AR>(sfp, slp, pb, o_node, p_rad, e.a_r, e.k_r, lam_c);
+      radial_pair<1, PLANE, PROD, BR - AR>(sfp, slp, pb, o_node, p_rad, e.a2, e.k2, lam_c);
     else
-      radial_pair<T, -1, PLANE, PROD, BR - AR>(sfp, slp, pb, o_node, p_rad, e.a_r, e.k_r, lam_c);
+      radial_pair<-1, PLANE, PROD, BR - AR>(sfp, slp, pb, o_node, p_rad, e.a2, e.k2, lam_c);
+    // alpha^2 and 2 alpha (1 - alpha) of |C_theta| at this node
+    auto azimuthal = [&](uint64_t at, uint64_t& a2, uint64_t& k2) {
+      const uint64_t alpha = fx_mul_frac(at, my_ratio);
+      a2 = fx_mul_frac(alpha, alpha);
+      k2 = 2 * (alpha - a2);
+    };
     {
-      const T at = e.a_w * my_invr, kt = at - at * at;
+      uint64_t a2, k2;
+      azimuthal(e.at, a2, k2);
       if (fl_c & 2)
-        azimuthal_pair<T, kWinR, PLANE, PROD, BT - AT>(sfp, lam_c, pb, o_node, p_az, at, kt);
+        azimuthal_pair<kWinR, PLANE, PROD, BT - AT>(sfp, lam_c, pb, o_node, p_az, a2, k2);
       else
-        azimuthal_pair<T, -kWinR, PLANE, PROD, BT - AT>(sfp, lam_c, pb, o_node, p_az, at, kt);
+        azimuthal_pair<-kWinR, PLANE, PROD, BT - AT>(sfp, lam_c, pb, o_node, p_az, a2, k2);
     }
     if (rowl < 4) {
       // halo rows: warps 0..3 take window rows 0, 1, TT + 2, TT + 3; rows
       // above the tile are read by labels whose upwind side is +theta
       const int rr = rowl < 2 ? rowl : TT + rowl;
-      const CourEntry<T> eh = ctab[rr * NP + pair];
+      const CourEntry eh = ctab[rr * NP + pair];
       const bool q1_up_pos = (eh.fl & 2) != 0;
-      const T ath = eh.a_w * my_invr, kth = ath - ath * ath;
+      uint64_t ath, kth;
+      azimuthal(eh.at, ath, kth);
       const int o = rr * kWinR + col;
       if (rowl < 2)
-        azimuthal_one<T, kWinR>(sfp + (q1_up_pos ? 0 : PLANE) + o, slp + (q1_up_pos ? 0 : PLANE) + o,
+        azimuthal_one<kWinR>(sfp + (q1_up_pos ? 0 : PLANE) + o, slp + (q1_up_pos ? 0 : PLANE) + o,
                                 pb + (q1_up_pos ? 0 : PROD) + AT + rr * kTileR + lane, BT - AT, ath, kth);
       else
-        azimuthal_one<T, -kWinR>(sfp + (q1_up_pos ? PLANE : 0) + o, slp + (q1_up_pos ? PLANE : 0) + o,
+        azimuthal_one<-kWinR>(sfp + (q1_up_pos ? PLANE : 0) + o, slp + (q1_up_pos ? PLANE : 0) + o,
                                  pb + (q1_up_pos ? PROD : 0) + AT + rr * kTileR + lane, BT - AT, ath, kth);
     }
     {
@@ -400,13 +418,13 @@ __global__ void __launch_bounds__(AdjSize<T>::threads, AdjTile<T>::min_blocks)
         const int h = (kSep ? rowl - 4 : rowl) * 32 + lane;
         if (h < 4 * TT) {
           const int hr = h >> 2, L = (h >> 1) & 1, j = h & 1;
-          const CourEntry<T> eh = ctab[(hr + 2) * NP + pair];
+          const CourEntry eh = ctab[(hr + 2) * NP + pair];
           const int uh = (eh.fl & 1) ? 1 : -1, uL = L ? -uh : uh;
           const int c = uL == 1 ? j - 2 : kTileR + j;
           const int o = (hr + 2) * kWinR + c + kLeft;
           const T* fw = sfp + L * PLANE + o;
           T MD, MP;
-          mwb_partials<T>(eh.a_r, eh.k_r, fw[0] - fw[uL], fw[uL] - fw[2 * uL], MD, MP);
+          fx_mwb_partials(fw[0] - fw[uL], fw[uL] - fw[2 * uL], eh.a2, eh.k2, MD, MP);
           const T lam = slp[L * PLANE + o];
           pb[L * PROD + AR + hr * RC + c + 2] = lam * MD;
           pb[L * PROD + BR + hr * RC + c + 2] = lam * MP;
@@ -475,7 +493,7 @@ cudaError_t launch_adjoint(const CUtensorMap* tmap_f, const CUtensorMap* tmap_l,
   ws.gwall = reinterpret_cast<T*>(scratch + scratch_part((size_t)9 * p.n_theta * 10 * sizeof(T)));
   ws.gdir = reinterpret_cast<T*>(reinterpret_cast<unsigned char*>(ws.gwall) +
                                  scratch_part((size_t)24 * p.n_theta * sizeof(T)));
-  constexpr int rows = sizeof(T) == 4 ? kAdjRows32 : kAdjRows64;
+  const int rows = p.adj_rows;
   AdjOrder order;
   order.nt = (p.n_r + kTileR - 1) / kTileR;
   order.ny = (p.n_theta + rows - 1) / rows;
@@ -486,12 +504,16 @@ cudaError_t launch_adjoint(const CUtensorMap* tmap_f, const CUtensorMap* tmap_l,
     // FP32: the packed two-nodes-per-thread pair kernel (adjoint_f32x2.cu)
     return launch_adjoint_pairs_f32(tmap_f, tmap_l, tmap_fn, tmap_ln, f, lam_in, lam_out, ws, order, p, d, stream);
   } else {
-    static std::atomic<unsigned long long> configured{0};
-    constexpr int smem = AdjSize<T>::smem;
-    const cudaError_t e = set_smem_once(adjoint_pair_kernel<T>, smem, configured);
-    if (e != cudaSuccess) return e;
-    return launch_overlapped(adjoint_pair_kernel<T>, dim3((unsigned)order.blocks()), AdjSize<T>::threads, smem, stream,
-                             *tmap_f, *tmap_l, f, lam_in, lam_out, ws, order, p, d);
+    auto go = [&](auto tt) {
+      constexpr int TT = decltype(tt)::value;
+      static std::atomic<unsigned long long> configured{0};
+      const cudaError_t e = set_smem_once(adjoint_pair_kernel<TT>, AdjSize<TT>::smem, configured);
+      if (e != cudaSuccess) return e;
+      return launch_overlapped(adjoint_pair_kernel<TT>, dim3((unsigned)order.blocks()), AdjSize<TT>::threads,
+                               AdjSize<TT>::smem, stream, *tmap_f, *tmap_l, f, lam_in, lam_out, ws, order, p, d);
+    };
+    return rows == kAdjRows64 ? go(std::integral_constant<int, kAdjRows64>{})
+                              : go(std::integral_constant<int, kAdjRows64Small>{});
   }
 }
 

@@ -116,4 +116,47 @@ __device__ __forceinline__ int64_t fx_mwb(int64_t D, int64_t Dp, const FxCourant
   return fx_signed(fx_mul(a, coef), s);
 }
 
+// A fraction (units of 2^-63) as a double.
+__device__ __forceinline__ double fx_fraction_to_double(uint64_t u) {
+  const int lz = __clzll((long long)u);
+  const uint64_t m = u << (lz & 63), r = (m >> 11) + ((m >> 10) & 1);
+  const uint32_t hi = (uint32_t)(r >> 32) + ((uint32_t)(1022 - lz) << 20);
+  return u == 0 ? 0.0 : __hiloint2double((int)hi, (int)(uint32_t)r);
+}
+
+// Partial derivatives of M of Eq. (28) (mwb_partials in adjoint_common.cuh) with
+// respect to D and Dp, from a2 = alpha^2 and k2 = 2 alpha (1 - alpha) in units of
+// 2^-63.  With v = |D| / (|D| + |Dp|): D and Dp of one sign, M_D = a2 + 2 k2 v -
+// k2 v^2 and M_Dp = -k2 v^2; of opposite signs, a2 + k2 and 0; D = 0, a2 + k2 / 2
+// and 0; Dp = 0, a2 + k2 and -k2 / 2.  v is formed on aligned integer mantissas
+// to ~2^-62 (three float quotient digits with exact remainders), so the only
+// FP64 operations are the caller's two differences.  Not finite: NaN.
+__device__ __forceinline__ void fx_mwb_partials(double D, double Dp, uint64_t a2, uint64_t k2, double& MD, double& MDp) {
+  const int hD = __double2hiint(D), hP = __double2hiint(Dp);
+  const uint32_t lD = (uint32_t)__double2loint(D), lP = (uint32_t)__double2loint(Dp);
+  const int eD = (hD >> 20) & 0x7ff, eP = (hP >> 20) & 0x7ff, e = max(eD, eP);
+  auto mantissa = [&](int h, uint32_t l, int ex) -> uint64_t {
+    const uint64_t m = ((uint64_t)(((uint32_t)h & 0xfffffu) | 0x100000u) << 32 | l) << 6;
+    return ex == 0 ? 0 : m >> min(e - ex, 63);
+  };
+  const uint64_t a = mantissa(hD, lD, eD), n = a + mantissa(hP, lP, eP);   // n < 2^60
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fx_float(n)));
+  const uint32_t i0 = __float_as_uint(__fadd_rn(fx_float(a) * r, 1.0f)) - 0x3f800000u;   // units of 2^-23
+  const int64_t rem0 = (int64_t)((a << 23) - n * (uint64_t)i0);
+  const int32_t i1 = __float2int_rn(fx_float(rem0) * r * 4194304.0f);                    // units of 2^-45
+  const int64_t rem1 = (int64_t)(((uint64_t)rem0 << 22) - n * (uint64_t)(int64_t)i1);
+  const int32_t i2 = __float2int_rn(fx_float(rem1) * r * 262144.0f);                     // units of 2^-63
+  const uint64_t v = ((uint64_t)i0 << 40) + (uint64_t)((int64_t)i1 * 262144) + (uint64_t)(int64_t)i2;
+  const uint64_t w = fx_mul_frac(k2, v), wv = fx_mul_frac(w, v);
+  const bool zD = (((uint32_t)hD << 1) | lD) == 0, zP = (((uint32_t)hP << 1) | lP) == 0;
+  const bool opposite = (hD ^ hP) < 0;
+  uint64_t md = a2 + 2 * w - wv, mp = wv;
+  if (opposite || zP) { md = a2 + k2; mp = zP ? k2 >> 1 : 0; }
+  if (zD || e == 0) { md = a2 + (k2 >> 1); mp = 0; }
+  const bool finite = e < 0x7ff;
+  MD = finite ? fx_fraction_to_double(md) : __hiloint2double(0x7ff80000, 0);
+  MDp = finite ? -fx_fraction_to_double(mp) : MD;
+}
+
 }  // namespace pclb

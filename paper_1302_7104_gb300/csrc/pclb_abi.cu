@@ -310,7 +310,15 @@ pclb_status encode_map(pclb_ctx* ctx, const void* base, int box_rows, CUtensorMa
   return PCLB_OK;
 }
 
-int adj_box_rows(const pclb_ctx* ctx) { return (ctx->prec == PCLB_FP64 ? kAdjRows64 : kAdjRows32) + 4; }
+int adj_box_rows(const pclb_ctx* ctx) { return ctx->sp.adj_rows + 4; }
+
+// Tile rows of the adjoint: 16 in FP32; in FP64 8, or 4 where tiles of 8 rows
+// would leave SMs (152) without one.
+int adj_tile_rows(const pclb_grid* g, pclb_precision prec) {
+  if (prec == PCLB_FP32) return kAdjRows32;
+  const long long tiles = (long long)((g->n_r + kTileR - 1) / kTileR) * ((g->n_theta + kAdjRows64 - 1) / kAdjRows64);
+  return tiles <= kSmallGridTilesAdj ? kAdjRows64Small : kAdjRows64;
+}
 
 // The node-phase descriptor of the FP32 adjoint: one tile, kTileR x kAdjRows32
 // (unused for FP64).
@@ -802,6 +810,7 @@ pclb_status pclb_create(const pclb_grid* grid, const pclb_dvm* dvm, double tau, 
   sp.decay = std::exp(-dt / tau);
   sp.scheme = PCLB_SCHEME_MWB;
   sp.tile_rows = step_tile_rows(grid, dvm, prec);
+  sp.adj_rows = adj_tile_rows(grid, prec);
   sp.wait_ns = kDefaultWaitNs;
   sp.bc_kind[0] = bc->kind[0];
   sp.bc_kind[1] = bc->kind[1];

@@ -40,6 +40,8 @@ constexpr int kGhostRows = 2;       // azimuthal ghost rows stored on each side
 // Tile rows of the adjoint kernel (its window holds f and lam for all labels).
 constexpr int kAdjRows32 = 16;
 constexpr int kAdjRows64 = 8;
+constexpr int kAdjRows64Small = 4;    // FP64 on grids of at most kSmallGridTilesAdj tiles of 8 rows
+constexpr int kSmallGridTilesAdj = 152;
 // Time a kernel waits for the TMA copies of its own window (mbarrier phase)
 // before it reports PCLB_FLAG_TIMEOUT and gives the tile up; the copies of a
 // tile given up get the default limit again to land before the CTA exits.
@@ -107,6 +109,7 @@ struct StepParams {
   const float* inv_r_f;       // [n_r] 1 / r_i in float
   const float4* cs_ff;        // [n_theta] cos theta_i, sin theta_i as float-float pairs (hi, lo, hi, lo)
   int tile_rows;              // tile rows of the step, kTileT or kTileTSmall
+  int adj_rows;               // tile rows of the adjoint
   uint32_t* status;           // device status word (PCLB_FLAG_*)
   uint64_t wait_ns;           // a step's wait for its own window copies before it gives the tile up
 };
