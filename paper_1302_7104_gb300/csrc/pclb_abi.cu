@@ -327,12 +327,12 @@ pclb_status encode_node_map(pclb_ctx* ctx, const void* base, CUtensorMap* out) {
   return encode_map(ctx, base, kAdjRows32, out, kTileR);
 }
 
-// Tile rows of the octagon's step: small tiles while the chip (152 SMs) could
-// not be filled with large ones.
+// Tile rows of the octagon's step: smaller tiles while the chip (152 SMs)
+// could not be filled with large ones.
 int step_tile_rows(const pclb_grid* g, const pclb_dvm* d, pclb_precision prec) {
   const long long tiles = (long long)((g->n_r + kTileR - 1) / kTileR) * ((g->n_theta + kTileT - 1) / kTileT);
-  return d->n_dirs == kNDirs && tiles <= (prec == PCLB_FP64 ? kSmallGridTiles64 : kSmallGridTiles32) ? kTileTSmall
-                                                                                                     : kTileT;
+  if (d->n_dirs != kNDirs || tiles > kSmallGridTiles) return kTileT;
+  return prec == PCLB_FP64 && tiles <= kTinyGridTiles64 ? 2 : kTileTSmall;
 }
 
 // Window rows of the step's TMA boxes (in FP64 the small tiles are the MWB

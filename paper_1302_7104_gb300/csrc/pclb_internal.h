@@ -28,9 +28,10 @@ constexpr int kTileT = 16;
 constexpr int kTileT32 = 16;
 constexpr int kStepThreads32 = 16 * kTileT32;
 constexpr int kCtasPerSm32 = 2;
-constexpr int kTileTSmall = 4;      // the steps of the octagon on small grids
-// at most this many 32 x 16 tiles: small tiles
-constexpr int kSmallGridTiles64 = 76, kSmallGridTiles32 = 76;
+// The octagon's steps on small grids: tiles of kTileTSmall rows on at most
+// kSmallGridTiles tiles of 32 x 16, in FP64 of two rows on at most kTinyGridTiles64.
+constexpr int kTileTSmall = 4;
+constexpr int kSmallGridTiles = 76, kTinyGridTiles64 = 8;
 constexpr int kWinR = kTileR + 8;   // 40 columns
 constexpr int kWinT = kTileT + 4;   // 20 rows
 constexpr int kLeft = 4;            // column of interior r0 inside the window
@@ -108,7 +109,7 @@ struct StepParams {
   const double* courant64;    // the same table in double: [n_theta + 4][pairs][4] (flags as value)
   const float* inv_r_f;       // [n_r] 1 / r_i in float
   const float4* cs_ff;        // [n_theta] cos theta_i, sin theta_i as float-float pairs (hi, lo, hi, lo)
-  int tile_rows;              // tile rows of the step, kTileT or kTileTSmall
+  int tile_rows;              // tile rows of the step: kTileT, kTileTSmall or (FP64) 2
   int adj_rows;               // tile rows of the adjoint
   uint32_t* status;           // device status word (PCLB_FLAG_*)
   uint64_t wait_ns;           // a step's wait for its own window copies before it gives the tile up

@@ -27,8 +27,9 @@
 // again and evaluated in FP64 throughout.
 //
 // TT = 16: one thread per node, for grids that fill the chip with such tiles.
-// TT = 4: the four shells of a row on four warps, for small grids, where the
-// time of one tile is the time of the step.
+// TT = 4 or 2: the shells of a row on four warps, or half shells on eight, for
+// small grids, where the time of one tile is the time of the step.
+// Consecutive steps overlap their set-up (programmatic dependent launch).
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -54,13 +55,14 @@ struct FxTab {
 
 template <int TT>
 struct FxSize {
-  static constexpr int split = 16 / TT;                       // warps per row
+  static constexpr int split = 16 / TT;                       // warps per row: 1, 4 or 8
+  static constexpr int dirs = split <= 4 ? kHalfDirs : 4 * kHalfDirs / split;   // direction pairs of a shell per warp
   static constexpr int plane = kWinR * (TT + 4);
   static constexpr int planes_bytes = kQ * plane * 8;
   static constexpr int tab_bytes = kPairsFx * TT * (int)sizeof(FxTab);
   static constexpr int ghost_bytes = kGhostScratch64<TT> * 8;
-  // split > 1: per node the shells' sums (S, X, Y), then w_1..4, w_0, a0, a1, u/E, rho
-  static constexpr int node_bytes = split > 1 ? 32 * TT * 12 * 8 : 0;
+  // split > 1: per node the shells' sums (S, X, Y), then w_1..4, a0, a1, u/E; split 8: the second halves' sums too
+  static constexpr int node_bytes = split > 1 ? 32 * TT * (split > 4 ? 24 : 12) * 8 : 0;
   static constexpr int scratch = ghost_bytes > node_bytes ? ghost_bytes : node_bytes;
   static constexpr int smem = planes_bytes + tab_bytes + scratch + 128;
   static_assert((plane * 8) % 128 == 0, "TMA destinations must stay 128-byte aligned");
@@ -133,7 +135,6 @@ __global__ void __launch_bounds__(kThreadsFx, 1)
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
     mbar_fence_init();
-    load(&bar[0]);
   }
   const double inv_r0 = p.inv_r[r0];
   if (tid < kPairsFx * TT) {   // Courant entries of the tile rows
@@ -147,6 +148,9 @@ __global__ void __launch_bounds__(kThreadsFx, 1)
     tab[pair * TT + rl] = t;
   }
   if (tid < kGroupsFx) top[tid] = 0;
+  pdl_wait();      // the step before this one has written f and read f_out
+  pdl_launch();    // the next one may start its set-up
+  if (tid == 0) load(&bar[0]);
   // The whole block gives the tile up if any thread's wait ran out (block
   // barriers follow, so the decision must be uniform); thread 0 then gives
   // the copies one more bounded chance to land before the block exits.
@@ -205,21 +209,32 @@ __global__ void __launch_bounds__(kThreadsFx, 1)
   const double decay = p.decay, omd = 1.0 - decay;
   EqParams<double> eq;
   double f0 = 0.0;
-  // the sums S, X = sum c_x f, Y of shell k (1 / sqrt 2 as a fraction of 2^63)
-  auto shell_sums = [&](int k, double o[3]) {
-    const int64_t* f = fx + (1 + (k - 1) * kNDirs) * PLANE + node;
-    int64_t S = 0, D[kHalfDirs];
+  // this warp's shells and direction pairs
+  constexpr int DIRS = SZ::dirs;
+  const int k_first = SPLIT == 1 ? 1 : split / (SPLIT / 4) + 1, k_last = SPLIT == 1 ? 4 : k_first;
+  const int i_first = SPLIT > 4 ? (split & 1) * DIRS : 0;
+  auto shell_exp = [&](int k) { return k == 1 ? ek[1] : (k == 2 ? ek[2] : (k == 3 ? ek[3] : ek[4])); };
+  // the sums S, X = sum c_x f, Y over those direction pairs of shell k
+  auto shell_sums = [&](int k, int64_t o[3]) {
+    const int64_t* f = fx + (1 + (k - 1) * kNDirs + i_first) * PLANE + node;
+    int64_t S = 0, D[DIRS];
 #pragma unroll
-    for (int i = 0; i < kHalfDirs; ++i) {
+    for (int i = 0; i < DIRS; ++i) {
       const int64_t a = f[i * PLANE], b = f[(i + kHalfDirs) * PLANE];
       S += a + b;
       D[i] = a - b;
     }
-    const int e = k == 1 ? ek[1] : (k == 2 ? ek[2] : (k == 3 ? ek[3] : ek[4]));
+    // x / sqrt 2 (the fraction in units of 2^-63)
     auto diagonal = [](int64_t x) { return fx_signed(fx_mul(fx_abs(x), 0x5a827999fcef3242ull), x >> 63); };
-    o[0] = fx_to_double(S, e);
-    o[1] = fx_to_double(D[0] + diagonal(D[1] - D[3]), e);
-    o[2] = fx_to_double(D[2] + diagonal(D[1] + D[3]), e);
+    o[0] = S;
+    if constexpr (DIRS == 4) {   // directions (1,0), (s,s), (0,1), (-s,s)
+      o[1] = D[0] + diagonal(D[1] - D[3]);
+      o[2] = D[2] + diagonal(D[1] + D[3]);
+    } else {
+      const int64_t g = diagonal(D[1]);
+      o[1] = i_first == 0 ? D[0] + g : -g;
+      o[2] = i_first == 0 ? g : D[0] + g;
+    }
   };
   // factors of (1 - d) f^eq: w_k = (1 - d) rho F_k
   auto factors = [&](const NodeState<double>& m) {
@@ -233,19 +248,32 @@ __global__ void __launch_bounds__(kThreadsFx, 1)
       double s0 = f0, sx = 0.0, sy = 0.0, se = 0.0;
 #pragma unroll 1
       for (int k = 1; k <= 4; ++k) {
-        double s[3];
+        int64_t s[3];
         shell_sums(k, s);
-        s0 += s[0];
-        sx = fma(d.speed[k], s[1], sx);
-        sy = fma(d.speed[k], s[2], sy);
-        se = fma(d.half_v2[k], s[0], se);
+        const int e = shell_exp(k);
+        const double S = fx_to_double(s[0], e);
+        s0 += S;
+        sx = fma(d.speed[k], fx_to_double(s[1], e), sx);
+        sy = fma(d.speed[k], fx_to_double(s[2], e), sy);
+        se = fma(d.half_v2[k], S, se);
       }
       factors(node_state64(s0, sx, sy, se));
     }
   } else {
-    // shell split + 1 by this warp, the state by the row's first warp
+    // this warp's part of the sums, the state by the row's first warp
     double* part = scratch + (rl * 32 + lane) * 12;
-    if (!general) shell_sums(split + 1, part + 3 * split);
+    int64_t s[3];
+    if (!general) shell_sums(k_first, s);
+    if constexpr (SPLIT > 4) {   // the halves of a shell
+      int64_t* second = reinterpret_cast<int64_t*>(scratch + 32 * TT * 12) + (rl * 32 + lane) * 12 + 3 * (k_first - 1);
+      if (!general && i_first != 0)
+        for (int j = 0; j < 3; ++j) second[j] = s[j];
+      __syncthreads();
+      if (!general && i_first == 0)
+        for (int j = 0; j < 3; ++j) s[j] += second[j];
+    }
+    if (!general && i_first == 0)
+      for (int j = 0; j < 3; ++j) part[3 * (k_first - 1) + j] = fx_to_double(s[j], shell_exp(k_first));
     __syncthreads();
     if (!general && split == 0) {
       f0 = fx_to_double(fx[node], ek[0]);
@@ -309,13 +337,13 @@ __global__ void __launch_bounds__(kThreadsFx, 1)
   int q_last = 0;
   double o1, o2;
 #pragma unroll 1
-  for (int k = SPLIT == 1 ? 1 : split + 1; k <= (SPLIT == 1 ? 4 : split + 1); ++k) {
-    const int e = k == 1 ? ek[1] : (k == 2 ? ek[2] : (k == 3 ? ek[3] : ek[4]));
+  for (int k = k_first; k <= k_last; ++k) {
+    const int e = shell_exp(k);
     // (1 - d) f^eq of the shell's pairs: ev +- od, ev = A + y^2 (B + y^2 C), od = y (O1 + y^2 O3)
     const double w = k == 1 ? eq.w[1] : (k == 2 ? eq.w[2] : (k == 3 ? eq.w[3] : eq.w[4])), wa = w * eq.a1;
     const double A = w * eq.a0, B = wa * d.half_v2[k], C = w * d.v4_24[k], O1 = wa * d.speed[k], O3 = w * d.v3_6[k];
 #pragma unroll 1
-    for (int i = 0; i < kHalfDirs; ++i) {
+    for (int i = i_first; i < i_first + DIRS; ++i) {
       const int q1 = 1 + (k - 1) * kNDirs + i, q2 = q1 + kHalfDirs;
       const double y = i == 0 ? eq.uxE : (i == 1 ? y1 : (i == 2 ? eq.uyE : y3)), y2 = y * y;
       const double ev = fma(y2, fma(y2, C, B), A), z = fma(y2, O3, O1);
@@ -351,18 +379,20 @@ static cudaError_t launch_tile_rows(const CUtensorMap* tmap_in, double* f_out, c
   const cudaError_t e = set_smem_once(step_kernel_f64<TT>, FxSize<TT>::smem, configured);
   if (e != cudaSuccess) return e;
   const dim3 grid((p.n_r + kTileR - 1) / kTileR, ty_end - ty_begin);
-  step_kernel_f64<TT><<<grid, kThreadsFx, FxSize<TT>::smem, stream>>>(*tmap_in, f_out, p, d, ty_begin);
-  return cudaGetLastError();
+  return launch_overlapped(step_kernel_f64<TT>, grid, kThreadsFx, FxSize<TT>::smem, stream, *tmap_in, f_out, p, d,
+                           ty_begin);
 }
 
 // Tile rows [ty_begin, ty_end) of kTileT nodes each.
 cudaError_t launch_step_f64_mwb(const CUtensorMap* tmap_in, double* f_out, const StepParams& p,
                                 const DvmConst<double>& d, cudaStream_t stream, int ty_begin, int ty_end) {
-  if (p.tile_rows == kTileT) return launch_tile_rows<kTileT>(tmap_in, f_out, p, d, stream, ty_begin, ty_end);
-  constexpr int per = kTileT / kTileTSmall;
-  const int last = (p.n_theta + kTileTSmall - 1) / kTileTSmall;
-  return launch_tile_rows<kTileTSmall>(tmap_in, f_out, p, d, stream, ty_begin * per,
-                                       ty_end * per < last ? ty_end * per : last);
+  const int per = kTileT / p.tile_rows, last = (p.n_theta + p.tile_rows - 1) / p.tile_rows;
+  const int b = ty_begin * per, e = ty_end * per < last ? ty_end * per : last;
+  switch (p.tile_rows) {
+    case 2: return launch_tile_rows<2>(tmap_in, f_out, p, d, stream, b, e);
+    case 4: return launch_tile_rows<4>(tmap_in, f_out, p, d, stream, b, e);
+    default: return launch_tile_rows<kTileT>(tmap_in, f_out, p, d, stream, b, e);
+  }
 }
 
 }  // namespace pclb
