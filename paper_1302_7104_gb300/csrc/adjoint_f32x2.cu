@@ -454,7 +454,7 @@ __device__ __forceinline__ void adjoint_tile(const CUtensorMap& tmap_f, const CU
     for (int side = 0; side < 2; ++side)
       if (side == 0 ? inner : outer)
         adjoint_walls<float, kTT>(f, lam_in, side, slots[side], t0, ws, *reinterpret_cast<WallShared<float, kTT>*>(ctab),
-                                  p, d);
+                                  nullptr, p, d);
   }
   auto prime_pairs = [&]() {
     for (int s = 0; s < kAS && s < kANP; ++s) issue_pair(s, s);

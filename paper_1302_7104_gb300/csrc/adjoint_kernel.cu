@@ -38,7 +38,8 @@
 // The FP64 kernel is bound by FP64 issue (a warp-wide operation per ~76 cycles
 // and quarter SM); the partials are therefore formed in integers
 // (fx_mwb_partials, 10 of 14 FP64 operations less per label and direction).
-// TT = 8 rows; 4 on grids whose tiles would leave SMs idle.
+// TT = 8 rows, one thread per node; on grids whose tiles would leave SMs idle
+// 4 rows and two threads per node (LS = 2), one label of each pair each.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -69,10 +70,11 @@ constexpr int kAdjStages = 2;   // ring depth of the pair-streaming kernel (2 me
 static_assert(sizeof(EqParams<float>) == 10 * sizeof(float) && sizeof(EqParams<double>) == 10 * sizeof(double),
               "ghost-state scratch holds 10 values per EqParams");
 
-template <int TT>
+// TT rows; LS = 2: two threads per node, one label of each pair each.
+template <int TT, int LS>
 struct AdjSize {
-  static constexpr int threads = 32 * TT;
-  static constexpr int min_blocks = 24 / TT;   // at most 85 registers
+  static constexpr int threads = 32 * TT * LS;
+  static constexpr int min_blocks = 2;   // what shared memory allows
   static constexpr int plane = kWinR * (TT + 4);
   static constexpr int npairs = 4 * kNDirs / 2;
   // products of one label: radial A, B over TT rows x 36 columns (tile
@@ -83,7 +85,9 @@ struct AdjSize {
   static constexpr int prod_bytes = 2 * 2 * prod * 8;             // 2 buffers x 2 labels
   static constexpr int ratio_bytes = kTileR * 8;
   static constexpr int tab_bytes = (TT + 4) * npairs * (int)sizeof(CourEntry);
-  static constexpr int smem = ring_bytes + prod_bytes + ratio_bytes + tab_bytes + 128;
+  static constexpr int ghost_bytes = 2 * 2 * TT * kQ * 8;         // both walls' ghost values
+  static constexpr int smem = ring_bytes + prod_bytes + ratio_bytes + tab_bytes + ghost_bytes + 128;
+  static_assert(LS == 1 || 2 * 12 * 32 * TT * 8 <= prod_bytes, "exchange of the node phase inside the product buffers");
   // the ring's planes are TMA destinations: 128-byte aligned
   static_assert((plane * 8) % 128 == 0, "TMA destinations must stay 128-byte aligned");
 };
@@ -91,95 +95,80 @@ struct AdjSize {
 namespace {
 
 
-// (rho, u_x, u_y, E) of one node for the cotangent of the equilibrium (FP64;
-// the FP32 pair kernel forms the state of its two nodes in float-float).
-__device__ __forceinline__ void adj_node_state(const double* f, int plane, const DvmConst<double>& d, double& rho,
-                                               double& ux, double& uy, double& E, bool& ok) {
-  const NodeState<double> m = node_moments(f, plane, d);
-  rho = m.rho; ux = m.ux; uy = m.uy; E = m.E; ok = m.ok;
-}
-
-
 // ---- the pair-streaming kernel's stencil pieces ------------------------------
-// Products of both labels of a pair at one node in one direction: q1 has its
-// upwind side at offset U, q2 (the opposite velocity) at -U.  sf, sl: the
-// pair's f and lam planes (q2 at +PLANE); o: the node in a plane; pr: its
-// product slot (M_D products; the M_Dp ones at +DB, q2's at +PROD).
-template <int U, int PLANE, int PROD, int DB>
-__device__ __forceinline__ void radial_pair(const double* sf, const double* sl, double* pb, int o, int pr, uint64_t a2,
-                                            uint64_t k2, double lam[2]) {
-#pragma unroll
-  for (int L = 0; L < 2; ++L) {
-    constexpr int kU[2] = {U, -U};
-    const double* f = sf + L * PLANE + o;
-    double MD, MP;
-    fx_mwb_partials(f[0] - f[kU[L]], f[kU[L]] - f[2 * kU[L]], a2, k2, MD, MP);
-    lam[L] = sl[L * PLANE + o];
-    pb[L * PROD + pr] = lam[L] * MD;
-    pb[L * PROD + pr + DB] = lam[L] * MP;
-  }
-}
-
-template <int U, int PLANE, int PROD, int DB>
-__device__ __forceinline__ void azimuthal_pair(const double* sf, const double lam[2], double* pb, int o, int pa,
-                                               uint64_t a2, uint64_t k2) {
-#pragma unroll
-  for (int L = 0; L < 2; ++L) {
-    constexpr int kU[2] = {U, -U};
-    const double* f = sf + L * PLANE + o;
-    double MD, MP;
-    fx_mwb_partials(f[0] - f[kU[L]], f[kU[L]] - f[2 * kU[L]], a2, k2, MD, MP);
-    pb[L * PROD + pa] = lam[L] * MD;
-    pb[L * PROD + pa + DB] = lam[L] * MP;
-  }
-}
-
-// One label at one halo node, upwind side at offset U.
-template <int U>
-__device__ __forceinline__ void azimuthal_one(const double* fw, const double* lw, double* pa, int DB, uint64_t a2,
-                                              uint64_t k2) {
+// lam(n) M_D(n), lam(n) M_Dp(n) of one label at one node in one direction, its
+// upwind neighbours at offsets u and 2u, to P and P + DB.
+__device__ __forceinline__ void products(const double* f, int u, double lam, double* P, int DB, uint64_t a2, uint64_t k2) {
   double MD, MP;
-  fx_mwb_partials(fw[0] - fw[U], fw[U] - fw[2 * U], a2, k2, MD, MP);
-  const double lam = lw[0];
-  pa[0] = lam * MD;
-  pa[DB] = lam * MP;
+  const double f1 = f[u];
+  fx_mwb_partials(f[0] - f1, f1 - f[2 * u], a2, k2, MD, MP);
+  P[0] = lam * MD;
+  P[DB] = lam * MP;
 }
 
-// Gather of the radial products at one node: the node n = c + j u reads f(n),
+// Gather of one label's products at one node: the node n = c + j u reads f(n),
 // f(n + u), f(n + 2 u), so dM(n)/df(c) collects M_D of n = c, M_Dp - M_D of
-// n = c - u and -M_Dp of n = c - 2u (u = U for q1, -U for q2).
-template <class T, int U, int PROD, int DB>
-__device__ __forceinline__ void gather_radial(const T* pb, int pr, T acc[2]) {
-  acc[0] = pb[pr] - pb[pr - U] + pb[pr + DB - U] - pb[pr + DB - 2 * U];
-  const T* p2 = pb + PROD;
-  acc[1] = p2[pr] - p2[pr + U] + p2[pr + DB + U] - p2[pr + DB + 2 * U];
+// n = c - u and -M_Dp of n = c - 2u.
+__device__ __forceinline__ double gather(const double* P, int DB, int u) { return P[0] - P[-u] + P[DB - u] - P[DB - 2 * u]; }
+
+// The azimuthal gather where the upwind side changes within the five rows: bit
+// o of neg set when row o - 2 has v_theta < 0 for this label (its reader of row 0
+// is then the row below it).
+__device__ __forceinline__ double gather_mixed(const double* P, int DB, int neg) {
+  double a = P[0];
+  if (neg & 2) a += P[DB - kTileR] - P[-kTileR];
+  if (!(neg & 8)) a += P[DB + kTileR] - P[kTileR];
+  if (neg & 1) a -= P[DB - 2 * kTileR];
+  if (!(neg & 16)) a -= P[DB + 2 * kTileR];
+  return a;
 }
 
-// Azimuthal gather when the rows -2 .. +2 around the node all have q1's
-// upwind side on the same side: the readers of the node sit at +V, +2V for
-// q1 and at -V, -2V for q2 (V = +-row stride).
-template <class T, int V, int PROD, int DB>
-__device__ __forceinline__ void gather_azimuthal(const T* pb, int pa, T acc[2]) {
-  acc[0] += pb[pa] + pb[pa + DB + V] - pb[pa + V] - pb[pa + DB + 2 * V];
-  const T* p2 = pb + PROD;
-  acc[1] += p2[pa] + p2[pa + DB - V] - p2[pa - V] - p2[pa + DB - 2 * V];
-}
-
-// The same where the upwind side changes within the five rows: bit o of neg
-// set when row o - 2 has v_theta < 0 for q1 (its reader of row 0 is then the
-// row below it).
-template <class T, int PROD, int DB>
-__device__ __forceinline__ void gather_azimuthal_mixed(const T* pb, int pa, int tneg, T acc[2]) {
+// The sums of eq_cotangent (adjoint_common.cuh) over shells k0 .. k1, and the
+// rest velocity's if l0 is given: A, Bx, By, Cs, Dx, Fq.
+template <class LamFn>
+__device__ __forceinline__ void cotangent_sums(double ux, double uy, double E, const DvmConst<double>& d, int k0, int k1,
+                                               const double* l0, LamFn lam, double o[6]) {
+  const double invE = recip_newton(E);
+  const double s = (ux * ux + uy * uy) * invE;
+  const double a1 = 1.0 - 0.5 * s, a0 = a1 + 0.125 * s * s;
+  const double uxE = ux * invE, uyE = uy * invE;
+  auto weight = [&](int k, double& F, double& Fd) {   // F_k(E) and its derivative
+    const double* c = d.Fc[k];
+    F = E * (c[0] + E * (c[1] + E * (c[2] + E * c[3])));
+    Fd = c[0] + E * (2.0 * c[1] + E * (3.0 * c[2] + E * 4.0 * c[3]));
+  };
 #pragma unroll
-  for (int L = 0; L < 2; ++L) {
-    const T* P = pb + L * PROD;
-    const int neg = L ? (tneg ^ 0x1f) : tneg;          // the partner has the opposite velocity
-    T a = P[pa];
-    if (neg & 2) a += P[pa + DB - kTileR] - P[pa - kTileR];
-    if (!(neg & 8)) a += P[pa + DB + kTileR] - P[pa + kTileR];
-    if (neg & 1) a -= P[pa + DB - 2 * kTileR];
-    if (!(neg & 16)) a -= P[pa + DB + 2 * kTileR];
-    acc[L] += a;
+  for (int j = 0; j < 6; ++j) o[j] = 0.0;
+  if (l0) {   // x = 0
+    double Fs = 0.0, Fds = 0.0;
+#pragma unroll
+    for (int k = 1; k <= 4; ++k) {
+      double F, Fd;
+      weight(k, F, Fd);
+      Fs += F;
+      Fds += Fd;
+    }
+    const double l0F = *l0 * (1.0 - d.B0 * Fs);
+    o[0] = l0F * a0;
+    o[3] = l0F * (-0.5 + 0.25 * s);
+    o[5] = *l0 * (-d.B0 * Fds) * a0;
+  }
+  constexpr int half = kNDirs / 2;
+#pragma unroll 1
+  for (int k = k0; k <= k1; ++k) {
+    double F, Fd, Ak = 0, Bxk = 0, Byk = 0, Ck = 0, Dk = 0;
+    weight(k, F, Fd);
+#pragma unroll
+    for (int i = 0; i < half; ++i) {
+      const int q = 1 + (k - 1) * kNDirs + i;
+      pair_terms<double>(d.vx[q], d.vy[q], uxE, uyE, s, a0, a1, lam(q), lam(q + half), Ak, Bxk, Byk, Ck, Dk);
+    }
+    o[0] += F * Ak;
+    o[1] += F * Bxk;
+    o[2] += F * Byk;
+    o[3] += F * Ck;
+    o[4] += F * Dk;
+    o[5] += Fd * Ak;
   }
 }
 
@@ -188,14 +177,14 @@ __device__ __forceinline__ void gather_azimuthal_mixed(const T* pb, int pa, int 
 // ---------------------------------------------------------------------------
 // Pair-streaming part.
 // ---------------------------------------------------------------------------
-template <int TT>
-__global__ void __launch_bounds__(AdjSize<TT>::threads, AdjSize<TT>::min_blocks)
+template <int TT, int LS>
+__global__ void __launch_bounds__(AdjSize<TT, LS>::threads, AdjSize<TT, LS>::min_blocks)
     adjoint_pair_kernel(const __grid_constant__ CUtensorMap tmap_f, const __grid_constant__ CUtensorMap tmap_l,
                         const double* __restrict__ f, const double* __restrict__ lam_in, double* __restrict__ lam_out,
                         const __grid_constant__ WallScratch<double> ws, const __grid_constant__ AdjOrder order,
                         const __grid_constant__ StepParams p, const __grid_constant__ DvmConst<double> d) {
   using T = double;
-  using SZ = AdjSize<TT>;
+  using SZ = AdjSize<TT, LS>;
   constexpr int PLANE = SZ::plane;
   constexpr int NP = SZ::npairs, RC = SZ::rcols, PROD = SZ::prod;
   constexpr int S = kAdjStages;
@@ -207,14 +196,17 @@ __global__ void __launch_bounds__(AdjSize<TT>::threads, AdjSize<TT>::min_blocks)
   T* prod = ring + S * 4 * PLANE;                             // [buffer][label][products]
   uint64_t* ratio = reinterpret_cast<uint64_t*>(prod + 2 * 2 * PROD);   // 1/r of the tile columns relative to the first
   CourEntry* ctab = reinterpret_cast<CourEntry*>(ratio + kTileR);        // [TT + 4][NP]
-  uint64_t* bar = reinterpret_cast<uint64_t*>(ctab + (TT + 4) * NP);     // [S]
+  T* gval = reinterpret_cast<T*>(ctab + (TT + 4) * NP);                  // [side][layer][TT][Q] ghost values
+  uint64_t* bar = reinterpret_cast<uint64_t*>(gval + 2 * 2 * TT * kQ);   // [S]
 
   int tx, ty;
   order.tile(blockIdx.x, tx, ty);
   const int r0 = tx * kTileR;
   const int t0 = ty * TT;
   const int tid = threadIdx.x;
-  const int lane = tid & 31, rowl = tid >> 5;
+  const int lane = tid & 31, warp = tid >> 5;
+  const int rowl = warp % TT;               // tile row
+  const int half_of = warp / TT;            // LS = 2: this thread's label of each pair (and half of the shells)
 
   // the planes of pair pr (labels q1, q1 + N_i/2) into stage s (thread 0)
   auto issue_pair = [&](int pr, int s) {
@@ -242,7 +234,8 @@ __global__ void __launch_bounds__(AdjSize<TT>::threads, AdjSize<TT>::min_blocks)
   static_assert(sizeof(WallShared<T, TT>) <= (TT + 4) * NP * sizeof(CourEntry), "wall scratch inside the Courant table");
   for (int side = 0; side < 2; ++side)
     if (side == 0 ? inner : outer)
-      adjoint_walls<T, TT>(f, lam_in, side, slots[side], t0, ws, *reinterpret_cast<WallShared<T, TT>*>(ctab), p, d);
+      adjoint_walls<T, TT>(f, lam_in, side, slots[side], t0, ws, *reinterpret_cast<WallShared<T, TT>*>(ctab),
+                           gval + side * 2 * TT * kQ, p, d);
   const double inv_r0 = p.inv_r[r0];
   if (tid < kTileR) ratio[tid] = r0 + tid < p.n_r ? fx_fraction(p.inv_r[r0 + tid] * recip_newton(inv_r0)) : 0;
   // Courant entries of the stored rows t0 .. t0 + TT + 3 (theta rows t0 - 2 .. t0 + TT + 1)
@@ -282,20 +275,60 @@ __global__ void __launch_bounds__(AdjSize<TT>::threads, AdjSize<TT>::min_blocks)
   const int srow = t + kGhostRows;
   const size_t plane_out = (size_t)p.rows * p.pitch;
   const T decay = (T)p.decay;
-  T gs[4] = {T(0), T(0), T(0), T(0)};
-  if (valid) {
+  T gs[4];
+  {
     // (1 - d) g of this node, read from global memory while the first pairs'
-    // windows land (the TMA copies then mostly hit L2)
-    const int plane = p.rows * p.pitch;
-    const size_t off = (size_t)srow * p.pitch + r;
+    // windows land (the TMA copies then mostly hit L2); threads without a node
+    // repeat the nearest one
+    const size_t plane = plane_out;
+    const size_t off = (size_t)(min(t, p.n_theta - 1) + kGhostRows) * p.pitch + min(r, p.n_r - 1);
+    const T* fn = f + off;
     const T* ln = lam_in + off;
-    T rho, ux, uy, E;
-    bool nok;
-    adj_node_state(f + off, plane, d, rho, ux, uy, E, nok);
-    if (!nok) atomicOr(p.status, PCLB_FLAG_NONPHYS);
-    T G[4], g[4];
-    eq_cotangent<T>(rho, ux, uy, E, d, [&](int q) -> T { return ln[(size_t)q * plane]; }, G);
-    to_moment_cotangent<T>(rho, ux, uy, E, G, g);
+    T* mine = prod + ((rowl * 32 + lane) * 2 + half_of) * 12;    // exchange of the two halves of the shells
+    const T* theirs = prod + ((rowl * 32 + lane) * 2 + (1 - half_of)) * 12;
+    const int k0 = LS == 1 ? 1 : 2 * half_of + 1, k1 = LS == 1 ? 4 : k0 + 1;
+    const T lam0 = ln[0];
+    T m[4] = {half_of == 0 ? fn[0] : T(0), T(0), T(0), T(0)};    // rho, j_x, j_y, e
+#pragma unroll 1
+    for (int k = k0; k <= k1; ++k) {
+      T S = T(0), D[kNDirs / 2];
+#pragma unroll
+      for (int i = 0; i < kNDirs / 2; ++i) {
+        const int q = 1 + (k - 1) * kNDirs + i;
+        const T a = fn[(size_t)q * plane], b = fn[(size_t)(q + kNDirs / 2) * plane];
+        S += a + b;
+        D[i] = a - b;
+      }
+      m[0] += S;
+      m[1] = fma(d.speed[k], fma(d.cx[2], D[1] - D[3], D[0]), m[1]);
+      m[2] = fma(d.speed[k], fma(d.cx[2], D[1] + D[3], D[2]), m[2]);
+      m[3] = fma(d.half_v2[k], S, m[3]);
+    }
+    if constexpr (LS == 2) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) mine[j] = m[j];
+      __syncthreads();
+#pragma unroll
+      for (int j = 0; j < 4; ++j) m[j] += theirs[j];
+    }
+    const NodeState<T> st = node_state64(m[0], m[1], m[2], m[3]);
+    if (valid && !st.ok) atomicOr(p.status, PCLB_FLAG_NONPHYS);
+    T c[6];
+    cotangent_sums(st.ux, st.uy, st.E, d, k0, k1, half_of == 0 ? &lam0 : nullptr,
+                   [&](int q) -> T { return ln[(size_t)q * plane]; }, c);
+    if constexpr (LS == 2) {
+#pragma unroll
+      for (int j = 0; j < 6; ++j) mine[4 + j] = c[j];
+      __syncthreads();
+#pragma unroll
+      for (int j = 0; j < 6; ++j) c[j] += theirs[4 + j];
+      __syncthreads();   // read before the pairs' products take the buffer
+    }
+    const T invE = recip_newton(st.E), s = (st.ux * st.ux + st.uy * st.uy) * invE, rE = st.rho * invE;
+    const T G[4] = {c[0], rE * (c[1] + T(2) * st.ux * c[3]), rE * (c[2] + T(2) * st.uy * c[3]),
+                    st.rho * (c[5] - (c[4] + s * c[3]) * invE)};
+    T g[4];
+    to_moment_cotangent<T>(st.rho, st.ux, st.uy, st.E, G, g);
 #pragma unroll
     for (int j = 0; j < 4; ++j) gs[j] = (T(1) - decay) * g[j];
     // the cotangent the ghost nodes return to the two nodes next to each wall
@@ -303,10 +336,10 @@ __global__ void __launch_bounds__(AdjSize<TT>::threads, AdjSize<TT>::min_blocks)
 #pragma unroll
       for (int j = 0; j < 4; ++j) gs[j] += ws.gwall[((size_t)(slots[side] * 2 + node) * p.n_theta + t) * 4 + j];
     };
-    if (r == 0) add_wall(0, 0);
-    if (r == 1) add_wall(0, 1);
-    if (r == p.n_r - 1) add_wall(1, 0);
-    if (r == p.n_r - 2) add_wall(1, 1);
+    if (valid && r == 0) add_wall(0, 0);
+    if (valid && r == 1) add_wall(0, 1);
+    if (valid && r == p.n_r - 1) add_wall(1, 0);
+    if (valid && r == p.n_r - 2) add_wall(1, 1);
   }
   const int o_node = row * kWinR + col;                 // this node in a window plane
   const int p_rad = AR + rowl * RC + lane + 2;          // its radial product slot
@@ -319,14 +352,9 @@ __global__ void __launch_bounds__(AdjSize<TT>::threads, AdjSize<TT>::min_blocks)
     if (t < 2) lam_out[(size_t)d.recv_hi[q] * plane_out + (size_t)(p.n_theta + kGhostRows + t) * p.pitch + r] = v;
   };
   // rest velocity: no convection
-  if (valid) store(0, decay * lam_in[(size_t)srow * p.pitch + r] + gs[0] + gs[3] * d.half_v2[0]);
+  if (valid && half_of == 0) store(0, decay * lam_in[(size_t)srow * p.pitch + r] + gs[0] + gs[3] * d.half_v2[0]);
 
-  // wall tiles: the ghost states of the rows this thread fills (warp 0: inner, warp 1: outer)
   const bool wall_tile = inner || outer;
-  const int gside = rowl == 0 ? 0 : 1;
-  const bool fills = wall_tile && rowl < 2 && lane < TT && t0 + lane < p.n_theta && (gside == 0 ? inner : outer);
-  const EqParams<T>* eg = ws.ghost + (size_t)(slots[gside] * 3) * p.n_theta + t0 + lane;   // layer l at + l n_theta
-  const bool gneq = (p.bc_kind[gside] & PCLB_BC_NEQ) != 0;   // its ghosts carry the wall node's departure
 
   bool ok = true;
   int brk = NP;                                         // the pair at which a wait timed out
@@ -340,95 +368,68 @@ __global__ void __launch_bounds__(AdjSize<TT>::threads, AdjSize<TT>::min_blocks)
     T* pb = prod + (pair & 1) * 2 * PROD;                // this pair's products: [label][...]
     if (ok) ok = p.wait_ns != 0 && mbar_wait_bounded(&bar[s], (uint32_t)((pair / S) & 1), p.wait_ns);
     if (wall_tile) {
-      // radial ghost columns of this pair's f planes (f = f^eq of the ghost
-      // states, plus the wall node's departure for non-equilibrium ghosts)
-      if (fills && ok) {
-        T* fw = const_cast<T*>(st) + (2 + lane) * kWinR;
-        const int c0 = gside == 0 ? kLeft : cw_out, stp = gside == 0 ? 1 : -1;
-        T dep1 = T(0), dep2 = T(0);
-        if (gneq) {
-          const EqParams<T> ea = eg[(size_t)2 * p.n_theta];
-          dep1 = fw[c0] - adj_feq<T>(ea, d, q1);
-          dep2 = fw[PLANE + c0] - adj_feq<T>(ea, d, q2);
-        }
-        for (int l = 0; l < 2; ++l) {
-          const int c = c0 - stp * (1 + l);
-          if (c < 0 || c >= kWinR) continue;
-          const EqParams<T> e = eg[(size_t)l * p.n_theta];
-          fw[c] = adj_feq<T>(e, d, q1) + dep1;
-          fw[PLANE + c] = adj_feq<T>(e, d, q2) + dep2;
-        }
+      // radial ghost columns of this pair's f planes: wall, layer, label, row
+      if (tid < 8 * TT && ok) {
+        const int rr = tid % TT, L = tid / TT & 1, l = tid / (2 * TT) & 1, side = tid / (4 * TT);
+        const int c = (side == 0 ? kLeft : cw_out) - (side == 0 ? 1 : -1) * (1 + l);
+        if ((side == 0 ? inner : outer) && t0 + rr < p.n_theta && c >= 0 && c < kWinR)
+          const_cast<T*>(st)[L * PLANE + (2 + rr) * kWinR + c] = gval[((side * 2 + l) * TT + rr) * kQ + (L ? q2 : q1)];
       }
       __syncthreads();
     }
 
     // (A) products lam(n) M_D(n), lam(n) M_Dp(n) of every node that can reach the
-    // tile.  Warp w forms those of tile row w at its 32 columns (both labels),
-    // warps 0..3 the halo rows -2, -1, TT, TT + 1 for the label whose upwind
-    // side points into the tile, and the next warps the halo columns.  The
-    // upwind sides are uniform across a warp (one row), so each warp takes a
-    // branch in which the stencil offsets are constants.
+    // tile: each thread those of its node (both labels, or its own), warps
+    // 0..3 the halo rows -2, -1, TT, TT + 1 for the label whose upwind side
+    // points into the tile, and the next warp the halo columns.
     const T* sfp = st;                                    // f q1, f q2 at +PLANE
     const T* slp = st + 2 * PLANE;                        // lam q1, lam q2 at +PLANE
     const CourEntry e = ctab[row * NP + pair];
     const int fl_c = e.fl;                                // flags of this node's row
-    T lam_c[2];                                           // lam^{n+1} of both labels at this node
-    if (fl_c & 1)
-      radial_pair<1, PLANE, PROD, BR - AR>(sfp, slp, pb, o_node, p_rad, e.a2, e.k2, lam_c);
-    else
-      radial_pair<-1, PLANE, PROD, BR - AR>(sfp, slp, pb, o_node, p_rad, e.a2, e.k2, lam_c);
-    // alpha^2 and 2 alpha (1 - alpha) of |C_theta| at this node
+    // label L's upwind offsets at this node's row
+    auto up_r = [&](int L) { return ((fl_c & 1) != 0) != (L != 0) ? 1 : -1; };
+    auto up_t = [&](int L) { return ((fl_c & 2) != 0) != (L != 0) ? kWinR : -kWinR; };
+    // alpha^2 and 2 alpha (1 - alpha) of |C_theta| at this thread's column
     auto azimuthal = [&](uint64_t at, uint64_t& a2, uint64_t& k2) {
       const uint64_t alpha = fx_mul_frac(at, my_ratio);
       a2 = fx_mul_frac(alpha, alpha);
       k2 = 2 * (alpha - a2);
     };
+    T lam_c[LS == 1 ? 2 : 1];                             // lam^{n+1} of the label(s) at this node
     {
       uint64_t a2, k2;
       azimuthal(e.at, a2, k2);
-      if (fl_c & 2)
-        azimuthal_pair<kWinR, PLANE, PROD, BT - AT>(sfp, lam_c, pb, o_node, p_az, a2, k2);
-      else
-        azimuthal_pair<-kWinR, PLANE, PROD, BT - AT>(sfp, lam_c, pb, o_node, p_az, a2, k2);
+#pragma unroll
+      for (int j = 0; j < (LS == 1 ? 2 : 1); ++j) {
+        const int L = LS == 1 ? j : half_of;
+        const T* fw = sfp + L * PLANE + o_node;
+        lam_c[j] = slp[L * PLANE + o_node];
+        products(fw, up_r(L), lam_c[j], pb + L * PROD + p_rad, BR - AR, e.a2, e.k2);
+        products(fw, up_t(L), lam_c[j], pb + L * PROD + p_az, BT - AT, a2, k2);
+      }
     }
-    if (rowl < 4) {
-      // halo rows: warps 0..3 take window rows 0, 1, TT + 2, TT + 3; rows
-      // above the tile are read by labels whose upwind side is +theta
-      const int rr = rowl < 2 ? rowl : TT + rowl;
+    if (warp < 4) {
+      // halo rows: window rows 0, 1, TT + 2, TT + 3; rows above the tile are
+      // read by labels whose upwind side is +theta
+      const int rr = warp < 2 ? warp : TT + warp;
       const CourEntry eh = ctab[rr * NP + pair];
       const bool q1_up_pos = (eh.fl & 2) != 0;
-      uint64_t ath, kth;
-      azimuthal(eh.at, ath, kth);
-      const int o = rr * kWinR + col;
-      if (rowl < 2)
-        azimuthal_one<kWinR>(sfp + (q1_up_pos ? 0 : PLANE) + o, slp + (q1_up_pos ? 0 : PLANE) + o,
-                                pb + (q1_up_pos ? 0 : PROD) + AT + rr * kTileR + lane, BT - AT, ath, kth);
-      else
-        azimuthal_one<-kWinR>(sfp + (q1_up_pos ? PLANE : 0) + o, slp + (q1_up_pos ? PLANE : 0) + o,
-                                 pb + (q1_up_pos ? PROD : 0) + AT + rr * kTileR + lane, BT - AT, ath, kth);
-    }
-    {
-      // halo columns: 4 per tile row (label, column); the warps after the first
-      // four take them, or warp 0 as well when the tile has too few rows.
-      // Upwind at larger r (+1) reads the tile from columns -2, -1, at
-      // smaller r from 32, 33.
-      constexpr int HW = (4 * TT + 31) / 32;
-      constexpr bool kSep = TT >= 4 + HW;
-      if (kSep ? (rowl >= 4 && rowl < 4 + HW) : rowl < HW) {
-        const int h = (kSep ? rowl - 4 : rowl) * 32 + lane;
-        if (h < 4 * TT) {
-          const int hr = h >> 2, L = (h >> 1) & 1, j = h & 1;
-          const CourEntry eh = ctab[(hr + 2) * NP + pair];
-          const int uh = (eh.fl & 1) ? 1 : -1, uL = L ? -uh : uh;
-          const int c = uL == 1 ? j - 2 : kTileR + j;
-          const int o = (hr + 2) * kWinR + c + kLeft;
-          const T* fw = sfp + L * PLANE + o;
-          T MD, MP;
-          fx_mwb_partials(fw[0] - fw[uL], fw[uL] - fw[2 * uL], eh.a2, eh.k2, MD, MP);
-          const T lam = slp[L * PLANE + o];
-          pb[L * PROD + AR + hr * RC + c + 2] = lam * MD;
-          pb[L * PROD + BR + hr * RC + c + 2] = lam * MP;
-        }
+      uint64_t a2, k2;
+      azimuthal(eh.at, a2, k2);
+      const int L = (warp < 2) == q1_up_pos ? 0 : 1, o = rr * kWinR + col;
+      products(sfp + L * PLANE + o, warp < 2 ? kWinR : -kWinR, slp[L * PLANE + o], pb + L * PROD + AT + rr * kTileR + lane,
+               BT - AT, a2, k2);
+    } else if (warp == 4) {
+      // halo columns: 4 per tile row (label, column).  Upwind at larger r (+1)
+      // reads the tile from columns -2, -1, at smaller r from 32, 33.
+      static_assert(4 * TT <= 32 && TT * LS >= 5, "halo columns: one warp");
+      if (lane < 4 * TT) {
+        const int hr = lane >> 2, L = (lane >> 1) & 1, j = lane & 1;
+        const CourEntry eh = ctab[(hr + 2) * NP + pair];
+        const int u = ((eh.fl & 1) != 0) != (L != 0) ? 1 : -1;
+        const int c = u == 1 ? j - 2 : kTileR + j;
+        const int o = L * PLANE + (hr + 2) * kWinR + c + kLeft;
+        products(sfp + o, u, slp[o], pb + L * PROD + AR + hr * RC + c + 2, BR - AR, eh.a2, eh.k2);
       }
     }
     if (__syncthreads_or(!ok)) {
@@ -441,35 +442,31 @@ __global__ void __launch_bounds__(AdjSize<TT>::threads, AdjSize<TT>::min_blocks)
       issue_pair(pair + S, s);
     }
 
-    // (B) gather at this node: node n = c + j u_n reads f(n), f(n + u_n),
-    // f(n + 2 u_n), so dM(n)/df(n) = M_D, dM(n)/df(n + u_n) = M_Dp - M_D,
-    // dM(n)/df(n + 2 u_n) = -M_Dp.
+    // (B) gather at this node
     if (valid) {
-      T acc[2];
-      if (fl_c & 1)
-        gather_radial<T, 1, PROD, BR - AR>(pb, p_rad, acc);
-      else
-        gather_radial<T, -1, PROD, BR - AR>(pb, p_rad, acc);
-      const int tneg = fl_c >> 2;                        // bit o: row o - 2 has v_theta < 0 for q1
-      if (tneg == 0)
-        gather_azimuthal<T, kTileR, PROD, BT - AT>(pb, p_az, acc);
-      else if (tneg == 31)
-        gather_azimuthal<T, -kTileR, PROD, BT - AT>(pb, p_az, acc);
-      else
-        gather_azimuthal_mixed<T, PROD, BT - AT>(pb, p_az, tneg, acc);
       const T A = gs[0] + gs[3] * d.half_v2[k];
       const T B = gs[1] * d.vx[q1] + gs[2] * d.vy[q1];
-      T o1 = decay * lam_c[0] + (A + B) - acc[0], o2 = decay * lam_c[1] + (A - B) - acc[1];
-      if (wall_tile) {
-        // non-equilibrium ghosts hand their cotangent straight to f_q of the wall node
-        for (int sd = 0; sd < 2; ++sd)
-          if ((p.bc_kind[sd] & PCLB_BC_NEQ) && r == (sd == 0 ? 0 : p.n_r - 1)) {
-            o1 += ws.gdir[((size_t)slots[sd] * p.n_theta + t) * kQ + q1];
-            o2 += ws.gdir[((size_t)slots[sd] * p.n_theta + t) * kQ + q2];
-          }
+      const int tneg = fl_c >> 2;                        // bit o: row o - 2 has v_theta < 0 for q1
+#pragma unroll
+      for (int j = 0; j < (LS == 1 ? 2 : 1); ++j) {
+        const int L = LS == 1 ? j : half_of, q = L ? q2 : q1;
+        const T* P = pb + L * PROD;
+        T acc = gather(P + p_rad, BR - AR, up_r(L));
+        // one side for all rows -2 .. +2 around the node: the readers sit
+        // upwind's opposite way; else row by row
+        if (tneg == 0 || tneg == 31)
+          acc += gather(P + p_az, BT - AT, (tneg == 0) == (L == 0) ? -kTileR : kTileR);
+        else
+          acc += gather_mixed(P + p_az, BT - AT, L ? tneg ^ 0x1f : tneg);
+        T o = decay * lam_c[j] + (L ? A - B : A + B) - acc;
+        if (wall_tile) {
+          // non-equilibrium ghosts hand their cotangent straight to f_q of the wall node
+          for (int sd = 0; sd < 2; ++sd)
+            if ((p.bc_kind[sd] & PCLB_BC_NEQ) && r == (sd == 0 ? 0 : p.n_r - 1))
+              o += ws.gdir[((size_t)slots[sd] * p.n_theta + t) * kQ + q];
+        }
+        store(q, o);
       }
-      store(q1, o1);
-      store(q2, o2);
     }
   }
   if (brk < NP && tid == 0) {
@@ -504,16 +501,16 @@ cudaError_t launch_adjoint(const CUtensorMap* tmap_f, const CUtensorMap* tmap_l,
     // FP32: the packed two-nodes-per-thread pair kernel (adjoint_f32x2.cu)
     return launch_adjoint_pairs_f32(tmap_f, tmap_l, tmap_fn, tmap_ln, f, lam_in, lam_out, ws, order, p, d, stream);
   } else {
-    auto go = [&](auto tt) {
-      constexpr int TT = decltype(tt)::value;
+    auto go = [&](auto tt, auto ls) {
+      constexpr int TT = decltype(tt)::value, LS = decltype(ls)::value;
       static std::atomic<unsigned long long> configured{0};
-      const cudaError_t e = set_smem_once(adjoint_pair_kernel<TT>, AdjSize<TT>::smem, configured);
+      const cudaError_t e = set_smem_once(adjoint_pair_kernel<TT, LS>, AdjSize<TT, LS>::smem, configured);
       if (e != cudaSuccess) return e;
-      return launch_overlapped(adjoint_pair_kernel<TT>, dim3((unsigned)order.blocks()), AdjSize<TT>::threads,
-                               AdjSize<TT>::smem, stream, *tmap_f, *tmap_l, f, lam_in, lam_out, ws, order, p, d);
+      return launch_overlapped(adjoint_pair_kernel<TT, LS>, dim3((unsigned)order.blocks()), AdjSize<TT, LS>::threads,
+                               AdjSize<TT, LS>::smem, stream, *tmap_f, *tmap_l, f, lam_in, lam_out, ws, order, p, d);
     };
-    return rows == kAdjRows64 ? go(std::integral_constant<int, kAdjRows64>{})
-                              : go(std::integral_constant<int, kAdjRows64Small>{});
+    if (rows == kAdjRows64) return go(std::integral_constant<int, kAdjRows64>{}, std::integral_constant<int, 1>{});
+    return go(std::integral_constant<int, kAdjRows64Small>{}, std::integral_constant<int, 2>{});
   }
 }
 

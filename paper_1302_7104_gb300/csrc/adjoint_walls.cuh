@@ -83,13 +83,16 @@ struct WallShared {
 
 // Rows t0 .. t0 + TT - 1 of wall `side` into `slot` of ws, by all threads of the
 // block (256); ends with a block barrier.  f, lam: the stored planes.
+// values: if given, the ghost values themselves, [layer][TT][Q] (the FP64
+// kernel copies them into its windows; forming them pair by pair took 36
+// FP64 operations per pair between two block barriers).
 //
 // Bound: latency.  The node states use FP64 (a warp-wide operation per ~76
 // cycles and quarter SM): they are formed once per row, a lane each, instead of
 // in every lane of a warp per row.
 template <class T, int TT>
 __device__ __noinline__ void adjoint_walls(const T* __restrict__ f, const T* __restrict__ lam, int side, int slot,
-                                           int t0, const WallScratch<T>& ws, WallShared<T, TT>& sh,
+                                           int t0, const WallScratch<T>& ws, WallShared<T, TT>& sh, T* values,
                                            const StepParams& p, const DvmConst<T>& d) {
   const int tid = threadIdx.x;
   const size_t plane = (size_t)p.rows * p.pitch;
@@ -141,8 +144,23 @@ __device__ __noinline__ void adjoint_walls(const T* __restrict__ f, const T* __r
     if (t0 + row < p.n_theta) ghost[(size_t)l * p.n_theta + t] = e;
   }
   __syncthreads();
-  // a pair of opposite velocities of one row per thread, 16 lanes a row
   constexpr int half = kNDirs / 2;
+  if (values) {
+    for (int it = tid; it < 2 * 4 * half * TT; it += blockDim.x) {   // layer, row, pair
+      const int pair = it % (4 * half), row = it / (4 * half) % TT, l = it / (4 * half * TT);
+      const int q1 = 1 + pair / half * kNDirs + pair % half, t = min(t0 + row, p.n_theta - 1);
+      const T* fa = f + (size_t)(t + kGhostRows) * p.pitch + ra;
+#pragma unroll
+      for (int L = 0; L < 2; ++L) {
+        const int q = q1 + L * half;
+        T v = adj_feq<T>(sh.eq[l][row], d, q);
+        if (neq) v += fa[(size_t)q * plane] - adj_feq<T>(sh.eq[2][row], d, q);
+        values[(l * TT + row) * kQ + q] = v;
+      }
+    }
+    __syncthreads();
+  }
+  // a pair of opposite velocities of one row per thread, 16 lanes a row
   for (int it = tid; it < 4 * half * TT; it += blockDim.x) {
     const int row = it / (4 * half), pair = it % (4 * half), t = min(t0 + row, p.n_theta - 1);
     const bool live = t0 + row < p.n_theta;
@@ -174,8 +192,15 @@ __device__ __noinline__ void adjoint_walls(const T* __restrict__ f, const T* __r
         const T f_a = fa[(size_t)q * plane], f_b = fb[(size_t)q * plane];
         // the ghost values as the step forms them (plus the departure f_q(a)
         // - f^eq_q(a) for non-equilibrium ghosts)
-        const T dep = neq ? f_a - adj_feq<T>(ea, d, q) : T(0);
-        const T g0 = adj_feq<T>(e0, d, q) + dep, g1 = adj_feq<T>(e1, d, q) + dep;
+        T g0, g1;
+        if (values) {
+          g0 = values[row * kQ + q];
+          g1 = values[(TT + row) * kQ + q];
+        } else {
+          const T dep = neq ? f_a - adj_feq<T>(ea, d, q) : T(0);
+          g0 = adj_feq<T>(e0, d, q) + dep;
+          g1 = adj_feq<T>(e1, d, q) + dep;
+        }
         T MDa, MPa, MDb, MPb;
         mwb_partials<T>(cr.a_r, cr.k_r, f_a - g0, g0 - g1, MDa, MPa);
         mwb_partials<T>(cr.a_r, cr.k_r, f_b - f_a, f_a - g0, MDb, MPb);
