@@ -79,6 +79,24 @@ __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 
+// Block barrier that warps may reach at different places of the code.
+__device__ __forceinline__ void block_barrier() { asm volatile("barrier.cta.sync 0;" ::: "memory"); }
+
+// Barrier `id` of the block's first `threads` threads; true for all of them if
+// pred holds for any.
+__device__ __forceinline__ bool barrier_or(int id, int threads, bool pred) {
+  uint32_t any;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %3, 0;\n\t"
+      "barrier.cta.red.or.pred q, %1, %2, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(any)
+      : "r"(id), "r"(threads), "r"((uint32_t)pred)
+      : "memory");
+  return any != 0;
+}
+
 // Programmatic dependent launch: wait for the grid launched before this one
 // on the stream (its results are then visible), and let the grid after this
 // one start.  Without the launch attribute both return at once.

@@ -26,20 +26,22 @@ struct Eq2 {
   f2 yh[kHalf], yl[kHalf];  // c_i . u / E, float-float
 };
 
-__device__ __forceinline__ Eq2 eq2(const State2& s, const DvmConst<float>& d) {
-  Eq2 q;
-  ff2 sum = ff2_of(bc2(0.f));
+// F_k(E) of Eq. (11a).
+__device__ __forceinline__ ff2 shell_weight2(const ff2& E, const DvmConst<float>& d, int k) {
+  ff2 a = ffc(d.Fc[k][3], d.Fc_lo[k][3]);
 #pragma unroll
-  for (int k = 1; k <= 4; ++k) {
-    ff2 a = ffc(d.Fc[k][3], d.Fc_lo[k][3]);
-#pragma unroll
-    for (int n = 2; n >= 0; --n) a = ff2_mul_add(a, s.E, ffc(d.Fc[k][n], d.Fc_lo[k][n]));
-    a = ff2_mul(a, s.E);                               // F_k(E)
-    sum = ff2_add(sum, a);
-    q.w[k] = ff2_round(ff2_mul(s.rho, a));
-  }
+  for (int n = 2; n >= 0; --n) a = ff2_mul_add(a, E, ffc(d.Fc[k][n], d.Fc_lo[k][n]));
+  return ff2_mul(a, E);
+}
+
+// rho F_0 from the sum of F_1 .. F_4.
+__device__ __forceinline__ f2 rest_weight2(const ff2& rho, const ff2& sum, const DvmConst<float>& d) {
   const ff2 f0 = ff2_add(ff2_of(bc2(1.f)), ff2_mul(ff2_of(bc2(-d.B0)), sum));   // F_0
-  q.w[0] = ff2_round(ff2_mul(s.rho, f0));
+  return ff2_round(ff2_mul(rho, f0));
+}
+
+// Everything but the weights.
+__device__ __forceinline__ void eq2_polynomial(const State2& s, Eq2& q) {
   const ff2 invE = ff2_recip(s.E);
   const ff2 uxE = ff2_mul(s.ux, invE), uyE = ff2_mul(s.uy, invE);
   const ff2 u2E = ff2_add(ff2_mul(s.ux, uxE), ff2_mul(s.uy, uyE));   // u^2 / E
@@ -55,6 +57,19 @@ __device__ __forceinline__ Eq2 eq2(const State2& s, const DvmConst<float>& d) {
   q.yh[1] = y1.hi;  q.yl[1] = y1.lo;
   q.yh[2] = uyE.hi; q.yl[2] = uyE.lo;
   q.yh[3] = y3.hi;  q.yl[3] = y3.lo;
+}
+
+__device__ __forceinline__ Eq2 eq2(const State2& s, const DvmConst<float>& d) {
+  Eq2 q;
+  ff2 sum = ff2_of(bc2(0.f));
+#pragma unroll
+  for (int k = 1; k <= 4; ++k) {
+    const ff2 a = shell_weight2(s.E, d, k);
+    sum = ff2_add(sum, a);
+    q.w[k] = ff2_round(ff2_mul(s.rho, a));
+  }
+  q.w[0] = rest_weight2(s.rho, sum, d);
+  eq2_polynomial(s, q);
   return q;
 }
 

@@ -53,6 +53,40 @@ __device__ __forceinline__ void shell_sums(const float* f, Stride stride, const 
   }
 }
 
+// The same sums with the planes of the shell at f (and of the shell added to it
+// at f_add, if given), the unit vectors those of any shell.
+__device__ __forceinline__ void group_sums32(const float* f, const float* f_add, int stride, const DvmConst<float>& d,
+                                             float& S, float& X, float& Xl, float& Y, float& Yl) {
+  S = 0.f; X = 0.f; Xl = 0.f; Y = 0.f; Yl = 0.f;
+#pragma unroll
+  for (int i = 0; i < kHalf; ++i) {
+    float fa = f[i * stride], fb = f[(i + kHalf) * stride];
+    if (f_add) {
+      fa += f_add[i * stride];
+      fb += f_add[(i + kHalf) * stride];
+    }
+    S += fa + fb;
+    const float dd = fa - fb;
+    X = fmaf(d.cx[1 + i], dd, X);
+    Xl = fmaf(d.cx_lo[1 + i], dd, Xl);
+    Y = fmaf(d.cy[1 + i], dd, Y);
+    Yl = fmaf(d.cy_lo[1 + i], dd, Yl);
+  }
+}
+
+// Velocity and temperature from the moments.
+__device__ __forceinline__ State32 state32_of(ff rho, ff jx, ff jy, ff e) {
+  State32 s;
+  const ff inv = ff_recip(rho);
+  s.rho = rho;
+  s.ux = ff_mul(jx, inv);
+  s.uy = ff_mul(jy, inv);
+  const ff ke = ff_add(ff_mul(jx, s.ux), ff_mul(jy, s.uy));      // |j|^2 / rho
+  s.E = ff_mul(ff_add(e, ff_scale(ke, -0.5f)), inv);
+  s.ok = (rho.hi > 0.f) && (s.E.hi > 0.f) && isfinite(e.hi) && isfinite(jx.hi) && isfinite(jy.hi);
+  return s;
+}
+
 // raw (if given): the moments rho, j_x, j_y and e = rho (E + u^2/2) themselves.
 template <class Stride>
 __device__ __forceinline__ State32 state32(const float* f, Stride stride, const DvmConst<float>& d, ff* raw = nullptr) {
@@ -78,34 +112,24 @@ __device__ __forceinline__ State32 state32(const float* f, Stride stride, const 
     e = ff_add(e, ff_mul(hv, ff_of(S)));
   }
   if (raw) { raw[0] = rho; raw[1] = jx; raw[2] = jy; raw[3] = e; }
-  State32 s;
-  const ff inv = ff_recip(rho);
-  s.rho = rho;
-  s.ux = ff_mul(jx, inv);
-  s.uy = ff_mul(jy, inv);
-  const ff ke = ff_add(ff_mul(jx, s.ux), ff_mul(jy, s.uy));      // |j|^2 / rho
-  s.E = ff_mul(ff_add(e, ff_scale(ke, -0.5f)), inv);
-  s.ok = (rho.hi > 0.f) && (s.E.hi > 0.f) && isfinite(e.hi) && isfinite(jx.hi) && isfinite(jy.hi);
-  return s;
+  return state32_of(rho, jx, jy, e);
 }
 
-// Weights and polynomial factors of Eq. (10) for a node state.
-__device__ __forceinline__ Eq32 eq32(const State32& s, const DvmConst<float>& d) {
-  Eq32 q;
-  ff sum = ff_of(0.f);
+// F_k(E) of Eq. (11a), and rho F_0 from the sum of F_1 .. F_4.
+__device__ __forceinline__ ff shell_weight32(ff E, const DvmConst<float>& d, int k) {
+  ff a{d.Fc[k][3], d.Fc_lo[k][3]};
 #pragma unroll
-  for (int k = 1; k <= 4; ++k) {
-    ff a{d.Fc[k][3], d.Fc_lo[k][3]};
-#pragma unroll
-    for (int n = 2; n >= 0; --n) a = ff_mul_add(a, s.E, ff{d.Fc[k][n], d.Fc_lo[k][n]});
-    a = ff_mul(a, s.E);                  // F_k(E)
-    sum = ff_add(sum, a);
-    const ff wk = ff_mul(s.rho, a);
-    q.w[k] = wk.hi + wk.lo;
-  }
+  for (int n = 2; n >= 0; --n) a = ff_mul_add(a, E, ff{d.Fc[k][n], d.Fc_lo[k][n]});
+  return ff_mul(a, E);
+}
+__device__ __forceinline__ float rest_weight32(ff rho, ff sum, const DvmConst<float>& d) {
   const ff f0 = ff_add(ff_of(1.f), ff_mul(ff_of(-d.B0), sum));   // F_0 = 1 - B0 sum F_k
-  const ff w0 = ff_mul(s.rho, f0);
-  q.w[0] = w0.hi + w0.lo;
+  const ff w0 = ff_mul(rho, f0);
+  return w0.hi + w0.lo;
+}
+
+// The polynomial factors of Eq. (10) for a node state.
+__device__ __forceinline__ void eq32_polynomial(const State32& s, const DvmConst<float>& d, Eq32& q) {
   const ff invE = ff_recip(s.E);
   const ff uxE = ff_mul(s.ux, invE), uyE = ff_mul(s.uy, invE);
   const ff u2E = ff_add(ff_mul(s.ux, uxE), ff_mul(s.uy, uyE));   // u^2 / E
@@ -121,6 +145,21 @@ __device__ __forceinline__ Eq32 eq32(const State32& s, const DvmConst<float>& d)
     q.yh[i] = y.hi;
     q.yl[i] = y.lo;
   }
+}
+
+// Weights and polynomial factors of Eq. (10) for a node state.
+__device__ __forceinline__ Eq32 eq32(const State32& s, const DvmConst<float>& d) {
+  Eq32 q;
+  ff sum = ff_of(0.f);
+#pragma unroll
+  for (int k = 1; k <= 4; ++k) {
+    const ff a = shell_weight32(s.E, d, k);
+    sum = ff_add(sum, a);
+    const ff wk = ff_mul(s.rho, a);
+    q.w[k] = wk.hi + wk.lo;
+  }
+  q.w[0] = rest_weight32(s.rho, sum, d);
+  eq32_polynomial(s, d, q);
   return q;
 }
 
@@ -131,15 +170,17 @@ __device__ __forceinline__ float x_of(float sh, float sl, float yh, float yl) {
 
 // Equilibrium of label q (direction i of shell k, sign +1 for the first of the
 // pair) from the node factors; used for ghost nodes.
-__device__ __forceinline__ float feq32(const Eq32& e, const DvmConst<float>& d, int k, int i, float sign) {
-  if (k == 0) return e.w[0] * e.a0;
+__device__ __forceinline__ float feq32_weighted(const Eq32& e, const DvmConst<float>& d, float w, int k, int i,
+                                                float sign) {
   const float x = sign * x_of(d.speed[k], d.speed_lo[k], e.yh[i], e.yl[i]);
   const float x2 = x * x;
   const float ev = fmaf(x2, fmaf(x2, 1.0f / 24.0f, e.a1h), e.a0);
   const float od = x * fmaf(x2, 1.0f / 6.0f, e.a1);
-  return e.w[k] * (ev + od);
+  return w * (ev + od);
 }
-
+__device__ __forceinline__ float feq32(const Eq32& e, const DvmConst<float>& d, int k, int i, float sign) {
+  return k == 0 ? e.w[0] * e.a0 : feq32_weighted(e, d, e.w[k], k, i, sign);
+}
 
 // Node state from given fields (rho, Cartesian u, E = T).
 __device__ __forceinline__ State32 state32_from_fields(float rho, float ux, float uy, float E) {

@@ -50,7 +50,10 @@ struct F32Size {
   static constexpr int plane = kWinR * (TT + 4);                 // floats per plane window
   static constexpr int planes_bytes = kQ * plane * 4;            // 105600 for TT = 16
   static constexpr int tab_bytes = kPairs * TT * 16;             // one float4 per (pair, row)
-  static constexpr int smem = planes_bytes + tab_bytes + 128;
+  // split: the node pairs' exchange, [4 groups][7] terms, f_0, then [4 shells][2] weights
+  static constexpr int pairs = 16 * TT;
+  static constexpr int exchange_bytes = split > 1 ? (29 + 8) * pairs * 8 : 0;
+  static constexpr int smem = planes_bytes + tab_bytes + exchange_bytes + 128;
   static constexpr int threads = kStepThreads32 + (split > 1 ? 64 : 0);   // two warps for the ghost columns
   // every plane window is a TMA destination: 128-byte aligned (a tile height
   // whose window breaks this faults with a misaligned address)
@@ -93,82 +96,119 @@ __device__ __forceinline__ void shell_sums2(const float* f, f2& S, f2& X, f2& Xl
   }
 }
 
-// Moments (Eqs. 3-5) and temperature recovery of the two nodes.  ready(g)
-// is called before plane group g (the rest plane and shell 1, then shells 2,
-// 3, 4) is first read, so the sums start while later groups still land.
+// What one group of shells adds to the moments (Eqs. 3-5) of the two nodes.
+// Groups: 0 shell 1; 1 shells 2 + 3 direction by direction, with the speed and
+// v^2/2 of shell 2; 2 shell 3 again with the differences v_3 - v_2, (v_3^2 -
+// v_2^2)/2 (S then does not enter rho); 3 shell 4.
+struct Terms2 {
+  f2 S;
+  ff2 jx, jy, e;
+};
+template <int G, int PL>
+__device__ __forceinline__ Terms2 group_terms2(const float* f, const DvmConst<float>& d) {
+  f2 S, X, Xl, Y, Yl;
+  shell_sums2<G == 0 ? 1 : (G == 1 ? 2 : (G == 2 ? 3 : 4)), G == 1 ? 3 : 0, PL>(f, S, X, Xl, Y, Yl);
+  constexpr int k = G == 0 ? 1 : (G == 1 ? 2 : 4);
+  const ff2 v = G == 2 ? ffc(d.dv23, d.dv23_lo) : ffc(d.speed[k], d.speed_lo[k]);
+  const ff2 h = G == 2 ? ffc(d.dh23, d.dh23_lo) : ffc(d.half_v2[k], d.half_v2_lo[k]);
+  return Terms2{S, ff2_mul(v, ff2{X, Xl}), ff2_mul(v, ff2{Y, Yl}), ff2_mul(h, ff2_of(S))};
+}
+
+// Adds the groups up in order and recovers velocity and temperature.
+struct Moments2 {
+  ff2 rho, jx, jy, e;
+  __device__ __forceinline__ explicit Moments2(f2 f0) : rho(ff2_of(f0)), jx(ff2_of(bc2(0.f))), jy(jx), e(jx) {}
+  template <int G>
+  __device__ __forceinline__ void add(const Terms2& t) {
+    if (G != 2) rho = ff2_add(rho, ff2_of(t.S));
+    jx = ff2_add(jx, t.jx);
+    jy = ff2_add(jy, t.jy);
+    e = ff2_add(e, t.e);
+  }
+  __device__ __forceinline__ State2 state() const {
+    State2 s;
+    const ff2 inv = ff2_recip(rho);
+    s.rho = rho;
+    s.ux = ff2_mul(jx, inv);
+    s.uy = ff2_mul(jy, inv);
+    const ff2 ke = ff2_add(ff2_mul(jx, s.ux), ff2_mul(jy, s.uy));    // |j|^2 / rho
+    s.E = ff2_mul(ff2_add(e, ff2_scale(ke, -0.5f)), inv);
+    return s;
+  }
+};
+
+// The state of the two nodes.  ready(g) is called before plane group g (the
+// rest plane and shell 1, then shells 2, 3, 4) is first read, so the sums start
+// while later groups still land.
 template <int PL, class Ready>
 __device__ __forceinline__ State2 state2(const float* f, const DvmConst<float>& d, Ready ready) {
   ready(0);
-  ff2 rho = ff2_of(ld2(f)), jx = ff2_of(bc2(0.f)), jy = jx, e = jx;
-  f2 S, X, Xl, Y, Yl;
-  // shell 1
-  shell_sums2<1, 0, PL>(f, S, X, Xl, Y, Yl);
-  rho = ff2_add(rho, ff2_of(S));
-  jx = ff2_add(jx, ff2_mul(ffc(d.speed[1], d.speed_lo[1]), ff2{X, Xl}));
-  jy = ff2_add(jy, ff2_mul(ffc(d.speed[1], d.speed_lo[1]), ff2{Y, Yl}));
-  e = ff2_add(e, ff2_mul(ffc(d.half_v2[1], d.half_v2_lo[1]), ff2_of(S)));
-  // shells 2 + 3 direction by direction, with the speed and v^2/2 of shell 2
+  Moments2 m(ld2(f));
+  m.template add<0>(group_terms2<0, PL>(f, d));
   ready(1);
   ready(2);
-  shell_sums2<2, 3, PL>(f, S, X, Xl, Y, Yl);
-  rho = ff2_add(rho, ff2_of(S));
-  jx = ff2_add(jx, ff2_mul(ffc(d.speed[2], d.speed_lo[2]), ff2{X, Xl}));
-  jy = ff2_add(jy, ff2_mul(ffc(d.speed[2], d.speed_lo[2]), ff2{Y, Yl}));
-  e = ff2_add(e, ff2_mul(ffc(d.half_v2[2], d.half_v2_lo[2]), ff2_of(S)));
-  // shell 3 again with the differences v_3 - v_2, (v_3^2 - v_2^2)/2
-  shell_sums2<3, 0, PL>(f, S, X, Xl, Y, Yl);
-  jx = ff2_add(jx, ff2_mul(ffc(d.dv23, d.dv23_lo), ff2{X, Xl}));
-  jy = ff2_add(jy, ff2_mul(ffc(d.dv23, d.dv23_lo), ff2{Y, Yl}));
-  e = ff2_add(e, ff2_mul(ffc(d.dh23, d.dh23_lo), ff2_of(S)));
-  // shell 4
+  m.template add<1>(group_terms2<1, PL>(f, d));
+  m.template add<2>(group_terms2<2, PL>(f, d));
   ready(3);
-  shell_sums2<4, 0, PL>(f, S, X, Xl, Y, Yl);
-  rho = ff2_add(rho, ff2_of(S));
-  jx = ff2_add(jx, ff2_mul(ffc(d.speed[4], d.speed_lo[4]), ff2{X, Xl}));
-  jy = ff2_add(jy, ff2_mul(ffc(d.speed[4], d.speed_lo[4]), ff2{Y, Yl}));
-  e = ff2_add(e, ff2_mul(ffc(d.half_v2[4], d.half_v2_lo[4]), ff2_of(S)));
+  m.template add<3>(group_terms2<3, PL>(f, d));
+  return m.state();
+}
 
-  State2 s;
-  const ff2 inv = ff2_recip(rho);
-  s.rho = rho;
-  s.ux = ff2_mul(jx, inv);
-  s.uy = ff2_mul(jy, inv);
-  const ff2 ke = ff2_add(ff2_mul(jx, s.ux), ff2_mul(jy, s.uy));    // |j|^2 / rho
-  s.E = ff2_mul(ff2_add(e, ff2_scale(ke, -0.5f)), inv);
-  return s;
+// The same with the groups spread over the four threads of a node pair (thread
+// `split` forms group `split`), which exchange them through x [group][7][pairs]
+// (`pairs` node pairs, this one `ip`).  barrier() joins the threads and tells
+// whether all of them have their planes.
+template <int PL, class Ready, class Barrier>
+__device__ __forceinline__ State2 state2_split(const float* f, const DvmConst<float>& d, int split, f2* x, int pairs,
+                                               int ip, Ready ready, Barrier barrier) {
+  Terms2 t;
+  switch (split) {
+    case 0: ready(0); t = group_terms2<0, PL>(f, d); break;
+    case 1: ready(1); ready(2); t = group_terms2<1, PL>(f, d); break;
+    case 2: ready(2); t = group_terms2<2, PL>(f, d); break;
+    default: ready(3); t = group_terms2<3, PL>(f, d); break;
+  }
+  f2* o = x + split * 7 * pairs + ip;
+  o[0] = t.S;
+  o[1 * pairs] = t.jx.hi; o[2 * pairs] = t.jx.lo;
+  o[3 * pairs] = t.jy.hi; o[4 * pairs] = t.jy.lo;
+  o[5 * pairs] = t.e.hi;  o[6 * pairs] = t.e.lo;
+  if (split == 0) x[28 * pairs + ip] = ld2(f);
+  barrier();
+  auto get = [&](int g) {
+    const f2* i = x + g * 7 * pairs + ip;
+    return Terms2{i[0], ff2{i[1 * pairs], i[2 * pairs]}, ff2{i[3 * pairs], i[4 * pairs]}, ff2{i[5 * pairs], i[6 * pairs]}};
+  };
+  Moments2 m(x[28 * pairs + ip]);
+  m.template add<0>(get(0));
+  m.template add<1>(get(1));
+  m.template add<2>(get(2));
+  m.template add<3>(get(3));
+  return m.state();
 }
 
 // Ghost columns of one wall (wall node at window column cw) for the tile's TT
 // rows, by one warp, Sec. II C 1: lane (row, node) forms the state of the wall
 // node a or of the next node b, then lane (row, layer) the layer's state and
-// its equilibrium; with TT = 4 the four groups of lanes hold the same states and
-// store a shell each.  (One lane per row forming both states and both layers
-// took about 8 of the 19 us of a small step.)
-template <int TT>
+// its equilibrium.  (One lane per row forming both states and both layers took
+// about 8 of the 19 us of a small step.)  With TT = 4 the four groups of lanes
+// share that work shell by shell, with shuffles: the sums of Eqs. 3-5, the
+// weights of Eq. 11 and the values stored; what does not depend on f is formed
+// before ready() waits for the planes.  Same operations, same results.
+template <int TT, class Ready>
 __device__ __noinline__ void ghost_columns_f32(float* sm, int lane, int side, int cw, int t0, const StepParams& p,
-                                               const DvmConst<float>& d) {
+                                               const DvmConst<float>& d, Ready ready) {
   constexpr int PL = F32Size<TT>::plane;
+  constexpr bool kShare = TT == 4;
+  static_assert(TT == 16 || TT == 4, "32 lanes: row, node, and for 4 rows the shell");
   const int step = side == 0 ? 1 : -1;
   const int row = 2 + lane % TT, layer = (lane / TT) & 1, group = lane / (2 * TT);
+  const int base = lane % (2 * TT);   // this lane's (row, node) in group 0
   const int t = min(t0 + lane % TT, p.n_theta - 1);
-  const State32 m = state32(sm + row * kWinR + cw + (layer == 0 ? 0 : step), PL, d);
-  // the other node's state (lane a holds a, lane b holds b)
-  auto other = [&](ff x) { return ff{__shfl_xor_sync(0xffffffffu, x.hi, TT), __shfl_xor_sync(0xffffffffu, x.lo, TT)}; };
-  const State32 o{other(m.rho), other(m.ux), other(m.uy), other(m.E),
-                  __shfl_xor_sync(0xffffffffu, (int)m.ok, TT) != 0};
-  const State32 a = layer == 0 ? m : o, b = layer == 0 ? o : m;
-  // Eq. (39), applied twice: g0 = 2a - b, g1 = 2 g0 - a = 3a - 2b.
-  auto extrapolated = [&](ff xa, ff xb) {
-    const ff g0 = ff_add(ff_scale(xa, 2.f), ff_neg(xb));
-    return layer == 0 ? g0 : ff_add(ff_scale(g0, 2.f), ff_neg(xa));
-  };
-  State32 g;
-  g.rho = extrapolated(a.rho, b.rho);
-  g.E = extrapolated(a.E, b.E);
-  g.ux = extrapolated(a.ux, b.ux);
-  g.uy = extrapolated(a.uy, b.uy);
   const int kind = p.bc_kind[side] & ~PCLB_BC_NEQ;
   const bool neq = (p.bc_kind[side] & PCLB_BC_NEQ) != 0;
+
+  State32 g;   // the layer's state: prescribed components first
   if (kind != PCLB_BC_EXTRAP) {
     const double c = p.cos_t[t], s = p.sin_t[t];
     const double* v = p.bc_vals + (size_t)((side * 2 + layer) * 4) * p.n_theta + t;
@@ -180,26 +220,91 @@ __device__ __noinline__ void ghost_columns_f32(float* sm, int lane, int side, in
       g.E = ff_from(v[3 * p.n_theta]);
     }
   }
+  // equilibrium factors of a state; with kShare w[1] holds the weight of
+  // shell group + 1
+  auto factors = [&](const State32& s) {
+    if constexpr (!kShare) {
+      return eq32(s, d);
+    } else {
+      Eq32 q;
+      const ff F = shell_weight32(s.E, d, group + 1);
+      ff sum = ff_of(0.f);
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        sum = ff_add(sum, ff{__shfl_sync(0xffffffffu, F.hi, base + k * 2 * TT), __shfl_sync(0xffffffffu, F.lo, base + k * 2 * TT)});
+      const ff wk = ff_mul(s.rho, F);
+      q.w[1] = wk.hi + wk.lo;
+      q.w[0] = rest_weight32(s.rho, sum, d);
+      eq32_polynomial(s, d, q);
+      return q;
+    }
+  };
+  Eq32 e;
+  if (kind == PCLB_BC_DIRICHLET) e = factors(g);
+
+  if (!ready()) return;   // uniform: the tile is given up
+  const float* fn = sm + row * kWinR + cw + (layer == 0 ? 0 : step);
+  State32 m;
+  if constexpr (!kShare) {
+    m = state32(fn, PL, d);
+  } else {
+    const int k = group + 1;   // groups: shells 1; 2 + 3; 3; 4
+    float S, X, Xl, Y, Yl;
+    group_sums32(fn + (1 + (k - 1) * kNDirs) * PL, group == 1 ? fn + (1 + 2 * kNDirs) * PL : nullptr, PL, d, S, X, Xl, Y, Yl);
+    const ff v = group == 2 ? ff{d.dv23, d.dv23_lo} : ff{d.speed[k], d.speed_lo[k]};
+    const ff h = group == 2 ? ff{d.dh23, d.dh23_lo} : ff{d.half_v2[k], d.half_v2_lo[k]};
+    const ff tx = ff_mul(v, ff{X, Xl}), ty = ff_mul(v, ff{Y, Yl}), te = ff_mul(h, ff_of(S));
+    ff rho = ff_of(fn[0]), jx = ff_of(0.f), jy = jx, en = jx;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int from = base + i * 2 * TT;
+      auto get = [&](float x) { return __shfl_sync(0xffffffffu, x, from); };
+      const float Si = get(S);
+      if (i != 2) rho = ff_add(rho, ff_of(Si));
+      jx = ff_add(jx, ff{get(tx.hi), get(tx.lo)});
+      jy = ff_add(jy, ff{get(ty.hi), get(ty.lo)});
+      en = ff_add(en, ff{get(te.hi), get(te.lo)});
+    }
+    m = state32_of(rho, jx, jy, en);
+  }
+  // the other node's state (lane a holds a, lane b holds b)
+  auto other = [&](ff x) { return ff{__shfl_xor_sync(0xffffffffu, x.hi, TT), __shfl_xor_sync(0xffffffffu, x.lo, TT)}; };
+  const State32 o{other(m.rho), other(m.ux), other(m.uy), other(m.E),
+                  __shfl_xor_sync(0xffffffffu, (int)m.ok, TT) != 0};
+  const State32 a = layer == 0 ? m : o, b = layer == 0 ? o : m;
+  // Eq. (39), applied twice: g0 = 2a - b, g1 = 2 g0 - a = 3a - 2b.
+  auto extrapolated = [&](ff xa, ff xb) {
+    const ff g0 = ff_add(ff_scale(xa, 2.f), ff_neg(xb));
+    return layer == 0 ? g0 : ff_add(ff_scale(g0, 2.f), ff_neg(xa));
+  };
+  if (kind != PCLB_BC_DIRICHLET) {
+    g.rho = extrapolated(a.rho, b.rho);
+    g.E = extrapolated(a.E, b.E);
+    if (kind == PCLB_BC_EXTRAP) {
+      g.ux = extrapolated(a.ux, b.ux);
+      g.uy = extrapolated(a.uy, b.uy);
+    }
+    e = factors(g);
+  }
+  // equilibrium of the wall node, for the departure it hands to its ghosts
+  Eq32 ea{};
+  if (neq) ea = factors(a);
   const int col = cw - step * (1 + layer);
   if (t0 + lane % TT >= p.n_theta) return;
   if (!(a.ok && b.ok && g.rho.hi > 0.f && g.E.hi > 0.f)) atomicOr(p.status, PCLB_FLAG_NONPHYS);
   if (col < 0 || col >= kWinR) return;
-  // equilibrium of the wall node, for the departure it hands to its ghosts
-  Eq32 ea{};
-  if (neq) ea = eq32(a, d);
   const float* fa = sm + row * kWinR + cw;
-  const Eq32 e = eq32(g, d);
   float* gp = sm + row * kWinR + col;
   if (group == 0) gp[0] = feq32(e, d, 0, 0, 1.f) + (neq ? fa[0] - feq32(ea, d, 0, 0, 1.f) : 0.f);
 #pragma unroll 1
-  for (int k = TT == 16 ? 1 : group + 1; k <= (TT == 16 ? 4 : group + 1); ++k)
+  for (int k = kShare ? group + 1 : 1; k <= (kShare ? group + 1 : 4); ++k)
 #pragma unroll
     for (int i = 0; i < kHalf; ++i) {
-      const int q = 1 + (k - 1) * kNDirs + i;
-      float v1 = feq32(e, d, k, i, 1.f), v2 = feq32(e, d, k, i, -1.f);
+      const int q = 1 + (k - 1) * kNDirs + i, kw = kShare ? 1 : k;
+      float v1 = feq32_weighted(e, d, e.w[kw], k, i, 1.f), v2 = feq32_weighted(e, d, e.w[kw], k, i, -1.f);
       if (neq) {
-        v1 += fa[q * PL] - feq32(ea, d, k, i, 1.f);
-        v2 += fa[(q + kHalf) * PL] - feq32(ea, d, k, i, -1.f);
+        v1 += fa[q * PL] - feq32_weighted(ea, d, ea.w[kw], k, i, 1.f);
+        v2 += fa[(q + kHalf) * PL] - feq32_weighted(ea, d, ea.w[kw], k, i, -1.f);
       }
       gp[q * PL] = v1;
       gp[(q + kHalf) * PL] = v2;
@@ -232,7 +337,8 @@ __global__ void __launch_bounds__(F32Size<TT>::threads, kCtasPerSm32)
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float* sm = reinterpret_cast<float*>(smem_raw);
   float4* tab = reinterpret_cast<float4*>(smem_raw + SZ::planes_bytes);
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + SZ::planes_bytes + SZ::tab_bytes);
+  f2* xch = reinterpret_cast<f2*>(smem_raw + SZ::planes_bytes + SZ::tab_bytes);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + SZ::planes_bytes + SZ::tab_bytes + SZ::exchange_bytes);
 
   const int r0 = blockIdx.x * kTileR;
   const int t0 = (blockIdx.y + ty0) * TT;   // ty0: first tile row of the launch
@@ -245,6 +351,31 @@ __global__ void __launch_bounds__(F32Size<TT>::threads, kCtasPerSm32)
     tma_prefetch_desc(&tmap_in);
     for (int g = 0; g < kGroups; ++g) mbar_init(&bar[g], 1);
     mbar_fence_init();
+  }
+  const int warp = tid >> 5, lane = tid & 31;
+  const int cw_out = p.n_r - 1 - r0 + kLeft;
+  const bool inner = r0 == 0, outer = cw_out <= kLeft + kTileR;   // tiles at a wall
+  bool ok = true;
+  auto ready = [&](int g) {
+    if (ok) ok = p.wait_ns != 0 && mbar_wait_bounded(&bar[g], 0, p.wait_ns);   // 0: give up at once
+  };
+  if constexpr (SPLIT > 1) {
+    if (warp >= kStepThreads32 / 32) {   // the ghost columns' warps: one per wall
+      const int side = warp - kStepThreads32 / 32;
+      const bool active = side == 0 ? inner : outer;
+      bool joined = false;
+      auto all = [&]() {   // after what does not depend on f
+        pdl_wait();
+        block_barrier();   // barriers initialised
+        joined = true;
+        for (int g = 0; g < kGroups; ++g) ready(g);
+        return ok = __all_sync(0xffffffffu, ok);
+      };
+      if (active) ghost_columns_f32<TT>(sm, lane, side, side == 0 ? kLeft : cw_out, t0, p, d, all);
+      if (!joined) block_barrier();
+      if (inner || outer) __syncthreads_or(!ok);
+      return;
+    }
   }
   // Courant entries of the tile rows: table layout [pair][row] (read before
   // the wait: no step writes them)
@@ -263,11 +394,9 @@ __global__ void __launch_bounds__(F32Size<TT>::threads, kCtasPerSm32)
     }
   }
   if (tid < kPairs * TT) tab[te_pair * TT + te_row] = te;
-  __syncthreads();   // table visible (while the copies are still landing)
-  bool ok = true;
+  block_barrier();   // table visible (while the copies are still landing)
 
   // ---- per-thread nodes: row rl, radial cells j2 and j2 + 1 -----------------
-  const int warp = tid >> 5, lane = tid & 31;
   const int rl = (2 * warp + (lane >> 4)) % TT;    // tile row
   const int split = SPLIT == 1 ? 0 : warp / (TT / 2);   // SPLIT > 1: shell split + 1; the two warps after those: ghost columns
   const int j2 = 2 * (lane & 15);                  // even radial offset 0..30
@@ -279,25 +408,15 @@ __global__ void __launch_bounds__(F32Size<TT>::threads, kCtasPerSm32)
   const bool v0 = row_ok && r < p.n_r, v1 = row_ok && r + 1 < p.n_r;
   const float* win = sm + row * kWinR + col;
 
-  const int cw_out = p.n_r - 1 - r0 + kLeft;
-  const bool inner = r0 == 0, outer = cw_out <= kLeft + kTileR;   // tiles at a wall
-  auto ready = [&](int g) {
-    if (ok) ok = p.wait_ns != 0 && mbar_wait_bounded(&bar[g], 0, p.wait_ns);   // 0: give up at once
-  };
-  if constexpr (SPLIT > 1) {
-    if (warp >= kStepThreads32 / 32) {   // the ghost columns' warps: one per wall
-      const int side = warp - kStepThreads32 / 32;
-      if (!inner && !outer) return;
-      for (int g = 0; g < kGroups; ++g) ready(g);
-      if (ok && (side == 0 ? inner : outer)) ghost_columns_f32<TT>(sm, lane, side, side == 0 ? kLeft : cw_out, t0, p, d);
-      __syncthreads_or(!ok);
-      return;
-    }
-  }
-
   Eq2 eq;
+  const int ip = (warp & (TT / 2 - 1)) * 32 + lane;   // node pair of the tile (SPLIT > 1)
   {
-    State2 s = state2<PL>(win, d, ready);
+    State2 s;
+    if constexpr (SPLIT == 1) {
+      s = state2<PL>(win, d, ready);
+    } else {
+      s = state2_split<PL>(win, d, split, xch, SZ::pairs, ip, ready, [&]() { ok = !barrier_or(1, kStepThreads32, !ok); });
+    }
     const bool ok0 = s.rho.hi.x > 0.f && s.E.hi.x > 0.f && isfinite(s.E.hi.x) && isfinite(s.ux.hi.x) &&
                      isfinite(s.uy.hi.x);
     const bool ok1 = s.rho.hi.y > 0.f && s.E.hi.y > 0.f && isfinite(s.E.hi.y) && isfinite(s.ux.hi.y) &&
@@ -308,14 +427,32 @@ __global__ void __launch_bounds__(F32Size<TT>::threads, kCtasPerSm32)
                s.ux.hi.x = 0.f; s.ux.lo.x = 0.f; s.uy.hi.x = 0.f; s.uy.lo.x = 0.f; }
     if (!v1) { s.rho.hi.y = 1.f; s.rho.lo.y = 0.f; s.E.hi.y = 1.f; s.E.lo.y = 0.f;
                s.ux.hi.y = 0.f; s.ux.lo.y = 0.f; s.uy.hi.y = 0.f; s.uy.lo.y = 0.f; }
-    eq = eq2(s, d);
+    if constexpr (SPLIT == 1) {
+      eq = eq2(s, d);
+    } else {   // this thread's shell only; the first thread of a pair also needs the sum of all four
+      const ff2 F = shell_weight2(s.E, d, split + 1);
+      xch[(29 + 2 * split) * SZ::pairs + ip] = F.hi;
+      xch[(30 + 2 * split) * SZ::pairs + ip] = F.lo;
+      eq.w[1] = ff2_round(ff2_mul(s.rho, F));
+      eq2_polynomial(s, eq);
+      barrier_or(1, kStepThreads32, false);
+      if (split == 0) {
+        ff2 sum = ff2_of(bc2(0.f));
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          sum = ff2_add(sum, ff2{xch[(29 + 2 * k) * SZ::pairs + ip], xch[(30 + 2 * k) * SZ::pairs + ip]});
+        eq.w[0] = rest_weight2(s.rho, sum, d);
+      }
+    }
   }
 
   // ---- radial ghost columns (tiles at a wall only) ----------------------------
   if (inner || outer) {
     if constexpr (SPLIT == 1) {
-      if (ok && inner && warp == 0) ghost_columns_f32<TT>(sm, lane, 0, kLeft, t0, p, d);
-      if (ok && outer && warp == 1) ghost_columns_f32<TT>(sm, lane, 1, cw_out, t0, p, d);
+      const bool here = __all_sync(0xffffffffu, ok);
+      auto landed = [&]() { return here; };
+      if (inner && warp == 0) ghost_columns_f32<TT>(sm, lane, 0, kLeft, t0, p, d, landed);
+      if (outer && warp == 1) ghost_columns_f32<TT>(sm, lane, 1, cw_out, t0, p, d, landed);
     }
     if (__syncthreads_or(!ok)) {   // ghost columns visible; a copy that timed out stops the tile
       if (tid == 0) {
@@ -409,7 +546,7 @@ __global__ void __launch_bounds__(F32Size<TT>::threads, kCtasPerSm32)
 #pragma unroll 1
   for (int k = SPLIT == 1 ? 1 : split + 1; k <= (SPLIT == 1 ? 4 : split + 1); ++k) {
     const f2 sh = bc2(d.speed[k]), sl = bc2(d.speed_lo[k]);
-    const f2 wk = k == 1 ? eq.w[1] : (k == 2 ? eq.w[2] : (k == 3 ? eq.w[3] : eq.w[4]));
+    const f2 wk = SPLIT > 1 || k == 1 ? eq.w[1] : (k == 2 ? eq.w[2] : (k == 3 ? eq.w[3] : eq.w[4]));
     const int qb = 1 + (k - 1) * kNDirs;
 #pragma unroll
     for (int i = 0; i < kHalf; ++i) {
