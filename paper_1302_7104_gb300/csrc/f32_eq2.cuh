@@ -87,4 +87,76 @@ __device__ __forceinline__ void feq_pair2(const Eq2& eq, f2 sh, f2 sl, int i, f2
   fm = fma2(neg2(wk), od, wev);
 }
 
+// Sums over one shell (plus, optionally, a second shell added direction by
+// direction) of f, c_x f and c_y f for both nodes, with the octagon's exact
+// unit vectors as float-float constants.  ld(q): the two nodes' f_q.
+template <int K, int KADD, class LD>
+__device__ __forceinline__ void shell_sums2(LD ld, f2& S, f2& X, f2& Xl, f2& Y, f2& Yl) {
+  S = bc2(0.f); X = bc2(0.f); Xl = bc2(0.f); Y = bc2(0.f); Yl = bc2(0.f);
+#pragma unroll
+  for (int i = 0; i < kHalf; ++i) {
+    const int q = 1 + (K - 1) * kNDirs + i;
+    f2 fa = ld(q), fb = ld(q + kHalf);
+    if (KADD > 0) {
+      const int qa = 1 + (KADD - 1) * kNDirs + i;
+      fa = add2(fa, ld(qa));
+      fb = add2(fb, ld(qa + kHalf));
+    }
+    S = add2(S, add2(fa, fb));
+    const f2 dd = sub2(fa, fb);
+    if (i == 0) {
+      X = add2(X, dd);
+    } else if (i == 2) {
+      Y = add2(Y, dd);
+    } else {
+      const float sx = i == 1 ? 1.f : -1.f;
+      X = fma2(bc2(sx * kS), dd, X);
+      Xl = fma2(bc2(sx * kSl), dd, Xl);
+      Y = fma2(bc2(kS), dd, Y);
+      Yl = fma2(bc2(kSl), dd, Yl);
+    }
+  }
+}
+
+// What one group of shells adds to the moments (Eqs. 3-5) of the two nodes.
+// Groups: 0 shell 1; 1 shells 2 + 3 direction by direction, with the speed and
+// v^2/2 of shell 2; 2 shell 3 again with the differences v_3 - v_2, (v_3^2 -
+// v_2^2)/2 (S then does not enter rho); 3 shell 4.
+struct Terms2 {
+  f2 S;
+  ff2 jx, jy, e;
+};
+template <int G, class LD>
+__device__ __forceinline__ Terms2 group_terms2(LD ld, const DvmConst<float>& d) {
+  f2 S, X, Xl, Y, Yl;
+  shell_sums2<G == 0 ? 1 : (G == 1 ? 2 : (G == 2 ? 3 : 4)), G == 1 ? 3 : 0>(ld, S, X, Xl, Y, Yl);
+  constexpr int k = G == 0 ? 1 : (G == 1 ? 2 : 4);
+  const ff2 v = G == 2 ? ffc(d.dv23, d.dv23_lo) : ffc(d.speed[k], d.speed_lo[k]);
+  const ff2 h = G == 2 ? ffc(d.dh23, d.dh23_lo) : ffc(d.half_v2[k], d.half_v2_lo[k]);
+  return Terms2{S, ff2_mul(v, ff2{X, Xl}), ff2_mul(v, ff2{Y, Yl}), ff2_mul(h, ff2_of(S))};
+}
+
+// Adds the groups up in order and recovers velocity and temperature.
+struct Moments2 {
+  ff2 rho, jx, jy, e;
+  __device__ __forceinline__ explicit Moments2(f2 f0) : rho(ff2_of(f0)), jx(ff2_of(bc2(0.f))), jy(jx), e(jx) {}
+  template <int G>
+  __device__ __forceinline__ void add(const Terms2& t) {
+    if (G != 2) rho = ff2_add(rho, ff2_of(t.S));
+    jx = ff2_add(jx, t.jx);
+    jy = ff2_add(jy, t.jy);
+    e = ff2_add(e, t.e);
+  }
+  __device__ __forceinline__ State2 state() const {
+    State2 s;
+    const ff2 inv = ff2_recip(rho);
+    s.rho = rho;
+    s.ux = ff2_mul(jx, inv);
+    s.uy = ff2_mul(jy, inv);
+    const ff2 ke = ff2_add(ff2_mul(jx, s.ux), ff2_mul(jy, s.uy));    // |j|^2 / rho
+    s.E = ff2_mul(ff2_add(e, ff2_scale(ke, -0.5f)), inv);
+    return s;
+  }
+};
+
 }  // namespace pclb

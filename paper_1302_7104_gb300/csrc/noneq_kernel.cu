@@ -1,4 +1,4 @@
-// Non-equilibrium manifestations of Sec. IV, one node per thread.
+// Non-equilibrium manifestations of Sec. IV.
 //
 // For the weights w_q = f_q (moments) or w_q = f_q - f^eq_q (departures) and
 // the velocities c_q = v_q (plain) or c_q = v_q - u (central), in polar
@@ -28,6 +28,7 @@
 
 #include "device_common.cuh"
 #include "dvm_generic.h"
+#include "f32_eq2.cuh"
 #include "f32_state.cuh"
 #include "gen_state.cuh"
 #include "pclb_internal.h"
@@ -37,31 +38,6 @@ namespace pclb {
 namespace {
 
 constexpr int kNeqThreads = 128;
-
-// rho, u and E of the node in the precision of the step kernels (float-float
-// moments in FP32), and rho E, 2 rho E^2 in double.
-__device__ __forceinline__ void neq_state(const float* f, size_t plane, const DvmConst<float>& d, float& rho,
-                                          float& ux, float& uy, bool& ok, double& rE, double& rE2) {
-  const State32 s = state32(f, plane, d);
-  const double R = (double)s.rho.hi + s.rho.lo, E = (double)s.E.hi + s.E.lo;
-  rho = (float)R;
-  ux = s.ux.hi + s.ux.lo;
-  uy = s.uy.hi + s.uy.lo;
-  ok = s.ok;
-  rE = R * E;
-  rE2 = 2.0 * R * E * E;
-}
-
-__device__ __forceinline__ void neq_state(const double* f, size_t plane, const DvmConst<double>& d, double& rho,
-                                          double& ux, double& uy, bool& ok, double& rE, double& rE2) {
-  const NodeState<double> m = node_moments(f, plane, d);
-  rho = m.rho;
-  ux = m.ux;
-  uy = m.uy;
-  ok = m.ok;
-  rE = m.rho_d * m.E_d;
-  rE2 = 2.0 * m.rho_d * m.E_d * m.E_d;
-}
 
 // Plain moments (12 components, order as above) from central ones C with
 // density R (0 for departures) and velocity (ur, ut), polar components.
@@ -91,20 +67,20 @@ __device__ __forceinline__ void plain_from_central(T R, T ur, T ut, const T* C, 
 
 }  // namespace
 
-template <class T>
+// FP64: one node per thread.
 __global__ void __launch_bounds__(kNeqThreads)
-    noneq_kernel(const T* __restrict__ f, T* __restrict__ out, int groups, const __grid_constant__ StepParams p,
-                 const __grid_constant__ DvmConst<T> d) {
+    noneq_kernel(const double* __restrict__ f, double* __restrict__ out, int groups,
+                 const __grid_constant__ StepParams p, const __grid_constant__ DvmConst<double> d) {
+  using T = double;
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   const int t = blockIdx.y;
   if (r >= p.n_r || t >= p.n_theta) return;
   const size_t plane = (size_t)p.rows * p.pitch;
   const T* fn = f + (size_t)(t + kGhostRows) * p.pitch + r;
-  T rho, ux, uy;
-  bool ok;
-  double rE, rE2;
-  neq_state(fn, plane, d, rho, ux, uy, ok, rE, rE2);
-  if (!ok) atomicOr(p.status, PCLB_FLAG_NONPHYS);
+  const NodeState<T> m = node_moments(fn, plane, d);
+  const T rho = m.rho, ux = m.ux, uy = m.uy;
+  const T rE = m.rho * m.E, rE2 = 2.0 * m.rho * m.E * m.E;
+  if (!m.ok) atomicOr(p.status, PCLB_FLAG_NONPHYS);
   const T cs = (T)p.cos_t[t], sn = (T)p.sin_t[t];
   const T u_r = ux * cs + uy * sn, u_t = uy * cs - ux * sn;
 
@@ -136,10 +112,10 @@ __global__ void __launch_bounds__(kNeqThreads)
   T D[12];
 #pragma unroll
   for (int c = 0; c < 12; ++c) D[c] = A[c];
-  D[0] = (T)((double)A[0] - rE);
-  D[2] = (T)((double)A[2] - rE);
-  D[9] = (T)((double)A[9] - rE2);
-  D[11] = (T)((double)A[11] - rE2);
+  D[0] = A[0] - rE;
+  D[2] = A[2] - rE;
+  D[9] = A[9] - rE2;
+  D[11] = A[11] - rE2;
 
   const size_t nodes = (size_t)p.n_theta * p.n_r, n = (size_t)t * p.n_r + r;
   int slot = 0;
@@ -155,6 +131,105 @@ __global__ void __launch_bounds__(kNeqThreads)
       for (int c = 0; c < 12; ++c) out_g[c] = D[c];
 #pragma unroll
     for (int c = 0; c < 12; ++c) out[(size_t)(slot * 12 + c) * nodes + n] = out_g[c];
+    ++slot;
+  }
+}
+
+// FP32: two radially adjacent nodes per thread in packed FP32x2 arithmetic, the
+// node state and rho E, 2 rho E^2 in float-float.  Bound: HBM, with issue close
+// behind (one node per thread and FP64 for the departures: 156 us on 1024 x
+// 2048, all four groups, at 83% issue and half the FP64 pipe).
+__global__ void __launch_bounds__(kNeqThreads)
+    noneq_f32_kernel(const float* __restrict__ f, float* __restrict__ out, int groups,
+                     const __grid_constant__ StepParams p, const __grid_constant__ DvmConst<float> d) {
+  const int r = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+  const int t = blockIdx.y;
+  if (r >= p.n_r || t >= p.n_theta) return;
+  const bool v1 = r + 1 < p.n_r;   // the second node exists (else its values, from the row's padding, are not stored)
+  const size_t plane = (size_t)p.rows * p.pitch;
+  const float* fn = f + (size_t)(t + kGhostRows) * p.pitch + r;
+  auto ld = [&](int q) { return __ldg(reinterpret_cast<const float2*>(fn + (size_t)q * plane)); };
+  Moments2 m(ld(0));
+  m.add<0>(group_terms2<0>(ld, d));
+  m.add<1>(group_terms2<1>(ld, d));
+  m.add<2>(group_terms2<2>(ld, d));
+  m.add<3>(group_terms2<3>(ld, d));
+  const State2 st = m.state();
+  auto physical = [](float rho, float E, float e, float jx, float jy) {
+    return rho > 0.f && E > 0.f && isfinite(e) && isfinite(jx) && isfinite(jy);
+  };
+  if (!physical(m.rho.hi.x, st.E.hi.x, m.e.hi.x, m.jx.hi.x, m.jy.hi.x) ||
+      (v1 && !physical(m.rho.hi.y, st.E.hi.y, m.e.hi.y, m.jx.hi.y, m.jy.hi.y)))
+    atomicOr(p.status, PCLB_FLAG_NONPHYS);
+  const f2 ux = ff2_round(st.ux), uy = ff2_round(st.uy), rho = ff2_round(st.rho);
+  const float cs = (float)p.cos_t[t], sn = (float)p.sin_t[t];
+  const f2 u_r = fma2(ux, bc2(cs), mul2(uy, bc2(sn))), u_t = fma2(uy, bc2(cs), neg2(mul2(ux, bc2(sn))));
+
+  // central moments of f (the sums with c.c, halved at the end)
+  f2 A[12];
+#pragma unroll
+  for (int c = 0; c < 12; ++c) A[c] = bc2(0.f);
+#pragma unroll
+  for (int q = 0; q < kQ; ++q) {
+    const f2 w = ld(q);
+    const f2 cr = sub2(bc2(fmaf(d.vx[q], cs, d.vy[q] * sn)), u_r), ct = sub2(bc2(fmaf(d.vy[q], cs, -(d.vx[q] * sn))), u_t);
+    const f2 cc = fma2(cr, cr, mul2(ct, ct));
+    const f2 wr = mul2(w, cr), wt = mul2(w, ct);
+    const f2 wrr = mul2(wr, cr), wrt = mul2(wr, ct), wtt = mul2(wt, ct);
+    A[0] = add2(A[0], wrr);
+    A[1] = add2(A[1], wrt);
+    A[2] = add2(A[2], wtt);
+    A[3] = fma2(wrr, cr, A[3]);
+    A[4] = fma2(wrr, ct, A[4]);
+    A[5] = fma2(wrt, ct, A[5]);
+    A[6] = fma2(wtt, ct, A[6]);
+    A[7] = fma2(cc, wr, A[7]);
+    A[8] = fma2(cc, wt, A[8]);
+    A[9] = fma2(cc, wrr, A[9]);
+    A[10] = fma2(cc, wrt, A[10]);
+    A[11] = fma2(cc, wtt, A[11]);
+  }
+#pragma unroll
+  for (int c = 7; c < 12; ++c) A[c] = mul2(A[c], bc2(0.5f));
+  // central departures: minus the equilibrium's (rho E I, 0, 0, 2 rho E^2 I)
+  const ff2 rE = ff2_mul(st.rho, st.E), rE2 = ff2_scale(ff2_mul(rE, st.E), 2.f);
+  auto less = [](f2 a, ff2 b) { return sub2(sub2(a, b.hi), b.lo); };
+  const f2 D0 = less(A[0], rE), D2 = less(A[2], rE), D9 = less(A[9], rE2), D11 = less(A[11], rE2);
+
+  const size_t nodes = (size_t)p.n_theta * p.n_r;
+  float* o = out + (size_t)t * p.n_r + r;
+  const bool wide = v1 && (reinterpret_cast<uintptr_t>(o) & 7) == 0 && (nodes & 1) == 0;
+  auto put = [&](int c, float x, float y) {
+    float* oc = o + (size_t)c * nodes;
+    if (wide) {
+      *reinterpret_cast<float2*>(oc) = make_float2(x, y);
+    } else {
+      oc[0] = x;
+      if (v1) oc[1] = y;
+    }
+  };
+  int slot = 0;
+#pragma unroll 1
+  for (int g = 0; g < 4; ++g) {
+    if (!(groups & (1 << g))) continue;
+    const bool dep = (g & 1) != 0;
+    float X[12], Y[12];
+#pragma unroll
+    for (int c = 0; c < 12; ++c) { X[c] = A[c].x; Y[c] = A[c].y; }
+    if (dep) {
+      X[0] = D0.x; X[2] = D2.x; X[9] = D9.x; X[11] = D11.x;
+      Y[0] = D0.y; Y[2] = D2.y; Y[9] = D9.y; Y[11] = D11.y;
+    }
+    if (g < 2) {
+      float PX[12], PY[12];
+      plain_from_central<float>(dep ? 0.f : rho.x, u_r.x, u_t.x, X, PX);
+      plain_from_central<float>(dep ? 0.f : rho.y, u_r.y, u_t.y, Y, PY);
+#pragma unroll
+      for (int c = 0; c < 12; ++c) put(slot * 12 + c, PX[c], PY[c]);
+    } else {
+#pragma unroll
+      for (int c = 0; c < 12; ++c) put(slot * 12 + c, X[c], Y[c]);
+    }
     ++slot;
   }
 }
@@ -278,8 +353,12 @@ template cudaError_t launch_noneq_gen<double>(const double*, double*, int, const
 template <class T>
 cudaError_t launch_noneq(const T* f, T* out, int groups, const StepParams& p, const DvmConst<T>& d,
                          cudaStream_t s) {
-  dim3 grid((p.n_r + kNeqThreads - 1) / kNeqThreads, p.n_theta);
-  noneq_kernel<T><<<grid, kNeqThreads, 0, s>>>(f, out, groups, p, d);
+  constexpr int per = sizeof(T) == 4 ? 2 : 1;   // nodes per thread
+  const dim3 grid((p.n_r + per * kNeqThreads - 1) / (per * kNeqThreads), p.n_theta);
+  if constexpr (sizeof(T) == 4)
+    noneq_f32_kernel<<<grid, kNeqThreads, 0, s>>>(f, out, groups, p, d);
+  else
+    noneq_kernel<<<grid, kNeqThreads, 0, s>>>(f, out, groups, p, d);
   return cudaGetLastError();
 }
 

@@ -65,92 +65,21 @@ __device__ __forceinline__ int group_planes(int g) { return g == 0 ? 1 + kNDirs 
 
 __device__ __forceinline__ f2 ld2(const float* p) { return *reinterpret_cast<const float2*>(p); }
 
-// Sums over one shell (plus, optionally, a second shell added direction by
-// direction) of f, c_x f and c_y f for both nodes, with the octagon's exact
-// unit vectors as float-float constants.
-template <int K, int KADD, int PL>
-__device__ __forceinline__ void shell_sums2(const float* f, f2& S, f2& X, f2& Xl, f2& Y, f2& Yl) {
-  S = bc2(0.f); X = bc2(0.f); Xl = bc2(0.f); Y = bc2(0.f); Yl = bc2(0.f);
-#pragma unroll
-  for (int i = 0; i < kHalf; ++i) {
-    const int q = 1 + (K - 1) * kNDirs + i;
-    f2 fa = ld2(f + q * PL), fb = ld2(f + (q + kHalf) * PL);
-    if (KADD > 0) {
-      const int qa = 1 + (KADD - 1) * kNDirs + i;
-      fa = add2(fa, ld2(f + qa * PL));
-      fb = add2(fb, ld2(f + (qa + kHalf) * PL));
-    }
-    S = add2(S, add2(fa, fb));
-    const f2 dd = sub2(fa, fb);
-    if (i == 0) {
-      X = add2(X, dd);
-    } else if (i == 2) {
-      Y = add2(Y, dd);
-    } else {
-      const float sx = i == 1 ? 1.f : -1.f;
-      X = fma2(bc2(sx * kS), dd, X);
-      Xl = fma2(bc2(sx * kSl), dd, Xl);
-      Y = fma2(bc2(kS), dd, Y);
-      Yl = fma2(bc2(kSl), dd, Yl);
-    }
-  }
-}
-
-// What one group of shells adds to the moments (Eqs. 3-5) of the two nodes.
-// Groups: 0 shell 1; 1 shells 2 + 3 direction by direction, with the speed and
-// v^2/2 of shell 2; 2 shell 3 again with the differences v_3 - v_2, (v_3^2 -
-// v_2^2)/2 (S then does not enter rho); 3 shell 4.
-struct Terms2 {
-  f2 S;
-  ff2 jx, jy, e;
-};
-template <int G, int PL>
-__device__ __forceinline__ Terms2 group_terms2(const float* f, const DvmConst<float>& d) {
-  f2 S, X, Xl, Y, Yl;
-  shell_sums2<G == 0 ? 1 : (G == 1 ? 2 : (G == 2 ? 3 : 4)), G == 1 ? 3 : 0, PL>(f, S, X, Xl, Y, Yl);
-  constexpr int k = G == 0 ? 1 : (G == 1 ? 2 : 4);
-  const ff2 v = G == 2 ? ffc(d.dv23, d.dv23_lo) : ffc(d.speed[k], d.speed_lo[k]);
-  const ff2 h = G == 2 ? ffc(d.dh23, d.dh23_lo) : ffc(d.half_v2[k], d.half_v2_lo[k]);
-  return Terms2{S, ff2_mul(v, ff2{X, Xl}), ff2_mul(v, ff2{Y, Yl}), ff2_mul(h, ff2_of(S))};
-}
-
-// Adds the groups up in order and recovers velocity and temperature.
-struct Moments2 {
-  ff2 rho, jx, jy, e;
-  __device__ __forceinline__ explicit Moments2(f2 f0) : rho(ff2_of(f0)), jx(ff2_of(bc2(0.f))), jy(jx), e(jx) {}
-  template <int G>
-  __device__ __forceinline__ void add(const Terms2& t) {
-    if (G != 2) rho = ff2_add(rho, ff2_of(t.S));
-    jx = ff2_add(jx, t.jx);
-    jy = ff2_add(jy, t.jy);
-    e = ff2_add(e, t.e);
-  }
-  __device__ __forceinline__ State2 state() const {
-    State2 s;
-    const ff2 inv = ff2_recip(rho);
-    s.rho = rho;
-    s.ux = ff2_mul(jx, inv);
-    s.uy = ff2_mul(jy, inv);
-    const ff2 ke = ff2_add(ff2_mul(jx, s.ux), ff2_mul(jy, s.uy));    // |j|^2 / rho
-    s.E = ff2_mul(ff2_add(e, ff2_scale(ke, -0.5f)), inv);
-    return s;
-  }
-};
-
 // The state of the two nodes.  ready(g) is called before plane group g (the
 // rest plane and shell 1, then shells 2, 3, 4) is first read, so the sums start
 // while later groups still land.
 template <int PL, class Ready>
 __device__ __forceinline__ State2 state2(const float* f, const DvmConst<float>& d, Ready ready) {
+  auto ld = [&](int q) { return ld2(f + q * PL); };
   ready(0);
-  Moments2 m(ld2(f));
-  m.template add<0>(group_terms2<0, PL>(f, d));
+  Moments2 m(ld(0));
+  m.template add<0>(group_terms2<0>(ld, d));
   ready(1);
   ready(2);
-  m.template add<1>(group_terms2<1, PL>(f, d));
-  m.template add<2>(group_terms2<2, PL>(f, d));
+  m.template add<1>(group_terms2<1>(ld, d));
+  m.template add<2>(group_terms2<2>(ld, d));
   ready(3);
-  m.template add<3>(group_terms2<3, PL>(f, d));
+  m.template add<3>(group_terms2<3>(ld, d));
   return m.state();
 }
 
@@ -161,12 +90,13 @@ __device__ __forceinline__ State2 state2(const float* f, const DvmConst<float>& 
 template <int PL, class Ready, class Barrier>
 __device__ __forceinline__ State2 state2_split(const float* f, const DvmConst<float>& d, int split, f2* x, int pairs,
                                                int ip, Ready ready, Barrier barrier) {
+  auto ld = [&](int q) { return ld2(f + q * PL); };
   Terms2 t;
   switch (split) {
-    case 0: ready(0); t = group_terms2<0, PL>(f, d); break;
-    case 1: ready(1); ready(2); t = group_terms2<1, PL>(f, d); break;
-    case 2: ready(2); t = group_terms2<2, PL>(f, d); break;
-    default: ready(3); t = group_terms2<3, PL>(f, d); break;
+    case 0: ready(0); t = group_terms2<0>(ld, d); break;
+    case 1: ready(1); ready(2); t = group_terms2<1>(ld, d); break;
+    case 2: ready(2); t = group_terms2<2>(ld, d); break;
+    default: ready(3); t = group_terms2<3>(ld, d); break;
   }
   f2* o = x + split * 7 * pairs + ip;
   o[0] = t.S;
