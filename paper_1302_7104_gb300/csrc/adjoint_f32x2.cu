@@ -753,10 +753,11 @@ cudaError_t launch_adjoint_pairs_f32(const CUtensorMap* tmap_f, const CUtensorMa
                                      const WallScratch<float>& ws, const AdjOrder& order, const StepParams& p,
                                      const DvmConst<float>& d, cudaStream_t s) {
   static std::atomic<unsigned long long> configured{0};
-  const cudaError_t e = set_smem_once(adjoint_pair_f32x2, kASmem, configured);
+  const cudaError_t e = set_smem_once(adjoint_pair_f32x2, std::max(kASmem, kOwnSmBytes), configured);
   if (e != cudaSuccess) return e;
-  return launch_overlapped(adjoint_pair_f32x2, dim3((unsigned)order.blocks()), kAThr, kASmem, s, *tmap_f, *tmap_l,
-                           *tmap_fn, *tmap_ln, f, lam_in, lam_out, ws, order, p, d);
+  return launch_overlapped(adjoint_pair_f32x2, dim3((unsigned)order.blocks()), kAThr,
+                           adjoint_smem(kASmem, order.blocks()), s, *tmap_f, *tmap_l, *tmap_fn, *tmap_ln, f, lam_in,
+                           lam_out, ws, order, p, d);
 }
 
 }  // namespace pclb

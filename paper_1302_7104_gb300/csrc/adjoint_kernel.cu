@@ -504,10 +504,10 @@ cudaError_t launch_adjoint(const CUtensorMap* tmap_f, const CUtensorMap* tmap_l,
     auto go = [&](auto tt, auto ls) {
       constexpr int TT = decltype(tt)::value, LS = decltype(ls)::value;
       static std::atomic<unsigned long long> configured{0};
-      const cudaError_t e = set_smem_once(adjoint_pair_kernel<TT, LS>, AdjSize<TT, LS>::smem, configured);
+      const cudaError_t e = set_smem_once(adjoint_pair_kernel<TT, LS>, std::max(AdjSize<TT, LS>::smem, kOwnSmBytes), configured);
       if (e != cudaSuccess) return e;
       return launch_overlapped(adjoint_pair_kernel<TT, LS>, dim3((unsigned)order.blocks()), AdjSize<TT, LS>::threads,
-                               AdjSize<TT, LS>::smem, stream, *tmap_f, *tmap_l, f, lam_in, lam_out, ws, order, p, d);
+                               adjoint_smem(AdjSize<TT, LS>::smem, order.blocks()), stream, *tmap_f, *tmap_l, f, lam_in, lam_out, ws, order, p, d);
     };
     if (rows == kAdjRows64) return go(std::integral_constant<int, kAdjRows64>{}, std::integral_constant<int, 1>{});
     return go(std::integral_constant<int, kAdjRows64Small>{}, std::integral_constant<int, 2>{});
