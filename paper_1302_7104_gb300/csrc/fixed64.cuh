@@ -14,6 +14,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "device_common.cuh"
+
 namespace pclb {
 
 // Exponents for which fx_to_double stays inside the normal range; NaN and
@@ -71,6 +73,11 @@ __device__ __forceinline__ uint64_t fx_abs(int64_t x) {
 }
 __device__ __forceinline__ int64_t fx_signed(uint64_t a, int64_t s) { return ((int64_t)a ^ s) - s; }   // s: 0 or -1
 
+// x / sqrt 2 for |x| < 2^61.
+__device__ __forceinline__ int64_t fx_diagonal(int64_t x) {
+  return fx_signed(fx_mul(fx_abs(x), 0x5a827999fcef3242ull), x >> 63);   // 2^63 / sqrt 2
+}
+
 __device__ __forceinline__ float fx_float(uint64_t u) {
   return fmaf(__uint2float_rn((uint32_t)(u >> 32)), 4294967296.0f, __uint2float_rn((uint32_t)u));
 }
@@ -114,6 +121,43 @@ __device__ __forceinline__ int64_t fx_mwb(int64_t D, int64_t Dp, const FxCourant
   const int32_t i1 = __float2int_rn(fmaf(c.k2, q, c.klo * v0));             // units of 2^-52
   const uint64_t coef = c.a2 + c.k40 * (uint64_t)i0 + (uint64_t)((int64_t)i1 * 2048);
   return fx_signed(fx_mul(a, coef), s);
+}
+
+// Largest biased exponent of the values, and whether fixed point with that
+// exponent stays clear of the ends of the double range (NaN and infinity do not).
+__device__ __forceinline__ int fx_exponent(int h0) { return (h0 >> 20) & 0x7ff; }
+template <class... H>
+__device__ __forceinline__ int fx_exponent(int h0, int h1, H... rest) {
+  return fx_exponent(max(h0 & 0x7fffffff, h1 & 0x7fffffff), rest...);
+}
+__device__ __forceinline__ bool fx_range(int e) { return e >= kFxMinExp && e <= kFxMaxExp; }
+
+// |D| (D - Dp) / (|D| + |Dp|) in FP64, small differences scaled up by a power of two.
+__device__ __forceinline__ double limiter64(double D, double Dp) {
+  const bool small = fmax(fabs(D), fabs(Dp)) < 0x1p-500;
+  if (small) { D *= 0x1p+500; Dp *= 0x1p+500; }
+  const double den = fabs(D) + fabs(Dp);
+  const double v = den >= 0x1p-1000 ? fabs(D) * recip_newton1(den) * (D - Dp) : 0.0;
+  return small ? v * 0x1p-500 : v;
+}
+
+// d x0 - M_r - M_theta of one label (Eqs. 19, 28): x0 the node, u1, u2 and v1, v2
+// its upwind neighbours in r and theta.  In fixed point on the exponent of the
+// largest of the five, or in FP64 outside its range (c: the pair's FP64 Courant
+// entry at the row).
+__device__ __forceinline__ double fx_carried(double x0, double u1, double u2, double v1, double v2, const FxCourant& cr,
+                                             const FxCourant& ct, uint64_t dfx, int64_t dsign, double decay,
+                                             const double* c, double inv_r) {
+  const int e = fx_exponent(__double2hiint(x0), __double2hiint(u1), __double2hiint(u2), __double2hiint(v1),
+                            __double2hiint(v2));
+  if (!fx_range(e)) {
+    const double D = x0 - u1, Dt = x0 - v1, at = c[2] * inv_r, kt = at - at * at;
+    return decay * x0 - c[0] * D - c[1] * limiter64(D, u1 - u2) - at * Dt - kt * limiter64(Dt, v1 - v2);
+  }
+  const int64_t x = fx_from_double(x0, e), a = fx_from_double(u1, e), b = fx_from_double(v1, e);
+  const int64_t keep = fx_signed(fx_mul(fx_abs(x), dfx), (x >> 63) ^ dsign);
+  return fx_to_double(keep - fx_mwb(x - a, a - fx_from_double(u2, e), cr) - fx_mwb(x - b, b - fx_from_double(v2, e), ct),
+                      e);
 }
 
 // A fraction (units of 2^-63) as a double.

@@ -29,9 +29,13 @@ constexpr int kTileT32 = 16;
 constexpr int kStepThreads32 = 16 * kTileT32;
 constexpr int kCtasPerSm32 = 2;
 // The octagon's steps on small grids: tiles of kTileTSmall rows on at most
-// kSmallGridTiles tiles of 32 x 16, in FP64 of two rows on at most kTinyGridTiles64.
+// kSmallGridTiles tiles of 32 x 16 (two waves of the 152 SMs), in FP64 of two
+// rows on at most kTinyGridTiles64 (one wave).  FP64, us per step with tiles
+// of 2 / 4 / 16 rows: 64 x 128 (16 tiles) 15.1 / 22.3 / 52.4, 64 x 256 (32)
+// 30.0 / 22.5 / 52.6, 128 x 304 (76) 59.6 / 44.5 / 52.6, 128 x 608 (152)
+// 112 / 88.6 / 53.6.
 constexpr int kTileTSmall = 4;
-constexpr int kSmallGridTiles = 76, kTinyGridTiles64 = 8;
+constexpr int kSmallGridTiles = 76, kTinyGridTiles64 = 19;
 constexpr int kWinR = kTileR + 8;   // 40 columns
 constexpr int kWinT = kTileT + 4;   // 20 rows
 constexpr int kLeft = 4;            // column of interior r0 inside the window

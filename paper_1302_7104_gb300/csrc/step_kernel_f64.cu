@@ -9,9 +9,9 @@
 // pipes; FP64 keeps the node state, the equilibrium factors and the final
 // sums (~7 operations per update), so results keep double precision.
 //
-// Tile work (one CTA, 512 threads; kTileR x TT nodes, 16 / TT warps per row):
+// Tile work (one CTA, 512 threads; kTileR x kTileT nodes, one per thread):
 //   1. one thread issues 33 TMA box copies (one per velocity plane) of the
-//      window [r0-4, r0+36) x [t0-2, t0+TT+2) into shared memory;
+//      window [r0-4, r0+36) x [t0-2, t0+18) into shared memory;
 //   2. tiles at a wall form the radial ghost columns in the window, in FP64
 //      (ghost_cols.cuh);
 //   3. the block finds the largest exponent of each shell's planes and
@@ -26,9 +26,7 @@
 // largest value (the fixed-point unit would be coarse for them) is loaded
 // again and evaluated in FP64 throughout.
 //
-// TT = 16: one thread per node, for grids that fill the chip with such tiles.
-// TT = 4 or 2: the shells of a row on four warps, or half shells on eight, for
-// small grids, where the time of one tile is the time of the step.
+// Grids that do not fill the chip with such tiles run step_small_f64.cu.
 // Consecutive steps overlap their set-up (programmatic dependent launch).
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -53,17 +51,11 @@ struct FxTab {
   int fl, pad;      // bit 0: v_r < 0, bit 1: v_theta < 0 for the first label of the pair
 };
 
-template <int TT>
 struct FxSize {
-  static constexpr int split = 16 / TT;                       // warps per row: 1, 4 or 8
-  static constexpr int dirs = split <= 4 ? kHalfDirs : 4 * kHalfDirs / split;   // direction pairs of a shell per warp
-  static constexpr int plane = kWinR * (TT + 4);
+  static constexpr int plane = kWinR * (kTileT + 4);
   static constexpr int planes_bytes = kQ * plane * 8;
-  static constexpr int tab_bytes = kPairsFx * TT * (int)sizeof(FxTab);
-  static constexpr int ghost_bytes = kGhostScratch64<TT> * 8;
-  // split > 1: per node the shells' sums (S, X, Y), then w_1..4, a0, a1, u/E; split 8: the second halves' sums too
-  static constexpr int node_bytes = split > 1 ? 32 * TT * (split > 4 ? 24 : 12) * 8 : 0;
-  static constexpr int scratch = ghost_bytes > node_bytes ? ghost_bytes : node_bytes;
+  static constexpr int tab_bytes = kPairsFx * kTileT * (int)sizeof(FxTab);
+  static constexpr int scratch = kGhostScratch64<kTileT> * 8;
   static constexpr int smem = planes_bytes + tab_bytes + scratch + 128;
   static_assert((plane * 8) % 128 == 0, "TMA destinations must stay 128-byte aligned");
   static_assert(smem <= 232448, "shared memory of one CTA");
@@ -85,20 +77,12 @@ __device__ __noinline__ void general_node(const double* w, const EqParams<double
     const double ev = eq.a0 + x2 * (eq.a1h + x2 * (1.0 / 24.0)), od = x * (eq.a1 + x2 * (1.0 / 6.0));
     const double wd = omd * eq.w[k];
     auto mwb = [&](const double* fp, double P, int s_r, int s_t) {
-      // |D| (D - Dp) / (|D| + |Dp|), small differences scaled up by a power of two
-      auto h = [](double D, double Dp) {
-        const bool small = fmax(fabs(D), fabs(Dp)) < 0x1p-500;
-        if (small) { D *= 0x1p+500; Dp *= 0x1p+500; }
-        const double den = fabs(D) + fabs(Dp);
-        const double v = den >= 0x1p-1000 ? fabs(D) * recip_newton1(den) * (D - Dp) : 0.0;
-        return small ? v * 0x1p-500 : v;
-      };
       const double f0 = fp[0], u1 = fp[s_r], v1 = fp[s_t], Dr = f0 - u1, Dt = f0 - v1;
       double o = fma(wd, P, decay * f0);
       o = fma(-ar, Dr, o);
-      o = fma(-kr, h(Dr, u1 - fp[2 * s_r]), o);
+      o = fma(-kr, limiter64(Dr, u1 - fp[2 * s_r]), o);
       o = fma(-at, Dt, o);
-      return fma(-kt, h(Dt, v1 - fp[2 * s_t]), o);
+      return fma(-kt, limiter64(Dt, v1 - fp[2 * s_t]), o);
     };
     store(q1, mwb(w + (size_t)q1 * PLANE, ev + od, sr, st));
     store(q2, mwb(w + (size_t)q2 * PLANE, ev - od, -sr, -st));
@@ -107,12 +91,11 @@ __device__ __noinline__ void general_node(const double* w, const EqParams<double
 
 }  // namespace
 
-template <int TT>
 __global__ void __launch_bounds__(kThreadsFx, 1)
     step_kernel_f64(const __grid_constant__ CUtensorMap tmap_in, double* __restrict__ f_out,
                     const __grid_constant__ StepParams p, const __grid_constant__ DvmConst<double> d, int ty0) {
-  using SZ = FxSize<TT>;
-  constexpr int PLANE = SZ::plane, SPLIT = SZ::split;
+  using SZ = FxSize;
+  constexpr int PLANE = SZ::plane, TT = kTileT;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   double* sm = reinterpret_cast<double*>(smem_raw);
   int64_t* fx = reinterpret_cast<int64_t*>(smem_raw);
@@ -202,100 +185,39 @@ __global__ void __launch_bounds__(kThreadsFx, 1)
   __syncthreads();
 
   // ---- the node state and the equilibrium factors ------------------------------
-  const int rl = warp % TT, split = warp / TT;   // tile row; the shells of this warp
+  const int rl = warp;   // tile row
   const int r = r0 + lane, t = t0 + rl;
   const int node = (rl + 2) * kWinR + kLeft + lane;
   const bool valid = r < p.n_r && t < p.n_theta;
   const double decay = p.decay, omd = 1.0 - decay;
   EqParams<double> eq;
   double f0 = 0.0;
-  // this warp's shells and direction pairs
-  constexpr int DIRS = SZ::dirs;
-  const int k_first = SPLIT == 1 ? 1 : split / (SPLIT / 4) + 1, k_last = SPLIT == 1 ? 4 : k_first;
-  const int i_first = SPLIT > 4 ? (split & 1) * DIRS : 0;
   auto shell_exp = [&](int k) { return k == 1 ? ek[1] : (k == 2 ? ek[2] : (k == 3 ? ek[3] : ek[4])); };
-  // the sums S, X = sum c_x f, Y over those direction pairs of shell k
-  auto shell_sums = [&](int k, int64_t o[3]) {
-    const int64_t* f = fx + (1 + (k - 1) * kNDirs + i_first) * PLANE + node;
-    int64_t S = 0, D[DIRS];
+  if (!general) {
+    f0 = fx_to_double(fx[node], ek[0]);
+    double s0 = f0, sx = 0.0, sy = 0.0, se = 0.0;
+#pragma unroll 1
+    for (int k = 1; k <= 4; ++k) {   // S, X = sum c_x f, Y: directions (1,0), (s,s), (0,1), (-s,s)
+      const int64_t* f = fx + (1 + (k - 1) * kNDirs) * PLANE + node;
+      int64_t S = 0, D[kHalfDirs];
 #pragma unroll
-    for (int i = 0; i < DIRS; ++i) {
-      const int64_t a = f[i * PLANE], b = f[(i + kHalfDirs) * PLANE];
-      S += a + b;
-      D[i] = a - b;
+      for (int i = 0; i < kHalfDirs; ++i) {
+        const int64_t a = f[i * PLANE], b = f[(i + kHalfDirs) * PLANE];
+        S += a + b;
+        D[i] = a - b;
+      }
+      const int e = shell_exp(k);
+      const double Sd = fx_to_double(S, e);
+      s0 += Sd;
+      sx = fma(d.speed[k], fx_to_double(D[0] + fx_diagonal(D[1] - D[3]), e), sx);
+      sy = fma(d.speed[k], fx_to_double(D[2] + fx_diagonal(D[1] + D[3]), e), sy);
+      se = fma(d.half_v2[k], Sd, se);
     }
-    // x / sqrt 2 (the fraction in units of 2^-63)
-    auto diagonal = [](int64_t x) { return fx_signed(fx_mul(fx_abs(x), 0x5a827999fcef3242ull), x >> 63); };
-    o[0] = S;
-    if constexpr (DIRS == 4) {   // directions (1,0), (s,s), (0,1), (-s,s)
-      o[1] = D[0] + diagonal(D[1] - D[3]);
-      o[2] = D[2] + diagonal(D[1] + D[3]);
-    } else {
-      const int64_t g = diagonal(D[1]);
-      o[1] = i_first == 0 ? D[0] + g : -g;
-      o[2] = i_first == 0 ? g : D[0] + g;
-    }
-  };
-  // factors of (1 - d) f^eq: w_k = (1 - d) rho F_k
-  auto factors = [&](const NodeState<double>& m) {
+    // factors of (1 - d) f^eq: w_k = (1 - d) rho F_k
+    const NodeState<double> m = node_state64(s0, sx, sy, se);
     eq = valid ? eq_params<double>(omd * m.rho, m.ux, m.uy, m.E, d) : eq_params<double>(1.0, 0.0, 0.0, 1.0, d);
     // not physical, or more than 2^8 below the window's largest value: too coarse a unit
     if (valid && !(m.ok && __double2hiint(m.rho) >= most - (8 << 20))) general = true;
-  };
-  if constexpr (SPLIT == 1) {
-    if (!general) {
-      f0 = fx_to_double(fx[node], ek[0]);
-      double s0 = f0, sx = 0.0, sy = 0.0, se = 0.0;
-#pragma unroll 1
-      for (int k = 1; k <= 4; ++k) {
-        int64_t s[3];
-        shell_sums(k, s);
-        const int e = shell_exp(k);
-        const double S = fx_to_double(s[0], e);
-        s0 += S;
-        sx = fma(d.speed[k], fx_to_double(s[1], e), sx);
-        sy = fma(d.speed[k], fx_to_double(s[2], e), sy);
-        se = fma(d.half_v2[k], S, se);
-      }
-      factors(node_state64(s0, sx, sy, se));
-    }
-  } else {
-    // this warp's part of the sums, the state by the row's first warp
-    double* part = scratch + (rl * 32 + lane) * 12;
-    int64_t s[3];
-    if (!general) shell_sums(k_first, s);
-    if constexpr (SPLIT > 4) {   // the halves of a shell
-      int64_t* second = reinterpret_cast<int64_t*>(scratch + 32 * TT * 12) + (rl * 32 + lane) * 12 + 3 * (k_first - 1);
-      if (!general && i_first != 0)
-        for (int j = 0; j < 3; ++j) second[j] = s[j];
-      __syncthreads();
-      if (!general && i_first == 0)
-        for (int j = 0; j < 3; ++j) s[j] += second[j];
-    }
-    if (!general && i_first == 0)
-      for (int j = 0; j < 3; ++j) part[3 * (k_first - 1) + j] = fx_to_double(s[j], shell_exp(k_first));
-    __syncthreads();
-    if (!general && split == 0) {
-      f0 = fx_to_double(fx[node], ek[0]);
-      double s0 = f0, sx = 0.0, sy = 0.0, se = 0.0;
-#pragma unroll
-      for (int k = 1; k <= 4; ++k) {
-        s0 += part[3 * (k - 1)];
-        sx = fma(d.speed[k], part[3 * (k - 1) + 1], sx);
-        sy = fma(d.speed[k], part[3 * (k - 1) + 2], sy);
-        se = fma(d.half_v2[k], part[3 * (k - 1)], se);
-      }
-      factors(node_state64(s0, sx, sy, se));
-#pragma unroll
-      for (int k = 1; k <= 4; ++k) part[k - 1] = eq.w[k];
-      part[4] = eq.a0; part[5] = eq.a1; part[6] = eq.uxE; part[7] = eq.uyE;
-    }
-    __syncthreads();
-    if (!general && split > 0) {
-#pragma unroll
-      for (int k = 1; k <= 4; ++k) eq.w[k] = part[k - 1];
-      eq.a0 = part[4]; eq.a1 = part[5]; eq.uxE = part[6]; eq.uyE = part[7];
-    }
   }
   general = __syncthreads_or(general);
 
@@ -316,7 +238,7 @@ __global__ void __launch_bounds__(kThreadsFx, 1)
     }
     if (!wait(&bar[1])) return;
     if (wall_tile) ghost_columns_f64<TT, PLANE>(sm, scratch, r0, t0, p, d);
-    if (split != 0 || !valid) return;
+    if (!valid) return;
     const NodeState<double> m = node_moments(sm + node, PLANE, d);
     if (!m.ok) atomicOr(p.status, PCLB_FLAG_NONPHYS);
     eq = eq_params<double>(m.rho, m.ux, m.uy, m.E, d);
@@ -326,7 +248,7 @@ __global__ void __launch_bounds__(kThreadsFx, 1)
     return;
   }
   if (!valid) return;
-  if (split == 0) store(0, fma(decay, f0, eq.w[0] * eq.a0));   // rest velocity: no convection
+  store(0, fma(decay, f0, eq.w[0] * eq.a0));   // rest velocity: no convection
   const uint64_t dfx = fx_fraction(fabs(decay));
   const int64_t dsign = decay < 0.0 ? -1 : 0;
   const uint64_t ratio = fx_fraction(p.inv_r[r] * recip_newton(inv_r0));   // 1/r relative to the tile's first column
@@ -337,13 +259,13 @@ __global__ void __launch_bounds__(kThreadsFx, 1)
   int q_last = 0;
   double o1, o2;
 #pragma unroll 1
-  for (int k = k_first; k <= k_last; ++k) {
+  for (int k = 1; k <= 4; ++k) {
     const int e = shell_exp(k);
     // (1 - d) f^eq of the shell's pairs: ev +- od, ev = A + y^2 (B + y^2 C), od = y (O1 + y^2 O3)
     const double w = k == 1 ? eq.w[1] : (k == 2 ? eq.w[2] : (k == 3 ? eq.w[3] : eq.w[4])), wa = w * eq.a1;
     const double A = w * eq.a0, B = wa * d.half_v2[k], C = w * d.v4_24[k], O1 = wa * d.speed[k], O3 = w * d.v3_6[k];
 #pragma unroll 1
-    for (int i = i_first; i < i_first + DIRS; ++i) {
+    for (int i = 0; i < kHalfDirs; ++i) {
       const int q1 = 1 + (k - 1) * kNDirs + i, q2 = q1 + kHalfDirs;
       const double y = i == 0 ? eq.uxE : (i == 1 ? y1 : (i == 2 ? eq.uyE : y3)), y2 = y * y;
       const double ev = fma(y2, fma(y2, C, B), A), z = fma(y2, O3, O1);
@@ -372,27 +294,21 @@ __global__ void __launch_bounds__(kThreadsFx, 1)
   store(q_last + kHalfDirs, o2);
 }
 
-template <int TT>
-static cudaError_t launch_tile_rows(const CUtensorMap* tmap_in, double* f_out, const StepParams& p,
-                                    const DvmConst<double>& d, cudaStream_t stream, int ty_begin, int ty_end) {
-  static std::atomic<unsigned long long> configured{0};   // per instantiation and device
-  const cudaError_t e = set_smem_once(step_kernel_f64<TT>, FxSize<TT>::smem, configured);
-  if (e != cudaSuccess) return e;
-  const dim3 grid((p.n_r + kTileR - 1) / kTileR, ty_end - ty_begin);
-  return launch_overlapped(step_kernel_f64<TT>, grid, kThreadsFx, FxSize<TT>::smem, stream, *tmap_in, f_out, p, d,
-                           ty_begin);
-}
+cudaError_t launch_step_small_f64(const CUtensorMap*, double*, const StepParams&, const DvmConst<double>&, cudaStream_t,
+                                  int, int);
 
 // Tile rows [ty_begin, ty_end) of kTileT nodes each.
 cudaError_t launch_step_f64_mwb(const CUtensorMap* tmap_in, double* f_out, const StepParams& p,
                                 const DvmConst<double>& d, cudaStream_t stream, int ty_begin, int ty_end) {
-  const int per = kTileT / p.tile_rows, last = (p.n_theta + p.tile_rows - 1) / p.tile_rows;
-  const int b = ty_begin * per, e = ty_end * per < last ? ty_end * per : last;
-  switch (p.tile_rows) {
-    case 2: return launch_tile_rows<2>(tmap_in, f_out, p, d, stream, b, e);
-    case 4: return launch_tile_rows<4>(tmap_in, f_out, p, d, stream, b, e);
-    default: return launch_tile_rows<kTileT>(tmap_in, f_out, p, d, stream, b, e);
+  if (p.tile_rows != kTileT) {
+    const int per = kTileT / p.tile_rows, last = (p.n_theta + p.tile_rows - 1) / p.tile_rows;
+    return launch_step_small_f64(tmap_in, f_out, p, d, stream, ty_begin * per, std::min(ty_end * per, last));
   }
+  static std::atomic<unsigned long long> configured{0};   // per device
+  const cudaError_t e = set_smem_once(step_kernel_f64, FxSize::smem, configured);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((p.n_r + kTileR - 1) / kTileR, ty_end - ty_begin);
+  return launch_overlapped(step_kernel_f64, grid, kThreadsFx, FxSize::smem, stream, *tmap_in, f_out, p, d, ty_begin);
 }
 
 }  // namespace pclb

@@ -94,3 +94,30 @@ def test_zero_planes_and_equal_neighbours():
     got, _ = _step(w, f)
     want = O.run(w, f, 1)
     assert np.max(np.abs(got - want)) <= 1e-12 * np.max(np.abs(want))
+
+
+# Tiles of 2 rows on at most 19 tiles of 32 x 16, of 4 rows up to 76: both
+# sides of that line, last tiles of one to three columns (the wall node or its
+# neighbour in another tile's columns) and of one row
+@pytest.mark.parametrize("n_r,n_t", [(32, 304), (32, 305), (608, 16), (609, 17), (33, 301), (34, 303), (35, 302), (3, 307)])
+@pytest.mark.parametrize("bc", [(I.BC_EXTRAP, I.BC_EXTRAP), (I.BC_WALL | I.BC_NEQ, I.BC_DIRICHLET | I.BC_NEQ)])
+def test_small_tiles_match_oracle(n_r, n_t, bc):
+    w = I.random_smooth(n_r, n_t, seed=n_r + n_t, bc_kind=bc, amp=0.02 if n_r < 8 else 0.2)
+    f = _noisy(w)
+    got, _ = _step(w, f, 2)
+    want = O.run(w, f, 2)
+    assert np.max(np.abs(got - want)) <= 2e-12 * np.max(np.abs(want))
+
+
+@pytest.mark.parametrize("ratio,scale", [(300.0, 2.0 ** -1000), (300.0, 1.0), (300.0, 2.0 ** 1000), (1e12, 1.0),
+                                         (1e12, 2.0 ** 1000)])
+def test_tiles_of_four_rows_outside_fixed_point(ratio, scale):
+    w = _contrast(I.random_smooth(64, 400, seed=8), ratio)
+    f = _noisy(w)
+    got, flags = _step(w, f * scale)
+    want = O.run(w, f, 1)
+    assert flags == 0
+    thin = np.s_[:, :, 20:32]
+    got = got / scale
+    assert np.max(np.abs(got - want)) <= 1e-12 * np.max(np.abs(want))
+    assert np.max(np.abs(got[thin] - want[thin])) <= 1e-12 * np.max(np.abs(want[thin]))
