@@ -14,7 +14,10 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "device_common.cuh"
+#include "pclb_internal.h"
 
 namespace pclb {
 
@@ -141,23 +144,64 @@ __device__ __forceinline__ double limiter64(double D, double Dp) {
   return small ? v * 0x1p-500 : v;
 }
 
-// d x0 - M_r - M_theta of one label (Eqs. 19, 28): x0 the node, u1, u2 and v1, v2
-// its upwind neighbours in r and theta.  In fixed point on the exponent of the
-// largest of the five, or in FP64 outside its range (c: the pair's FP64 Courant
-// entry at the row).
-__device__ __forceinline__ double fx_carried(double x0, double u1, double u2, double v1, double v2, const FxCourant& cr,
-                                             const FxCourant& ct, uint64_t dfx, int64_t dsign, double decay,
-                                             const double* c, double inv_r) {
+// The compared schemes (Sec. II B 3) in upwind form: M = alpha D + c ((D' or D)
+// - (D or Dp)), c = alpha (1 - alpha) / 2 (Warming-Beam, Lax-Wendroff) or alpha / 2
+// (second-order upwind), D' = f(downwind) - f of Lax-Wendroff.
+struct FxLinear {
+  uint64_t a, c;   // units of 2^-63
+};
+template <int SCH>
+using FxCoef = std::conditional_t<SCH == PCLB_SCHEME_MWB, FxCourant, FxLinear>;
+
+template <int SCH>
+__device__ __forceinline__ FxCoef<SCH> fx_coef(uint64_t alpha) {
+  if constexpr (SCH == PCLB_SCHEME_MWB) return fx_courant(alpha);
+  else return FxLinear{alpha, (SCH == PCLB_SCHEME_UPWIND2 ? alpha : alpha - fx_mul_frac(alpha, alpha)) >> 1};
+}
+
+// M of node value x0, upwind values u1, u2 and (Lax-Wendroff) downwind value d1,
+// all below 2^59.
+template <int SCH>
+__device__ __forceinline__ int64_t fx_increment(int64_t x0, int64_t u1, int64_t u2, int64_t d1, const FxCoef<SCH>& c) {
+  const int64_t D = x0 - u1;
+  if constexpr (SCH == PCLB_SCHEME_MWB) {
+    return fx_mwb(D, u1 - u2, c);
+  } else {
+    const int64_t E = SCH == PCLB_SCHEME_LW ? d1 - x0 - D : D - (u1 - u2);
+    return fx_signed(fx_mul(fx_abs(D), c.a), D >> 63) + fx_signed(fx_mul(fx_abs(E), c.c), E >> 63);
+  }
+}
+
+// The same in FP64; a = |C|, K = |C| (1 - |C|).
+template <int SCH>
+__device__ __forceinline__ double increment64(double a, double K, double x0, double u1, double u2, double d1) {
+  const double D = x0 - u1, Dp = u1 - u2;
+  if (SCH == PCLB_SCHEME_MWB) return fma(a, D, K * limiter64(D, Dp));
+  if (SCH == PCLB_SCHEME_LW) return a * D + 0.5 * K * ((d1 - x0) - D);
+  return a * D + 0.5 * (SCH == PCLB_SCHEME_WB ? K : a) * (D - Dp);
+}
+
+// d x0 - M_r - M_theta of one label (Eqs. 19, 28): x0 the node, u1 and v1 its
+// upwind neighbours in r and theta, u2 and v2 the next ones (Lax-Wendroff: the
+// downwind neighbours).  In fixed point on the exponent of the largest of
+// them, or in FP64 outside its range (c: the pair's FP64 Courant entry at the row).
+template <int SCH>
+__device__ __forceinline__ double fx_carried(double x0, double u1, double u2, double v1, double v2,
+                                             const FxCoef<SCH>& cr, const FxCoef<SCH>& ct, uint64_t dfx, int64_t dsign,
+                                             double decay, const double* c, double inv_r) {
   const int e = fx_exponent(__double2hiint(x0), __double2hiint(u1), __double2hiint(u2), __double2hiint(v1),
                             __double2hiint(v2));
   if (!fx_range(e)) {
-    const double D = x0 - u1, Dt = x0 - v1, at = c[2] * inv_r, kt = at - at * at;
-    return decay * x0 - c[0] * D - c[1] * limiter64(D, u1 - u2) - at * Dt - kt * limiter64(Dt, v1 - v2);
+    const double at = c[2] * inv_r;
+    return decay * x0 - increment64<SCH>(c[0], c[1], x0, u1, u2, u2) - increment64<SCH>(at, at - at * at, x0, v1, v2, v2);
   }
-  const int64_t x = fx_from_double(x0, e), a = fx_from_double(u1, e), b = fx_from_double(v1, e);
-  const int64_t keep = fx_signed(fx_mul(fx_abs(x), dfx), (x >> 63) ^ dsign);
-  return fx_to_double(keep - fx_mwb(x - a, a - fx_from_double(u2, e), cr) - fx_mwb(x - b, b - fx_from_double(v2, e), ct),
-                      e);
+  const int64_t i0 = fx_from_double(x0, e);
+  auto M = [&](double n1, double n2, const FxCoef<SCH>& k) {
+    const int64_t f = fx_from_double(n2, e);
+    return fx_increment<SCH>(i0, fx_from_double(n1, e), f, f, k);
+  };
+  const int64_t keep = fx_signed(fx_mul(fx_abs(i0), dfx), (i0 >> 63) ^ dsign);
+  return fx_to_double(keep - M(u1, u2, cr) - M(v1, v2, ct), e);
 }
 
 // A fraction (units of 2^-63) as a double.

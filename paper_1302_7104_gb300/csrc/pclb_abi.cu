@@ -335,16 +335,10 @@ int step_tile_rows(const pclb_grid* g, const pclb_dvm* d, pclb_precision prec) {
   return prec == PCLB_FP64 && tiles <= kTinyGridTiles64 ? 2 : kTileTSmall;
 }
 
-// Window rows of the step's TMA boxes (in FP64 the small tiles are the MWB
-// step's only, the other schemes run 16-row tiles).
-int step_box_rows(const pclb_ctx* ctx) {
-  return (ctx->prec == PCLB_FP32 || ctx->scheme == PCLB_SCHEME_MWB ? ctx->sp.tile_rows : kTileT) + 4;
-}
-
-// Both f buffers' descriptors for the current scheme.
+// Both f buffers' descriptors.
 pclb_status make_tmaps(pclb_ctx* ctx) {
   for (int w = 0; w < 2; ++w) {
-    const pclb_status st = encode_map(ctx, ctx->ws + ctx->lay.f[w], step_box_rows(ctx), &ctx->tmap[w]);
+    const pclb_status st = encode_map(ctx, ctx->ws + ctx->lay.f[w], ctx->sp.tile_rows + 4, &ctx->tmap[w]);
     if (st != PCLB_OK) return st;
   }
   return PCLB_OK;
@@ -968,7 +962,7 @@ pclb_status pclb_step_states(pclb_ctx* ctx, const void* f_from, void* f_to) {
                             ctx->stream);
   } else {
     CUtensorMap map;
-    pclb_status st = encode_map(ctx, f_from, step_box_rows(ctx), &map);
+    pclb_status st = encode_map(ctx, f_from, ctx->sp.tile_rows + 4, &map);
     if (st != PCLB_OK) return st;
     e = ctx->prec == PCLB_FP32 ? launch_step_f32(&map, (float*)f_to, ctx->sp, ctx->dvm32, ctx->stream)
                                : launch_step<double>(&map, (double*)f_to, ctx->sp, ctx->dvm64, ctx->stream);
@@ -1236,7 +1230,7 @@ pclb_status pclb_set_scheme(pclb_ctx* ctx, int32_t scheme, int32_t relaxation) {
   ctx->relaxation = relaxation;
   ctx->sp.scheme = scheme;
   ctx->sp.decay = relaxation == PCLB_RELAX_EULER ? 1.0 - ctx->dt / ctx->tau : std::exp(-ctx->dt / ctx->tau);
-  return make_tmaps(ctx);   // the FP64 schemes differ in their tiles
+  return PCLB_OK;
 }
 
 pclb_status pclb_set_wait_limit(pclb_ctx* ctx, uint64_t limit_ns) {

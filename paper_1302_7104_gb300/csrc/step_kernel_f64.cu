@@ -1,5 +1,5 @@
-// Fused FP64 time step (Eq. 38 with the MWB increments of Eq. 28): one launch
-// advances every node.  The other convection schemes run step_kernel.cu.
+// Fused FP64 time step (Eq. 38 with the MWB increments of Eq. 28 or those of
+// the compared schemes): one launch advances every node.
 //
 // What bounds it: FP64 issue.  A quarter SM starts one warp-wide FP64
 // operation per 64-76 cycles (measured), so the ~34 FP64 operations per update
@@ -45,16 +45,18 @@ constexpr int kPairsFx = 4 * kNDirs / 2;   // pairs of opposite velocities
 constexpr int kHalfDirs = kNDirs / 2;
 constexpr int kGroupsFx = 5;               // exponent groups: the rest plane and the four shells
 
+template <int SCH>
 struct FxTab {
-  FxCourant r;      // radial
+  FxCoef<SCH> r;    // radial
   uint64_t at;      // |C_theta| at the tile's first column, units 2^-63
   int fl, pad;      // bit 0: v_r < 0, bit 1: v_theta < 0 for the first label of the pair
 };
 
+template <int SCH>
 struct FxSize {
   static constexpr int plane = kWinR * (kTileT + 4);
   static constexpr int planes_bytes = kQ * plane * 8;
-  static constexpr int tab_bytes = kPairsFx * kTileT * (int)sizeof(FxTab);
+  static constexpr int tab_bytes = kPairsFx * kTileT * (int)sizeof(FxTab<SCH>);
   static constexpr int scratch = kGhostScratch64<kTileT> * 8;
   static constexpr int smem = planes_bytes + tab_bytes + scratch + 128;
   static_assert((plane * 8) % 128 == 0, "TMA destinations must stay 128-byte aligned");
@@ -63,7 +65,7 @@ struct FxSize {
 
 // The pairs of one node in FP64 throughout, for the tiles described above: w
 // the node in the window (doubles), planes PLANE apart.
-template <int PLANE, class Store>
+template <int SCH, int PLANE, class Store>
 __device__ __noinline__ void general_node(const double* w, const EqParams<double>& eq, const double* courant, double inv_r,
                                           double decay, const DvmConst<double>& d, Store store) {
   const double omd = 1.0 - decay;
@@ -71,35 +73,33 @@ __device__ __noinline__ void general_node(const double* w, const EqParams<double
   for (int pair = 0; pair < kPairsFx; ++pair) {
     const int k = 1 + pair / kHalfDirs, q1 = 1 + (k - 1) * kNDirs + pair % kHalfDirs, q2 = q1 + kHalfDirs;
     const double* e = courant + pair * 4;
-    const double ar = e[0], kr = e[1], at = e[2] * inv_r, kt = at - at * at;
+    const double at = e[2] * inv_r, kt = at - at * at;
     const int fl = (int)e[3], sr = (fl & 1) ? 1 : -1, st = (fl & 2) ? kWinR : -kWinR;
     const double x = d.vx[q1] * eq.uxE + d.vy[q1] * eq.uyE, x2 = x * x;
     const double ev = eq.a0 + x2 * (eq.a1h + x2 * (1.0 / 24.0)), od = x * (eq.a1 + x2 * (1.0 / 6.0));
     const double wd = omd * eq.w[k];
-    auto mwb = [&](const double* fp, double P, int s_r, int s_t) {
-      const double f0 = fp[0], u1 = fp[s_r], v1 = fp[s_t], Dr = f0 - u1, Dt = f0 - v1;
-      double o = fma(wd, P, decay * f0);
-      o = fma(-ar, Dr, o);
-      o = fma(-kr, limiter64(Dr, u1 - fp[2 * s_r]), o);
-      o = fma(-at, Dt, o);
-      return fma(-kt, limiter64(Dt, v1 - fp[2 * s_t]), o);
+    auto value = [&](const double* fp, double P, int s_r, int s_t) {
+      const double o = fma(wd, P, decay * fp[0]);
+      return o - increment64<SCH>(e[0], e[1], fp[0], fp[s_r], fp[2 * s_r], fp[-s_r]) -
+             increment64<SCH>(at, kt, fp[0], fp[s_t], fp[2 * s_t], fp[-s_t]);
     };
-    store(q1, mwb(w + (size_t)q1 * PLANE, ev + od, sr, st));
-    store(q2, mwb(w + (size_t)q2 * PLANE, ev - od, -sr, -st));
+    store(q1, value(w + (size_t)q1 * PLANE, ev + od, sr, st));
+    store(q2, value(w + (size_t)q2 * PLANE, ev - od, -sr, -st));
   }
 }
 
 }  // namespace
 
+template <int SCH>
 __global__ void __launch_bounds__(kThreadsFx, 1)
     step_kernel_f64(const __grid_constant__ CUtensorMap tmap_in, double* __restrict__ f_out,
                     const __grid_constant__ StepParams p, const __grid_constant__ DvmConst<double> d, int ty0) {
-  using SZ = FxSize;
+  using SZ = FxSize<SCH>;
   constexpr int PLANE = SZ::plane, TT = kTileT;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   double* sm = reinterpret_cast<double*>(smem_raw);
   int64_t* fx = reinterpret_cast<int64_t*>(smem_raw);
-  FxTab* tab = reinterpret_cast<FxTab*>(smem_raw + SZ::planes_bytes);                      // [pair][row]
+  FxTab<SCH>* tab = reinterpret_cast<FxTab<SCH>*>(smem_raw + SZ::planes_bytes);          // [pair][row]
   double* scratch = reinterpret_cast<double*>(smem_raw + SZ::planes_bytes + SZ::tab_bytes);
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + SZ::planes_bytes + SZ::tab_bytes + SZ::scratch);
   int* top = reinterpret_cast<int*>(bar + 2);   // [kGroupsFx] largest high words
@@ -123,8 +123,8 @@ __global__ void __launch_bounds__(kThreadsFx, 1)
   if (tid < kPairsFx * TT) {   // Courant entries of the tile rows
     const int pair = tid / TT, rl = tid % TT;
     const double* e = p.courant64 + ((size_t)(min(t0 + rl, p.n_theta - 1) + kGhostRows) * kPairsFx + pair) * 4;
-    FxTab t;
-    t.r = fx_courant(fx_fraction(e[0]));
+    FxTab<SCH> t;
+    t.r = fx_coef<SCH>(fx_fraction(e[0]));
     t.at = fx_fraction(e[2] * inv_r0);
     t.fl = (int)e[3];
     t.pad = 0;
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(kThreadsFx, 1)
     eq = eq_params<double>(m.rho, m.ux, m.uy, m.E, d);
     const double fe = eq.w[0] * eq.a0;
     store(0, fe + (sm[node] - fe) * decay);
-    general_node<PLANE>(sm + node, eq, p.courant64 + (size_t)(t + kGhostRows) * kPairsFx * 4, p.inv_r[r], decay, d, store);
+    general_node<SCH, PLANE>(sm + node, eq, p.courant64 + (size_t)(t + kGhostRows) * kPairsFx * 4, p.inv_r[r], decay, d, store);
     return;
   }
   if (!valid) return;
@@ -269,16 +269,17 @@ __global__ void __launch_bounds__(kThreadsFx, 1)
       const int q1 = 1 + (k - 1) * kNDirs + i, q2 = q1 + kHalfDirs;
       const double y = i == 0 ? eq.uxE : (i == 1 ? y1 : (i == 2 ? eq.uyE : y3)), y2 = y * y;
       const double ev = fma(y2, fma(y2, C, B), A), z = fma(y2, O3, O1);
-      const FxTab& te = tab[((k - 1) * kHalfDirs + i) * TT + rl];
-      const FxCourant cr = te.r, ct = fx_courant(fx_mul_frac(te.at, ratio));
+      const FxTab<SCH>& te = tab[((k - 1) * kHalfDirs + i) * TT + rl];
+      const FxCoef<SCH> cr = te.r, ct = fx_coef<SCH>(fx_mul_frac(te.at, ratio));
       const int fl = te.fl;
       const int sr = (fl & 1) ? 1 : -1;               // v_r < 0 for q1: upwind at larger r
       const int st = (fl & 2) ? kWinR : -kWinR;       // v_theta < 0 for q1: upwind at larger theta
       // d f - M_r - M_theta of a label whose upwind neighbours sit at s_r and s_t
       auto carried = [&](const int64_t* x, int s_r, int s_t) {
-        const int64_t x0 = x[0], u1 = x[s_r], u2 = x[2 * s_r], v1 = x[s_t], v2 = x[2 * s_t];
+        const int64_t x0 = x[0];
         const int64_t keep = fx_signed(fx_mul(fx_abs(x0), dfx), (x0 >> 63) ^ dsign);
-        return fx_to_double(keep - fx_mwb(x0 - u1, u1 - u2, cr) - fx_mwb(x0 - v1, v1 - v2, ct), e);
+        return fx_to_double(keep - fx_increment<SCH>(x0, x[s_r], x[2 * s_r], x[-s_r], cr) -
+                                fx_increment<SCH>(x0, x[s_t], x[2 * s_t], x[-s_t], ct), e);
       };
       const double g1 = carried(fx + q1 * PLANE + node, sr, st), g2 = carried(fx + q2 * PLANE + node, -sr, -st);
       if (q_last) {
@@ -294,21 +295,42 @@ __global__ void __launch_bounds__(kThreadsFx, 1)
   store(q_last + kHalfDirs, o2);
 }
 
+template <int SCH>
 cudaError_t launch_step_small_f64(const CUtensorMap*, double*, const StepParams&, const DvmConst<double>&, cudaStream_t,
                                   int, int);
 
-// Tile rows [ty_begin, ty_end) of kTileT nodes each.
-cudaError_t launch_step_f64_mwb(const CUtensorMap* tmap_in, double* f_out, const StepParams& p,
-                                const DvmConst<double>& d, cudaStream_t stream, int ty_begin, int ty_end) {
+template <int SCH>
+static cudaError_t launch_scheme(const CUtensorMap* tmap_in, double* f_out, const StepParams& p,
+                                 const DvmConst<double>& d, cudaStream_t stream, int ty_begin, int ty_end) {
   if (p.tile_rows != kTileT) {
     const int per = kTileT / p.tile_rows, last = (p.n_theta + p.tile_rows - 1) / p.tile_rows;
-    return launch_step_small_f64(tmap_in, f_out, p, d, stream, ty_begin * per, std::min(ty_end * per, last));
+    return launch_step_small_f64<SCH>(tmap_in, f_out, p, d, stream, ty_begin * per, std::min(ty_end * per, last));
   }
-  static std::atomic<unsigned long long> configured{0};   // per device
-  const cudaError_t e = set_smem_once(step_kernel_f64, FxSize::smem, configured);
+  static std::atomic<unsigned long long> configured{0};   // per instantiation and device
+  const cudaError_t e = set_smem_once(step_kernel_f64<SCH>, FxSize<SCH>::smem, configured);
   if (e != cudaSuccess) return e;
   const dim3 grid((p.n_r + kTileR - 1) / kTileR, ty_end - ty_begin);
-  return launch_overlapped(step_kernel_f64, grid, kThreadsFx, FxSize::smem, stream, *tmap_in, f_out, p, d, ty_begin);
+  return launch_overlapped(step_kernel_f64<SCH>, grid, kThreadsFx, FxSize<SCH>::smem, stream, *tmap_in, f_out, p, d,
+                           ty_begin);
 }
+
+// Tile rows [ty_begin, ty_end) of the grid, kTileT nodes each (ty_end < 0: to
+// the last tile row); an empty range launches nothing.  tmap_in: boxes of
+// p.tile_rows + 4 window rows.
+template <class T>
+cudaError_t launch_step(const CUtensorMap* tmap_in, T* f_out, const StepParams& p, const DvmConst<T>& d,
+                        cudaStream_t stream, int ty_begin, int ty_end) {
+  if (ty_end < 0) ty_end = (p.n_theta + kTileT - 1) / kTileT;
+  if (ty_begin < 0 || ty_end <= ty_begin) return cudaSuccess;
+  switch (p.scheme) {
+    case PCLB_SCHEME_WB: return launch_scheme<PCLB_SCHEME_WB>(tmap_in, f_out, p, d, stream, ty_begin, ty_end);
+    case PCLB_SCHEME_LW: return launch_scheme<PCLB_SCHEME_LW>(tmap_in, f_out, p, d, stream, ty_begin, ty_end);
+    case PCLB_SCHEME_UPWIND2: return launch_scheme<PCLB_SCHEME_UPWIND2>(tmap_in, f_out, p, d, stream, ty_begin, ty_end);
+    default: return launch_scheme<PCLB_SCHEME_MWB>(tmap_in, f_out, p, d, stream, ty_begin, ty_end);
+  }
+}
+
+template cudaError_t launch_step<double>(const CUtensorMap*, double*, const StepParams&, const DvmConst<double>&,
+                                         cudaStream_t, int, int);
 
 }  // namespace pclb

@@ -1,4 +1,4 @@
-// The FP64 MWB step (Eq. 38 with Eq. 28) on small grids, where the time of one
+// The FP64 step (Eq. 38) on small grids, where the time of one
 // tile is the time of the step: tiles of 32 (r) x TT (theta) nodes, TT = 2 or 4.
 //
 // As in step_kernel_f64.cu the sums and the convection increments are formed in
@@ -31,20 +31,21 @@ constexpr int kHalfDirs = kNDirs / 2;
 constexpr int kPairsSm = 4 * kHalfDirs;
 constexpr int kPairWarps = 16;
 
+template <int SCH>
 struct SmTab {
-  FxCourant r;      // radial
+  FxCoef<SCH> r;    // radial
   uint64_t at;      // |C_theta| at the tile's first column, units of 2^-63
   int64_t fl;       // bit 0: v_r < 0, bit 1: v_theta < 0 for the first label of the pair
 };
 
-template <int TT>
+template <int SCH, int TT>
 struct SmSize {
   static constexpr int split = kPairWarps / TT;             // warps per row: 4 or 8
   static constexpr int dirs = split == 4 ? 4 : 2;           // direction pairs of its shell per warp
   static constexpr int threads = 32 * (kPairWarps + TT + 2);
   static constexpr int plane = kWinR * (TT + 4);
   static constexpr int planes_bytes = kQ * plane * 8;
-  static constexpr int tab_bytes = kPairsSm * TT * (int)sizeof(SmTab);
+  static constexpr int tab_bytes = kPairsSm * TT * (int)sizeof(SmTab<SCH>);
   // per node the shells' sums (S, X, Y), the equilibrium factors w_1 .. w_4, a0, a1, u / E
   static constexpr int node_bytes = TT * 32 * (12 + 8) * 8;
   // per wall, slot (ghost layer 0, 1, wall node) and row the factors w_0 .. w_4, a0, a1, a1h, u / E
@@ -116,15 +117,15 @@ __device__ __forceinline__ NodeState<double> state_of_sums(double f0, const doub
 
 }  // namespace
 
-template <int TT>
-__global__ void __launch_bounds__(SmSize<TT>::threads, 1)
+template <int SCH, int TT>
+__global__ void __launch_bounds__(SmSize<SCH, TT>::threads, 1)
     step_small_f64(const __grid_constant__ CUtensorMap tmap_in, double* __restrict__ f_out,
                    const __grid_constant__ StepParams p, const __grid_constant__ DvmConst<double> d, int ty0) {
-  using SZ = SmSize<TT>;
+  using SZ = SmSize<SCH, TT>;
   constexpr int PLANE = SZ::plane, SPLIT = SZ::split, DIRS = SZ::dirs;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   double* sm = reinterpret_cast<double*>(smem_raw);
-  SmTab* tab = reinterpret_cast<SmTab*>(smem_raw + SZ::planes_bytes);                        // [pair][row]
+  SmTab<SCH>* tab = reinterpret_cast<SmTab<SCH>*>(smem_raw + SZ::planes_bytes);            // [pair][row]
   double* sums = reinterpret_cast<double*>(smem_raw + SZ::planes_bytes + SZ::tab_bytes);   // [row][lane][12]
   double* fac = sums + TT * 32 * 12;                                                         // [row][lane][8]
   double* gfac = fac + TT * 32 * 8;                                                          // [side][slot][row][10]
@@ -150,8 +151,8 @@ __global__ void __launch_bounds__(SmSize<TT>::threads, 1)
   if (tid < kPairsSm * TT) {   // Courant entries of the tile rows
     const int pair = tid / TT, rl = tid % TT;
     const double* e = p.courant64 + ((size_t)(min(t0 + rl, p.n_theta - 1) + kGhostRows) * kPairsSm + pair) * 4;
-    SmTab t;
-    t.r = fx_courant(fx_fraction(e[0]));
+    SmTab<SCH> t;
+    t.r = fx_coef<SCH>(fx_fraction(e[0]));
     t.at = fx_fraction(e[2] * inv_r0);
     t.fl = (int64_t)e[3];
     tab[pair * TT + rl] = t;
@@ -317,13 +318,15 @@ __global__ void __launch_bounds__(SmSize<TT>::threads, 1)
 #pragma unroll
   for (int j = 0; j < DIRS; ++j) {
     const int i = i_first + j, q1 = 1 + (k - 1) * kNDirs + i;
-    const SmTab& te = tab[((k - 1) * kHalfDirs + i) * TT + rl];
-    const FxCourant cr = te.r, ct = fx_courant(fx_mul_frac(te.at, ratio));
+    const SmTab<SCH>& te = tab[((k - 1) * kHalfDirs + i) * TT + rl];
+    const FxCoef<SCH> cr = te.r, ct = fx_coef<SCH>(fx_mul_frac(te.at, ratio));
     const int fl = (int)te.fl;
     const int sr = (fl & 1) ? 1 : -1;               // v_r < 0 for q1: upwind at larger r
     const int st = (fl & 2) ? kWinR : -kWinR;       // v_theta < 0 for q1: upwind at larger theta
     auto carried = [&](const double* x, int s_r, int s_t) {
-      return fx_carried(x[0], x[s_r], x[2 * s_r], x[s_t], x[2 * s_t], cr, ct, dfx, dsign, decay, c64 + 4 * i, inv_r);
+      constexpr int far = SCH == PCLB_SCHEME_LW ? -1 : 2;
+      return fx_carried<SCH>(x[0], x[s_r], x[far * s_r], x[s_t], x[far * s_t], cr, ct, dfx, dsign, decay, c64 + 4 * i,
+                             inv_r);
     };
     gq[j][0] = carried(sm + q1 * PLANE + node, sr, st);
     gq[j][1] = carried(sm + (q1 + kHalfDirs) * PLANE + node, -sr, -st);
@@ -344,22 +347,31 @@ __global__ void __launch_bounds__(SmSize<TT>::threads, 1)
   }
 }
 
-// Tile rows [ty_begin, ty_end) of p.tile_rows nodes each.
-template <int TT>
+template <int SCH, int TT>
 static cudaError_t launch_small(const CUtensorMap* tmap_in, double* f_out, const StepParams& p, const DvmConst<double>& d,
                                 cudaStream_t stream, int ty_begin, int ty_end) {
   static std::atomic<unsigned long long> configured{0};   // per instantiation and device
-  const cudaError_t e = set_smem_once(step_small_f64<TT>, SmSize<TT>::smem, configured);
+  constexpr int smem = SmSize<SCH, TT>::smem, threads = SmSize<SCH, TT>::threads;
+  const cudaError_t e = set_smem_once(step_small_f64<SCH, TT>, smem, configured);
   if (e != cudaSuccess) return e;
   const dim3 grid((p.n_r + kTileR - 1) / kTileR, ty_end - ty_begin);
-  return launch_overlapped(step_small_f64<TT>, grid, SmSize<TT>::threads, SmSize<TT>::smem, stream, *tmap_in, f_out, p, d,
-                           ty_begin);
+  return launch_overlapped(step_small_f64<SCH, TT>, grid, threads, smem, stream, *tmap_in, f_out, p, d, ty_begin);
 }
 
+// Tile rows [ty_begin, ty_end) of p.tile_rows nodes each.
+template <int SCH>
 cudaError_t launch_step_small_f64(const CUtensorMap* tmap_in, double* f_out, const StepParams& p,
                                   const DvmConst<double>& d, cudaStream_t stream, int ty_begin, int ty_end) {
-  return p.tile_rows == 2 ? launch_small<2>(tmap_in, f_out, p, d, stream, ty_begin, ty_end)
-                          : launch_small<4>(tmap_in, f_out, p, d, stream, ty_begin, ty_end);
+  return p.tile_rows == 2 ? launch_small<SCH, 2>(tmap_in, f_out, p, d, stream, ty_begin, ty_end)
+                          : launch_small<SCH, 4>(tmap_in, f_out, p, d, stream, ty_begin, ty_end);
 }
+#define PCLB_SMALL(SCH)                                                                                             \
+  template cudaError_t launch_step_small_f64<SCH>(const CUtensorMap*, double*, const StepParams&,                   \
+                                                  const DvmConst<double>&, cudaStream_t, int, int);
+PCLB_SMALL(PCLB_SCHEME_MWB)
+PCLB_SMALL(PCLB_SCHEME_WB)
+PCLB_SMALL(PCLB_SCHEME_LW)
+PCLB_SMALL(PCLB_SCHEME_UPWIND2)
+#undef PCLB_SMALL
 
 }  // namespace pclb

@@ -121,3 +121,32 @@ def test_tiles_of_four_rows_outside_fixed_point(ratio, scale):
     got = got / scale
     assert np.max(np.abs(got - want)) <= 1e-12 * np.max(np.abs(want))
     assert np.max(np.abs(got[thin] - want[thin])) <= 1e-12 * np.max(np.abs(want[thin]))
+
+
+# The compared schemes in fixed point, tiles of 2, 4 and 16 rows (6, 50 and
+# 164 tiles of 32 x 16), and with magnitudes outside fixed point's range
+@pytest.mark.parametrize("scheme", [P.SCHEME_WB, P.SCHEME_LW, P.SCHEME_UPWIND2])
+@pytest.mark.parametrize("n_r,n_t", [(35, 33), (65, 259), (97, 643)])
+@pytest.mark.parametrize("bc", [(I.BC_EXTRAP, I.BC_EXTRAP), (I.BC_WALL | I.BC_NEQ, I.BC_DIRICHLET | I.BC_NEQ)])
+@pytest.mark.parametrize("relax", [P.RELAX_EXACT, P.RELAX_EULER])
+def test_compared_schemes_match_oracle(scheme, n_r, n_t, bc, relax):
+    w = I.random_smooth(n_r, n_t, seed=n_r, bc_kind=bc)
+    w.scheme, w.relaxation = scheme, relax
+    f = _noisy(w)
+    got, flags = _step(w, f, 2)
+    want = O.run(w, f, 2)
+    assert flags == 0
+    assert np.max(np.abs(got - want)) <= 2e-12 * np.max(np.abs(want))
+
+
+@pytest.mark.parametrize("scheme", [P.SCHEME_WB, P.SCHEME_LW, P.SCHEME_UPWIND2])
+@pytest.mark.parametrize("n_t", [40, 1300])
+@pytest.mark.parametrize("scale", [2.0 ** -950, 2.0 ** 950])
+def test_compared_schemes_of_any_magnitude(scheme, n_t, scale):
+    w = I.random_smooth(64, n_t, seed=9)
+    w.scheme = scheme
+    f = _noisy(w)
+    got, flags = _step(w, f * scale)
+    want = O.run(w, f, 1)
+    assert flags == 0
+    assert np.max(np.abs(got / scale - want)) <= 1e-12 * np.max(np.abs(want))
