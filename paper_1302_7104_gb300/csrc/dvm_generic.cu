@@ -1,18 +1,11 @@
-// The FP64 step and the field kernels (both precisions) for the larger
-// velocity sets of Table I, N_i = 16 and 24 directions per shell (Q = 65,
-// 97): the same model (Eqs. 2-5, 10-11, 19 or 18, 28 or the other convection
-// schemes, 38-40), one thread per node, stencil values read from global
-// memory (L1/L2), the moments, the temperature and the equilibrium factors in
-// double.  These sets serve the paper's velocity-set comparison; their FP32
-// step is the tiled kernel of dvm_tiled32.cu, the tuned TMA kernels cover
-// N_i = 8.
-//
-// Radial ghost nodes (Sec. II C 1) are formed once per wall row by
-// gen_ghost_kernel into a small buffer [side][layer][n_theta][Q] (f = f^eq of
-// the extrapolated or prescribed state, plus the wall node's departure from
-// equilibrium for non-equilibrium ghosts); the azimuthal ghost rows (Eq. 40)
-// are stored rows, written by the producer of the seam rows with the label
-// rotation, as in the rest of the library.
+// The field kernels (both precisions) for the larger velocity sets of Table I,
+// N_i = 16 and 24 directions per shell (Q = 65, 97): the same model (Eqs. 2-5,
+// 10-11), one thread per node, the moments, the temperature and the equilibrium
+// factors in double (FP64) or float-float (FP32).  These sets serve the
+// paper's velocity-set comparison; their steps are dvm_step_f64.cu and the tiled
+// FP32 kernel of dvm_tiled32.cu.  The azimuthal ghost rows (Eq. 40) are stored
+// rows, written by the producer of the seam rows with the label rotation, as in
+// the rest of the library.
 #include <cfloat>
 #include <cmath>
 #include <cstddef>
@@ -92,11 +85,6 @@ __device__ GenEq gen_eq(double rho, double ux, double uy, double E, const DvmG& 
   return e;
 }
 
-__device__ __forceinline__ double gen_feq(const GenEq& e, const DvmG& d, int q) {
-  const double x = d.vx[q] * e.uxE + d.vy[q] * e.uyE;
-  return e.w[d.shell[q]] * (e.a0 + x * (e.a1 + x * (e.a1h + x * (1.0 / 6.0 + x * (1.0 / 24.0)))));
-}
-
 // The equilibrium factors in the arithmetic type C of the per-velocity work
 // (float for FP32 storage, double for FP64), rounded from the double ones.
 template <class C>
@@ -121,23 +109,6 @@ __device__ __forceinline__ void gen_feq_pair(const GenEqC<C>& e, C vx, C vy, int
   const C od = x * (e.a1 + x2 * C(1.0 / 6.0));
   fp = e.w[k] * (ev + od);
   fm = e.w[k] * (ev - od);
-}
-
-// Convection increment in upwind form from a = |C|, K = a (1 - a), the node
-// value f0, its upwind neighbours u1, u2 and (Lax-Wendroff) the downwind one d1.
-// The limiter ratio |D| / (|D| + |Dp|) with the correctly rounded quotient
-// (0 when the sum is below the smallest normal number).
-template <int SCH>
-__device__ __forceinline__ double gen_convect(double a, double K, double f0, double u1, double u2, double d1) {
-  const double D = f0 - u1, Dp = u1 - u2;
-  if (SCH == PCLB_SCHEME_MWB) {
-    const double den = fabs(D) + fabs(Dp);
-    const double h = den >= DBL_MIN ? fabs(D) * (D - Dp) / den : 0.0;
-    return a * D + K * h;
-  }
-  if (SCH == PCLB_SCHEME_WB) return a * D + 0.5 * K * (D - Dp);
-  if (SCH == PCLB_SCHEME_UPWIND2) return a * D + 0.5 * a * (D - Dp);
-  return a * D + 0.5 * K * ((d1 - f0) - D);
 }
 
 // Store of label q at interior node (t, r), and of the azimuthal ghost rows
@@ -283,126 +254,6 @@ __global__ void __launch_bounds__(kGenThreads)
   put(temp, m.E);
 }
 
-// Radial ghost layers of wall `side` at row t: layer l sits at r = -1 - l
-// (inner) or n_r + l (outer).  Eq. (39) applied twice to the wall node a and
-// the next node b: g0 = 2a - b, g1 = 2 g0 - a, for the components the
-// boundary kind extrapolates; the others prescribed.
-__global__ void __launch_bounds__(kGenThreads)
-    gen_ghost_kernel(const double* __restrict__ f, double* __restrict__ ghost, const __grid_constant__ StepParams p,
-                     const __grid_constant__ DvmG d) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  const int side = blockIdx.y;
-  if (t >= p.n_theta) return;
-  const size_t plane = (size_t)p.rows * p.pitch;
-  const int ra = side == 0 ? 0 : p.n_r - 1, step = side == 0 ? 1 : -1;
-  const double* fa = f + (size_t)(t + kGhostRows) * p.pitch + ra;
-  const GenState a = gen_moments_node(fa, plane, d);
-  const GenState b = gen_moments_node(fa + step, plane, d);
-  double g[2][4];
-  g[0][0] = 2.0 * a.rho - b.rho;  g[1][0] = 2.0 * g[0][0] - a.rho;
-  g[0][1] = 2.0 * a.ux - b.ux;    g[1][1] = 2.0 * g[0][1] - a.ux;
-  g[0][2] = 2.0 * a.uy - b.uy;    g[1][2] = 2.0 * g[0][2] - a.uy;
-  g[0][3] = 2.0 * a.E - b.E;      g[1][3] = 2.0 * g[0][3] - a.E;
-  const int kind = p.bc_kind[side] & ~PCLB_BC_NEQ;
-  const bool neq = (p.bc_kind[side] & PCLB_BC_NEQ) != 0;
-  if (kind != PCLB_BC_EXTRAP) {
-    const double c = p.cos_t[t], s = p.sin_t[t];
-    for (int l = 0; l < 2; ++l) {
-      const double* v = p.bc_vals + (size_t)((side * 2 + l) * 4) * p.n_theta + t;
-      const double ur = v[1 * p.n_theta], ut = v[2 * p.n_theta];
-      g[l][1] = ur * c - ut * s;
-      g[l][2] = ur * s + ut * c;
-      if (kind == PCLB_BC_DIRICHLET) {
-        g[l][0] = v[0];
-        g[l][3] = v[3 * p.n_theta];
-      }
-    }
-  }
-  bool ok = a.ok && b.ok;
-  const GenEq ea = gen_eq(a.rho, a.ux, a.uy, a.E, d);
-  for (int l = 0; l < 2; ++l) {
-    ok = ok && g[l][0] > 0.0 && g[l][3] > 0.0;
-    const GenEq e = gen_eq(g[l][0], g[l][1], g[l][2], g[l][3], d);
-    double* out = ghost + ((size_t)(side * 2 + l) * p.n_theta + t) * d.q;
-    for (int q = 0; q < d.q; ++q) {
-      double v = gen_feq(e, d, q);
-      if (neq) v += fa[(size_t)q * plane] - gen_feq(ea, d, q);
-      out[q] = v;
-    }
-  }
-  if (!ok) atomicOr(p.status, PCLB_FLAG_NONPHYS);
-}
-
-// One FP64 step (Eq. 38) at node (t, r): moments and equilibrium factors in
-// double, then per pair of opposite velocities (sharing the Courant entry
-// and the even and odd parts of the equilibrium polynomial) the relaxation
-// (decay d = exp(-dt/tau) or 1 - dt/tau) minus the convection increments in r
-// and theta.
-template <int SCH>
-__global__ void __launch_bounds__(kGenThreads)
-    gen_step_kernel(const double* __restrict__ f, double* __restrict__ f_out, const double* __restrict__ ghost,
-                    const __grid_constant__ StepParams p, const __grid_constant__ DvmG d) {
-  using T = double;
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  const int t = blockIdx.y;
-  if (r >= p.n_r) return;
-  const size_t plane = (size_t)p.rows * p.pitch;
-  const int srow = t + kGhostRows;
-  const T* fn = f + (size_t)srow * p.pitch + r;
-  const GenState m = gen_moments_node(fn, plane, d);
-  const GenEqC<T> e = gen_eq_c<T>(gen_eq(m.rho, m.ux, m.uy, m.E, d));
-  if (!m.ok) atomicOr(p.status, PCLB_FLAG_NONPHYS);
-  const T decay = (T)p.decay;
-  // value of label q (plane fq) at radial index rr of row t (a ghost layer
-  // outside the grid)
-  auto fr = [&](const T* fq, int q, int rr) -> T {
-    if (rr < 0) return ghost[((size_t)(0 * 2 + (-1 - rr)) * p.n_theta + t) * d.q + q];
-    if (rr >= p.n_r) return ghost[((size_t)(1 * 2 + (rr - p.n_r)) * p.n_theta + t) * d.q + q];
-    return fq[rr - r];
-  };
-  // value of plane fq at stored row srow + dt_rows of column r
-  const ptrdiff_t pitch = p.pitch;
-  auto ft = [&](const T* fq, int dt_rows) -> T { return fq[dt_rows * pitch]; };
-  // label q at this node and at the azimuthal ghost rows it feeds (Eq. 40)
-  T* out_row = f_out + (size_t)srow * p.pitch + r;
-  T* out_lo = t >= p.n_theta - 2 ? f_out + (size_t)(t - (p.n_theta - 2)) * p.pitch + r : nullptr;
-  T* out_hi = t < 2 ? f_out + (size_t)(p.n_theta + kGhostRows + t) * p.pitch + r : nullptr;
-  auto put = [&](int q, T v) {
-    out_row[(size_t)q * plane] = v;
-    if (out_lo) out_lo[(size_t)d.recv_lo[q] * plane] = v;
-    if (out_hi) out_hi[(size_t)d.recv_hi[q] * plane] = v;
-  };
-  {
-    const T f0 = fn[0];
-    const T fe = e.w[0] * e.a0;
-    put(0, fe + (f0 - fe) * decay);
-  }
-  const int half = d.n_dirs / 2, npairs = 2 * d.n_dirs;
-  const T inv_r = (T)p.inv_r[r];
-  const bool lw = SCH == PCLB_SCHEME_LW;
-  for (int k = 1; k <= 4; ++k)
-    for (int i = 0; i < half; ++i) {
-      const int q1 = 1 + (k - 1) * d.n_dirs + i, q2 = q1 + half;
-      const double* ce = p.courant64 + ((size_t)srow * npairs + (k - 1) * half + i) * 4;
-      const T ar = ce[0], kr = ce[1], at = ce[2] * inv_r;
-      const int fl = (int)ce[3];
-      const T kt = at - at * at;
-      const int sr = (fl & 1) ? 1 : -1;   // v_r < 0 for q1: upwind at larger r
-      const int st = (fl & 2) ? 1 : -1;   // v_theta < 0 for q1: upwind at larger theta
-      T fe[2];
-      gen_feq_pair<T>(e, d.vx[q1], d.vy[q1], k, fe[0], fe[1]);
-      for (int L = 0; L < 2; ++L) {
-        const int q = L ? q2 : q1, s_r = L ? -sr : sr, s_t = L ? -st : st;
-        const T* fq = fn + (size_t)q * plane;
-        const T a = fq[0];
-        const T cr = gen_convect<SCH>(ar, kr, a, fr(fq, q, r + s_r), fr(fq, q, r + 2 * s_r),
-                                      lw ? fr(fq, q, r - s_r) : T(0));
-        const T ct = gen_convect<SCH>(at, kt, a, ft(fq, s_t), ft(fq, 2 * s_t), lw ? ft(fq, -s_t) : T(0));
-        put(q, fe[L] + (a - fe[L]) * decay - cr - ct);
-      }
-    }
-}
-
 // Global integrals with weight r dr dtheta (as pclb_diagnostics): per block a
 // fixed grid-stride subset in a fixed order, then one thread sums the blocks.
 // The node state in double: FP64 storage by double sums, FP32 by the
@@ -455,16 +306,6 @@ __global__ void __launch_bounds__(kGenThreads)
     }
 }
 
-template <int SCH>
-cudaError_t gen_step_scheme(const double* f, double* f_out, double* ghost, const StepParams& p, const DvmG& d,
-                            cudaStream_t s) {
-  // one thread per wall row, in warps, so that the rows spread over the SMs
-  gen_ghost_kernel<<<dim3((p.n_theta + 31) / 32, 2), 32, 0, s>>>(f, ghost, p, d);
-  gen_step_kernel<SCH><<<dim3((p.n_r + kGenThreads - 1) / kGenThreads, p.n_theta), kGenThreads, 0, s>>>(
-      f, f_out, ghost, p, d);
-  return cudaGetLastError();
-}
-
 }  // namespace
 
 template <class T>
@@ -501,16 +342,6 @@ cudaError_t gen_launch_pack(const T* f, T* out, const StepParams& p, const DvmG&
 template <class T>
 cudaError_t gen_launch_unpack(const T* in, T* f, const StepParams& p, const DvmG& d, cudaStream_t s) {
   return launch_copy_rows<T, true>(in, f, d.q, p, recv_labels(d, d.q), s);
-}
-
-cudaError_t gen_launch_step_f64(const double* f, double* f_out, double* ghost, const StepParams& p, const DvmG& d,
-                                cudaStream_t s) {
-  switch (p.scheme) {
-    case PCLB_SCHEME_WB: return gen_step_scheme<PCLB_SCHEME_WB>(f, f_out, ghost, p, d, s);
-    case PCLB_SCHEME_LW: return gen_step_scheme<PCLB_SCHEME_LW>(f, f_out, ghost, p, d, s);
-    case PCLB_SCHEME_UPWIND2: return gen_step_scheme<PCLB_SCHEME_UPWIND2>(f, f_out, ghost, p, d, s);
-    default: return gen_step_scheme<PCLB_SCHEME_MWB>(f, f_out, ghost, p, d, s);
-  }
 }
 
 void fill_dvm_generic32(DvmG32& c, const pclb_dvm& d, const DvmG& g) {

@@ -23,8 +23,8 @@ struct DvmG32 {
 
 void fill_dvm_generic32(DvmG32& c, const pclb_dvm& d, const DvmG& g);
 
-// One FP64 step of the N_i = 16 or 24 set (dvm_generic.cu): the radial ghost
-// layers into ghost [side][layer][n_theta][Q], then one thread per node.
+// One FP64 step of the N_i = 16 or 24 set (dvm_step_f64.cu): the radial ghost
+// layers into ghost [side][layer][n_theta][Q], then the nodes.
 cudaError_t gen_launch_step_f64(const double* f, double* f_out, double* ghost, const StepParams& p, const DvmG& d,
                                 cudaStream_t s);
 

@@ -150,3 +150,30 @@ def test_compared_schemes_of_any_magnitude(scheme, n_t, scale):
     want = O.run(w, f, 1)
     assert flags == 0
     assert np.max(np.abs(got / scale - want)) <= 1e-12 * np.max(np.abs(want))
+
+
+# N_i = 16 and 24: blocks of 32 nodes of a row, four wall rows per ghost block
+@pytest.mark.parametrize("n_dirs", [16, 24])
+@pytest.mark.parametrize("scheme,relax", [(P.SCHEME_MWB, P.RELAX_EXACT), (P.SCHEME_WB, P.RELAX_EULER),
+                                          (P.SCHEME_LW, P.RELAX_EXACT), (P.SCHEME_UPWIND2, P.RELAX_EULER)])
+@pytest.mark.parametrize("n_r,n_t", [(3, 2), (32, 5), (33, 9), (66, 4)])
+@pytest.mark.parametrize("bc", [(I.BC_EXTRAP, I.BC_EXTRAP), (I.BC_WALL | I.BC_NEQ, I.BC_DIRICHLET | I.BC_NEQ)])
+def test_larger_sets_match_oracle(n_dirs, scheme, relax, n_r, n_t, bc):
+    w = I.random_smooth(n_r, n_t, seed=n_r + n_t, bc_kind=bc, amp=0.02 if n_r < 8 else 0.2, tau=0.05,
+                        n_dirs=n_dirs, n_f=n_dirs)
+    w.scheme, w.relaxation = scheme, relax
+    f = _noisy(w)
+    got, _ = _step(w, f, 2)
+    want = O.run(w, f, 2)
+    assert np.max(np.abs(got - want)) <= 2e-12 * np.max(np.abs(want))
+
+
+@pytest.mark.parametrize("n_dirs", [16, 24])
+@pytest.mark.parametrize("scale", [2.0 ** -950, 2.0 ** 950])
+def test_larger_sets_of_any_magnitude(n_dirs, scale):
+    w = _contrast(I.random_smooth(64, 24, seed=10, n_dirs=n_dirs, n_f=n_dirs), 300.0)
+    f = _noisy(w)
+    got, flags = _step(w, f * scale)
+    want = O.run(w, f, 1)
+    assert flags == 0
+    assert np.max(np.abs(got / scale - want)) <= 1e-12 * np.max(np.abs(want))
