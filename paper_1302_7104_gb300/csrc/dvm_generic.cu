@@ -23,12 +23,6 @@ namespace {
 
 constexpr int kGenThreads = 128;
 
-struct GenEq {
-  double w[5];              // rho F_k(E) (Eq. 11); w[0] = rho (1 - B0 sum_k F_k)
-  double a0, a1, a1h;       // coefficients of the polynomial of Eq. (10)
-  double uxE, uyE;          // u / E
-};
-
 struct GenState {
   double rho, ux, uy, E;
   bool ok;
@@ -67,50 +61,6 @@ __device__ GenState gen_moments_node(const double* f, size_t plane, const DvmG& 
   return gen_state_of(s0, sx, sy, se);
 }
 
-__device__ GenEq gen_eq(double rho, double ux, double uy, double E, const DvmG& d) {
-  GenEq e;
-  double Fs = 0.0;
-  for (int k = 1; k <= 4; ++k) {
-    const double F = E * (d.Fc[k][0] + E * (d.Fc[k][1] + E * (d.Fc[k][2] + E * d.Fc[k][3])));
-    e.w[k] = rho * F;
-    Fs += F;
-  }
-  e.w[0] = rho * (1.0 - d.B0 * Fs);
-  const double u2E = (ux * ux + uy * uy) / E;
-  e.a1 = 1.0 - 0.5 * u2E;
-  e.a0 = e.a1 + 0.125 * u2E * u2E;
-  e.a1h = 0.5 * e.a1;
-  e.uxE = ux / E;
-  e.uyE = uy / E;
-  return e;
-}
-
-// The equilibrium factors in the arithmetic type C of the per-velocity work
-// (float for FP32 storage, double for FP64), rounded from the double ones.
-template <class C>
-struct GenEqC {
-  C w[5], a0, a1, a1h, uxE, uyE;
-};
-
-template <class C>
-__device__ __forceinline__ GenEqC<C> gen_eq_c(const GenEq& e) {
-  GenEqC<C> c;
-  for (int k = 0; k < 5; ++k) c.w[k] = (C)e.w[k];
-  c.a0 = (C)e.a0; c.a1 = (C)e.a1; c.a1h = (C)e.a1h; c.uxE = (C)e.uxE; c.uyE = (C)e.uyE;
-  return c;
-}
-
-// f^eq of velocity (vx, vy) of shell k, Eq. (10), as even and odd parts in x
-// = v.u/E: P(x) = ev + od, P(-x) = ev - od (the opposite velocity).
-template <class C>
-__device__ __forceinline__ void gen_feq_pair(const GenEqC<C>& e, C vx, C vy, int k, C& fp, C& fm) {
-  const C x = vx * e.uxE + vy * e.uyE, x2 = x * x;
-  const C ev = e.a0 + x2 * (e.a1h + x2 * C(1.0 / 24.0));
-  const C od = x * (e.a1 + x2 * C(1.0 / 6.0));
-  fp = e.w[k] * (ev + od);
-  fm = e.w[k] * (ev - od);
-}
-
 // Store of label q at interior node (t, r), and of the azimuthal ghost rows
 // of the receiving labels when t is a seam row (Eq. 40).
 template <class T>
@@ -123,30 +73,6 @@ __device__ __forceinline__ void gen_store(T* f, const StepParams& p, const DvmG&
 }
 
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kGenThreads)
-    gen_set_state_kernel(double* __restrict__ f, const double* __restrict__ rho, const double* __restrict__ u_r,
-                         const double* __restrict__ u_t, const double* __restrict__ temp,
-                         const __grid_constant__ StepParams p, const __grid_constant__ DvmG d) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  const int t = blockIdx.y;
-  if (r >= p.n_r) return;
-  const size_t n = (size_t)t * p.n_r + r;
-  const double c = p.cos_t[t], s = p.sin_t[t];
-  const double R = rho[n], ur = u_r[n], ut = u_t[n], E = temp[n];  // E = T
-  if (!(R > 0.0 && E > 0.0)) atomicOr(p.status, PCLB_FLAG_NONPHYS);
-  const GenEqC<double> e = gen_eq_c<double>(gen_eq(R, ur * c - ut * s, ur * s + ut * c, E, d));
-  gen_store<double>(f, p, d, 0, t, r, e.w[0] * e.a0);
-  const int half = d.n_dirs / 2;
-  for (int k = 1; k <= 4; ++k)
-    for (int i = 0; i < half; ++i) {
-      const int q = 1 + (k - 1) * d.n_dirs + i;
-      double fp, fm;
-      gen_feq_pair<double>(e, d.vx[q], d.vy[q], k, fp, fm);
-      gen_store<double>(f, p, d, q, t, r, fp);
-      gen_store<double>(f, p, d, q + half, t, r, fm);
-    }
-}
-
 __global__ void __launch_bounds__(kGenThreads)
     gen_moments_kernel(const double* __restrict__ f, double* rho, double* u_r, double* u_t, double* temp,
                        const __grid_constant__ StepParams p, const __grid_constant__ DvmG d) {
@@ -313,7 +239,7 @@ cudaError_t gen_launch_set_state(T* f, const T* rho, const T* ur, const T* ut, c
                                  const DvmG& d, const DvmG32& c, cudaStream_t s) {
   const dim3 grid((p.n_r + kGenThreads - 1) / kGenThreads, p.n_theta);
   if constexpr (sizeof(T) == 8)
-    gen_set_state_kernel<<<grid, kGenThreads, 0, s>>>(f, rho, ur, ut, temp, p, d);
+    return gen_launch_set_state_f64(f, rho, ur, ut, temp, p, d, s);
   else if (d.n_dirs == 16)
     gen_set_state_f32_kernel<16><<<grid, kGenThreads, 0, s>>>(f, rho, ur, ut, temp, p, d, c);
   else

@@ -23,6 +23,10 @@ struct DvmG32 {
 
 void fill_dvm_generic32(DvmG32& c, const pclb_dvm& d, const DvmG& g);
 
+// f^eq of the fields in FP64 (dvm_step_f64.cu).
+cudaError_t gen_launch_set_state_f64(double* f, const double* rho, const double* ur, const double* ut,
+                                     const double* temp, const StepParams& p, const DvmG& d, cudaStream_t s);
+
 // One FP64 step of the N_i = 16 or 24 set (dvm_step_f64.cu): the radial ghost
 // layers into ghost [side][layer][n_theta][Q], then the nodes.
 cudaError_t gen_launch_step_f64(const double* f, double* f_out, double* ghost, const StepParams& p, const DvmG& d,

@@ -1,5 +1,5 @@
-// One FP64 step (Eq. 38) of the N_i = 16 and 24 velocity sets: the radial ghost
-// layers, then the nodes.
+// The FP64 initial state and step (Eq. 38) of the N_i = 16 and 24 velocity sets;
+// a step is two launches, the radial ghost layers and the nodes.
 //
 // What bounds it: FP64 issue (a quarter SM starts one warp-wide FP64 operation
 // per 64-76 cycles).  The convection increments, ~36 FP64 operations per update
@@ -9,9 +9,9 @@
 // share the directions (H / 4 of the H pairs each, over the four shells), a fifth
 // forms the states from their sums while they convect.  On small grids this
 // also gives every node four threads.
-// N_i = 16, 512 x 512: 703 us per step (1639 before, one thread per node and all
-// of it in FP64); 64 x 64: 38 us (236, of which 150 the ghosts, one thread per
-// wall row; now a warp per row).
+// N_i = 16, 512 x 512: 367 us per step (1639 before, one thread per node and all
+// of it in FP64), the FP64 pipe 81% busy; 64 x 64: 32 us (236, of which 150 the
+// ghosts, one thread per wall row; now a warp per row).
 #include <cuda_runtime.h>
 
 #include "device_common.cuh"
@@ -48,6 +48,71 @@ __device__ __forceinline__ GenFactors gen_factors(double rho, double ux, double 
   g.a1 = fma(-0.5, s, 1.0);
   g.a0 = fma(0.125 * s, s, g.a1);
   return g;
+}
+
+// What the nodes of a block share with the warps that own the directions: per
+// shell A, B, C, O1, O3 of scale f^eq = A + y^2 (B + y^2 C) +- y (O1 + y^2 O3), y
+// = c_i.u / E, and u / (E v_1) (DvmG holds c_i v_1), for 32 nodes.
+struct GenPoly {
+  double c[4][5][32], uxv[32], uyv[32];
+};
+__device__ __forceinline__ void put_poly(GenPoly& o, int lane, const GenFactors& g, int nd, const DvmG& d) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const double w = g.w[k + 1], v = d.vx[1 + k * nd], hv = d.half_v2[k + 1], wa = w * g.a1, wh = w * hv;
+    o.c[k][0][lane] = w * g.a0;
+    o.c[k][1][lane] = wa * hv;
+    o.c[k][2][lane] = wh * hv * (1.0 / 6.0);
+    o.c[k][3][lane] = wa * v;
+    o.c[k][4][lane] = wh * v * (1.0 / 3.0);
+  }
+  const double iv = recip_newton(d.vx[1]);
+  o.uxv[lane] = g.uxE * iv;
+  o.uyv[lane] = g.uyE * iv;
+}
+
+// f^eq of a block's 32 nodes from their fields, the directions over four warps.
+// Bound: FP64 issue (90%), 3.4 operations per label with the direction's y shared
+// by the shells (5.5 with x = v_q.u / E of each pair, and a thread per node):
+// 512 x 512, N_i = 16, 130 us (197).
+template <int ND>
+__global__ void __launch_bounds__(32 * kParts)
+    gen_set_state64(double* __restrict__ f, const double* __restrict__ rho, const double* __restrict__ u_r,
+                    const double* __restrict__ u_t, const double* __restrict__ temp,
+                    const __grid_constant__ StepParams p, const __grid_constant__ DvmG d) {
+  constexpr int H = ND / 2, DIRS = H / kParts;
+  __shared__ GenPoly poly;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int r = blockIdx.x * 32 + lane, t = blockIdx.y;
+  const size_t plane = (size_t)p.rows * p.pitch;
+  auto put = [&](int q, double v) {
+    f[(size_t)q * plane + (size_t)(t + kGhostRows) * p.pitch + r] = v;
+    if (t >= p.n_theta - 2) f[(size_t)d.recv_lo[q] * plane + (size_t)(t - (p.n_theta - 2)) * p.pitch + r] = v;
+    if (t < 2) f[(size_t)d.recv_hi[q] * plane + (size_t)(p.n_theta + kGhostRows + t) * p.pitch + r] = v;
+  };
+  if (warp == 0) {
+    const size_t n = (size_t)t * p.n_r + min(r, p.n_r - 1);
+    const double c = p.cos_t[t], s = p.sin_t[t];
+    const double R = rho[n], ur = u_r[n], ut = u_t[n], E = temp[n];   // E = T
+    if (!(R > 0.0 && E > 0.0)) atomicOr(p.status, PCLB_FLAG_NONPHYS);
+    const GenFactors g = gen_factors(R, ur * c - ut * s, ur * s + ut * c, E, d);
+    put_poly(poly, lane, g, ND, d);
+    if (r < p.n_r) put(0, g.w[0] * g.a0);
+  }
+  __syncthreads();
+  if (r >= p.n_r) return;
+#pragma unroll 1
+  for (int j = 0; j < DIRS; ++j) {
+    const int i = warp + kParts * j;
+    const double y = fma(d.vx[1 + i], poly.uxv[lane], d.vy[1 + i] * poly.uyv[lane]), y2 = y * y;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const double(&c)[5][32] = poly.c[k];
+      const double ev = fma(y2, fma(y2, c[2][lane], c[1][lane]), c[0][lane]), z = fma(y2, c[4][lane], c[3][lane]);
+      put(1 + k * ND + i, fma(y, z, ev));
+      put(1 + k * ND + i + H, fma(-y, z, ev));
+    }
+  }
 }
 
 // Radial ghost layers of wall blockIdx.y, a warp per row: layer l sits at r = -1
@@ -169,13 +234,14 @@ struct GenTab {
 };
 
 template <int SCH, int ND>
-__global__ void __launch_bounds__(32 * (kParts + 1), 3)
+__global__ void __launch_bounds__(32 * (kParts + 1), 5)
     gen_step_kernel(const double* __restrict__ f, double* __restrict__ f_out, const double* __restrict__ ghost,
                     const __grid_constant__ StepParams p, const __grid_constant__ DvmG d) {
   constexpr int H = ND / 2, NP = 4 * H, DIRS = H / kParts;
   __shared__ GenTab<SCH> tab[NP];
   __shared__ double part[kParts][4][32];
-  __shared__ double fac[22][32];   // per shell A, B, C, O1, O3 of (1 - d) f^eq = A + x^2 (B + x^2 C) +- x (O1 + x^2 O3); u / E
+  __shared__ double carried[2 * DIRS * 4][32 * kParts];   // d f - M_r - M_theta of each thread's labels
+  __shared__ GenPoly poly;   // of (1 - d) f^eq
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int r0 = blockIdx.x * 32, r = r0 + lane, t = blockIdx.y;
   const bool valid = r < p.n_r;
@@ -214,17 +280,7 @@ __global__ void __launch_bounds__(32 * (kParts + 1), 3)
     const NodeState<double> m = node_state64(s[0], s[1], s[2], s[3]);
     if (valid && !m.ok) atomicOr(p.status, PCLB_FLAG_NONPHYS);
     const GenFactors g = gen_factors(omd * m.rho, m.ux, m.uy, m.E, d);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const double w = g.w[k + 1], wa = w * g.a1;
-      fac[5 * k + 0][lane] = w * g.a0;
-      fac[5 * k + 1][lane] = 0.5 * wa;
-      fac[5 * k + 2][lane] = w * (1.0 / 24.0);
-      fac[5 * k + 3][lane] = wa;
-      fac[5 * k + 4][lane] = w * (1.0 / 6.0);
-    }
-    fac[20][lane] = g.uxE;
-    fac[21][lane] = g.uyE;
+    put_poly(poly, lane, g, ND, d);
     __syncthreads();
     if (valid) put(0, fma(decay, f0, g.w[0] * g.a0));   // rest velocity: no convection
     return;
@@ -260,40 +316,38 @@ __global__ void __launch_bounds__(32 * (kParts + 1), 3)
     if (rr >= p.n_r) return ghost[((size_t)(2 + rr - p.n_r) * p.n_theta + t) * d.q + q];
     return fq[rr - rc];
   };
-  double gq[DIRS][4][2];
+  // (rolled: unrolled, the loop was 64 KB of code and instruction fetch held it up, 703 us a step against 376)
+#pragma unroll 1
+  for (int n = 0; n < 4 * DIRS; ++n) {
+    const int k = n & 3, i = warp + kParts * (n >> 2), pair = k * H + i, q1 = 1 + k * ND + i;
+    const GenTab<SCH>& e = tab[pair];
+    const FxCoef<SCH> cr = e.r, ct = fx_coef<SCH>(fx_mul_frac(e.at, ratio));
+    const int fl = (int)e.fl;
 #pragma unroll
-  for (int j = 0; j < DIRS; ++j)
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int pair = k * H + warp + kParts * j, q1 = 1 + k * ND + warp + kParts * j;
-      const GenTab<SCH>& e = tab[pair];
-      const FxCoef<SCH> cr = e.r, ct = fx_coef<SCH>(fx_mul_frac(e.at, ratio));
-      const int fl = (int)e.fl;
-#pragma unroll
-      for (int L = 0; L < 2; ++L) {
-        const int sr = ((fl & 1) != 0) != (L != 0) ? 1 : -1;               // upwind at larger r
-        const ptrdiff_t st = ((fl & 2) != 0) != (L != 0) ? p.pitch : -(ptrdiff_t)p.pitch;   // upwind at larger theta
-        constexpr int far = SCH == PCLB_SCHEME_LW ? -1 : 2;
-        const int q = q1 + L * H;
-        const double* x = fn + (size_t)q * plane;
-        gq[j][k][L] = fx_carried<SCH>(x[0], radial(x, q, rc + sr), radial(x, q, rc + far * sr), x[st], x[far * st], cr,
-                                      ct, dfx, dsign, decay, c64 + 4 * pair, inv_r);
-      }
+    for (int L = 0; L < 2; ++L) {
+      const int sr = ((fl & 1) != 0) != (L != 0) ? 1 : -1;               // upwind at larger r
+      const ptrdiff_t st = ((fl & 2) != 0) != (L != 0) ? p.pitch : -(ptrdiff_t)p.pitch;   // upwind at larger theta
+      constexpr int far = SCH == PCLB_SCHEME_LW ? -1 : 2;
+      const int q = q1 + L * H;
+      const double* x = fn + (size_t)q * plane;
+      carried[2 * n + L][threadIdx.x] =
+          fx_carried<SCH>(x[0], radial(x, q, rc + sr), radial(x, q, rc + far * sr), x[st], x[far * st], cr, ct, dfx,
+                          dsign, decay, c64 + 4 * pair, inv_r);
     }
+  }
   __syncthreads();
   if (!valid) return;
-  const double uxE = fac[20][lane], uyE = fac[21][lane];
+#pragma unroll 1
+  for (int j = 0; j < DIRS; ++j) {
+    const int i = warp + kParts * j;
+    const double y = fma(d.vx[1 + i], poly.uxv[lane], d.vy[1 + i] * poly.uyv[lane]), y2 = y * y;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const double A = fac[5 * k][lane], B = fac[5 * k + 1][lane], C = fac[5 * k + 2][lane], O1 = fac[5 * k + 3][lane],
-                 O3 = fac[5 * k + 4][lane];
-#pragma unroll
-    for (int j = 0; j < DIRS; ++j) {
-      const int q = 1 + k * ND + warp + kParts * j;
-      const double x = fma(d.vx[q], uxE, d.vy[q] * uyE), x2 = x * x;
-      const double ev = fma(x2, fma(x2, C, B), A), z = fma(x2, O3, O1);
-      put(q, fma(x, z, ev + gq[j][k][0]));
-      put(q + H, fma(-x, z, ev + gq[j][k][1]));
+    for (int k = 0; k < 4; ++k) {
+      const double(&c)[5][32] = poly.c[k];
+      const double ev = fma(y2, fma(y2, c[2][lane], c[1][lane]), c[0][lane]), z = fma(y2, c[4][lane], c[3][lane]);
+      const int q = 1 + k * ND + i, n = 4 * j + k;
+      put(q, fma(y, z, ev + carried[2 * n][threadIdx.x]));
+      put(q + H, fma(-y, z, ev + carried[2 * n + 1][threadIdx.x]));
     }
   }
 }
@@ -320,6 +374,16 @@ cudaError_t gen_step_scheme(const double* f, double* f_out, double* ghost, const
 }
 
 }  // namespace
+
+cudaError_t gen_launch_set_state_f64(double* f, const double* rho, const double* ur, const double* ut,
+                                     const double* temp, const StepParams& p, const DvmG& d, cudaStream_t s) {
+  const dim3 grid((p.n_r + 31) / 32, p.n_theta);
+  if (d.n_dirs == 16)
+    gen_set_state64<16><<<grid, 32 * kParts, 0, s>>>(f, rho, ur, ut, temp, p, d);
+  else
+    gen_set_state64<24><<<grid, 32 * kParts, 0, s>>>(f, rho, ur, ut, temp, p, d);
+  return cudaGetLastError();
+}
 
 cudaError_t gen_launch_step_f64(const double* f, double* f_out, double* ghost, const StepParams& p, const DvmG& d,
                                 cudaStream_t s) {
