@@ -318,11 +318,10 @@ __device__ __forceinline__ void to_moment_cotangent2(f2 rho, f2 ux, f2 uy, f2 E,
 }
 
 // Phase (A) for one label at this thread's two nodes, its upwind offsets U
-// (columns) and V (window rows) as constants: the products of the MWB
-// partials in r and theta; returns lam of the two nodes.
-template <int U, int V>
-__device__ __forceinline__ f2 products_label(const float* w, const float* wl, float* P, int p_rad, int p_az, f2 a_r,
-                                             f2 k_r, f2 a_t, f2 k_t) {
+// (columns) and V (window rows): the products of the MWB partials in r and
+// theta; returns lam of the two nodes.
+__device__ __forceinline__ f2 products_label(int U, const float* w, const float* wl, int V, float* P, int p_rad,
+                                             int p_az, f2 a_r, f2 k_r, f2 a_t, f2 k_t) {
   const f2 C = lds2(w);
   const f2 S2 = lds2(w + 2 * U);                            // f(n + 2u) of both nodes
   const f2 u1 = U > 0 ? mk2(C.y, S2.x) : mk2(S2.y, C.x);     // f(n + u)
@@ -340,18 +339,16 @@ __device__ __forceinline__ f2 products_label(const float* w, const float* wl, fl
 
 // Phase (A) for both labels of a pair: q1's upwind offsets UR, VT, q2's the
 // opposite ones.
-template <int UR, int VT>
-__device__ __forceinline__ void products_pair(const float* sf, const float* sl, float* pb, int o, int p_rad, int p_az,
-                                              f2 a_r, f2 k_r, f2 a_t, f2 k_t, f2 lam_c[2]) {
-  lam_c[0] = products_label<UR, VT>(sf + o, sl + o, pb, p_rad, p_az, a_r, k_r, a_t, k_t);
-  lam_c[1] = products_label<-UR, -VT>(sf + kAPl + o, sl + kAPl + o, pb + kProd, p_rad, p_az, a_r, k_r, a_t, k_t);
+__device__ __forceinline__ void products_pair(int UR, const float* sf, const float* sl, int VT, float* pb, int o,
+                                              int p_rad, int p_az, f2 a_r, f2 k_r, f2 a_t, f2 k_t, f2 lam_c[2]) {
+  lam_c[0] = products_label(UR, sf + o, sl + o, VT, pb, p_rad, p_az, a_r, k_r, a_t, k_t);
+  lam_c[1] = products_label(-UR, sf + kAPl + o, sl + kAPl + o, -VT, pb + kProd, p_rad, p_az, a_r, k_r, a_t, k_t);
 }
 
 // Products of one halo row (window row rr) at the node pair jj, jj + 1, for
 // the label whose upwind side points into the tile: V = +row for the rows
 // below the tile, -row for those above.
-template <int V>
-__device__ __forceinline__ void halo_row(const float* sf, const float* sl, float* pb, const float4* ctab,
+__device__ __forceinline__ void halo_row(int V, const float* sf, const float* sl, float* pb, const float4* ctab,
                                          const float* invr, int pair, int rr, int jj) {
   const float4 eh = ctab[rr * kANP + pair];
   const bool q1_up_pos = (__float_as_int(eh.w) & 2) != 0;
@@ -370,8 +367,7 @@ __device__ __forceinline__ void halo_row(const float* sf, const float* sl, float
 
 // Radial gather of one label at the two nodes (upwind offset U): A(c) -
 // A(c - u) + B(c - u) - B(c - 2u).
-template <int U>
-__device__ __forceinline__ f2 gather_radial2(const float* P, int p_rad) {
+__device__ __forceinline__ f2 gather_radial2(int U, const float* P, int p_rad) {
   const f2 A0 = lds2(P + kAR + p_rad), B0 = lds2(P + kBR + p_rad);
   const f2 An = lds2(P + kAR + p_rad - 2 * U), Bn = lds2(P + kBR + p_rad - 2 * U);
   const f2 Au = U > 0 ? mk2(An.y, A0.x) : mk2(A0.y, An.x);
@@ -381,8 +377,7 @@ __device__ __forceinline__ f2 gather_radial2(const float* P, int p_rad) {
 
 // Azimuthal gather of one label where the rows -2 .. +2 around the node all
 // have their upwind side on one side: the readers of the node at +W, +2W.
-template <int W>
-__device__ __forceinline__ f2 gather_az2(const float* P) {
+__device__ __forceinline__ f2 gather_az2(const float* P, int W) {
   constexpr int DB = kBT - kAT;
   return sub2(sub2(add2(lds2(P), lds2(P + DB + W)), lds2(P + W)), lds2(P + DB + 2 * W));
 }
@@ -622,24 +617,20 @@ __device__ __forceinline__ void adjoint_tile(const CUtensorMap& tmap_f, const CU
     const f2 a_r = bc2(ce.x), k_r = bc2(ce.y);
     const f2 a_t = mul2(bc2(ce.z), my_invr), k_t = fma2(neg2(a_t), a_t, a_t);
     f2 lam_c[2];
-    // bit 0: q1 reads n + 1, n + 2 in r; bit 1: q1 reads the rows above.  The
-    // two rows of a warp nearly always agree (a label's upwind side changes
-    // at a few theta rows only), so the branch is uniform in practice.
-    switch (fl_c & 3) {
-      case 0: products_pair<-1, -kWinR>(sf, sl, pb, o_node, p_rad, p_az, a_r, k_r, a_t, k_t, lam_c); break;
-      case 1: products_pair<1, -kWinR>(sf, sl, pb, o_node, p_rad, p_az, a_r, k_r, a_t, k_t, lam_c); break;
-      case 2: products_pair<-1, kWinR>(sf, sl, pb, o_node, p_rad, p_az, a_r, k_r, a_t, k_t, lam_c); break;
-      default: products_pair<1, kWinR>(sf, sl, pb, o_node, p_rad, p_az, a_r, k_r, a_t, k_t, lam_c); break;
-    }
+    // bit 0: q1 reads n + 1, n + 2 in r; bit 1: q1 reads the rows above.  Both
+    // offsets are variables: with an instance of the code for each case (four
+    // here, two each for the halo rows and the gathers) the loop waited for
+    // instruction fetches (2.4 of 11 stall cycles per issue; 103 us on 512 x 1024
+    // against 96; a loop over the two labels as well: 100).
+    const int VT = (fl_c & 2) ? kWinR : -kWinR;
+    products_pair((fl_c & 1) ? 1 : -1, sf, sl, VT, pb, o_node, p_rad, p_az, a_r, k_r, a_t, k_t, lam_c);
     if (tid < 64) {
       // halo rows (window rows 0, 1, kTT + 2, kTT + 3), the label whose
       // upwind side points into the tile: warp 0 the rows below the tile
       // (read by the label with its upwind side at +theta), warp 1 the rows
       // above it
-      if (tid < 32)
-        halo_row<kWinR>(sf, sl, pb, ctab, invr, pair, tid >> 4, 2 * (tid & 15));
-      else
-        halo_row<-kWinR>(sf, sl, pb, ctab, invr, pair, kTT + 2 + ((tid >> 4) & 1), 2 * (tid & 15));
+      halo_row(tid < 32 ? kWinR : -kWinR, sf, sl, pb, ctab, invr, pair, (tid < 32 ? 0 : kTT + 2) + ((tid >> 4) & 1),
+               2 * (tid & 15));
     } else if (tid < 96) {
       // halo columns: per tile row and label the two columns whose upwind
       // stencils reach the tile, -2, -1 (upwind at larger r) or 32, 33
@@ -673,22 +664,15 @@ __device__ __forceinline__ void adjoint_tile(const CUtensorMap& tmap_f, const CU
     // n = c - u and -M_Dp of n = c - 2u
     if (v0 || v1) {
       f2 acc[2];
-      if (fl_c & 1) {
-        acc[0] = gather_radial2<1>(pb, p_rad);
-        acc[1] = gather_radial2<-1>(pb + kProd, p_rad);
-      } else {
-        acc[0] = gather_radial2<-1>(pb, p_rad);
-        acc[1] = gather_radial2<1>(pb + kProd, p_rad);
-      }
+      acc[0] = gather_radial2((fl_c & 1) ? 1 : -1, pb, p_rad);
+      acc[1] = gather_radial2((fl_c & 1) ? -1 : 1, pb + kProd, p_rad);
       const int tneg = fl_c >> 2;                  // bit o: row o - 2 has v_theta < 0 for q1
       constexpr int DB = kBT - kAT;
-      if (tneg == 0) {
-        // q1's readers at +V, +2V, q2's at -V, -2V (V = one row)
-        acc[0] = add2(acc[0], gather_az2<kTileR>(pb + p_az));
-        acc[1] = add2(acc[1], gather_az2<-kTileR>(pb + kProd + p_az));
-      } else if (tneg == 31) {
-        acc[0] = add2(acc[0], gather_az2<-kTileR>(pb + p_az));
-        acc[1] = add2(acc[1], gather_az2<kTileR>(pb + kProd + p_az));
+      if (tneg == 0 || tneg == 31) {
+        // q1's readers at +W, +2W, q2's at -W, -2W
+        const int W = tneg == 0 ? kTileR : -kTileR;
+        acc[0] = add2(acc[0], gather_az2(pb + p_az, W));
+        acc[1] = add2(acc[1], gather_az2(pb + kProd + p_az, -W));
       } else {
 #pragma unroll
         for (int L = 0; L < 2; ++L) {
