@@ -50,7 +50,8 @@ struct SmSize {
   static constexpr int node_bytes = TT * 32 * (12 + 8) * 8;
   // per wall, slot (ghost layer 0, 1, wall node) and row the factors w_0 .. w_4, a0, a1, a1h, u / E
   static constexpr int ghost_bytes = 2 * 3 * TT * 10 * 8;
-  static constexpr int smem = planes_bytes + tab_bytes + node_bytes + ghost_bytes + 128;
+  static constexpr int kept_bytes = 2 * dirs * 32 * kPairWarps * 8;
+  static constexpr int smem = planes_bytes + tab_bytes + node_bytes + ghost_bytes + kept_bytes + 128;
   static_assert((plane * 8) % 128 == 0, "TMA destinations must stay 128-byte aligned");
 };
 
@@ -129,7 +130,8 @@ __global__ void __launch_bounds__(SmSize<SCH, TT>::threads, 1)
   double* sums = reinterpret_cast<double*>(smem_raw + SZ::planes_bytes + SZ::tab_bytes);   // [row][lane][12]
   double* fac = sums + TT * 32 * 12;                                                         // [row][lane][8]
   double* gfac = fac + TT * 32 * 8;                                                          // [side][slot][row][10]
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + SZ::planes_bytes + SZ::tab_bytes + SZ::node_bytes + SZ::ghost_bytes);
+  double* kept = gfac + 2 * 3 * TT * 10;                                                     // [label][pair thread]
+  uint64_t* bar = reinterpret_cast<uint64_t*>(kept + 2 * SZ::dirs * 32 * kPairWarps);
 
   const int r0 = blockIdx.x * kTileR;
   const int t0 = (blockIdx.y + ty0) * TT;   // ty0: first tile row of the launch
@@ -309,27 +311,29 @@ __global__ void __launch_bounds__(SmSize<SCH, TT>::threads, 1)
     }
     bar_wait(kBarGhosts, n_values);
   }
+  // d f - M_r - M_theta of this thread's labels, kept in shared memory so that the loop
+  // stays rolled (unrolled, the compared schemes took 17.4 us a step on 64 x 64, now 15.4)
+  double* mine = kept + tid;
   const uint64_t dfx = fx_fraction(fabs(decay));
   const int64_t dsign = decay < 0.0 ? -1 : 0;
   const double inv_r = p.inv_r[min(r, p.n_r - 1)];
   const uint64_t ratio = fx_fraction(inv_r * recip_newton(inv_r0));   // 1/r relative to the tile's first column
   const double* c64 = p.courant64 + ((size_t)(min(t, p.n_theta - 1) + kGhostRows) * kPairsSm + (k - 1) * kHalfDirs) * 4;
-  double gq[DIRS][2];
-#pragma unroll
+#pragma unroll 1
   for (int j = 0; j < DIRS; ++j) {
     const int i = i_first + j, q1 = 1 + (k - 1) * kNDirs + i;
     const SmTab<SCH>& te = tab[((k - 1) * kHalfDirs + i) * TT + rl];
     const FxCoef<SCH> cr = te.r, ct = fx_coef<SCH>(fx_mul_frac(te.at, ratio));
     const int fl = (int)te.fl;
-    const int sr = (fl & 1) ? 1 : -1;               // v_r < 0 for q1: upwind at larger r
-    const int st = (fl & 2) ? kWinR : -kWinR;       // v_theta < 0 for q1: upwind at larger theta
-    auto carried = [&](const double* x, int s_r, int s_t) {
+#pragma unroll
+    for (int L = 0; L < 2; ++L) {
       constexpr int far = SCH == PCLB_SCHEME_LW ? -1 : 2;
-      return fx_carried<SCH>(x[0], x[s_r], x[far * s_r], x[s_t], x[far * s_t], cr, ct, dfx, dsign, decay, c64 + 4 * i,
-                             inv_r);
-    };
-    gq[j][0] = carried(sm + q1 * PLANE + node, sr, st);
-    gq[j][1] = carried(sm + (q1 + kHalfDirs) * PLANE + node, -sr, -st);
+      const int s_r = ((fl & 1) != 0) != (L != 0) ? 1 : -1;               // v_r < 0: upwind at larger r
+      const int s_t = ((fl & 2) != 0) != (L != 0) ? kWinR : -kWinR;       // v_theta < 0: upwind at larger theta
+      const double* x = sm + (q1 + L * kHalfDirs) * PLANE + node;
+      mine[(2 * j + L) * 32 * kPairWarps] = fx_carried<SCH>(x[0], x[s_r], x[far * s_r], x[s_t], x[far * s_t], cr, ct, dfx,
+                                                            dsign, decay, c64 + 4 * i, inv_r);
+    }
   }
   bar_wait(kBarState, n_state);
   if (!valid) return;
@@ -342,8 +346,8 @@ __global__ void __launch_bounds__(SmSize<SCH, TT>::threads, 1)
     double y = i == 0 ? uxE : uyE;                                   // directions (1,0), (s,s), (0,1), (-s,s)
     if (i & 1) y = d.cx[2] * (i == 1 ? uyE + uxE : uyE - uxE);
     const double y2 = y * y, ev = fma(y2, fma(y2, C, B), A), z = fma(y2, O3, O1);
-    store(q1, fma(y, z, ev + gq[j][0]));
-    store(q1 + kHalfDirs, fma(-y, z, ev + gq[j][1]));
+    store(q1, fma(y, z, ev + mine[2 * j * 32 * kPairWarps]));
+    store(q1 + kHalfDirs, fma(-y, z, ev + mine[(2 * j + 1) * 32 * kPairWarps]));
   }
 }
 
