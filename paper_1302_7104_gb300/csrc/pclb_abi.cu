@@ -312,8 +312,7 @@ pclb_status encode_map(pclb_ctx* ctx, const void* base, int box_rows, CUtensorMa
 
 int adj_box_rows(const pclb_ctx* ctx) { return ctx->sp.adj_rows + 4; }
 
-// Tile rows of the adjoint: 16 in FP32; in FP64 8, or 4 where tiles of 8 rows
-// would leave SMs (152) without one.
+// Tile rows of the adjoint: 16 in FP32; in FP64 8, or 4 on small grids.
 int adj_tile_rows(const pclb_grid* g, pclb_precision prec) {
   if (prec == PCLB_FP32) return kAdjRows32;
   const long long tiles = (long long)((g->n_r + kTileR - 1) / kTileR) * ((g->n_theta + kAdjRows64 - 1) / kAdjRows64);

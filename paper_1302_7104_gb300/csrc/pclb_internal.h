@@ -33,20 +33,22 @@ constexpr int kCtasPerSm32 = 2;
 // rows on at most kTinyGridTiles64 (one wave).  FP64, us per step with tiles
 // of 2 / 4 / 16 rows: 64 x 128 (16 tiles) 15.1 / 22.3 / 52.4, 64 x 256 (32)
 // 30.0 / 22.5 / 52.6, 128 x 304 (76) 59.6 / 44.5 / 52.6, 128 x 608 (152)
-// 112 / 88.6 / 53.6.
+// 112 / 88.6 / 53.6.  FP32, us per step with 4 / 16: 64 x 128 7.5 / 13.1, 64 x
+// 608 (76) 8.9 / 13.3, 128 x 400 (100) 15.0 / 13.5.
 constexpr int kTileTSmall = 4;
 constexpr int kSmallGridTiles = 76, kTinyGridTiles64 = 19;
 constexpr int kWinR = kTileR + 8;   // 40 columns
-constexpr int kWinT = kTileT + 4;   // 20 rows
 constexpr int kLeft = 4;            // column of interior r0 inside the window
-constexpr int kStepThreads = 256;   // 8 warps; each thread owns 2 nodes (rows w and w + 8)
 constexpr int kPitchAlign = 32;     // row pitch in elements (128 B for float)
 constexpr int kGhostRows = 2;       // azimuthal ghost rows stored on each side
 // Tile rows of the adjoint kernel (its window holds f and lam for all labels).
 constexpr int kAdjRows32 = 16;
 constexpr int kAdjRows64 = 8;
 constexpr int kAdjRows64Small = 4;    // FP64 on grids of at most kSmallGridTilesAdj tiles of 8 rows
-constexpr int kSmallGridTilesAdj = 152;
+// us per adjoint step with tiles of 4 / 8 rows: 64 x 304 (76 tiles of 8) 102 /
+// 150, 128 x 304 (152) 155 / 150, 128 x 400 (200) 212 / 252, 128 x 608 (304) 279 /
+// 254: up to three of the small ones to an SM (152).
+constexpr int kSmallGridTilesAdj = 228;
 // Time a kernel waits for the TMA copies of its own window (mbarrier phase)
 // before it reports PCLB_FLAG_TIMEOUT and gives the tile up; the copies of a
 // tile given up get the default limit again to land before the CTA exits.

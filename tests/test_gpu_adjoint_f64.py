@@ -89,3 +89,16 @@ def test_non_finite_values_stay_local_and_are_flagged():
     far = np.ones(f.shape, dtype=bool)
     far[:, 8:17, 46:55] = False
     assert not bad[far].any()
+
+
+# the line between tiles of 4 and 8 rows: 228 tiles of 32 x 8
+@pytest.mark.parametrize("n_r,n_t", [(32, 1824), (33, 905), (32, 1825)])
+def test_adjoint_matches_oracle_beside_the_line_of_the_tile_rule(n_r, n_t):
+    w = I.random_smooth(n_r, n_t, seed=n_t, bc_kind=(I.BC_WALL | I.BC_NEQ, I.BC_EXTRAP))
+    f = _state(w)
+    lam = np.random.default_rng(4).normal(size=f.shape)
+    got, flags = _adjoint(w, f, lam)
+    q, t, r = _sample(w, n_r + n_t)
+    want = O.adjoint_entries(w, f, lam, q, t, r)
+    assert flags == 0
+    assert np.max(np.abs(got[q, t, r] - want)) <= 1e-12 * np.max(np.abs(lam))
