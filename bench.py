@@ -362,7 +362,7 @@ def run_ours(args):
                    "reverse_step_ms": t_rev * 1e3, "reverse_ratio_to_forward": t_rev / per_launch,
                    "roofline": {"bound": "hbm", "achieved": alg / t_adj / 1e9, "peak": hbm, "unit": "GB/s",
                                 "frac": alg / t_adj / 1e9 / hbm, "alg_bytes_per_launch": alg,
-                                "kernel": "pclb::adjoint_pair_f32x2 (+ adjoint_wall_kernel on a side stream)"}}
+                                "kernel": "pclb::adjoint_pair_f32x2"}}
         del state
 
     # non-equilibrium manifestations (Sec. IV), all four groups, on the same state
@@ -385,7 +385,7 @@ def run_ours(args):
         noneq = {"ms": t_n * 1e3, "groups": 4, "fields": 48,
                  "roofline": {"bound": "hbm", "achieved": nbytes / t_n / 1e9, "peak": hbm, "unit": "GB/s",
                               "frac": nbytes / t_n / 1e9 / hbm, "alg_bytes_per_launch": nbytes,
-                              "kernel": "pclb::noneq_kernel<float>"}}
+                              "kernel": "pclb::noneq_f32_kernel"}}
         del out
     g.close()
 

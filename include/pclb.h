@@ -49,7 +49,8 @@
  * float-float velocity constants.  The adjoint step (PCLB_FP32) takes each
  * node's state from the same float-float moments, rounded to float, and
  * evaluates the cotangents in float (the ghost states at the walls in
- * double).  PCLB_FP64 computes everything in double.
+ * double).  PCLB_FP64 keeps double precision throughout; its step forms sums,
+ * differences and convection increments in 64-bit fixed point.
  */
 #ifndef PCLB_H
 #define PCLB_H
