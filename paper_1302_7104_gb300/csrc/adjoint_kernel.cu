@@ -39,7 +39,10 @@
 // and quarter SM); the partials are therefore formed in integers
 // (fx_mwb_partials, 10 of 14 FP64 operations less per label and direction).
 // TT = 8 rows, one thread per node; on grids whose tiles would leave SMs idle
-// 4 rows and two threads per node (LS = 2), one label of each pair each.
+// 4 rows and two threads per node (LS = 2), one label of each pair each, or 2
+// rows and four threads (LS = 4), which also work on two pairs at a time (half
+// the barriers): 64 x 128, 72.5 us per adjoint step with LS = 4, 102 with LS = 2,
+// 150 with 8 rows.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -70,10 +73,12 @@ constexpr int kAdjStages = 2;   // ring depth of the pair-streaming kernel (2 me
 static_assert(sizeof(EqParams<float>) == 10 * sizeof(float) && sizeof(EqParams<double>) == 10 * sizeof(double),
               "ghost-state scratch holds 10 values per EqParams");
 
-// TT rows; LS = 2: two threads per node, one label of each pair each.
+// TT rows; LS = 2: two threads per node, one label of each pair each; LS = 4:
+// four, and two pairs at a time.
 template <int TT, int LS>
 struct AdjSize {
   static constexpr int threads = 32 * TT * LS;
+  static constexpr int pp = LS == 4 ? 2 : 1;   // pairs at a time
   static constexpr int min_blocks = 2;   // what shared memory allows
   static constexpr int plane = kWinR * (TT + 4);
   static constexpr int npairs = 4 * kNDirs / 2;
@@ -81,13 +86,13 @@ struct AdjSize {
   // columns -2 .. 33), azimuthal A, B over TT + 4 rows (-2 .. TT + 1) x 32
   static constexpr int rcols = kTileR + 4;
   static constexpr int prod = 2 * TT * rcols + 2 * (TT + 4) * kTileR;
-  static constexpr int ring_bytes = kAdjStages * 4 * plane * 8;   // f, f', lam, lam' per stage
-  static constexpr int prod_bytes = 2 * 2 * prod * 8;             // 2 buffers x 2 labels
+  static constexpr int ring_bytes = kAdjStages * pp * 4 * plane * 8;   // f, f', lam, lam' per stage and pair
+  static constexpr int prod_bytes = 2 * pp * 2 * prod * 8;             // 2 buffers x 2 labels of each pair
   static constexpr int ratio_bytes = kTileR * 8;
   static constexpr int tab_bytes = (TT + 4) * npairs * (int)sizeof(CourEntry);
   static constexpr int ghost_bytes = 2 * 2 * TT * kQ * 8;         // both walls' ghost values
   static constexpr int smem = ring_bytes + prod_bytes + ratio_bytes + tab_bytes + ghost_bytes + 128;
-  static_assert(LS == 1 || 2 * 12 * 32 * TT * 8 <= prod_bytes, "exchange of the node phase inside the product buffers");
+  static_assert(LS == 1 || LS * 12 * 32 * TT * 8 <= prod_bytes, "exchange of the node phase inside the product buffers");
   // the ring's planes are TMA destinations: 128-byte aligned
   static_assert((plane * 8) % 128 == 0, "TMA destinations must stay 128-byte aligned");
 };
@@ -187,14 +192,14 @@ __global__ void __launch_bounds__(AdjSize<TT, LS>::threads, AdjSize<TT, LS>::min
   using SZ = AdjSize<TT, LS>;
   constexpr int PLANE = SZ::plane;
   constexpr int NP = SZ::npairs, RC = SZ::rcols, PROD = SZ::prod;
-  constexpr int S = kAdjStages;
+  constexpr int S = kAdjStages, PP = SZ::pp, NIT = NP / PP;   // stages; pairs at a time, iterations
   // offsets inside one label's products
   constexpr int AR = 0, BR = TT * RC, AT = 2 * TT * RC, BT = 2 * TT * RC + (TT + 4) * kTileR;
-  constexpr uint32_t kStageBytes = (uint32_t)(4 * PLANE * sizeof(T));
+  constexpr uint32_t kStageBytes = (uint32_t)(PP * 4 * PLANE * sizeof(T));
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  T* ring = reinterpret_cast<T*>(smem_raw);                 // [stage][f q1, f q2, lam q1, lam q2][PLANE]
-  T* prod = ring + S * 4 * PLANE;                             // [buffer][label][products]
-  uint64_t* ratio = reinterpret_cast<uint64_t*>(prod + 2 * 2 * PROD);   // 1/r of the tile columns relative to the first
+  T* ring = reinterpret_cast<T*>(smem_raw);                 // [stage][pair][f q1, f q2, lam q1, lam q2][PLANE]
+  T* prod = ring + S * PP * 4 * PLANE;                        // [buffer][pair][label][products]
+  uint64_t* ratio = reinterpret_cast<uint64_t*>(prod + 2 * PP * 2 * PROD);   // 1/r of the tile columns relative to the first
   CourEntry* ctab = reinterpret_cast<CourEntry*>(ratio + kTileR);        // [TT + 4][NP]
   T* gval = reinterpret_cast<T*>(ctab + (TT + 4) * NP);                  // [side][layer][TT][Q] ghost values
   uint64_t* bar = reinterpret_cast<uint64_t*>(gval + 2 * 2 * TT * kQ);   // [S]
@@ -206,18 +211,22 @@ __global__ void __launch_bounds__(AdjSize<TT, LS>::threads, AdjSize<TT, LS>::min
   const int tid = threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5;
   const int rowl = warp % TT;               // tile row
-  const int half_of = warp / TT;            // LS = 2: this thread's label of each pair (and half of the shells)
+  const int part = warp / TT;               // of LS threads per node
+  const int half_of = part & 1, pair_of = part >> 1;   // this thread's label of a pair, and pair of those at a time
 
-  // the planes of pair pr (labels q1, q1 + N_i/2) into stage s (thread 0)
-  auto issue_pair = [&](int pr, int s) {
-    const int k = 1 + pr / (kNDirs / 2);
-    const int q1 = 1 + (k - 1) * kNDirs + pr % (kNDirs / 2), q2 = q1 + kNDirs / 2;
-    T* st = ring + s * 4 * PLANE;
+  // the planes of iteration it's pairs (labels q1, q1 + N_i/2) into stage s (thread 0)
+  auto issue_pairs = [&](int it, int s) {
     mbar_arrive_expect_tx(&bar[s], kStageBytes);
-    tma_load_3d(st, &tmap_f, r0 - kLeft, t0, q1, &bar[s]);
-    tma_load_3d(st + PLANE, &tmap_f, r0 - kLeft, t0, q2, &bar[s]);
-    tma_load_3d(st + 2 * PLANE, &tmap_l, r0 - kLeft, t0, q1, &bar[s]);
-    tma_load_3d(st + 3 * PLANE, &tmap_l, r0 - kLeft, t0, q2, &bar[s]);
+#pragma unroll
+    for (int j = 0; j < PP; ++j) {
+      const int pr = it * PP + j, k = 1 + pr / (kNDirs / 2);
+      const int q1 = 1 + (k - 1) * kNDirs + pr % (kNDirs / 2), q2 = q1 + kNDirs / 2;
+      T* st = ring + (s * PP + j) * 4 * PLANE;
+      tma_load_3d(st, &tmap_f, r0 - kLeft, t0, q1, &bar[s]);
+      tma_load_3d(st + PLANE, &tmap_f, r0 - kLeft, t0, q2, &bar[s]);
+      tma_load_3d(st + 2 * PLANE, &tmap_l, r0 - kLeft, t0, q1, &bar[s]);
+      tma_load_3d(st + 3 * PLANE, &tmap_l, r0 - kLeft, t0, q2, &bar[s]);
+    }
   };
   if (tid == 0) {
     tma_prefetch_desc(&tmap_f);
@@ -264,7 +273,7 @@ __global__ void __launch_bounds__(AdjSize<TT, LS>::threads, AdjSize<TT, LS>::min
   }
   __syncthreads();
   if (tid == 0)
-    for (int s = 0; s < S && s < NP; ++s) issue_pair(s, s);
+    for (int s = 0; s < S && s < NIT; ++s) issue_pairs(s, s);
 
   // ---- this thread's node -----------------------------------------------------
   const int row = 2 + rowl;
@@ -284,11 +293,11 @@ __global__ void __launch_bounds__(AdjSize<TT, LS>::threads, AdjSize<TT, LS>::min
     const size_t off = (size_t)(min(t, p.n_theta - 1) + kGhostRows) * p.pitch + min(r, p.n_r - 1);
     const T* fn = f + off;
     const T* ln = lam_in + off;
-    T* mine = prod + ((rowl * 32 + lane) * 2 + half_of) * 12;    // exchange of the two halves of the shells
-    const T* theirs = prod + ((rowl * 32 + lane) * 2 + (1 - half_of)) * 12;
-    const int k0 = LS == 1 ? 1 : 2 * half_of + 1, k1 = LS == 1 ? 4 : k0 + 1;
+    T* all = prod + (rowl * 32 + lane) * LS * 12;                // exchange of the node's threads, which share the shells
+    T* mine = all + part * 12;
+    const int k0 = LS == 1 ? 1 : 4 / LS * part + 1, k1 = k0 + 4 / LS - 1;
     const T lam0 = ln[0];
-    T m[4] = {half_of == 0 ? fn[0] : T(0), T(0), T(0), T(0)};    // rho, j_x, j_y, e
+    T m[4] = {part == 0 ? fn[0] : T(0), T(0), T(0), T(0)};    // rho, j_x, j_y, e
 #pragma unroll 1
     for (int k = k0; k <= k1; ++k) {
       T S = T(0), D[kNDirs / 2];
@@ -304,24 +313,26 @@ __global__ void __launch_bounds__(AdjSize<TT, LS>::threads, AdjSize<TT, LS>::min
       m[2] = fma(d.speed[k], fma(d.cx[2], D[1] + D[3], D[2]), m[2]);
       m[3] = fma(d.half_v2[k], S, m[3]);
     }
-    if constexpr (LS == 2) {
+    // the sums of the node's threads' values j0 .. j0 + n - 1
+    auto exchange = [&](T* v, int j0, int n) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) mine[j] = m[j];
+      for (int j = 0; j < n; ++j) mine[j0 + j] = v[j];
       __syncthreads();
 #pragma unroll
-      for (int j = 0; j < 4; ++j) m[j] += theirs[j];
-    }
+      for (int j = 0; j < n; ++j) {
+        v[j] = all[j0 + j];
+#pragma unroll
+        for (int o = 1; o < LS; ++o) v[j] += all[o * 12 + j0 + j];
+      }
+    };
+    if constexpr (LS > 1) exchange(m, 0, 4);
     const NodeState<T> st = node_state64(m[0], m[1], m[2], m[3]);
     if (valid && !st.ok) atomicOr(p.status, PCLB_FLAG_NONPHYS);
     T c[6];
-    cotangent_sums(st.ux, st.uy, st.E, d, k0, k1, half_of == 0 ? &lam0 : nullptr,
+    cotangent_sums(st.ux, st.uy, st.E, d, k0, k1, part == 0 ? &lam0 : nullptr,
                    [&](int q) -> T { return ln[(size_t)q * plane]; }, c);
-    if constexpr (LS == 2) {
-#pragma unroll
-      for (int j = 0; j < 6; ++j) mine[4 + j] = c[j];
-      __syncthreads();
-#pragma unroll
-      for (int j = 0; j < 6; ++j) c[j] += theirs[4 + j];
+    if constexpr (LS > 1) {
+      exchange(c, 4, 6);
       __syncthreads();   // read before the pairs' products take the buffer
     }
     const T invE = recip_newton(st.E), s = (st.ux * st.ux + st.uy * st.uy) * invE, rE = st.rho * invE;
@@ -352,28 +363,32 @@ __global__ void __launch_bounds__(AdjSize<TT, LS>::threads, AdjSize<TT, LS>::min
     if (t < 2) lam_out[(size_t)d.recv_hi[q] * plane_out + (size_t)(p.n_theta + kGhostRows + t) * p.pitch + r] = v;
   };
   // rest velocity: no convection
-  if (valid && half_of == 0) store(0, decay * lam_in[(size_t)srow * p.pitch + r] + gs[0] + gs[3] * d.half_v2[0]);
+  if (valid && part == 0) store(0, decay * lam_in[(size_t)srow * p.pitch + r] + gs[0] + gs[3] * d.half_v2[0]);
 
   const bool wall_tile = inner || outer;
 
   bool ok = true;
-  int brk = NP;                                         // the pair at which a wait timed out
+  int brk = NIT;                                        // the iteration at which a wait timed out
 #pragma unroll 1
-  for (int pair = 0; pair < NP; ++pair) {
+  for (int it = 0; it < NIT; ++it) {
+    const int pair = it * PP + pair_of;
     const int k = 1 + pair / (kNDirs / 2);
     const int q1 = 1 + (k - 1) * kNDirs + pair % (kNDirs / 2);
     const int q2 = q1 + kNDirs / 2;                      // opposite velocity
-    const int s = pair % S;
-    const T* st = ring + s * 4 * PLANE;
-    T* pb = prod + (pair & 1) * 2 * PROD;                // this pair's products: [label][...]
-    if (ok) ok = p.wait_ns != 0 && mbar_wait_bounded(&bar[s], (uint32_t)((pair / S) & 1), p.wait_ns);
+    const int s = it % S;
+    T* stage = ring + s * PP * 4 * PLANE;
+    T* buffer = prod + (it & 1) * PP * 2 * PROD;
+    const T* st = stage + pair_of * 4 * PLANE;
+    T* pb = buffer + pair_of * 2 * PROD;                 // this pair's products: [label][...]
+    if (ok) ok = p.wait_ns != 0 && mbar_wait_bounded(&bar[s], (uint32_t)((it / S) & 1), p.wait_ns);
     if (wall_tile) {
-      // radial ghost columns of this pair's f planes: wall, layer, label, row
-      if (tid < 8 * TT && ok) {
-        const int rr = tid % TT, L = tid / TT & 1, l = tid / (2 * TT) & 1, side = tid / (4 * TT);
-        const int c = (side == 0 ? kLeft : cw_out) - (side == 0 ? 1 : -1) * (1 + l);
+      // radial ghost columns of the pairs' f planes: pair, wall, layer, label, row
+      if (tid < 8 * TT * PP && ok) {
+        const int rr = tid % TT, L = tid / TT & 1, l = tid / (2 * TT) & 1, side = tid / (4 * TT) & 1, j = tid / (8 * TT);
+        const int c = (side == 0 ? kLeft : cw_out) - (side == 0 ? 1 : -1) * (1 + l), pr = it * PP + j;
+        const int q = 1 + pr / (kNDirs / 2) * kNDirs + pr % (kNDirs / 2) + L * (kNDirs / 2);
         if ((side == 0 ? inner : outer) && t0 + rr < p.n_theta && c >= 0 && c < kWinR)
-          const_cast<T*>(st)[L * PLANE + (2 + rr) * kWinR + c] = gval[((side * 2 + l) * TT + rr) * kQ + (L ? q2 : q1)];
+          stage[(j * 4 + L) * PLANE + (2 + rr) * kWinR + c] = gval[((side * 2 + l) * TT + rr) * kQ + q];
       }
       __syncthreads();
     }
@@ -408,38 +423,40 @@ __global__ void __launch_bounds__(AdjSize<TT, LS>::threads, AdjSize<TT, LS>::min
         products(fw, up_t(L), lam_c[j], pb + L * PROD + p_az, BT - AT, a2, k2);
       }
     }
-    if (warp < 4) {
+    if (warp < 4 * PP) {
       // halo rows: window rows 0, 1, TT + 2, TT + 3; rows above the tile are
       // read by labels whose upwind side is +theta
-      const int rr = warp < 2 ? warp : TT + warp;
-      const CourEntry eh = ctab[rr * NP + pair];
+      const int h = warp & 3, j = warp >> 2, rr = h < 2 ? h : TT + h;
+      const CourEntry eh = ctab[rr * NP + it * PP + j];
       const bool q1_up_pos = (eh.fl & 2) != 0;
       uint64_t a2, k2;
       azimuthal(eh.at, a2, k2);
-      const int L = (warp < 2) == q1_up_pos ? 0 : 1, o = rr * kWinR + col;
-      products(sfp + L * PLANE + o, warp < 2 ? kWinR : -kWinR, slp[L * PLANE + o], pb + L * PROD + AT + rr * kTileR + lane,
-               BT - AT, a2, k2);
-    } else if (warp == 4) {
-      // halo columns: 4 per tile row (label, column).  Upwind at larger r (+1)
-      // reads the tile from columns -2, -1, at smaller r from 32, 33.
-      static_assert(4 * TT <= 32 && TT * LS >= 5, "halo columns: one warp");
-      if (lane < 4 * TT) {
-        const int hr = lane >> 2, L = (lane >> 1) & 1, j = lane & 1;
-        const CourEntry eh = ctab[(hr + 2) * NP + pair];
+      const int L = (h < 2) == q1_up_pos ? 0 : 1, o = rr * kWinR + col;
+      const T* w = stage + j * 4 * PLANE + L * PLANE + o;
+      products(w, h < 2 ? kWinR : -kWinR, w[2 * PLANE], buffer + (j * 2 + L) * PROD + AT + rr * kTileR + lane, BT - AT, a2,
+               k2);
+    }
+    if (warp == (PP == 1 ? 4 : TT * LS - 1)) {
+      // halo columns: 4 per pair and tile row (label, column).  Upwind at larger r
+      // (+1) reads the tile from columns -2, -1, at smaller r from 32, 33.
+      static_assert(4 * TT * PP <= 32 && TT * LS >= 5 && TT * LS >= 4 * PP, "halo rows and columns: a warp each");
+      if (lane < 4 * TT * PP) {
+        const int hr = (lane >> 2) % TT, j = lane / (4 * TT), L = (lane >> 1) & 1, i = lane & 1;
+        const CourEntry eh = ctab[(hr + 2) * NP + it * PP + j];
         const int u = ((eh.fl & 1) != 0) != (L != 0) ? 1 : -1;
-        const int c = u == 1 ? j - 2 : kTileR + j;
-        const int o = L * PLANE + (hr + 2) * kWinR + c + kLeft;
-        products(sfp + o, u, slp[o], pb + L * PROD + AR + hr * RC + c + 2, BR - AR, eh.a2, eh.k2);
+        const int c = u == 1 ? i - 2 : kTileR + i;
+        const T* w = stage + (j * 4 + L) * PLANE + (hr + 2) * kWinR + c + kLeft;
+        products(w, u, w[2 * PLANE], buffer + (j * 2 + L) * PROD + AR + hr * RC + c + 2, BR - AR, eh.a2, eh.k2);
       }
     }
     if (__syncthreads_or(!ok)) {
-      brk = pair;
+      brk = it;
       break;
     }
-    // the stage of this pair is free: the planes of pair + S start now
-    if (tid == 0 && pair + S < NP) {
+    // the stage is free: the planes of iteration it + S start now
+    if (tid == 0 && it + S < NIT) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      issue_pair(pair + S, s);
+      issue_pairs(it + S, s);
     }
 
     // (B) gather at this node
@@ -469,11 +486,11 @@ __global__ void __launch_bounds__(AdjSize<TT, LS>::threads, AdjSize<TT, LS>::min
       }
     }
   }
-  if (brk < NP && tid == 0) {
+  if (brk < NIT && tid == 0) {
     // a copy did not land in time: report it, give the copies still in
     // flight (the last one issued into each stage) a bounded time to finish
     atomicOr(p.status, PCLB_FLAG_TIMEOUT);
-    const int issued = brk + S < NP ? brk + S : NP;
+    const int issued = brk + S < NIT ? brk + S : NIT;
     for (int s = 0; s < S && s < issued; ++s) {
       const int last = s + ((issued - 1 - s) / S) * S;
       mbar_wait_bounded(&bar[s], (uint32_t)((last / S) & 1), kDefaultWaitNs);
@@ -510,7 +527,8 @@ cudaError_t launch_adjoint(const CUtensorMap* tmap_f, const CUtensorMap* tmap_l,
                                adjoint_smem(AdjSize<TT, LS>::smem, order.blocks()), stream, *tmap_f, *tmap_l, f, lam_in, lam_out, ws, order, p, d);
     };
     if (rows == kAdjRows64) return go(std::integral_constant<int, kAdjRows64>{}, std::integral_constant<int, 1>{});
-    return go(std::integral_constant<int, kAdjRows64Small>{}, std::integral_constant<int, 2>{});
+    if (rows == kAdjRows64Small) return go(std::integral_constant<int, kAdjRows64Small>{}, std::integral_constant<int, 2>{});
+    return go(std::integral_constant<int, kAdjRows64Tiny>{}, std::integral_constant<int, 4>{});
   }
 }
 

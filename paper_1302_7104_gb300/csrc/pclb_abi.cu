@@ -316,6 +316,7 @@ int adj_box_rows(const pclb_ctx* ctx) { return ctx->sp.adj_rows + 4; }
 int adj_tile_rows(const pclb_grid* g, pclb_precision prec) {
   if (prec == PCLB_FP32) return kAdjRows32;
   const long long tiles = (long long)((g->n_r + kTileR - 1) / kTileR) * ((g->n_theta + kAdjRows64 - 1) / kAdjRows64);
+  if (tiles <= kTinyGridTilesAdj) return kAdjRows64Tiny;
   return tiles <= kSmallGridTilesAdj ? kAdjRows64Small : kAdjRows64;
 }
 

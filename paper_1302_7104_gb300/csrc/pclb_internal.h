@@ -49,6 +49,10 @@ constexpr int kAdjRows64Small = 4;    // FP64 on grids of at most kSmallGridTile
 // 150, 128 x 304 (152) 155 / 150, 128 x 400 (200) 212 / 252, 128 x 608 (304) 279 /
 // 254: up to three of the small ones to an SM (152).
 constexpr int kSmallGridTilesAdj = 228;
+// 2 rows on at most kTinyGridTilesAdj (one of their blocks to an SM): 64 x 152
+// (38) 72.6 us against 102 with 4 rows, 64 x 304 (76) 103 against 101.
+constexpr int kAdjRows64Tiny = 2;
+constexpr int kTinyGridTilesAdj = 38;
 // Time a kernel waits for the TMA copies of its own window (mbarrier phase)
 // before it reports PCLB_FLAG_TIMEOUT and gives the tile up; the copies of a
 // tile given up get the default limit again to land before the CTA exits.

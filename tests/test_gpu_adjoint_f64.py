@@ -102,3 +102,18 @@ def test_adjoint_matches_oracle_beside_the_line_of_the_tile_rule(n_r, n_t):
     want = O.adjoint_entries(w, f, lam, q, t, r)
     assert flags == 0
     assert np.max(np.abs(got[q, t, r] - want)) <= 1e-12 * np.max(np.abs(lam))
+
+
+# tiles of 2 rows up to 38 tiles of 32 x 8: both sides, last tiles of one row and of one to three columns
+@pytest.mark.parametrize("n_r,n_t", [(32, 304), (32, 305), (33, 150), (34, 31), (35, 2), (3, 9), (99, 21)])
+@pytest.mark.parametrize("bc", [(I.BC_EXTRAP, I.BC_EXTRAP), (I.BC_WALL | I.BC_NEQ, I.BC_DIRICHLET | I.BC_NEQ)])
+def test_tiles_of_two_rows_match_oracle(n_r, n_t, bc):
+    w = I.random_smooth(n_r, n_t, seed=n_r + n_t, bc_kind=bc, amp=0.02 if n_r < 8 else 0.2)
+    f = _state(w)
+    lam = np.random.default_rng(8).normal(size=f.shape)
+    got, flags = _adjoint(w, f, lam)
+    q, t, r = _sample(w, n_r + n_t)
+    t = np.clip(t, 0, n_t - 1)
+    want = O.adjoint_entries(w, f, lam, q, t, r)
+    assert flags == 0
+    assert np.max(np.abs(got[q, t, r] - want)) <= 1e-12 * np.max(np.abs(lam))
