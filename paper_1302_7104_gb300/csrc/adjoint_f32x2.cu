@@ -387,7 +387,7 @@ __device__ __forceinline__ f2 gather_az2(const float* P, int W) {
 template <bool WALLS>
 __device__ __forceinline__ void adjoint_tile(const CUtensorMap& tmap_f, const CUtensorMap& tmap_l,
                                              const CUtensorMap& tmap_fn, const CUtensorMap& tmap_ln,
-                                             const float* __restrict__ f, const float* __restrict__ lam_in,
+                                             const float* f, const float* lam_in,
                                              float* __restrict__ lam_out, const WallScratch<float>& ws, int tx, int ty,
                                              bool last_tile, const StepParams& p, const DvmConst<float>& d) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -719,7 +719,7 @@ __device__ __forceinline__ void adjoint_tile(const CUtensorMap& tmap_f, const CU
 __global__ void __launch_bounds__(kAThr, 3)
     adjoint_pair_f32x2(const __grid_constant__ CUtensorMap tmap_f, const __grid_constant__ CUtensorMap tmap_l,
                        const __grid_constant__ CUtensorMap tmap_fn, const __grid_constant__ CUtensorMap tmap_ln,
-                       const float* __restrict__ f, const float* __restrict__ lam_in, float* __restrict__ lam_out,
+                       const float* f, const float* lam_in, float* __restrict__ lam_out,
                        const __grid_constant__ WallScratch<float> ws, const __grid_constant__ AdjOrder order,
                        const __grid_constant__ StepParams p, const __grid_constant__ DvmConst<float> d) {
   int tx, ty;

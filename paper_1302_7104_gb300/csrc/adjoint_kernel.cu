@@ -185,7 +185,7 @@ __device__ __forceinline__ void cotangent_sums(double ux, double uy, double E, c
 template <int TT, int LS>
 __global__ void __launch_bounds__(AdjSize<TT, LS>::threads, AdjSize<TT, LS>::min_blocks)
     adjoint_pair_kernel(const __grid_constant__ CUtensorMap tmap_f, const __grid_constant__ CUtensorMap tmap_l,
-                        const double* __restrict__ f, const double* __restrict__ lam_in, double* __restrict__ lam_out,
+                        const double* f, const double* lam_in, double* __restrict__ lam_out,
                         const __grid_constant__ WallScratch<double> ws, const __grid_constant__ AdjOrder order,
                         const __grid_constant__ StepParams p, const __grid_constant__ DvmConst<double> d) {
   using T = double;

@@ -91,7 +91,7 @@ struct WallShared {
 // cycles and quarter SM): they are formed once per row, a lane each, instead of
 // in every lane of a warp per row.
 template <class T, int TT>
-__device__ __noinline__ void adjoint_walls(const T* __restrict__ f, const T* __restrict__ lam, int side, int slot,
+__device__ __noinline__ void adjoint_walls(const T* f, const T* lam, int side, int slot,
                                            int t0, const WallScratch<T>& ws, WallShared<T, TT>& sh, T* values,
                                            const StepParams& p, const DvmConst<T>& d) {
   const int tid = threadIdx.x;

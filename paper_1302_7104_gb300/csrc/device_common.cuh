@@ -99,7 +99,9 @@ __device__ __forceinline__ bool barrier_or(int id, int threads, bool pred) {
 
 // Programmatic dependent launch: wait for the grid launched before this one
 // on the stream (its results are then visible), and let the grid after this
-// one start.  Without the launch attribute both return at once.
+// one start.  Without the launch attribute both return at once.  What a kernel
+// reads after pdl_wait() comes through pointers without const __restrict__: loads
+// through those count as invariant and may be moved above it.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

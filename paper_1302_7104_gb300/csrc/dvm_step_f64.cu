@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(32 * kParts)
 // the states and the factors.  Bound by the latency of ~150 dependent operations.
 template <int ND>
 __global__ void __launch_bounds__(32 * kGhostWarps)
-    gen_ghost_kernel(const double* __restrict__ f, double* __restrict__ ghost, const __grid_constant__ StepParams p,
+    gen_ghost_kernel(const double* f, double* __restrict__ ghost, const __grid_constant__ StepParams p,
                      const __grid_constant__ DvmG d) {
   constexpr int H = ND / 2, NP = 4 * H, N = (NP + 31) / 32;
   __shared__ GenFactors fac[kGhostWarps][3];
@@ -235,7 +235,7 @@ struct GenTab {
 
 template <int SCH, int ND>
 __global__ void __launch_bounds__(32 * (kParts + 1), 5)
-    gen_step_kernel(const double* __restrict__ f, double* __restrict__ f_out, const double* __restrict__ ghost,
+    gen_step_kernel(const double* f, double* __restrict__ f_out, const double* ghost,
                     const __grid_constant__ StepParams p, const __grid_constant__ DvmG d) {
   constexpr int H = ND / 2, NP = 4 * H, DIRS = H / kParts;
   __shared__ GenTab<SCH> tab[NP];

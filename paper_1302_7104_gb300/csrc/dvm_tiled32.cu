@@ -56,7 +56,7 @@ struct TiledSize {
   static constexpr int smem = ring_bytes + tab_bytes + ghost_bytes + 8 * kTStages + 64;
 };
 
-__device__ __forceinline__ f2 ldg2(const float* p) { return __ldg(reinterpret_cast<const float2*>(p)); }
+__device__ __forceinline__ f2 ldg2(const float* p) { return *reinterpret_cast<const float2*>(p); }
 __device__ __forceinline__ f2 lds2(const float* p) { return *reinterpret_cast<const float2*>(p); }
 
 __device__ __forceinline__ float rcp_approx_t(float x) {
@@ -193,7 +193,7 @@ __device__ __forceinline__ ff2 ff2_from_double(double v) {
 // two halves of the packed arithmetic.  Writes their equilibrium factors (11
 // pairs) and those of the wall node (11) to out.
 template <int ND>
-__device__ __noinline__ void tiled_ghost_state(const float* __restrict__ f, float* out, int side, int t,
+__device__ __noinline__ void tiled_ghost_state(const float* f, float* out, int side, int t,
                                                const StepParams& p, const DvmG32& c) {
   const size_t plane = (size_t)p.rows * p.pitch;
   const int ra = side == 0 ? 0 : p.n_r - 1, rb = side == 0 ? 1 : p.n_r - 2;
@@ -201,7 +201,7 @@ __device__ __noinline__ void tiled_ghost_state(const float* __restrict__ f, floa
   const float* fb = f + (size_t)(t + kGhostRows) * p.pitch + rb;
   // node a in the low half, node b in the high half
   ff2 m[4];
-  tiled_moments<ND>([&](int q) { return mk2(__ldg(fa + (size_t)q * plane), __ldg(fb + (size_t)q * plane)); }, c,
+  tiled_moments<ND>([&](int q) { return mk2(fa[(size_t)q * plane], fb[(size_t)q * plane]); }, c,
                     m[0], m[1], m[2], m[3]);
   bool ok = phys_x(m[0], m[1], m[2], m[3]) && phys_y(m[0], m[1], m[2], m[3]);
   const TEq ea = tiled_factors(m[0], m[1], m[2], m[3], c);
@@ -300,7 +300,7 @@ __device__ __forceinline__ void tupd(const float* w, f2 nar, f2 nkr, f2 nat, f2 
 // instantiations): 12% faster than two CTAs at 124 registers.
 template <int ND, int SCH>
 __global__ void __launch_bounds__(kTThreads, 3)
-    tiled_step_f32(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ f, float* __restrict__ f_out,
+    tiled_step_f32(const __grid_constant__ CUtensorMap tmap, const float* f, float* __restrict__ f_out,
                    const __grid_constant__ StepParams p, const __grid_constant__ DvmG d,
                    const __grid_constant__ DvmG32 c) {
   using TS = TiledSize<ND>;
