@@ -8,7 +8,9 @@
 // shell in the tile's window: one unit is at most 2^-58 of the largest value,
 // finer than the double's own spacing for every value within 2^-5 of it, where
 // the conversion is exact.  Sums and differences of these numbers are exact;
-// products drop less than two units.
+// conversions and products round to the nearest unit.  (Both used to drop what is
+// below a unit: next to gas 20 times as dense, thin gas then lost 1e-16 of its
+// mass in every step.)
 #pragma once
 
 #include <cuda_runtime.h>
@@ -25,48 +27,61 @@ namespace pclb {
 // infinity (0x7ff) are outside.
 constexpr int kFxMinExp = 128, kFxMaxExp = 1900;
 
-// f as fixed point; its biased exponent must not exceed ek.
+// f as fixed point, rounded to the nearest (ties to even, decided on five bits
+// below the unit); its biased exponent must not exceed ek.
 __device__ __forceinline__ int64_t fx_from_double(double f, int ek) {
   const int hi = __double2hiint(f);
   const uint32_t mh = ((uint32_t)hi & 0xfffffu) | 0x100000u;
-  uint64_t m = ((uint64_t)mh << 32 | (uint32_t)__double2loint(f)) << 6;
+  uint64_t m = ((uint64_t)mh << 32 | (uint32_t)__double2loint(f)) << 11;
   m >>= min(ek - ((hi >> 20) & 0x7ff), 63);
+  m = (m + (15u + (((uint32_t)m >> 5) & 1u))) >> 5;
   const int64_t s = hi >> 31;
   return (int64_t)(m ^ s) - s;
 }
 
-// The double nearest x 2^(ek - 1081) (|x| < 2^63).
+// The double nearest x 2^(ek - 1081) (|x| < 2^63), ties to even: of the few bits
+// that drop out, every fourth pattern or so is a tie.
 __device__ __forceinline__ double fx_to_double(int64_t x, int ek) {
   const int64_t s = x >> 63;
   uint64_t u = (uint64_t)((x ^ s) - s);
   const int lz = __clzll((long long)u);
   u <<= lz & 63;                                        // leading bit at 63
-  const uint64_t r = (u >> 11) + ((u >> 10) & 1);       // 53 bits, the carry runs into the exponent
+  const uint32_t ul = (uint32_t)u;
+  const uint64_t r = (u >> 11) + ((ul & 0x7ffu) + ((ul >> 11) & 1u) > 0x400u ? 1 : 0);   // 53 bits, the carry runs into the exponent
   const uint32_t hi = (uint32_t)(r >> 32) + ((uint32_t)(ek + 4 - lz) << 20) + ((uint32_t)s & 0x80000000u);
   return u == 0 ? 0.0 : __hiloint2double((int)hi, (int)(uint32_t)r);
 }
 
-// c in [0, 1] as a fraction in units of 2^-63 (c < 2^-960 counts as 0).
+// c in [0, 1] as a fraction in units of 2^-63, rounded (c < 2^-960 counts as 0).
 __device__ __forceinline__ uint64_t fx_fraction(double c) {
   const int hi = __double2hiint(c);
   const uint32_t mh = ((uint32_t)hi & 0xfffffu) | 0x100000u;
   const uint64_t m = ((uint64_t)mh << 32 | (uint32_t)__double2loint(c)) << 11;   // 2^63 <= m < 2^64
   const int sh = 1023 - (hi >> 20);                     // c = m 2^-63 2^-sh
-  const uint64_t one = 1ull << 63, x = sh > 63 ? 0 : m >> sh;
+  const uint64_t one = 1ull << 63, x = sh > 63 ? 0 : (sh < 1 ? m : ((m >> (sh - 1)) + 1) >> 1);
   return x < one ? x : one;
 }
 
-// a c 2^-63 for a < 2^61, c <= 2^63 (below the exact product by less than 2).
+// a c 2^-63 for a < 2^61, c <= 2^63, to the nearest (the error is below 1/2 + 2^-31).
 __device__ __forceinline__ uint64_t fx_mul(uint64_t a, uint64_t c) {
   const uint32_t al = (uint32_t)a, ah = (uint32_t)(a >> 32), cl = (uint32_t)c, ch = (uint32_t)(c >> 32);
-  const uint64_t mid = (uint64_t)al * ch + (uint64_t)ah * cl;
+  // in units of 2^32, with half a unit of the result: < 2^63 + 2^61 + 2^33
+  const uint64_t mid = (uint64_t)al * ch + ((uint64_t)ah * cl + 0x40000000u) + __umulhi(al, cl);
   return (uint64_t)(2u * ah) * ch + (mid >> 31);
 }
 
-// a c 2^-63 for fractions a, c <= 2^63.
+// a c 2^-64, else as fx_mul.
+__device__ __forceinline__ uint64_t fx_mul_half(uint64_t a, uint64_t c) {
+  const uint32_t al = (uint32_t)a, ah = (uint32_t)(a >> 32), cl = (uint32_t)c, ch = (uint32_t)(c >> 32);
+  const uint64_t mid = (uint64_t)al * ch + ((uint64_t)ah * cl + 0x80000000u) + __umulhi(al, cl);
+  return (uint64_t)ah * ch + (mid >> 32);
+}
+
+// a c 2^-63 for fractions a, c <= 2^63, to the nearest.
 __device__ __forceinline__ uint64_t fx_mul_frac(uint64_t a, uint64_t c) {
   const uint32_t al = (uint32_t)a, ah = (uint32_t)(a >> 32), cl = (uint32_t)c, ch = (uint32_t)(c >> 32);
-  const uint64_t mid = (uint64_t)al * ch + (uint64_t)ah * cl;   // < 2^64: the low words are below 2^32
+  // < 2^64: a high word is 2^31 only where the low word is 0
+  const uint64_t mid = (uint64_t)al * ch + ((uint64_t)ah * cl + 0x40000000u) + __umulhi(al, cl);
   return 2 * ((uint64_t)ah * ch) + (mid >> 31);
 }
 
@@ -109,7 +124,7 @@ __device__ __forceinline__ FxCourant fx_courant(uint64_t alpha) {
 
 // M of Eq. (28) in upwind form, |D|, |Dp| < 2^60.  v is formed to ~2^-46: a
 // float quotient rounded to i0 2^-23, its exact integer remainder, and the
-// remainder's float quotient.  Where D = 0 the quotients may be anything (0 / 0):
+// remainder's float quotient; 2 K v is then good to K 2^-45 + 2^-62.  Where D = 0 the quotients may be anything (0 / 0):
 // the result is c |D| = 0 in integers.
 __device__ __forceinline__ int64_t fx_mwb(int64_t D, int64_t Dp, const FxCourant& c) {
   const int64_t s = D >> 63;
@@ -121,8 +136,11 @@ __device__ __forceinline__ int64_t fx_mwb(int64_t D, int64_t Dp, const FxCourant
   const uint32_t i0 = __float_as_uint(__fadd_rn(v0, 1.0f)) - 0x3f800000u;   // v0 in units of 2^-23, rounded
   const int64_t rem = (int64_t)((num << 23) - n * (uint64_t)i0);            // |rem| <= 4 n < 2^63
   const float q = fx_float(rem) * r;                                        // the rest of v, units of 2^-23
-  const int32_t i1 = __float2int_rn(fmaf(c.k2, q, c.klo * v0));             // units of 2^-52
-  const uint64_t coef = c.a2 + c.k40 * (uint64_t)i0 + (uint64_t)((int64_t)i1 * 2048);
+  const float k = fmaf(c.k2, q, c.klo * v0);                                // the rest of 2 K v, units of 2^-52
+  const int32_t i1 = __float2int_rn(k);
+  // and what i1 rounds off, units of 2^-63 (a D far larger than the node's own value, times 2^-53, is not small beside it)
+  const int32_t i2 = __float_as_int(fmaf(k - __int2float_rn(i1), 2048.0f, 12582912.0f)) - 0x4b400000;
+  const uint64_t coef = c.a2 + c.k40 * (uint64_t)i0 + (uint64_t)((int64_t)i1 * 2048 + i2);
   return fx_signed(fx_mul(a, coef), s);
 }
 
@@ -144,8 +162,8 @@ __device__ __forceinline__ double limiter64(double D, double Dp) {
   return small ? v * 0x1p-500 : v;
 }
 
-// The compared schemes (Sec. II B 3) in upwind form: M = alpha D + c ((D' or D)
-// - (D or Dp)), c = alpha (1 - alpha) / 2 (Warming-Beam, Lax-Wendroff) or alpha / 2
+// The compared schemes (Sec. II B 3) in upwind form: M = alpha D + c/2 ((D' or D)
+// - (D or Dp)), c = alpha (1 - alpha) (Warming-Beam, Lax-Wendroff) or alpha
 // (second-order upwind), D' = f(downwind) - f of Lax-Wendroff.
 struct FxLinear {
   uint64_t a, c;   // units of 2^-63
@@ -156,7 +174,7 @@ using FxCoef = std::conditional_t<SCH == PCLB_SCHEME_MWB, FxCourant, FxLinear>;
 template <int SCH>
 __device__ __forceinline__ FxCoef<SCH> fx_coef(uint64_t alpha) {
   if constexpr (SCH == PCLB_SCHEME_MWB) return fx_courant(alpha);
-  else return FxLinear{alpha, (SCH == PCLB_SCHEME_UPWIND2 ? alpha : alpha - fx_mul_frac(alpha, alpha)) >> 1};
+  else return FxLinear{alpha, SCH == PCLB_SCHEME_UPWIND2 ? alpha : alpha - fx_mul_frac(alpha, alpha)};
 }
 
 // M of node value x0, upwind values u1, u2 and (Lax-Wendroff) downwind value d1,
@@ -168,7 +186,7 @@ __device__ __forceinline__ int64_t fx_increment(int64_t x0, int64_t u1, int64_t 
     return fx_mwb(D, u1 - u2, c);
   } else {
     const int64_t E = SCH == PCLB_SCHEME_LW ? d1 - x0 - D : D - (u1 - u2);
-    return fx_signed(fx_mul(fx_abs(D), c.a), D >> 63) + fx_signed(fx_mul(fx_abs(E), c.c), E >> 63);
+    return fx_signed(fx_mul(fx_abs(D), c.a), D >> 63) + fx_signed(fx_mul_half(fx_abs(E), c.c), E >> 63);
   }
 }
 
