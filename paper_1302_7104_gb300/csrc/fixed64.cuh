@@ -23,6 +23,8 @@
 
 namespace pclb {
 
+constexpr int kHalfDirs = kNDirs / 2;
+
 // Exponents for which fx_to_double stays inside the normal range; NaN and
 // infinity (0x7ff) are outside.
 constexpr int kFxMinExp = 128, kFxMaxExp = 1900;
@@ -153,13 +155,67 @@ __device__ __forceinline__ int fx_exponent(int h0, int h1, H... rest) {
 }
 __device__ __forceinline__ bool fx_range(int e) { return e >= kFxMinExp && e <= kFxMaxExp; }
 
-// |D| (D - Dp) / (|D| + |Dp|) in FP64, small differences scaled up by a power of two.
-__device__ __forceinline__ double limiter64(double D, double Dp) {
-  const bool small = fmax(fabs(D), fabs(Dp)) < 0x1p-500;
+// c in [0, 1] as a 2^-(63 + s), with 61 leading bits or more in a (subnormal c: 0).
+struct FxScaled {
+  uint64_t a;
+  int s;
+};
+__device__ __forceinline__ FxScaled fx_scaled(double c) {
+  const int hi = __double2hiint(c), sh = 1023 - (hi >> 20);   // c = m 2^-63 2^-sh
+  const uint32_t mh = ((uint32_t)hi & 0xfffffu) | 0x100000u;
+  const uint64_t m = ((uint64_t)mh << 32 | (uint32_t)__double2loint(c)) << 11;
+  if (sh >= 1023) return FxScaled{0, 0};
+  if (sh < 1) return FxScaled{1ull << 63, 0};
+  return sh < 2 ? FxScaled{m >> 1, 0} : FxScaled{m >> 2, sh - 2};
+}
+
+// u 2^-(63 + s) as a double; 0 below its normal range.
+__device__ __forceinline__ double fx_fraction_to_double(uint64_t u, int s) {
+  const int lz = __clzll((long long)u), e = 1022 - lz - s;
+  const uint64_t m = u << (lz & 63), r = (m >> 11) + ((m >> 10) & 1);
+  const uint32_t hi = (uint32_t)(r >> 32) + ((uint32_t)e << 20);
+  return u == 0 || e < 1 ? 0.0 : __hiloint2double((int)hi, (int)(uint32_t)r);
+}
+
+// |D| / (|D| + |Dp|) = v 2^-(63 + s), to ~2^-62 of it: three float quotient digits
+// with exact remainders, on integer mantissas aligned to the larger of the two.
+// e: the larger biased exponent (0: both below the normal range, v may be anything).
+__device__ __forceinline__ FxScaled fx_switch(double D, double Dp, int& e) {
+  const int hD = __double2hiint(D), hP = __double2hiint(Dp);
+  const int eD = (hD >> 20) & 0x7ff, eP = (hP >> 20) & 0x7ff;
+  e = max(eD, eP);
+  auto mantissa = [](int h, double x, int ex) -> uint64_t {
+    const uint64_t m = ((uint64_t)(((uint32_t)h & 0xfffffu) | 0x100000u) << 32 | (uint32_t)__double2loint(x)) << 6;
+    return ex == 0 ? 0 : m;
+  };
+  const uint64_t mD = mantissa(hD, D, eD);
+  const uint64_t n = (mD >> min(e - eD, 63)) + (mantissa(hP, Dp, eP) >> min(e - eP, 63));   // < 2^60
+  // |D| below |Dp| by whole powers of two: they go into s, so that v keeps its bits
+  const uint64_t a = e > eD ? mD >> 1 : mD;
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fx_float(n)));
+  const uint32_t i0 = __float_as_uint(__fadd_rn(fx_float(a) * r, 1.0f)) - 0x3f800000u;   // units of 2^-23
+  const int64_t rem0 = (int64_t)((a << 23) - n * (uint64_t)i0);
+  const int32_t i1 = __float2int_rn(fx_float(rem0) * r * 4194304.0f);                    // units of 2^-45
+  const int64_t rem1 = (int64_t)(((uint64_t)rem0 << 22) - n * (uint64_t)(int64_t)i1);
+  const int32_t i2 = __float2int_rn(fx_float(rem1) * r * 262144.0f);                     // units of 2^-63
+  return FxScaled{((uint64_t)i0 << 40) + (uint64_t)((int64_t)i1 * 262144) + (uint64_t)(int64_t)i2, max(e - eD - 1, 0)};
+}
+
+// M of Eq. (28) from doubles, good to the last places of D times the coefficient
+// whatever the sizes of D, Dp and alpha: four FP64 operations with the differences.
+__device__ __forceinline__ double mwb64(double alpha, double D, double Dp) {
+  const FxScaled c = fx_scaled(alpha);
+  const uint64_t a2 = fx_mul_frac(c.a, c.a >> min(c.s, 63)), k2 = 2 * (c.a - a2);
+  auto big = [](double x) { return ((__double2hiint(x) >> 20) & 0x7ff) >= 500; };
+  const bool small = !big(D) && !big(Dp);   // scaled up: a difference may be subnormal
   if (small) { D *= 0x1p+500; Dp *= 0x1p+500; }
-  const double den = fabs(D) + fabs(Dp);
-  const double v = den >= 0x1p-1000 ? fabs(D) * recip_newton1(den) * (D - Dp) : 0.0;
-  return small ? v * 0x1p-500 : v;
+  int e;
+  const FxScaled v = fx_switch(D, Dp, e);
+  const bool opposite = (__double2hiint(D) ^ __double2hiint(Dp)) < 0;
+  const uint64_t w = opposite ? k2 : fx_mul_frac(k2, v.a) >> min(v.s, 63);
+  const double M = e < 0x7ff ? D * fx_fraction_to_double(a2 + w, c.s) : __hiloint2double(0x7ff80000, 0);
+  return small ? M * 0x1p-500 : M;
 }
 
 // The compared schemes (Sec. II B 3) in upwind form: M = alpha D + c/2 ((D' or D)
@@ -190,11 +246,12 @@ __device__ __forceinline__ int64_t fx_increment(int64_t x0, int64_t u1, int64_t 
   }
 }
 
-// The same in FP64; a = |C|, K = |C| (1 - |C|).
+// The same from doubles; a = |C|.
 template <int SCH>
-__device__ __forceinline__ double increment64(double a, double K, double x0, double u1, double u2, double d1) {
+__device__ __forceinline__ double increment64(double a, double x0, double u1, double u2, double d1) {
   const double D = x0 - u1, Dp = u1 - u2;
-  if (SCH == PCLB_SCHEME_MWB) return fma(a, D, K * limiter64(D, Dp));
+  if constexpr (SCH == PCLB_SCHEME_MWB) return mwb64(a, D, Dp);
+  const double K = a - a * a;
   if (SCH == PCLB_SCHEME_LW) return a * D + 0.5 * K * ((d1 - x0) - D);
   return a * D + 0.5 * (SCH == PCLB_SCHEME_WB ? K : a) * (D - Dp);
 }
@@ -202,16 +259,16 @@ __device__ __forceinline__ double increment64(double a, double K, double x0, dou
 // d x0 - M_r - M_theta of one label (Eqs. 19, 28): x0 the node, u1 and v1 its
 // upwind neighbours in r and theta, u2 and v2 the next ones (Lax-Wendroff: the
 // downwind neighbours).  In fixed point on the exponent of the largest of
-// them, or in FP64 outside its range (c: the pair's FP64 Courant entry at the row).
+// them, or in FP64 outside its range and where x0 is more than 2^5 smaller, so
+// that a unit would be coarse for it (c: the pair's FP64 Courant entry at the row).
 template <int SCH>
 __device__ __forceinline__ double fx_carried(double x0, double u1, double u2, double v1, double v2,
                                              const FxCoef<SCH>& cr, const FxCoef<SCH>& ct, uint64_t dfx, int64_t dsign,
                                              double decay, const double* c, double inv_r) {
   const int e = fx_exponent(__double2hiint(x0), __double2hiint(u1), __double2hiint(u2), __double2hiint(v1),
                             __double2hiint(v2));
-  if (!fx_range(e)) {
-    const double at = c[2] * inv_r;
-    return decay * x0 - increment64<SCH>(c[0], c[1], x0, u1, u2, u2) - increment64<SCH>(at, at - at * at, x0, v1, v2, v2);
+  if (!fx_range(e) || fx_exponent(__double2hiint(x0)) < e - 5) {
+    return fma(decay, x0, -increment64<SCH>(c[0], x0, u1, u2, u2)) - increment64<SCH>(c[2] * inv_r, x0, v1, v2, v2);
   }
   const int64_t i0 = fx_from_double(x0, e);
   auto M = [&](double n1, double n2, const FxCoef<SCH>& k) {
@@ -222,12 +279,52 @@ __device__ __forceinline__ double fx_carried(double x0, double u1, double u2, do
   return fx_to_double(keep - M(u1, u2, cr) - M(v1, v2, ct), e);
 }
 
-// A fraction (units of 2^-63) as a double.
-__device__ __forceinline__ double fx_fraction_to_double(uint64_t u) {
-  const int lz = __clzll((long long)u);
-  const uint64_t m = u << (lz & 63), r = (m >> 11) + ((m >> 10) & 1);
-  const uint32_t hi = (uint32_t)(r >> 32) + ((uint32_t)(1022 - lz) << 20);
-  return u == 0 ? 0.0 : __hiloint2double((int)hi, (int)(uint32_t)r);
+// The sums S, X = sum c_x f, Y = sum c_y f of a shell at one node: f its first
+// label, planes `plane` apart.
+__device__ __forceinline__ void shell_sums64(const double* f, size_t plane, const DvmConst<double>& d, double o[3]) {
+  double a[kHalfDirs], b[kHalfDirs];
+#pragma unroll
+  for (int i = 0; i < kHalfDirs; ++i) {
+    a[i] = f[i * plane];
+    b[i] = f[(i + kHalfDirs) * plane];
+  }
+  auto hi = [](double x) { return __double2hiint(x); };
+  const int e = fx_exponent(hi(a[0]), hi(a[1]), hi(a[2]), hi(a[3]), hi(b[0]), hi(b[1]), hi(b[2]), hi(b[3]));
+  if (!fx_range(e)) {
+    double S = 0.0, D[kHalfDirs];
+#pragma unroll
+    for (int i = 0; i < kHalfDirs; ++i) {
+      S += a[i] + b[i];
+      D[i] = a[i] - b[i];
+    }
+    o[0] = S;
+    o[1] = fma(d.cx[2], D[1] - D[3], D[0]);
+    o[2] = fma(d.cx[2], D[1] + D[3], D[2]);
+    return;
+  }
+  int64_t S = 0, D[kHalfDirs];
+#pragma unroll
+  for (int i = 0; i < kHalfDirs; ++i) {
+    const int64_t x = fx_from_double(a[i], e), y = fx_from_double(b[i], e);
+    S += x + y;
+    D[i] = x - y;
+  }
+  o[0] = fx_to_double(S, e);
+  o[1] = fx_to_double(D[0] + fx_diagonal(D[1] - D[3]), e);
+  o[2] = fx_to_double(D[2] + fx_diagonal(D[1] + D[3]), e);
+}
+
+// Node state from the rest value and the four shells' sums.
+__device__ __forceinline__ NodeState<double> state_of_sums(double f0, const double* s, const DvmConst<double>& d) {
+  double s0 = f0, sx = 0.0, sy = 0.0, se = 0.0;
+#pragma unroll
+  for (int k = 1; k <= 4; ++k) {
+    s0 += s[3 * (k - 1)];
+    sx = fma(d.speed[k], s[3 * (k - 1) + 1], sx);
+    sy = fma(d.speed[k], s[3 * (k - 1) + 2], sy);
+    se = fma(d.half_v2[k], s[3 * (k - 1)], se);
+  }
+  return node_state64(s0, sx, sy, se);
 }
 
 // Partial derivatives of M of Eq. (28) (mwb_partials in adjoint_common.cuh) with
@@ -261,8 +358,8 @@ __device__ __forceinline__ void fx_mwb_partials(double D, double Dp, uint64_t a2
   if (opposite || zP) { md = a2 + k2; mp = zP ? k2 >> 1 : 0; }
   if (zD || e == 0) { md = a2 + (k2 >> 1); mp = 0; }
   const bool finite = e < 0x7ff;
-  MD = finite ? fx_fraction_to_double(md) : __hiloint2double(0x7ff80000, 0);
-  MDp = finite ? -fx_fraction_to_double(mp) : MD;
+  MD = finite ? fx_fraction_to_double(md, 0) : __hiloint2double(0x7ff80000, 0);
+  MDp = finite ? -fx_fraction_to_double(mp, 0) : MD;
 }
 
 }  // namespace pclb

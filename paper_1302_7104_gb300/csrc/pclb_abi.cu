@@ -25,7 +25,7 @@ namespace pclb {
 cudaError_t launch_step_f32(const CUtensorMap*, float*, const StepParams&, const DvmConst<float>&,
                             cudaStream_t, int ty_begin = 0, int ty_end = -1);
 template <class T>
-cudaError_t launch_step(const CUtensorMap*, T*, const StepParams&, const DvmConst<T>&, cudaStream_t,
+cudaError_t launch_step(const CUtensorMap*, const T*, T*, const StepParams&, const DvmConst<T>&, cudaStream_t,
                         int ty_begin = 0, int ty_end = -1);
 template <class T>
 cudaError_t launch_set_state(T*, const T*, const T*, const T*, const T*, const StepParams&,
@@ -431,7 +431,7 @@ pclb_status do_step(pclb_ctx* ctx, int n) {
     } else if constexpr (sizeof(T) == 4)
       e = launch_step_f32(&ctx->tmap[src], fbuf<float>(ctx, dst), ctx->sp, ctx->dvm32, ctx->stream);
     else
-      e = launch_step<T>(&ctx->tmap[src], fbuf<T>(ctx, dst), ctx->sp, dvm_of<T>(ctx), ctx->stream);
+      e = launch_step<T>(&ctx->tmap[src], fbuf<T>(ctx, src), fbuf<T>(ctx, dst), ctx->sp, dvm_of<T>(ctx), ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "step kernel launch");
     ctx->cur = dst;
   }
@@ -582,7 +582,7 @@ pclb_status run_host_slabs(pclb_ctx* ctx, const void* const in[4], int n, void* 
       return launch_step_f32(&ctx->tmap[src], fbuf<float>(ctx, 1 - src), ctx->sp, ctx->dvm32, cs(s), tile0(s),
                              tile0(s + 1));
     else
-      return launch_step<T>(&ctx->tmap[src], fbuf<T>(ctx, 1 - src), ctx->sp, dvm_of<T>(ctx), cs(s), tile0(s),
+      return launch_step<T>(&ctx->tmap[src], fbuf<T>(ctx, src), fbuf<T>(ctx, 1 - src), ctx->sp, dvm_of<T>(ctx), cs(s), tile0(s),
                             tile0(s + 1));
   };
   // moments of slab s of buffer b into the staging area (on the slab's
@@ -965,7 +965,7 @@ pclb_status pclb_step_states(pclb_ctx* ctx, const void* f_from, void* f_to) {
     pclb_status st = encode_map(ctx, f_from, ctx->sp.tile_rows + 4, &map);
     if (st != PCLB_OK) return st;
     e = ctx->prec == PCLB_FP32 ? launch_step_f32(&map, (float*)f_to, ctx->sp, ctx->dvm32, ctx->stream)
-                               : launch_step<double>(&map, (double*)f_to, ctx->sp, ctx->dvm64, ctx->stream);
+                               : launch_step<double>(&map, (const double*)f_from, (double*)f_to, ctx->sp, ctx->dvm64, ctx->stream);
   }
   return e == cudaSuccess ? PCLB_OK : cuda_fail(ctx, e, "step kernel launch");
 }

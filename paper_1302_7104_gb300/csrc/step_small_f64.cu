@@ -27,7 +27,6 @@ namespace pclb {
 
 namespace {
 
-constexpr int kHalfDirs = kNDirs / 2;
 constexpr int kPairsSm = 4 * kHalfDirs;
 constexpr int kPairWarps = 16;
 
@@ -65,55 +64,6 @@ __device__ __forceinline__ void bar_arrive(int id, int threads) {
 __device__ __forceinline__ void bar_wait(int id, int threads) {
   __syncwarp();
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-
-// The sums S, X = sum c_x f, Y = sum c_y f of a shell at one node: f its first
-// label, planes PLANE apart.
-template <int PLANE>
-__device__ __forceinline__ void shell_sums64(const double* f, const DvmConst<double>& d, double o[3]) {
-  double a[kHalfDirs], b[kHalfDirs];
-#pragma unroll
-  for (int i = 0; i < kHalfDirs; ++i) {
-    a[i] = f[i * PLANE];
-    b[i] = f[(i + kHalfDirs) * PLANE];
-  }
-  auto hi = [](double x) { return __double2hiint(x); };
-  const int e = fx_exponent(hi(a[0]), hi(a[1]), hi(a[2]), hi(a[3]), hi(b[0]), hi(b[1]), hi(b[2]), hi(b[3]));
-  if (!fx_range(e)) {
-    double S = 0.0, D[kHalfDirs];
-#pragma unroll
-    for (int i = 0; i < kHalfDirs; ++i) {
-      S += a[i] + b[i];
-      D[i] = a[i] - b[i];
-    }
-    o[0] = S;
-    o[1] = fma(d.cx[2], D[1] - D[3], D[0]);
-    o[2] = fma(d.cx[2], D[1] + D[3], D[2]);
-    return;
-  }
-  int64_t S = 0, D[kHalfDirs];
-#pragma unroll
-  for (int i = 0; i < kHalfDirs; ++i) {
-    const int64_t x = fx_from_double(a[i], e), y = fx_from_double(b[i], e);
-    S += x + y;
-    D[i] = x - y;
-  }
-  o[0] = fx_to_double(S, e);
-  o[1] = fx_to_double(D[0] + fx_diagonal(D[1] - D[3]), e);
-  o[2] = fx_to_double(D[2] + fx_diagonal(D[1] + D[3]), e);
-}
-
-// Node state from the rest value and the four shells' sums.
-__device__ __forceinline__ NodeState<double> state_of_sums(double f0, const double* s, const DvmConst<double>& d) {
-  double s0 = f0, sx = 0.0, sy = 0.0, se = 0.0;
-#pragma unroll
-  for (int k = 1; k <= 4; ++k) {
-    s0 += s[3 * (k - 1)];
-    sx = fma(d.speed[k], s[3 * (k - 1) + 1], sx);
-    sy = fma(d.speed[k], s[3 * (k - 1) + 2], sy);
-    se = fma(d.half_v2[k], s[3 * (k - 1)], se);
-  }
-  return node_state64(s0, sx, sy, se);
 }
 
 }  // namespace
@@ -229,7 +179,7 @@ __global__ void __launch_bounds__(SmSize<SCH, TT>::threads, 1)
       const double* s = sums + (grow * 32 + col - kLeft) * 12;
       if (col < kLeft || col >= kLeft + kTileR) {
 #pragma unroll 1
-        for (int k = 1; k <= 4; ++k) shell_sums64<PLANE>(f + (1 + (k - 1) * kNDirs) * PLANE, d, own + 3 * (k - 1));
+        for (int k = 1; k <= 4; ++k) shell_sums64(f + (1 + (k - 1) * kNDirs) * PLANE, PLANE, d, own + 3 * (k - 1));
         s = own;
       }
       m = state_of_sums(f[0], s, d);
@@ -276,7 +226,7 @@ __global__ void __launch_bounds__(SmSize<SCH, TT>::threads, 1)
   const int part = warp / TT, k = part / (SPLIT / 4) + 1, i_first = part % (SPLIT / 4) * DIRS;
   if (i_first == 0) {
     double s[3];
-    shell_sums64<PLANE>(sm + (1 + (k - 1) * kNDirs) * PLANE + node, d, s);
+    shell_sums64(sm + (1 + (k - 1) * kNDirs) * PLANE + node, PLANE, d, s);
     double* o = sums + (rl * 32 + lane) * 12 + 3 * (k - 1);
     o[0] = s[0]; o[1] = s[1]; o[2] = s[2];
     bar_arrive(kBarSums, n_sums);

@@ -57,6 +57,34 @@ def test_rounding_has_no_preferred_sign(n_r, n_t, n_dirs, scheme):
 
 
 @pytest.mark.parametrize("n_r,n_t,n_dirs", GRIDS)
+def test_cold_gas_beside_hot_gas_keeps_its_own_precision(n_r, n_t, n_dirs):
+    """T falls from 3 to 1 and rho from 64 to 1 inside a tile: the fourth
+    shell's values fall by ~2^13.  Cold nodes away from the jump, shell by shell:
+    the largest error against eight roundings (2^-50) of the shell's own scale
+    there, rho times the largest term of the polynomial F_k(T), which bounds what
+    double arithmetic can resolve of it (F_k is a difference of such terms)."""
+    w = I.random_smooth(n_r, n_t, seed=5, n_dirs=n_dirs, n_f=n_dirs, amp=0.1)
+    hot = np.arange(n_r) < 16
+    w.T = np.where(hot, 3.0, 1.0) * w.T
+    w.rho = np.where(hot, 64.0, 1.0) * w.rho
+    f = _noisy(w, noise=1e-3)
+    got, flags = _step(w, f)
+    want = O.run(w, f, 1)
+    assert flags == 0
+    cold = np.s_[:, 20:32]
+    v2 = [s * s for s in w.speeds]
+    T = w.T[cold].max()
+    for k in range(1, 5):
+        a, b, c = (v2[j] for j in range(1, 5) if j != k)
+        den = v2[k] * (v2[k] - a) * (v2[k] - b) * (v2[k] - c)
+        terms = (w.B[1] * a * b * c, w.B[2] * (a * b + b * c + c * a), w.B[3] * (a + b + c), w.B[4])
+        scale = w.rho[cold].max() * max(abs(x / den) * T ** (n + 1) for n, x in enumerate(terms))
+        q = slice(1 + (k - 1) * n_dirs, 1 + k * n_dirs)
+        err = np.abs(got[q, :, 20:32] - want[q, :, 20:32]).max()
+        assert err <= 2.0 ** -50 * scale, (k, err / scale)
+
+
+@pytest.mark.parametrize("n_r,n_t,n_dirs", GRIDS)
 def test_mass_drift_of_a_long_run_beside_dense_gas(n_r, n_t, n_dirs):
     """Columns of thin gas (1/20) beside dense gas at rest relative to one
     another, 100 steps of a tiny time step: every step multiplies the thin
