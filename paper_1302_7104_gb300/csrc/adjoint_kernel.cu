@@ -57,13 +57,15 @@
 
 namespace pclb {
 
-// Courant entry of one pair of opposite velocities at one theta row, in units
-// of 2^-63: alpha^2 and 2 alpha (1 - alpha) of alpha = |C_r|, and |C_theta| at
-// the tile's first column; flag bit 0 set when v_r < 0 and bit 1 when v_theta
-// < 0 for the first label of the pair.
+// Courant entry of one pair of opposite velocities at one theta row: alpha^2 and
+// 2 alpha (1 - alpha) of alpha = |C_r| in units of 2^-(63 + sr), and |C_theta| at
+// the tile's first column in units of 2^-(63 + st) (in plain units of 2^-63 the
+// partials of an alpha of 1e-10 had 30 digits left); flag bit 0 set when v_r <
+// 0 and bit 1 when v_theta < 0 for the first label of the pair.
 struct alignas(32) CourEntry {
   uint64_t a2, k2, at;
   int fl;
+  int16_t sr, st;
 };
 
 // bytes of one part of the wall scratch, aligned for the next
@@ -103,10 +105,11 @@ namespace {
 // ---- the pair-streaming kernel's stencil pieces ------------------------------
 // lam(n) M_D(n), lam(n) M_Dp(n) of one label at one node in one direction, its
 // upwind neighbours at offsets u and 2u, to P and P + DB.
-__device__ __forceinline__ void products(const double* f, int u, double lam, double* P, int DB, uint64_t a2, uint64_t k2) {
+__device__ __forceinline__ void products(const double* f, int u, double lam, double* P, int DB, uint64_t a2, uint64_t k2,
+                                         int s) {
   double MD, MP;
   const double f1 = f[u];
-  fx_mwb_partials(f[0] - f1, f1 - f[2 * u], a2, k2, MD, MP);
+  fx_mwb_partials(f[0] - f1, f1 - f[2 * u], a2, k2, s, MD, MP);
   P[0] = lam * MD;
   P[DB] = lam * MP;
 }
@@ -250,13 +253,14 @@ __global__ void __launch_bounds__(AdjSize<TT, LS>::threads, AdjSize<TT, LS>::min
   // Courant entries of the stored rows t0 .. t0 + TT + 3 (theta rows t0 - 2 .. t0 + TT + 1)
   for (int i = tid; i < (TT + 4) * NP; i += blockDim.x) {
     const int srow = t0 + i / NP, pr = i % NP;
-    CourEntry e{0, 0, 0, 0};
+    CourEntry e{0, 0, 0, 0, 0, 0};
     if (srow < p.rows) {
       const double* c = p.courant64 + ((size_t)srow * NP + pr) * 4;
-      const uint64_t alpha = fx_fraction(c[0]);
-      e.a2 = fx_mul_frac(alpha, alpha);
-      e.k2 = 2 * (alpha - e.a2);
-      e.at = fx_fraction(c[2] * inv_r0);
+      const FxScaled r = fx_scaled(c[0]), th = fx_scaled(c[2] * inv_r0);
+      fx_partial_coefs(r, e.a2, e.k2);
+      e.at = th.a;
+      e.sr = (int16_t)r.s;
+      e.st = (int16_t)th.s;
       e.fl = (int)c[3];
     }
     ctab[i] = e;
@@ -405,22 +409,20 @@ __global__ void __launch_bounds__(AdjSize<TT, LS>::threads, AdjSize<TT, LS>::min
     auto up_r = [&](int L) { return ((fl_c & 1) != 0) != (L != 0) ? 1 : -1; };
     auto up_t = [&](int L) { return ((fl_c & 2) != 0) != (L != 0) ? kWinR : -kWinR; };
     // alpha^2 and 2 alpha (1 - alpha) of |C_theta| at this thread's column
-    auto azimuthal = [&](uint64_t at, uint64_t& a2, uint64_t& k2) {
-      const uint64_t alpha = fx_mul_frac(at, my_ratio);
-      a2 = fx_mul_frac(alpha, alpha);
-      k2 = 2 * (alpha - a2);
+    auto azimuthal = [&](const CourEntry& x, uint64_t& a2, uint64_t& k2) {
+      fx_partial_coefs(FxScaled{fx_mul_frac(x.at, my_ratio), x.st}, a2, k2);
     };
     T lam_c[LS == 1 ? 2 : 1];                             // lam^{n+1} of the label(s) at this node
     {
       uint64_t a2, k2;
-      azimuthal(e.at, a2, k2);
+      azimuthal(e, a2, k2);
 #pragma unroll
       for (int j = 0; j < (LS == 1 ? 2 : 1); ++j) {
         const int L = LS == 1 ? j : half_of;
         const T* fw = sfp + L * PLANE + o_node;
         lam_c[j] = slp[L * PLANE + o_node];
-        products(fw, up_r(L), lam_c[j], pb + L * PROD + p_rad, BR - AR, e.a2, e.k2);
-        products(fw, up_t(L), lam_c[j], pb + L * PROD + p_az, BT - AT, a2, k2);
+        products(fw, up_r(L), lam_c[j], pb + L * PROD + p_rad, BR - AR, e.a2, e.k2, e.sr);
+        products(fw, up_t(L), lam_c[j], pb + L * PROD + p_az, BT - AT, a2, k2, e.st);
       }
     }
     if (warp < 4 * PP) {
@@ -430,11 +432,11 @@ __global__ void __launch_bounds__(AdjSize<TT, LS>::threads, AdjSize<TT, LS>::min
       const CourEntry eh = ctab[rr * NP + it * PP + j];
       const bool q1_up_pos = (eh.fl & 2) != 0;
       uint64_t a2, k2;
-      azimuthal(eh.at, a2, k2);
+      azimuthal(eh, a2, k2);
       const int L = (h < 2) == q1_up_pos ? 0 : 1, o = rr * kWinR + col;
       const T* w = stage + j * 4 * PLANE + L * PLANE + o;
       products(w, h < 2 ? kWinR : -kWinR, w[2 * PLANE], buffer + (j * 2 + L) * PROD + AT + rr * kTileR + lane, BT - AT, a2,
-               k2);
+               k2, eh.st);
     }
     if (warp == (PP == 1 ? 4 : TT * LS - 1)) {
       // halo columns: 4 per pair and tile row (label, column).  Upwind at larger r
@@ -446,7 +448,7 @@ __global__ void __launch_bounds__(AdjSize<TT, LS>::threads, AdjSize<TT, LS>::min
         const int u = ((eh.fl & 1) != 0) != (L != 0) ? 1 : -1;
         const int c = u == 1 ? i - 2 : kTileR + i;
         const T* w = stage + (j * 4 + L) * PLANE + (hr + 2) * kWinR + c + kLeft;
-        products(w, u, w[2 * PLANE], buffer + (j * 2 + L) * PROD + AR + hr * RC + c + 2, BR - AR, eh.a2, eh.k2);
+        products(w, u, w[2 * PLANE], buffer + (j * 2 + L) * PROD + AR + hr * RC + c + 2, BR - AR, eh.a2, eh.k2, eh.sr);
       }
     }
     if (__syncthreads_or(!ok)) {

@@ -202,11 +202,19 @@ __device__ __forceinline__ FxScaled fx_switch(double D, double Dp, int& e) {
   return FxScaled{((uint64_t)i0 << 40) + (uint64_t)((int64_t)i1 * 262144) + (uint64_t)(int64_t)i2, max(e - eD - 1, 0)};
 }
 
+// alpha^2 and 2 alpha (1 - alpha) of alpha = c.a 2^-(63 + c.s), in units of 2^-(63 + c.s):
+// they keep their digits however small alpha is.
+__device__ __forceinline__ void fx_partial_coefs(FxScaled c, uint64_t& a2, uint64_t& k2) {
+  a2 = fx_mul_frac(c.a, c.a >> min(c.s, 63));
+  k2 = 2 * (c.a - a2);
+}
+
 // M of Eq. (28) from doubles, good to the last places of D times the coefficient
 // whatever the sizes of D, Dp and alpha: four FP64 operations with the differences.
 __device__ __forceinline__ double mwb64(double alpha, double D, double Dp) {
   const FxScaled c = fx_scaled(alpha);
-  const uint64_t a2 = fx_mul_frac(c.a, c.a >> min(c.s, 63)), k2 = 2 * (c.a - a2);
+  uint64_t a2, k2;
+  fx_partial_coefs(c, a2, k2);
   auto big = [](double x) { return ((__double2hiint(x) >> 20) & 0x7ff) >= 500; };
   const bool small = !big(D) && !big(Dp);   // scaled up: a difference may be subnormal
   if (small) { D *= 0x1p+500; Dp *= 0x1p+500; }
@@ -329,37 +337,26 @@ __device__ __forceinline__ NodeState<double> state_of_sums(double f0, const doub
 
 // Partial derivatives of M of Eq. (28) (mwb_partials in adjoint_common.cuh) with
 // respect to D and Dp, from a2 = alpha^2 and k2 = 2 alpha (1 - alpha) in units of
-// 2^-63.  With v = |D| / (|D| + |Dp|): D and Dp of one sign, M_D = a2 + 2 k2 v -
+// 2^-(63 + s).  With v = |D| / (|D| + |Dp|): D and Dp of one sign, M_D = a2 + 2 k2 v -
 // k2 v^2 and M_Dp = -k2 v^2; of opposite signs, a2 + k2 and 0; D = 0, a2 + k2 / 2
-// and 0; Dp = 0, a2 + k2 and -k2 / 2.  v is formed on aligned integer mantissas
-// to ~2^-62 (three float quotient digits with exact remainders), so the only
-// FP64 operations are the caller's two differences.  Not finite: NaN.
-__device__ __forceinline__ void fx_mwb_partials(double D, double Dp, uint64_t a2, uint64_t k2, double& MD, double& MDp) {
+// and 0; Dp = 0, a2 + k2 and -k2 / 2.  v is formed on integer mantissas
+// (fx_switch), so the only FP64 operations are the caller's two differences.  Not
+// finite: NaN.
+__device__ __forceinline__ void fx_mwb_partials(double D, double Dp, uint64_t a2, uint64_t k2, int s, double& MD, double& MDp) {
+  int e;
+  const FxScaled v = fx_switch(D, Dp, e);
+  const uint64_t w = fx_mul_frac(k2, v.a), wv = fx_mul_frac(w, v.a);   // times 2^-v.s and 2^-2v.s
   const int hD = __double2hiint(D), hP = __double2hiint(Dp);
-  const uint32_t lD = (uint32_t)__double2loint(D), lP = (uint32_t)__double2loint(Dp);
-  const int eD = (hD >> 20) & 0x7ff, eP = (hP >> 20) & 0x7ff, e = max(eD, eP);
-  auto mantissa = [&](int h, uint32_t l, int ex) -> uint64_t {
-    const uint64_t m = ((uint64_t)(((uint32_t)h & 0xfffffu) | 0x100000u) << 32 | l) << 6;
-    return ex == 0 ? 0 : m >> min(e - ex, 63);
-  };
-  const uint64_t a = mantissa(hD, lD, eD), n = a + mantissa(hP, lP, eP);   // n < 2^60
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fx_float(n)));
-  const uint32_t i0 = __float_as_uint(__fadd_rn(fx_float(a) * r, 1.0f)) - 0x3f800000u;   // units of 2^-23
-  const int64_t rem0 = (int64_t)((a << 23) - n * (uint64_t)i0);
-  const int32_t i1 = __float2int_rn(fx_float(rem0) * r * 4194304.0f);                    // units of 2^-45
-  const int64_t rem1 = (int64_t)(((uint64_t)rem0 << 22) - n * (uint64_t)(int64_t)i1);
-  const int32_t i2 = __float2int_rn(fx_float(rem1) * r * 262144.0f);                     // units of 2^-63
-  const uint64_t v = ((uint64_t)i0 << 40) + (uint64_t)((int64_t)i1 * 262144) + (uint64_t)(int64_t)i2;
-  const uint64_t w = fx_mul_frac(k2, v), wv = fx_mul_frac(w, v);
-  const bool zD = (((uint32_t)hD << 1) | lD) == 0, zP = (((uint32_t)hP << 1) | lP) == 0;
+  const bool zD = (((uint32_t)hD << 1) | (uint32_t)__double2loint(D)) == 0;
+  const bool zP = (((uint32_t)hP << 1) | (uint32_t)__double2loint(Dp)) == 0;
   const bool opposite = (hD ^ hP) < 0;
-  uint64_t md = a2 + 2 * w - wv, mp = wv;
-  if (opposite || zP) { md = a2 + k2; mp = zP ? k2 >> 1 : 0; }
+  uint64_t md = a2 + 2 * (w >> min(v.s, 63)) - (wv >> min(2 * v.s, 63)), mp = wv;
+  int sp = s + 2 * v.s;
+  if (opposite || zP) { md = a2 + k2; mp = zP ? k2 >> 1 : 0; sp = s; }
   if (zD || e == 0) { md = a2 + (k2 >> 1); mp = 0; }
   const bool finite = e < 0x7ff;
-  MD = finite ? fx_fraction_to_double(md, 0) : __hiloint2double(0x7ff80000, 0);
-  MDp = finite ? -fx_fraction_to_double(mp, 0) : MD;
+  MD = finite ? fx_fraction_to_double(md, s) : __hiloint2double(0x7ff80000, 0);
+  MDp = finite ? -fx_fraction_to_double(mp, sp) : MD;
 }
 
 }  // namespace pclb
