@@ -1,11 +1,12 @@
 // The field kernels (both precisions) for the larger velocity sets of Table I,
 // N_i = 16 and 24 directions per shell (Q = 65, 97): the same model (Eqs. 2-5,
 // 10-11), one thread per node, the moments, the temperature and the equilibrium
-// factors in double (FP64) or float-float (FP32).  These sets serve the
+// factors in double (FP32: gen_state.cuh, the equilibrium in float-float).  These sets serve the
 // paper's velocity-set comparison; their steps are dvm_step_f64.cu and the tiled
 // FP32 kernel of dvm_tiled32.cu.  The azimuthal ghost rows (Eq. 40) are stored
 // rows, written by the producer of the seam rows with the label rotation, as in
 // the rest of the library.
+#include <algorithm>
 #include <cfloat>
 #include <cmath>
 #include <cstddef>
@@ -22,22 +23,6 @@ namespace pclb {
 namespace {
 
 constexpr int kGenThreads = 128;
-
-struct GenState {
-  double rho, ux, uy, E;
-  bool ok;
-};
-
-// Velocity and temperature from the sums rho, rho u, rho (E + u^2/2).
-__device__ __forceinline__ GenState gen_state_of(double s0, double sx, double sy, double se) {
-  GenState m;
-  m.rho = s0;
-  m.ux = sx / s0;
-  m.uy = sy / s0;
-  m.E = (se - 0.5 * (sx * m.ux + sy * m.uy)) / s0;
-  m.ok = s0 > 0.0 && m.E > 0.0 && isfinite(m.E) && isfinite(m.ux) && isfinite(m.uy);
-  return m;
-}
 
 // Moments (Eqs. 3-5): rho = sum f, rho u = sum f v, rho (E + u^2/2) = sum f
 // v^2/2, over the pairs of opposite velocities (2.5 FP64 operations per label
@@ -162,37 +147,45 @@ __global__ void __launch_bounds__(kGenThreads)
 template <int ND>
 __global__ void __launch_bounds__(kGenThreads)
     gen_moments_f32_kernel(const float* __restrict__ f, float* rho, float* u_r, float* u_t, float* temp,
-                           const __grid_constant__ StepParams p, const __grid_constant__ DvmG32 c) {
+                           const __grid_constant__ StepParams p, const __grid_constant__ DvmG d,
+                           const __grid_constant__ DvmG32 c) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   const int t = blockIdx.y;
   if (r >= p.n_r) return;
   const size_t plane = (size_t)p.rows * p.pitch;
-  const State32 m = gen_state32<ND>(f + (size_t)(t + kGhostRows) * p.pitch + r, plane, c);
+  const float* fn = f + (size_t)(t + kGhostRows) * p.pitch + r;
   const size_t n = (size_t)t * p.n_r + r;
-  const float4 cs = p.cs_ff[t];
-  const ff co{cs.x, cs.y}, si{cs.z, cs.w};
-  auto put = [&](float* o, ff x) {
-    if (o) o[n] = x.hi + x.lo;
-  };
-  put(rho, m.rho);
-  put(u_r, ff_add(ff_mul(m.ux, co), ff_mul(m.uy, si)));
-  put(u_t, ff_add(ff_mul(m.uy, co), ff_neg(ff_mul(m.ux, si))));
-  put(temp, m.E);
+  const State32 s = gen_state32<ND>(fn, plane, c);
+  if (gen_in_range(s)) {
+    const float4 cs = p.cs_ff[t];
+    const ff co{cs.x, cs.y}, si{cs.z, cs.w};
+    auto put = [&](float* o, ff x) {
+      if (o) o[n] = x.hi + x.lo;
+    };
+    put(rho, s.rho);
+    put(u_r, ff_add(ff_mul(s.ux, co), ff_mul(s.uy, si)));
+    put(u_t, ff_add(ff_mul(s.uy, co), ff_neg(ff_mul(s.ux, si))));
+    put(temp, s.E);
+    return;
+  }
+  const GenState m = gen_state_f32<ND>(fn, plane, d, c);
+  const double co = p.cos_t[t], si = p.sin_t[t];
+  if (rho) rho[n] = (float)m.rho;
+  if (u_r) u_r[n] = (float)(m.ux * co + m.uy * si);
+  if (u_t) u_t[n] = (float)(m.uy * co - m.ux * si);
+  if (temp) temp[n] = (float)m.E;
 }
 
 // Global integrals with weight r dr dtheta (as pclb_diagnostics): per block a
-// fixed grid-stride subset in a fixed order, then one thread sums the blocks.
-// The node state in double: FP64 storage by double sums, FP32 by the
-// float-float sums of gen_state32.
+// fixed grid-stride subset in a fixed order, the blocks' partials by six warps
+// (diag_final_kernel).  The node state in double.
 template <int ND>
 __device__ __forceinline__ GenState gen_diag_state(const double* f, size_t plane, const DvmG& d, const DvmG32&) {
   return gen_moments_node(f, plane, d);
 }
 template <int ND>
-__device__ __forceinline__ GenState gen_diag_state(const float* f, size_t plane, const DvmG&, const DvmG32& c) {
-  const State32 s = gen_state32<ND>(f, plane, c);
-  return GenState{(double)s.rho.hi + s.rho.lo, (double)s.ux.hi + s.ux.lo, (double)s.uy.hi + s.uy.lo,
-                  (double)s.E.hi + s.E.lo, s.ok};
+__device__ __forceinline__ GenState gen_diag_state(const float* f, size_t plane, const DvmG& d, const DvmG32& c) {
+  return gen_state_int<ND>(f, plane, d, c);
 }
 
 template <class T, int ND>
@@ -206,11 +199,11 @@ __global__ void __launch_bounds__(kGenThreads)
   for (size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x; n < n_nodes; n += (size_t)gridDim.x * blockDim.x) {
     const int t = (int)(n / p.n_r), r = (int)(n % p.n_r);
     const GenState m = gen_diag_state<ND>(f + (size_t)(t + kGhostRows) * p.pitch + r, plane, d, c);
-    const double w = (r_in + r * dr) * dr * dth;
-    v[0] += w * m.rho;
-    v[1] += w * m.rho * m.ux;
-    v[2] += w * m.rho * m.uy;
-    v[3] += w * m.rho * (m.E + 0.5 * (m.ux * m.ux + m.uy * m.uy));
+    const double w = (r_in + r * dr) * dr * dth * m.rho;
+    v[0] += w;
+    v[1] = fma(w, m.ux, v[1]);
+    v[2] = fma(w, m.uy, v[2]);
+    v[3] = fma(w, fma(0.5, m.ux * m.ux + m.uy * m.uy, m.E), v[3]);
     v[4] = fmin(v[4], m.rho);
     v[5] = fmin(v[5], m.E);
   }
@@ -254,9 +247,9 @@ cudaError_t gen_launch_moments(const T* f, T* rho, T* ur, T* ut, T* temp, const 
   if constexpr (sizeof(T) == 8)
     gen_moments_kernel<<<grid, kGenThreads, 0, s>>>(f, rho, ur, ut, temp, p, d);
   else if (d.n_dirs == 16)
-    gen_moments_f32_kernel<16><<<grid, kGenThreads, 0, s>>>(f, rho, ur, ut, temp, p, c);
+    gen_moments_f32_kernel<16><<<grid, kGenThreads, 0, s>>>(f, rho, ur, ut, temp, p, d, c);
   else
-    gen_moments_f32_kernel<24><<<grid, kGenThreads, 0, s>>>(f, rho, ur, ut, temp, p, c);
+    gen_moments_f32_kernel<24><<<grid, kGenThreads, 0, s>>>(f, rho, ur, ut, temp, p, d, c);
   return cudaGetLastError();
 }
 
@@ -293,6 +286,28 @@ void fill_dvm_generic32(DvmG32& c, const pclb_dvm& d, const DvmG& g) {
     for (int j = 0; j < 2; ++j) {
       hi[j][i] = (float)u[j];
       lo[j][i] = (float)(u[j] - (double)hi[j][i]);
+    }
+  }
+  {
+    // fractions of the power of two above the largest speed; cos and sin as they are
+    double v = 0.0, hv = 0.0;
+    for (int k = 1; k < 5; ++k) {
+      v = std::max(v, d.speeds[k]);
+      hv = std::max(hv, g.half_v2[k]);
+    }
+    std::frexp(v, &c.fx_exp_v);
+    std::frexp(hv, &c.fx_exp_hv);
+    c.fx_ok = std::isfinite(hv) && std::abs(c.fx_exp_v) < 200 && std::abs(c.fx_exp_hv) < 400;
+    auto fraction = [](double x) { return (uint64_t)std::nearbyint(std::ldexp(std::fabs(x), 63)); };   // |x| <= 1
+    for (int k = 1; k < 5 && c.fx_ok; ++k) {
+      c.fx_speed[k - 1] = fraction(std::ldexp(d.speeds[k], -c.fx_exp_v));
+      c.fx_half_v2[k - 1] = fraction(std::ldexp(g.half_v2[k], -c.fx_exp_hv));
+    }
+    for (int i = 0; i < nd / 2; ++i) {
+      const double phi = 2.0 * M_PI * i / nd;
+      c.fx_cx[i] = fraction(std::cos(phi));
+      c.fx_cy[i] = fraction(std::sin(phi));   // >= 0 in the first half
+      c.fx_neg_x |= (std::cos(phi) < 0.0 ? 1 : 0) << i;
     }
   }
   // the same velocities as DvmG (opposite directions exactly antisymmetric)

@@ -19,6 +19,11 @@ struct DvmG32 {
   float dv23h, dv23l, dh23h, dh23l;            // v_3 - v_2 and (v_3^2 - v_2^2) / 2
   float Fch[5][4], Fcl[5][4];                  // F_k(E) = sum_n Fc[k][n-1] E^n (Eq. 11a)
   float B0h, B0l;                              // F_0 = 1 - B0 sum_k F_k (Eq. 11b)
+  // For sums in integers (gen_state.cuh): v_k = fx_speed[k-1] 2^(fx_exp_v - 63), v_k^2 / 2
+  // = fx_half_v2[k-1] 2^(fx_exp_hv - 63), the unit vectors' |x| and y in 2^-63; fx_neg_x bit
+  // i: x < 0; fx_ok: the speeds are such that this holds.
+  uint64_t fx_speed[4], fx_half_v2[4], fx_cx[kMaxPairsG], fx_cy[kMaxPairsG];
+  int fx_exp_v, fx_exp_hv, fx_neg_x, fx_ok;
 };
 
 void fill_dvm_generic32(DvmG32& c, const pclb_dvm& d, const DvmG& g);

@@ -236,9 +236,8 @@ __global__ void __launch_bounds__(kNeqThreads)
 
 // The same for the N_i = 16 and 24 sets of Table I (Q = 65, 97, built to
 // reproduce the same equilibrium moments, Eqs. 6-9): the node's moments in
-// double, or in float-float for FP32 storage (one pass over its Q values), the
-// central moments in the storage type with the velocities of the set (float
-// tables for FP32).
+// double (FP32 storage: gen_state.cuh), the central moments in the storage type
+// with the velocities of the set (float tables for FP32).
 template <class T, int ND>
 __global__ void __launch_bounds__(kNeqThreads)
     noneq_gen_kernel(const T* __restrict__ f, T* __restrict__ out, int groups, const __grid_constant__ StepParams p,
@@ -252,10 +251,18 @@ __global__ void __launch_bounds__(kNeqThreads)
   double s0, uxd, uyd, E;
   if constexpr (sizeof(T) == 4) {
     const State32 m = gen_state32<ND>(fn, plane, c);
-    s0 = (double)m.rho.hi + m.rho.lo;
-    uxd = (double)m.ux.hi + m.ux.lo;
-    uyd = (double)m.uy.hi + m.uy.lo;
-    E = (double)m.E.hi + m.E.lo;
+    if (gen_in_range(m)) {
+      s0 = (double)m.rho.hi + m.rho.lo;
+      uxd = (double)m.ux.hi + m.ux.lo;
+      uyd = (double)m.uy.hi + m.uy.lo;
+      E = (double)m.E.hi + m.E.lo;
+    } else {
+      const GenState x = gen_state_f32<ND>(fn, plane, d, c);
+      s0 = x.rho;
+      uxd = x.ux;
+      uyd = x.uy;
+      E = x.E;
+    }
   } else {
     double sx = 0.0, sy = 0.0, se = 0.0;
     s0 = 0.0;

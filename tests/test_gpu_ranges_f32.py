@@ -1,0 +1,85 @@
+"""FP32 states of any magnitude: fields, integrals and initial states against the
+same expressions in extended precision on the host, from the FP32 values
+themselves.
+
+Every one of these is defined by sums that the library forms to double
+precision or better, so a float result may differ by its own rounding (2^-24)
+and a double one by a few roundings of the sums.
+"""
+import math
+
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_1302_7104_gb300 import inputs as I
+from paper_1302_7104_gb300 import pclb as P
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+LD = np.longdouble
+HALF_ULP = 2.0 ** -24 * (1.0 + 1e-5)
+
+
+def _state(n_dirs, scale, n_r=70, n_t=30):
+    w = I.random_smooth(n_r, n_t, seed=3, n_dirs=n_dirs, n_f=n_dirs)
+    f = O.set_state(w) * (1.0 + 0.01 * np.random.default_rng(1).normal(size=(w.q, n_t, n_r)))
+    return w, (f * scale).astype(np.float32)
+
+
+def _moments(w, f):
+    """rho, j_x, j_y, e and the sums of |terms| of j_x."""
+    f = f.astype(LD)
+    rho, jx, jy, e, size = f.sum(0), 0, 0, 0, 0
+    for k in range(1, 5):
+        for i in range(w.n_dirs):
+            sgn, phi = (1.0 if i < w.n_dirs // 2 else -1.0), 2.0 * math.pi * (i % (w.n_dirs // 2)) / w.n_dirs
+            q = 1 + (k - 1) * w.n_dirs + i
+            vx, vy = LD(w.speeds[k] * sgn * math.cos(phi)), LD(w.speeds[k] * sgn * math.sin(phi))
+            jx, jy, size = jx + vx * f[q], jy + vy * f[q], size + abs(vx * f[q])
+            e = e + LD(0.5 * w.speeds[k] ** 2) * f[q]
+    return rho, jx, jy, e, size
+
+
+def _area(w):
+    dr, dth = (w.r_out - w.r_in) / (w.n_r - 1), 2.0 * math.pi * w.n_f / (w.n_dirs * w.n_theta)
+    return ((w.r_in + np.arange(w.n_r) * LD(dr)) * dr * dth)[None, :]
+
+
+SCALES = [1.0, 2.0 ** -100, 2.0 ** -120, 2.0 ** 121, 2.0 ** 124]
+
+
+@pytest.mark.parametrize("n_dirs", [16, 24])
+@pytest.mark.parametrize("scale", SCALES)
+def test_integrals_of_the_larger_sets_in_double(n_dirs, scale):
+    """Tolerance: 16 roundings (2^-53) of the sums of the terms' sizes."""
+    w, f = _state(n_dirs, scale)
+    with P.PCLB(w, precision="fp32") as g:
+        d = g.set_f(torch.as_tensor(f, device="cuda")).diagnostics()
+        assert g.status_flags() == 0
+    rho, jx, jy, e, size = _moments(w, f)
+    a, T = _area(w), (e - (jx * jx + jy * jy) / (2 * rho)) / rho
+    tol = 16.0 * 2.0 ** -53
+    assert abs(d[0] - (a * rho).sum()) <= tol * (a * rho).sum()
+    assert abs(d[1] - (a * jx).sum()) <= tol * (a * size).sum()
+    assert abs(d[2] - (a * jy).sum()) <= tol * (a * size).sum()
+    assert abs(d[3] - (a * e).sum()) <= tol * (a * e).sum()
+    assert d[4] == float(rho.min()) or abs(d[4] - rho.min()) <= tol * rho.min()
+    assert abs(d[5] - T.min()) <= tol * T.min()
+
+
+@pytest.mark.parametrize("n_dirs", [16, 24])
+@pytest.mark.parametrize("scale", SCALES)
+def test_fields_of_the_larger_sets_round_once(n_dirs, scale):
+    w, f = _state(n_dirs, scale)
+    with P.PCLB(w, precision="fp32") as g:
+        got = [x.cpu().numpy().astype(LD) for x in g.set_f(torch.as_tensor(f, device="cuda")).moments()]
+        assert g.status_flags() == 0
+    rho, jx, jy, e, size = _moments(w, f)
+    th = (np.arange(1, w.n_theta + 1) * (2.0 * math.pi * w.n_f / (w.n_dirs * w.n_theta)))[:, None]
+    c, s = np.cos(th), np.sin(th)
+    want = [rho, (jx * c + jy * s) / rho, (jy * c - jx * s) / rho, (e - (jx * jx + jy * jy) / (2 * rho)) / rho]
+    for x, y in zip(got, want):
+        room = 32.0 * 2.0 ** -53 * (size / rho)      # roundings of the sums
+        assert (abs(x - y) <= HALF_ULP * abs(y) + (room if y is not rho else 32.0 * 2.0 ** -53 * rho)).all()
