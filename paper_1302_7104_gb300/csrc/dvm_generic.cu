@@ -74,6 +74,25 @@ __global__ void __launch_bounds__(kGenThreads)
   if (temp) temp[n] = m.E;
 }
 
+// f^eq of one node in double, rounded once per label: fields outside the range of
+// the float-float form below.
+static __device__ __noinline__ void gen_set_node(float* f, const StepParams& p, const DvmG& d, int t, int r, double R,
+                                                 double ur, double ut, double E) {
+  const double c = p.cos_t[t], s = p.sin_t[t], ux = ur * c - ut * s, uy = ur * s + ut * c;
+  const double uxE = ux / E, uyE = uy / E, u2E = (ux * ux + uy * uy) / E;
+  const double a1 = 1.0 - 0.5 * u2E, a0 = a1 + 0.125 * u2E * u2E;
+  double Fs = 0.0;
+#pragma unroll 1
+  for (int q = 4 * d.n_dirs; q >= 0; --q) {   // the rest velocity last: F_0 = 1 - B0 (F_1 + .. + F_4)
+    const int k = d.shell[q];
+    const double F = k == 0 ? 1.0 - d.B0 * Fs
+                            : E * (d.Fc[k][0] + E * (d.Fc[k][1] + E * (d.Fc[k][2] + E * d.Fc[k][3])));
+    if (k > 0 && q == 1 + (k - 1) * d.n_dirs) Fs += F;
+    const double x = d.vx[q] * uxE + d.vy[q] * uyE;
+    gen_store<float>(f, p, d, q, t, r, (float)(R * F * (a0 + x * (a1 + x * (0.5 * a1 + x * (1.0 / 6.0 + x * (1.0 / 24.0)))))));
+  }
+}
+
 // FP32 storage: f = f^eq of the fields, evaluated in float-float and rounded
 // once per label.  Per node and shell the polynomial of Eq. (10) in x = v_k
 // y_i, y_i = c_i.u/E, is folded into w ev = A + y^2 (B + y^2 C) and w od = y
@@ -92,6 +111,12 @@ __global__ void __launch_bounds__(kGenThreads)
   const size_t n = (size_t)t * p.n_r + r;
   const ff R = ff_of(rho[n]), E = ff_of(temp[n]), ur = ff_of(u_r[n]), ut = ff_of(u_t[n]);   // E = T
   if (!(R.hi > 0.f && E.hi > 0.f)) atomicOr(p.status, PCLB_FLAG_NONPHYS);
+  // the low parts stay normal numbers or nearly so, and nothing overflows
+  if (!(R.hi >= 0x1p-60f && R.hi <= 0x1p+60f && E.hi >= 0x1p-20f && E.hi <= 0x1p+10f &&
+        ur.hi * ur.hi + ut.hi * ut.hi <= 256.f * E.hi)) {
+    gen_set_node(f, p, d, t, r, R.hi, ur.hi, ut.hi, E.hi);
+    return;
+  }
   const float4 cs = p.cs_ff[t];
   const ff co{cs.x, cs.y}, si{cs.z, cs.w};
   const ff ux = ff_add(ff_mul(ur, co), ff_neg(ff_mul(ut, si))), uy = ff_add(ff_mul(ur, si), ff_mul(ut, co));

@@ -83,3 +83,45 @@ def test_fields_of_the_larger_sets_round_once(n_dirs, scale):
     for x, y in zip(got, want):
         room = 32.0 * 2.0 ** -53 * (size / rho)      # roundings of the sums
         assert (abs(x - y) <= HALF_ULP * abs(y) + (room if y is not rho else 32.0 * 2.0 ** -53 * rho)).all()
+
+
+@pytest.mark.parametrize("n_dirs", [16, 24])
+@pytest.mark.parametrize("rho,T,u", [(1.0, 1.0, 0.3), (2.0 ** -100, 1.0, 0.3), (2.0 ** -124, 1.0, 0.3), (2.0 ** 100, 1.0, 0.3),
+                                     (2.0 ** 120, 0.5, 0.3), (1.0, 2.0 ** -40, 0.0), (2.0 ** -60, 2.0 ** -60, 0.0),
+                                     (1.0, 2.0 ** 25, 1.0), (1.0, 1e-3, 1.0)])
+def test_initial_states_of_the_larger_sets_round_once(n_dirs, rho, T, u):
+    """f^eq (Eqs. 10-11) of fields around (rho, T, u), label by label: half a
+    unit in the last place (of the smallest normal number below it), and 64
+    roundings of double on the shell's largest term."""
+    w = I.random_smooth(40, 20, seed=3, n_dirs=n_dirs, n_f=n_dirs)
+    rng = np.random.default_rng(2)
+    fields = [(np.asarray(x) * (1.0 + 0.1 * rng.random(w.rho.shape))).astype(np.float32) for x in (rho, u, -0.5 * u, T)]
+    with P.PCLB(w, precision="fp32") as g:
+        got = g.set_state(*[torch.as_tensor(x, device="cuda") for x in fields]).get_f().cpu().numpy().astype(LD)
+        assert g.status_flags() == 0
+    R, ur, ut, E = (x.astype(LD) for x in fields)
+    th = (np.arange(1, w.n_theta + 1) * (2.0 * math.pi * w.n_f / (w.n_dirs * w.n_theta)))[:, None]
+    c, s = np.cos(th), np.sin(th)
+    ux, uy = ur * c - ut * s, ur * s + ut * c
+    z = (ux * ux + uy * uy) / E
+    a1 = 1 - z / 2
+    a0 = a1 + z * z / 8
+    v2, Fs, sizes = [LD(v) ** 2 for v in w.speeds], 0, 0
+    for k in range(4, -1, -1):
+        if k:
+            a, b, e = (v2[j] for j in range(1, 5) if j != k)
+            den = v2[k] * (v2[k] - a) * (v2[k] - b) * (v2[k] - e)
+            terms = [w.B[1] * a * b * e, w.B[2] * (a * b + b * e + e * a), w.B[3] * (a + b + e), w.B[4]]
+            F = sum(t / den * E ** (n + 1) for n, t in enumerate(terms))
+            size = sum(abs(t / den) * E ** (n + 1) for n, t in enumerate(terms))
+            Fs, sizes = Fs + F, sizes + size
+        else:
+            F, size = 1 - w.B[0] * Fs, 1 + w.B[0] * sizes
+        for i in range(w.n_dirs if k else 1):
+            sgn, phi = (1.0 if i < w.n_dirs // 2 else -1.0), 2.0 * math.pi * (i % (w.n_dirs // 2)) / w.n_dirs
+            x = (w.speeds[k] * sgn * math.cos(phi) * ux + w.speeds[k] * sgn * math.sin(phi) * uy) / E
+            poly = a0 + x * (a1 + x * (a1 / 2 + x * (LD(1) / 6 + x / 24)))
+            room = 64.0 * 2.0 ** -53 * R * size * (1 + z + z * z + abs(x) ** 4)
+            want = R * F * poly
+            q = 1 + (k - 1) * w.n_dirs + i if k else 0
+            assert (abs(got[q] - want) <= np.maximum(HALF_ULP * abs(want), 2.0 ** -150) + room).all(), (k, i)
