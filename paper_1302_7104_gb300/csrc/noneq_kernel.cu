@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kNeqThreads)
   const float cs = (float)p.cos_t[t], sn = (float)p.sin_t[t];
   const f2 u_r = fma2(ux, bc2(cs), mul2(uy, bc2(sn))), u_t = fma2(uy, bc2(cs), neg2(mul2(ux, bc2(sn))));
 
-  // central moments of f (the sums with c.c, halved at the end)
+  // central moments of f
   f2 A[12];
 #pragma unroll
   for (int c = 0; c < 12; ++c) A[c] = bc2(0.f);
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kNeqThreads)
   for (int q = 0; q < kQ; ++q) {
     const f2 w = ld(q);
     const f2 cr = sub2(bc2(fmaf(d.vx[q], cs, d.vy[q] * sn)), u_r), ct = sub2(bc2(fmaf(d.vy[q], cs, -(d.vx[q] * sn))), u_t);
-    const f2 cc = fma2(cr, cr, mul2(ct, ct));
+    const f2 h = mul2(bc2(0.5f), fma2(cr, cr, mul2(ct, ct)));
     const f2 wr = mul2(w, cr), wt = mul2(w, ct);
     const f2 wrr = mul2(wr, cr), wrt = mul2(wr, ct), wtt = mul2(wt, ct);
     A[0] = add2(A[0], wrr);
@@ -183,18 +183,29 @@ __global__ void __launch_bounds__(kNeqThreads)
     A[4] = fma2(wrr, ct, A[4]);
     A[5] = fma2(wrt, ct, A[5]);
     A[6] = fma2(wtt, ct, A[6]);
-    A[7] = fma2(cc, wr, A[7]);
-    A[8] = fma2(cc, wt, A[8]);
-    A[9] = fma2(cc, wrr, A[9]);
-    A[10] = fma2(cc, wrt, A[10]);
-    A[11] = fma2(cc, wtt, A[11]);
+    A[7] = fma2(h, wr, A[7]);
+    A[8] = fma2(h, wt, A[8]);
+    A[9] = fma2(h, wrr, A[9]);
+    A[10] = fma2(h, wrt, A[10]);
+    A[11] = fma2(h, wtt, A[11]);
   }
-#pragma unroll
-  for (int c = 7; c < 12; ++c) A[c] = mul2(A[c], bc2(0.5f));
-  // central departures: minus the equilibrium's (rho E I, 0, 0, 2 rho E^2 I)
+  // central departures: minus the equilibrium's (rho E I, 0, 0, 2 rho E^2 I), in
+  // double where the float-float products have no room
   const ff2 rE = ff2_mul(st.rho, st.E), rE2 = ff2_scale(ff2_mul(rE, st.E), 2.f);
   auto less = [](f2 a, ff2 b) { return sub2(sub2(a, b.hi), b.lo); };
-  const f2 D0 = less(A[0], rE), D2 = less(A[2], rE), D9 = less(A[9], rE2), D11 = less(A[11], rE2);
+  f2 D0 = less(A[0], rE), D2 = less(A[2], rE), D9 = less(A[9], rE2), D11 = less(A[11], rE2);
+  auto room = [](float x, float y) { return x >= 0x1p-96f && y >= 0x1p-96f && x <= 0x1p+120f && y <= 0x1p+120f; };
+  if (!(room(rE.hi.x, rE2.hi.x) && room(rE.hi.y, rE2.hi.y))) {
+    auto exact = [](ff rho, ff E, float a0, float a2, float a9, float a11, float& d0, float& d2, float& d9, float& d11) {
+      const double R = (double)rho.hi + rho.lo, e = (double)E.hi + E.lo, x = R * e, y = 2.0 * R * e * e;
+      d0 = (float)(a0 - x);
+      d2 = (float)(a2 - x);
+      d9 = (float)(a9 - y);
+      d11 = (float)(a11 - y);
+    };
+    exact(ff{st.rho.hi.x, st.rho.lo.x}, ff{st.E.hi.x, st.E.lo.x}, A[0].x, A[2].x, A[9].x, A[11].x, D0.x, D2.x, D9.x, D11.x);
+    exact(ff{st.rho.hi.y, st.rho.lo.y}, ff{st.E.hi.y, st.E.lo.y}, A[0].y, A[2].y, A[9].y, A[11].y, D0.y, D2.y, D9.y, D11.y);
+  }
 
   const size_t nodes = (size_t)p.n_theta * p.n_r;
   float* o = out + (size_t)t * p.n_r + r;

@@ -125,3 +125,33 @@ def test_initial_states_of_the_larger_sets_round_once(n_dirs, rho, T, u):
             want = R * F * poly
             q = 1 + (k - 1) * w.n_dirs + i if k else 0
             assert (abs(got[q] - want) <= np.maximum(HALF_ULP * abs(want), 2.0 ** -150) + room).all(), (k, i)
+
+
+def test_manifestations_near_the_largest_float():
+    """The octagon's central manifestations at a power-of-two scale at which the
+    sums of Sec. IV, taken in float label by label, just stay finite: they are
+    finite, and those of the unscaled state to the few roundings by which the node's
+    velocity may differ (its reciprocal density has no room for a low part)."""
+    w, f = _state(8, 1.0, n_r=41, n_t=12)
+    with P.PCLB(w, precision="fp32") as g:
+        base = g.set_f(torch.as_tensor(f, device="cuda")).noneq(P.NEQ_MSTAR | P.NEQ_DSTAR).cpu().numpy()
+        rho, jx, jy, e, _ = _moments(w, f)
+        ux, uy = (jx / rho).astype(np.float32), (jy / rho).astype(np.float32)
+        peak, total, size = 0.0, np.zeros((12,) + f.shape[1:], np.float32), np.zeros((12,) + f.shape[1:])
+        th = (np.arange(1, w.n_theta + 1) * (2.0 * math.pi * w.n_f / (w.n_dirs * w.n_theta)))[:, None].astype(np.float32)
+        c, s = np.cos(th), np.sin(th)
+        for q in range(w.q):
+            k, i = (0, 0) if q == 0 else (1 + (q - 1) // 8, (q - 1) % 8)
+            vx, vy = np.float32(w.speeds[k] * math.cos(math.pi * i / 4)), np.float32(w.speeds[k] * math.sin(math.pi * i / 4))
+            cr, ct = (vx - ux) * c + (vy - uy) * s, (vy - uy) * c - (vx - ux) * s
+            h = np.float32(0.5) * (cr * cr + ct * ct)
+            for n, x in enumerate((cr * cr, cr * ct, ct * ct, cr ** 3, cr * cr * ct, cr * ct * ct, ct ** 3, h * cr, h * ct,
+                                   h * cr * cr, h * cr * ct, h * ct * ct)):
+                total[n] += f[q] * x
+                size[n] += np.abs(f[q] * x)
+            peak = max(peak, np.abs(total).max())
+        scale = 2.0 ** (127 - math.floor(math.log2(1.02 * peak)))
+        got = g.set_f(torch.as_tensor((f * np.float32(scale)), device="cuda")).noneq(P.NEQ_MSTAR | P.NEQ_DSTAR).cpu().numpy()
+    assert np.isfinite(got).all()
+    for g in (0, 1):   # 2^-20 of the terms' size
+        assert (np.abs(got[g] / scale - base[g]) <= 2.0 ** -20 * size).all()
