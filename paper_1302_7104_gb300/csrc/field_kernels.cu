@@ -203,6 +203,18 @@ __global__ void diag_partial_kernel(const double* __restrict__ f, double* partia
   diag_block_reduce(acc, mn, partials);
 }
 
+// The moments rho, j, e of `rows` nodes of a column added up in double.
+__device__ __noinline__ void column_sums_double(const float* f, size_t plane, int pitch, int rows,
+                                                const DvmConst<float>& d, double v[4]) {
+  v[0] = v[1] = v[2] = v[3] = 0.0;
+  for (int t = 0; t < rows; ++t) {
+    ff m[4];
+    const State32 st = state32(f + (size_t)t * pitch, plane, d, m);
+    const float bad[4] = {0.f, st.ux.hi - st.ux.hi, st.uy.hi - st.uy.hi, st.E.hi - st.E.hi};   // NaN as in the kernel
+    for (int i = 0; i < 4; ++i) v[i] += (double)m[i].hi + m[i].lo + bad[i];
+  }
+}
+
 // FP32: the same integrals from the raw float-float moments (rho, j, e =
 // rho (E + u^2/2)), without FP64 work per node: a thread adds up to `rows`
 // nodes of one column in float-float and enters the double sums once, weighted
@@ -238,8 +250,14 @@ __global__ void __launch_bounds__(kDiagThreads32, 2)
     }
     any = true;
     const double w = (r_in + r * dr) * dr * dth;
+    double v[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) acc[i] += w * ((double)s[i].hi + s[i].lo);
+    for (int i = 0; i < 4; ++i) v[i] = (double)s[i].hi + s[i].lo;
+    // the rows' moments may be floats and their sums not
+    if (!(isfinite(s[0].hi) && isfinite(s[1].hi) && isfinite(s[2].hi) && isfinite(s[3].hi)))
+      column_sums_double(f + (size_t)(t0 + kGhostRows) * p.pitch + r, plane, p.pitch, t1 - t0, d, v);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i] += w * v[i];
   }
   const double mn[2] = {any && mh[0] < FLT_MAX ? (double)mh[0] + ml[0] : DBL_MAX,
                         any && mh[1] < FLT_MAX ? (double)mh[1] + ml[1] : DBL_MAX};

@@ -155,3 +155,18 @@ def test_manifestations_near_the_largest_float():
     assert np.isfinite(got).all()
     for g in (0, 1):   # 2^-20 of the terms' size
         assert (np.abs(got[g] / scale - base[g]) <= 2.0 ** -20 * size).all()
+
+
+def test_integrals_near_the_largest_float():
+    """The octagon's integrals where each node's moments are finite floats but a
+    few of them together are not: those of the unscaled state, to the rounding of
+    the sums (the grid is large enough for several rows per thread)."""
+    w = I.random_smooth(1024, 1300, seed=3)
+    with P.PCLB(w, precision="fp32") as g:
+        f = g.set_state().get_f()
+        base = g.diagnostics()
+        scale = 2.0 ** 125
+        got = g.set_f(f * scale).diagnostics()
+        assert g.status_flags() == 0
+    assert np.isfinite(got).all()
+    assert np.abs(got[:6] / scale ** np.array([1, 1, 1, 1, 1, 0]) - base[:6]).max() <= 1e-6 * base[0]
