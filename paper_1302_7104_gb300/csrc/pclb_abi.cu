@@ -74,7 +74,7 @@ namespace {
 
 thread_local char g_err[512] = "";
 constexpr int kDefaultTimeoutMs = 120000;
-constexpr int kSpinUs = 2000;   // bounded_sync polls without pause this long
+constexpr int kSpinUs = 2000;   // bounded_sync polls without sleeping this long
 
 struct HostCtx : pclb_ctx {
   std::vector<double> cos_t, sin_t, inv_r, bc_vals;
@@ -355,7 +355,7 @@ pclb_status bounded_sync(pclb_ctx* ctx, int timeout_ms) {
   }
   const auto t0 = std::chrono::steady_clock::now();
   pclb_status st = PCLB_OK;
-  int sleep_us = 1;
+  int sleep_us = 1, polls = 0;
   while (true) {
     e = cudaEventQuery(ev);
     if (e == cudaSuccess) break;
@@ -368,9 +368,14 @@ pclb_status bounded_sync(pclb_ctx* ctx, int timeout_ms) {
       st = fail(ctx, PCLB_ETIMEOUT, "stream did not finish within %d ms", timeout_ms);
       break;
     }
-    // Short waits poll without a pause: the shortest sleep costs the host
-    // ~55 us, as long as a whole kernel here.
-    if (waited < std::chrono::microseconds(kSpinUs)) continue;
+    // Short waits poll without a sleep, the shortest of which costs the host
+    // ~55 us, as long as a whole kernel here; every few polls offer the core to
+    // other threads (a wait that held on took a third of it from a thread
+    // computing there).
+    if (waited < std::chrono::microseconds(kSpinUs)) {
+      if (++polls % 16 == 0) std::this_thread::yield();
+      continue;
+    }
     std::this_thread::sleep_for(std::chrono::microseconds(sleep_us));
     if (sleep_us < 20) sleep_us *= 2;
   }
