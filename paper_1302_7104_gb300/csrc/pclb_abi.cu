@@ -74,7 +74,8 @@ namespace {
 
 thread_local char g_err[512] = "";
 constexpr int kDefaultTimeoutMs = 120000;
-constexpr int kSpinUs = 2000;   // bounded_sync polls without sleeping this long
+constexpr int kSpinUs = 2000;   // bounded_sync polls without sleeping this long,
+constexpr int kYieldUs = 50;    // offering the core to other threads this often
 
 struct HostCtx : pclb_ctx {
   std::vector<double> cos_t, sin_t, inv_r, bc_vals;
@@ -355,7 +356,8 @@ pclb_status bounded_sync(pclb_ctx* ctx, int timeout_ms) {
   }
   const auto t0 = std::chrono::steady_clock::now();
   pclb_status st = PCLB_OK;
-  int sleep_us = 1, polls = 0;
+  int sleep_us = 1;
+  std::chrono::steady_clock::duration offered{0};
   while (true) {
     e = cudaEventQuery(ev);
     if (e == cudaSuccess) break;
@@ -369,11 +371,14 @@ pclb_status bounded_sync(pclb_ctx* ctx, int timeout_ms) {
       break;
     }
     // Short waits poll without a sleep, the shortest of which costs the host
-    // ~55 us, as long as a whole kernel here; every few polls offer the core to
-    // other threads (a wait that held on took a third of it from a thread
-    // computing there).
+    // ~55 us, as long as a whole kernel here; they offer the core to other threads
+    // every kYieldUs (a wait that held on took a third of it from a thread
+    // computing there; an offer every 16 polls cost a wait ~5 us).
     if (waited < std::chrono::microseconds(kSpinUs)) {
-      if (++polls % 16 == 0) std::this_thread::yield();
+      if (waited >= offered + std::chrono::microseconds(kYieldUs)) {
+        std::this_thread::yield();
+        offered = std::chrono::steady_clock::now() - t0;
+      }
       continue;
     }
     std::this_thread::sleep_for(std::chrono::microseconds(sleep_us));

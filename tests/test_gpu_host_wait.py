@@ -33,9 +33,9 @@ def _share(work, seconds=0.4):
 
 
 def test_short_waits_leave_the_core_to_other_threads():
-    """Waits of up to ~2 ms poll instead of sleeping; every few polls offer the
-    core, so a thread that computes there keeps most of it (half to two thirds,
-    if the wait held on).  The best of three runs, as the machine may be busy."""
+    """Waits of up to ~2 ms poll instead of sleeping; every now and then they offer
+    the core, so a thread that computes there keeps nearly all of it (0.69, if
+    the wait held on).  The best of three runs, as the machine may be busy."""
     if not hasattr(os, "sched_setaffinity"):
         pytest.skip("no affinity calls")
     w = I.kh(n_r=2048, n_theta=2048)
