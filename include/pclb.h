@@ -50,7 +50,10 @@
  * node's state from the same float-float moments, rounded to float, and
  * evaluates the cotangents in float (the ghost states at the walls in
  * double).  PCLB_FP64 keeps double precision throughout; its step forms sums,
- * differences and convection increments in 64-bit fixed point.
+ * differences and convection increments in 64-bit fixed point, rounded to units of
+ * 2^-58 of the largest value that enters (of a stencil, or of a shell in a
+ * tile), where that is no coarser than the rounding of double arithmetic at the node,
+ * and in double elsewhere.
  */
 #ifndef PCLB_H
 #define PCLB_H

@@ -41,8 +41,8 @@
 // TT = 8 rows, one thread per node; on grids whose tiles would leave SMs idle
 // 4 rows and two threads per node (LS = 2), one label of each pair each, or 2
 // rows and four threads (LS = 4), which also work on two pairs at a time (half
-// the barriers): 64 x 128, 72.5 us per adjoint step with LS = 4, 102 with LS = 2,
-// 150 with 8 rows.
+// the barriers): 64 x 128, 73.3 us per adjoint step with LS = 4, 103 with LS = 2,
+// 154 with 8 rows.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -81,7 +81,7 @@ template <int TT, int LS>
 struct AdjSize {
   static constexpr int threads = 32 * TT * LS;
   static constexpr int pp = LS == 4 ? 2 : 1;   // pairs at a time
-  static constexpr int min_blocks = 2;   // what shared memory allows
+  static constexpr int min_blocks = 2;   // what shared memory allows with 8 rows, and 124 registers with fewer
   static constexpr int plane = kWinR * (TT + 4);
   static constexpr int npairs = 4 * kNDirs / 2;
   // products of one label: radial A, B over TT rows x 36 columns (tile

@@ -182,17 +182,6 @@ __device__ __forceinline__ float feq32(const Eq32& e, const DvmConst<float>& d, 
   return k == 0 ? e.w[0] * e.a0 : feq32_weighted(e, d, e.w[k], k, i, sign);
 }
 
-// Node state from given fields (rho, Cartesian u, E = T).
-__device__ __forceinline__ State32 state32_from_fields(float rho, float ux, float uy, float E) {
-  State32 s;
-  s.rho = ff_of(rho);
-  s.ux = ff_of(ux);
-  s.uy = ff_of(uy);
-  s.E = ff_of(E);
-  s.ok = rho > 0.f && E > 0.f;
-  return s;
-}
-
 // Node state (rho, u_x, u_y, E) in double for the global diagnostics, from the
 // FP32 path's float-float moments or the FP64 path's plain sums.
 __device__ __forceinline__ void node_state_double(const float* f, size_t plane, const DvmConst<float>& d,

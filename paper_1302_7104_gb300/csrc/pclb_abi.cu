@@ -163,7 +163,7 @@ Layout make_layout(const pclb_grid* g, const pclb_dvm* d, pclb_precision prec) {
   L.stage = off; off = align_up(off + (size_t)8 * g->n_r * g->n_theta * es, 256);
   L.adj_scratch = off; off = align_up(off + adjoint_scratch_bytes(g->n_theta, (int)es), 256);
   L.gen_ghost = off;
-  if (d->n_dirs != kNDirs) off = align_up(off + 4 * (size_t)g->n_theta * Q * es, 256);
+  if (d->n_dirs != kNDirs && prec == PCLB_FP64) off = align_up(off + 4 * (size_t)g->n_theta * Q * es, 256);
   L.total = off;
   return L;
 }
@@ -313,7 +313,7 @@ pclb_status encode_map(pclb_ctx* ctx, const void* base, int box_rows, CUtensorMa
 
 int adj_box_rows(const pclb_ctx* ctx) { return ctx->sp.adj_rows + 4; }
 
-// Tile rows of the adjoint: 16 in FP32; in FP64 8, or 4 on small grids.
+// Tile rows of the adjoint: 16 in FP32; in FP64 8, or 4 or 2 on small grids.
 int adj_tile_rows(const pclb_grid* g, pclb_precision prec) {
   if (prec == PCLB_FP32) return kAdjRows32;
   const long long tiles = (long long)((g->n_r + kTileR - 1) / kTileR) * ((g->n_theta + kAdjRows64 - 1) / kAdjRows64);

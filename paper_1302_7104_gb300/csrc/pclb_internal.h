@@ -31,9 +31,9 @@ constexpr int kCtasPerSm32 = 2;
 // The octagon's steps on small grids: tiles of kTileTSmall rows on at most
 // kSmallGridTiles tiles of 32 x 16 (two waves of the 152 SMs), in FP64 of two
 // rows on at most kTinyGridTiles64 (one wave).  FP64, us per step with tiles
-// of 2 / 4 / 16 rows: 64 x 128 (16 tiles) 15.1 / 22.3 / 52.4, 64 x 256 (32)
-// 30.0 / 22.5 / 52.6, 128 x 304 (76) 59.6 / 44.5 / 52.6, 128 x 608 (152)
-// 112 / 88.6 / 53.6.  FP32, us per step with 4 / 16: 64 x 128 7.5 / 13.1, 64 x
+// of 2 / 4 / 16 rows: 64 x 128 (16 tiles) 16.5 / 24.2 / 54.0, 64 x 256 (32)
+// 32.5 / 24.5 / 54.1, 128 x 304 (76) 65.2 / 48.5 / 53.7, 128 x 608 (152)
+// 123 / 96.7 / 55.0.  FP32, us per step with 4 / 16: 64 x 128 7.5 / 13.1, 64 x
 // 608 (76) 8.9 / 13.3, 128 x 400 (100) 15.0 / 13.5.
 constexpr int kTileTSmall = 4;
 constexpr int kSmallGridTiles = 76, kTinyGridTiles64 = 19;
@@ -45,12 +45,13 @@ constexpr int kGhostRows = 2;       // azimuthal ghost rows stored on each side
 constexpr int kAdjRows32 = 16;
 constexpr int kAdjRows64 = 8;
 constexpr int kAdjRows64Small = 4;    // FP64 on grids of at most kSmallGridTilesAdj tiles of 8 rows
-// us per adjoint step with tiles of 4 / 8 rows: 64 x 304 (76 tiles of 8) 102 /
-// 150, 128 x 304 (152) 155 / 150, 128 x 400 (200) 212 / 252, 128 x 608 (304) 279 /
-// 254: up to three of the small ones to an SM (152).
+// us per adjoint step with tiles of 4 / 8 rows: 64 x 304 (76 tiles of 8) 104 /
+// 154, 128 x 304 (152) 157 / 154, 128 x 400 (200) 213 / 256, 128 x 608 (304) 281 /
+// 258: up to three of the small ones per SM (152 SMs, two at a time).  With
+// more than 152 of the large ones some SMs hold two and take as long as 304 do.
 constexpr int kSmallGridTilesAdj = 228;
 // 2 rows on at most kTinyGridTilesAdj (one of their blocks to an SM): 64 x 152
-// (38) 72.6 us against 102 with 4 rows, 64 x 304 (76) 103 against 101.
+// (38) 73.4 us against 104 with 4 rows, 64 x 304 (76) 104 against 104.
 constexpr int kAdjRows64Tiny = 2;
 constexpr int kTinyGridTilesAdj = 38;
 // Time a kernel waits for the TMA copies of its own window (mbarrier phase)
@@ -137,7 +138,7 @@ struct Layout {
   size_t diag_out;            // double [8]
   size_t stage;               // host-I/O staging: 8 fields [n_theta][n_r]
   size_t adj_scratch;         // the adjoint's wall scratch (adjoint_walls.cuh)
-  size_t gen_ghost;           // N_i = 16, 24: radial ghost values [side][layer][n_theta][Q]
+  size_t gen_ghost;           // N_i = 16, 24, FP64: radial ghost values [side][layer][n_theta][Q]
   size_t total;
 };
 
@@ -181,7 +182,9 @@ inline cudaError_t launch_overlapped(void (*fn)(P...), dim3 grid, int threads, i
 // Its blocks are placed while the step before it still holds most SMs, and
 // would pile up on the free ones; where there is an SM for each (152), they ask
 // for more than half of one.  A step and an adjoint step, without and with: FP64
-// 64 x 128 172 and 119 us, 64 x 256 180 and 127; FP32 128 x 304 68.6 and 52.6.
+// 64 x 128 121 and 92 us, 64 x 256 182 and 129; FP32 128 x 304 69.6 and 51.6.
+// Contexts on streams of their own lose nothing by it (adjoint steps of four, FP64
+// 64 x 128: 60 us each, FP32 128 x 304: 14.4).
 inline int adjoint_smem(int smem, int blocks) { return blocks <= 152 && smem < kOwnSmBytes ? kOwnSmBytes : smem; }
 
 size_t adjoint_scratch_bytes(int n_theta, int elem);
