@@ -9,7 +9,7 @@
 // share the directions (H / 4 of the H pairs each, over the four shells), a fifth
 // forms the states from their sums while they convect.  On small grids this
 // also gives every node four threads.
-// N_i = 16, 512 x 512: 388 us per step (1639 before, one thread per node and all
+// N_i = 16, 512 x 512: 379 us per step (1639 before, one thread per node and all
 // of it in FP64); 64 x 64: 33 us (236, of which 150 the ghosts, one thread per wall
 // row; now a warp per row).
 #include <cuda_runtime.h>

@@ -126,8 +126,8 @@ __device__ __forceinline__ FxCourant fx_courant(uint64_t alpha) {
 
 // M of Eq. (28) in upwind form, |D|, |Dp| < 2^60.  v is formed to ~2^-46: a
 // float quotient rounded to i0 2^-23, its exact integer remainder, and the
-// remainder's float quotient; 2 K v is then good to K 2^-45 + 2^-62.  Where D = 0 the quotients may be anything (0 / 0):
-// the result is c |D| = 0 in integers.
+// remainder's float quotient; 2 K v is then good to K 2^-45 + 2^-62.  Where D = 0
+// the quotients may be anything (0 / 0): the result is c |D| = 0 in integers.
 __device__ __forceinline__ int64_t fx_mwb(int64_t D, int64_t Dp, const FxCourant& c) {
   const int64_t s = D >> 63;
   const uint64_t a = (uint64_t)((D ^ s) - s), n = a + fx_abs(Dp);
@@ -140,7 +140,7 @@ __device__ __forceinline__ int64_t fx_mwb(int64_t D, int64_t Dp, const FxCourant
   const float q = fx_float(rem) * r;                                        // the rest of v, units of 2^-23
   const float k = fmaf(c.k2, q, c.klo * v0);                                // the rest of 2 K v, units of 2^-52
   const int32_t i1 = __float2int_rn(k);
-  // and what i1 rounds off, units of 2^-63 (a D far larger than the node's own value, times 2^-53, is not small beside it)
+  // and what i1 rounds off, units of 2^-63 (2^-53 of a D far larger than the node's own value is not small beside it)
   const int32_t i2 = __float_as_int(fmaf(k - __int2float_rn(i1), 2048.0f, 12582912.0f)) - 0x4b400000;
   const uint64_t coef = c.a2 + c.k40 * (uint64_t)i0 + (uint64_t)((int64_t)i1 * 2048 + i2);
   return fx_signed(fx_mul(a, coef), s);
@@ -264,6 +264,14 @@ __device__ __forceinline__ double increment64(double a, double x0, double u1, do
   return a * D + 0.5 * (SCH == PCLB_SCHEME_WB ? K : a) * (D - Dp);
 }
 
+// fx_carried from doubles; a call, as it is rare and long (within the loop, N_i =
+// 24 on 1024 x 1024 took 2.09 ms a step against 2.02).
+template <int SCH>
+__device__ __noinline__ double carried64(double x0, double u1, double u2, double v1, double v2, double decay, double ar,
+                                         double at) {
+  return fma(decay, x0, -increment64<SCH>(ar, x0, u1, u2, u2)) - increment64<SCH>(at, x0, v1, v2, v2);
+}
+
 // d x0 - M_r - M_theta of one label (Eqs. 19, 28): x0 the node, u1 and v1 its
 // upwind neighbours in r and theta, u2 and v2 the next ones (Lax-Wendroff: the
 // downwind neighbours).  In fixed point on the exponent of the largest of
@@ -276,7 +284,7 @@ __device__ __forceinline__ double fx_carried(double x0, double u1, double u2, do
   const int e = fx_exponent(__double2hiint(x0), __double2hiint(u1), __double2hiint(u2), __double2hiint(v1),
                             __double2hiint(v2));
   if (!fx_range(e) || fx_exponent(__double2hiint(x0)) < e - 5) {
-    return fma(decay, x0, -increment64<SCH>(c[0], x0, u1, u2, u2)) - increment64<SCH>(c[2] * inv_r, x0, v1, v2, v2);
+    return carried64<SCH>(x0, u1, u2, v1, v2, decay, c[0], c[2] * inv_r);
   }
   const int64_t i0 = fx_from_double(x0, e);
   auto M = [&](double n1, double n2, const FxCoef<SCH>& k) {

@@ -31,9 +31,9 @@ constexpr int kCtasPerSm32 = 2;
 // The octagon's steps on small grids: tiles of kTileTSmall rows on at most
 // kSmallGridTiles tiles of 32 x 16 (two waves of the 152 SMs), in FP64 of two
 // rows on at most kTinyGridTiles64 (one wave).  FP64, us per step with tiles
-// of 2 / 4 / 16 rows: 64 x 128 (16 tiles) 16.5 / 24.2 / 54.0, 64 x 256 (32)
-// 32.5 / 24.5 / 54.1, 128 x 304 (76) 65.2 / 48.5 / 53.7, 128 x 608 (152)
-// 123 / 96.7 / 55.0.  FP32, us per step with 4 / 16: 64 x 128 7.5 / 13.1, 64 x
+// of 2 / 4 / 16 rows: 64 x 128 (16 tiles) 16.4 / 24.2 / 53.2, 64 x 256 (32)
+// 32.5 / 24.5 / 53.3, 128 x 304 (76) 65.2 / 48.5 / 53.3, 128 x 608 (152)
+// 123 / 96.7 / 54.2.  FP32, us per step with 4 / 16: 64 x 128 7.5 / 13.1, 64 x
 // 608 (76) 8.9 / 13.3, 128 x 400 (100) 15.0 / 13.5.
 constexpr int kTileTSmall = 4;
 constexpr int kSmallGridTiles = 76, kTinyGridTiles64 = 19;

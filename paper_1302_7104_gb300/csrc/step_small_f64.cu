@@ -15,7 +15,7 @@
 //     (Sec. II C 1) from the same sums; the pair warps turn them into values.
 // 100 x 20 with non-equilibrium walls: 16.8 us per step (206 us with all of it in
 // FP64 and the ghost columns row by row; 15.4 us with conversions and products
-// that dropped what is below a unit); 64 x 128: 16.5 us.
+// that dropped what is below a unit); 64 x 128: 16.4 us.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(SmSize<SCH, TT>::threads, 1)
     bar_wait(kBarGhosts, n_values);
   }
   // d f - M_r - M_theta of this thread's labels, kept in shared memory so that the loop
-  // stays rolled (unrolled, the compared schemes took 13% more on 64 x 64, now 16.5 us a step)
+  // stays rolled (unrolled, the compared schemes took 13% more on 64 x 64, now 16.3 us a step)
   double* mine = kept + tid;
   const uint64_t dfx = fx_fraction(fabs(decay));
   const int64_t dsign = decay < 0.0 ? -1 : 0;
