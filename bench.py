@@ -26,6 +26,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import subprocess
 import sys
 import threading
@@ -90,12 +91,18 @@ _KERNEL_SOURCES = {
 }
 
 
+def _code_only(text: str) -> str:
+    """C++ source without its comments and with every run of white space as one blank."""
+    text = re.sub(r"//[^\n]*|/\*.*?\*/", " ", text, flags=re.S)
+    return " ".join(text.split())
+
+
 def _kernel_hash(tag: str = "fp32") -> str:
-    """Hash of the sources of the FP32 ("fp32") or FP64 ("fp64") step kernel."""
+    """Hash of the code (comments aside) of the FP32 ("fp32") or FP64 ("fp64") step kernel's sources."""
     h = hashlib.sha256()
     for rel in _KERNEL_SOURCES[tag]:
-        with open(os.path.join(ROOT, rel), "rb") as fh:
-            h.update(fh.read())
+        with open(os.path.join(ROOT, rel), encoding="utf-8") as fh:
+            h.update(_code_only(fh.read()).encode())
     return h.hexdigest()[:16]
 
 
